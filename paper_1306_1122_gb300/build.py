@@ -32,8 +32,7 @@ UNITS = {
     "pairsum_f32_nv.cu": [],
     "pairsum_f32_split.cu": [],
     "pairsum_f64.cu": [],
-    "pairsum_ff.cu": [],
-    "pairsum_dif.cu": [],
+    "pairsum_re.cu": [],
     "vjp.cu": [],
     "noalloc.cu": [],
     "pxe.cu": [],

@@ -16,9 +16,6 @@
 
 using namespace dbie;
 
-#ifndef DBIE_FF_SPLIT_TARGET_PCT
-#define DBIE_FF_SPLIT_TARGET_PCT 200   // the same for the float-float re-evaluation pass
-#endif
 #ifndef DBIE_SPLIT_TARGET_PCT
 #define DBIE_SPLIT_TARGET_PCT 200
 #endif
@@ -77,27 +74,26 @@ struct Misc {
   int32_t work;
   int32_t near_cnt;
   int32_t bad;
-  int32_t pad[2];
+  int32_t zero;             // an empty queue's count
+  int32_t pad;
+  PlanHdr plan2;            // an empty queue's plan
 };
 
 struct SolveBufs {
   DBuf probs, ppos, lam0, sd, si, q_cnt_pass, item_off, ctrl, out, res, codes, corr;
   DBuf qpos[2], qlam[2], q_cnt[2], act[2], near[2];
-  DBuf msc, fout, fq_cnt_pass, fitem_off;            // certified decisions
-  DBuf fpos[2], flam[2], fq_cnt[2], ref[2];
-  DBuf dout, dq_cnt_pass, ditem_off;                  // its difference level
-  DBuf dpos[2], dlam[2], dlam0[2], dq_cnt[2];
+  DBuf msc, fout, fpos[2], flam[2], ref[2];           // certified decisions
+  DBuf dout, dpos[2], dlam[2], dlam0[2];              // its difference level
   cudaGraphExec_t exec = nullptr;
   std::vector<unsigned char> key;   // launch arguments the cached graph was captured with
   std::vector<cudaEvent_t> ev;      // profiling events inside the graph (6 per round)
   void release() {
     for (DBuf* b : {&probs, &ppos, &lam0, &sd, &si, &q_cnt_pass, &item_off, &ctrl, &out, &res,
-                    &codes, &corr, &msc, &fout, &fq_cnt_pass, &fitem_off, &dout, &dq_cnt_pass,
-                    &ditem_off})
+                    &codes, &corr, &msc, &fout, &dout})
       b->release();
     for (int s = 0; s < 2; ++s)
       for (DBuf* b : {&qpos[s], &qlam[s], &q_cnt[s], &act[s], &near[s], &fpos[s], &flam[s],
-                      &fq_cnt[s], &ref[s], &dpos[s], &dlam[s], &dlam0[s], &dq_cnt[s]})
+                      &ref[s], &dpos[s], &dlam[s], &dlam0[s]})
         b->release();
     if (exec) cudaGraphExecDestroy(exec);
     exec = nullptr;
@@ -117,17 +113,15 @@ struct SolveCtrl {
   int32_t pad;
   unsigned long long stat_queries;
   double stat_pairs;
-  // certified decisions: the float-float re-evaluation pass of each round
-  PlanHdr fplan;
-  int32_t fwork;
-  int32_t ref_cnt[2];
+  // certified decisions: the re-evaluation pass of each round (float-float and differences)
+  PlanHdr fplan, dplan, noplan;
+  int32_t rework[2];        // item counters of the pass (two launches while profiling)
+  int32_t zero;             // an empty queue's count
   int32_t pad2;
+  int32_t ref_cnt[2];
+  int32_t f_cnt[2], d_cnt[2];
   unsigned long long stat_ties;
   double stat_ff_pairs;
-  // and its difference level
-  PlanHdr dplan;
-  int32_t dwork;
-  int32_t pad3;
   unsigned long long stat_difs;
   double stat_dif_pairs;
 };
@@ -175,6 +169,7 @@ struct dbie_ctx {
   DBuf st_in, st_out, st_aux;     // host-memory staging
   DBuf qpos, qlam, near_list, out, ptiles;
   DBuf qlam0, dmsc;                // dbie_eval_difference: reference lambdas, bound sums
+  DBuf sctab;                     // sine and cosine table of the float-float kernels
   DBuf trace;                     // DBIE_TRACE_ITEMS builds: item timeline of the last pass
   int64_t trace_items = 0;
   DBuf tv32, tv64, probv;         // noise-variance tiles and their problem descriptor
@@ -314,6 +309,24 @@ dbie_status launch_kernel(const KernelRef& k, int grid, void* args, cudaStream_t
   return DBIE_OK;
 }
 
+// A pair-sum launch of a single call, between events while profiling is on.
+dbie_status timed_launch(dbie_ctx* c, const KernelRef& k, int grid, void* args, double pairs,
+                         cudaStream_t s) {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (c->profiling) {
+    e0 = take_event(c);
+    e1 = take_event(c);
+    CUDA_TRY(cudaEventRecord(e0, s));
+  }
+  DBIE_TRY(launch_kernel(k, grid, args, s));
+  if (c->profiling) {
+    CUDA_TRY(cudaEventRecord(e1, s));
+    c->pending.push_back({e0, e1});
+    c->pending_pairs.push_back(pairs);
+  }
+  return DBIE_OK;
+}
+
 int var_of(bool grad, bool dlam) {
   return grad ? (dlam ? VAR_OBJL : VAR_OBJ) : (dlam ? VAR_VL : VAR_V);
 }
@@ -326,6 +339,44 @@ KernelRef g1_ref(dbie_ctx* c, int var, bool tied, bool fp64, int rows = -1) {
   return g1_ref_f32(var, tied, c->cfg[var][tied ? 1 : 0], r);
 }
 
+// Float-float sums of n queries of this context, or with lam_ref (float64, as lam) the
+// difference sums between the two lambdas.  Results are in c->out, described by c->misc, as a
+// pass of one query per item.
+dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float* d_xyz,
+                        const float* d_lamf, const double* d_lamd, const double* lam_ref,
+                        cudaStream_t s) {
+  Misc* m = c->misc.as<Misc>();
+  const bool dif = lam_ref != nullptr;
+  if (dif)
+    launch_pack_eval(n, d_xyz, nullptr, lam_ref, c->qpos.as<float4>(), c->qlam0.as<Lam4>(),
+                     nullptr, nullptr, 0, 0.0, s);
+  launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(), nullptr,
+                   nullptr, 0, 0.0, s);
+  const KernelRef k = reeval_ref(var, tied, dif);
+  const int grid = persistent_grid(k, c->device);
+  const int64_t items = reeval_items(n, grid);
+  if (items > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
+  const int nsum = 3 * nsum_per_comp(var);
+  DBIE_TRY(ensure(c->out, sizeof(double) * items * nsum));
+  launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, 0, 1, 1, (int)n, s);
+  CUDA_TRY(cudaMemsetAsync(&m->zero, 0, sizeof(int32_t), s));
+  const ReList list{m->q_cnt, c->qpos.as<float4>(), c->qlam.as<Lam4>(),
+                    dif ? c->qlam0.as<Lam4>() : nullptr, c->out.as<double>(), &m->plan};
+  ReList none = list;
+  none.cnt = &m->zero;
+  none.plan = &m->plan2;
+  ReArgs a{};
+  a.probs = c->prob.as<ProbDesc>();
+  a.f = dif ? none : list;
+  a.d = dif ? list : none;
+  a.work = &m->work;
+  a.sctab = c->sctab.as<float4>();
+  a.rows = c->ntiles * RE_ROWS_PER_TILE;
+  DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
+  CUDA_TRY(cudaGetLastError());
+  return DBIE_OK;
+}
+
 // One pair-sum pass over n queries of this context (single problem): pack, plan, sweep,
 // near-field correction.  Results are in c->out as item chunks described by c->misc.
 dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, int64_t n,
@@ -334,13 +385,14 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   Misc* m = c->misc.as<Misc>();
   DBIE_TRY(ensure(c->qpos, sizeof(float4) * n));
   DBIE_TRY(ensure(c->qlam, sizeof(Lam4) * n));
+  if (ffp) return pass_reeval(c, var, tied, n, d_xyz, d_lamf, nullptr, nullptr, s);
   // (the noise variance sums positive terms: FP32 is accurate there without a near field)
-  const bool near_on = !fp64 && !ffp && o.near_z > 0 && var != VAR_NV;
+  const bool near_on = !fp64 && o.near_z > 0 && var != VAR_NV;
   if (near_on) DBIE_TRY(ensure(c->near_list, sizeof(int32_t) * n));
   CUDA_TRY(cudaMemsetAsync(&m->near_cnt, 0, sizeof(int32_t), s));
   launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(),
                    c->near_list.as<int32_t>(), &m->near_cnt, near_on ? 1 : 0, o.near_z, s);
-  const KernelRef k = ffp ? g1_ref_ff(var, tied) : g1_ref(c, var, tied, fp64);
+  const KernelRef k = g1_ref(c, var, tied, fp64);
   const int grid = persistent_grid(k, c->device);
   const int64_t nblk = (n + k.qper - 1) / k.qper;
   const int64_t target = std::max<int64_t>(1, (int64_t)grid * DBIE_SPLIT_TARGET_PCT / 100);
@@ -372,18 +424,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   a.trace = c->trace.as<unsigned long long>();
   c->trace_items = nitems;
 #endif
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (c->profiling) {
-    e0 = take_event(c);
-    e1 = take_event(c);
-    CUDA_TRY(cudaEventRecord(e0, s));
-  }
-  DBIE_TRY(launch_kernel(k, grid, &a, s));
-  if (c->profiling) {
-    CUDA_TRY(cudaEventRecord(e1, s));
-    c->pending.push_back({e0, e1});
-    c->pending_pairs.push_back((double)n * (double)c->nquad);
-  }
+  DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
   if (near_on)
     launch_nearfield(var, tied, c->prob.as<ProbDesc>(), c->near_list.as<int32_t>(), &m->near_cnt,
                      c->qpos.as<float4>(), c->qlam.as<Lam4>(), &m->plan, m->item_off,
@@ -511,7 +552,7 @@ void dbie_destroy(dbie_ctx* c) {
                   &c->st_aux, &c->qpos, &c->qlam, &c->near_list, &c->out, &c->ptiles, &c->tv32,
                   &c->tv64, &c->probv, &c->b0raw, &c->vtmp, &c->pxe_corr, &c->pxe_pos,
                   &c->pxe_list, &c->pxe_w, &c->pxe_part, &c->pxe_bins, &c->trace, &c->qlam0,
-                  &c->dmsc})
+                  &c->dmsc, &c->sctab})
     b->release();
   c->sb.release();
   for (auto& pr : c->pending) {
@@ -671,6 +712,8 @@ dbie_status dbie_create(dbie_ctx** out, int32_t nx, int32_t ny, double x0, doubl
   if ((st = ensure(c->prob, sizeof(ProbDesc))) != DBIE_OK) return bail(st);
   if ((st = ensure(c->err, sizeof(unsigned))) != DBIE_OK) return bail(st);
   if ((st = ensure(c->misc, sizeof(Misc))) != DBIE_OK) return bail(st);
+  if ((st = ensure(c->sctab, sizeof(float4) * SINCOS_TABLE)) != DBIE_OK) return bail(st);
+  launch_fill_sincos(c->sctab.as<float4>(), s);
   if (cudaMemsetAsync(c->err.p, 0, sizeof(unsigned), s) != cudaSuccess ||
       cudaMemsetAsync(c->misc.p, 0, sizeof(Misc), s) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -841,34 +884,7 @@ dbie_status dbie_eval_difference(dbie_ctx* c, int64_t n, const float* xyz,
   DBIE_TRY(ensure(c->qpos, sizeof(float4) * n));
   DBIE_TRY(ensure(c->qlam, sizeof(Lam4) * n));
   DBIE_TRY(ensure(c->qlam0, sizeof(Lam4) * n));
-  launch_pack_eval(n, xyz, nullptr, lambda_ref, c->qpos.as<float4>(), c->qlam0.as<Lam4>(), nullptr,
-                   nullptr, 0, 0.0, s);
-  launch_pack_eval(n, xyz, nullptr, lambda, c->qpos.as<float4>(), c->qlam.as<Lam4>(), nullptr,
-                   nullptr, 0, 0.0, s);
-  const KernelRef k = g1_ref_dif(tied != 0);
-  const int grid = persistent_grid(k, c->device);
-  const int64_t nblk = (n + k.qper - 1) / k.qper;
-  const int64_t target = std::max<int64_t>(1, (int64_t)grid * DBIE_SPLIT_TARGET_PCT / 100);
-  int64_t nsplit = 1;
-  if (nblk < target) nsplit = std::min<int64_t>((target + nblk - 1) / nblk, c->ntiles);
-  const int64_t nitems = nblk * nsplit;
-  if (nitems > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
-  DBIE_TRY(ensure(c->out, sizeof(double) * nitems * 12 * k.qper));
-  launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, (int)nitems, (int)nsplit, k.qper,
-                     (int)n, s);
-  G1Args a{};
-  a.probs = c->prob.as<ProbDesc>();
-  a.nprob = 1;
-  a.plan = &m->plan;
-  a.item_off = m->item_off;
-  a.q_cnt = m->q_cnt;
-  a.work = &m->work;
-  a.qpos = c->qpos.as<float4>();
-  a.qlam = c->qlam.as<Lam4>();
-  a.qlam0 = c->qlam0.as<Lam4>();
-  a.out = c->out.as<double>();
-  a.err = c->err.as<unsigned>();
-  DBIE_TRY(launch_kernel(k, grid, &a, s));
+  DBIE_TRY(pass_reeval(c, VAR_OBJ, tied != 0, n, xyz, nullptr, lambda, lambda_ref, s));
   double* msc = nullptr;
   if (dS_bound) {
     DBIE_TRY(ensure(c->dmsc, sizeof(double) * 18 * n));
@@ -876,7 +892,7 @@ dbie_status dbie_eval_difference(dbie_ctx* c, int64_t n, const float* xyz,
     launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n,
                (int)std::min<int64_t>((n + 127) / 128, 32LL * c->sm_count), s);
   }
-  launch_dif_debug(n, &m->plan, m->item_off, c->out.as<double>(), c->qlam.as<Lam4>(),
+  launch_dif_debug(n, &m->plan, c->out.as<double>(), c->qlam.as<Lam4>(),
                    c->qlam0.as<Lam4>(), msc, msc ? msc + 15 * n : nullptr, tied ? 1 : 3, dS,
                    dS_bound, s);
   CUDA_TRY(cudaGetLastError());
@@ -1354,19 +1370,16 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   // the persistent grid): more items balance the queue, fewer items mean fewer partial sums.
   const int target = (int)((int64_t)grid * DBIE_SPLIT_TARGET_PCT / 100);
   const int64_t items_cap = std::max<int64_t>((Qcap + k.qper - 1) / k.qper + nprob, 2LL * target) + 1;
-  // float-float re-evaluation pass (at most 2 queries per point and round)
-  const KernelRef kf = g1_ref_ff(VAR_OBJ, tied);
-  const int grid_ff = cert ? persistent_grid(kf, c->device) : 0;
-  const int target_ff = std::max(1, (int)((int64_t)grid_ff * DBIE_FF_SPLIT_TARGET_PCT / 100));
-  const int64_t fitems_cap = std::max<int64_t>((2 * N + kf.qper - 1) / kf.qper + nprob,
-                                               2LL * target_ff) + 1;
-  // difference level of the re-evaluation (values near the point's float-float reference)
+  // re-evaluation pass (at most 2 float-float and 2 difference queries per point and round); the
+  // difference level re-evaluates values near the point's float-float reference
   const bool dif_on = cert && o.certify_ref > 0;
-  const KernelRef kd = g1_ref_dif(tied);
-  const int grid_dif = dif_on ? persistent_grid(kd, c->device) : 0;
-  const int target_dif = std::max(1, (int)((int64_t)grid_dif * DBIE_FF_SPLIT_TARGET_PCT / 100));
-  const int64_t ditems_cap = std::max<int64_t>((2 * N + kd.qper - 1) / kd.qper + nprob,
-                                               2LL * target_dif) + 1;
+  const KernelRef kr = reeval_ref(VAR_OBJ, tied, dif_on);
+  const KernelRef kv = reeval_ref(VAR_V, tied, false);   // certified B
+  const int grid_re = cert ? persistent_grid(kr, c->device) : 0;
+  const int grid_v = cert ? persistent_grid(kv, c->device) : 0;
+  int max_rows = 0;
+  for (int p = 0; p < nprob; ++p)
+    max_rows = std::max(max_rows, ctxs[p]->ntiles * RE_ROWS_PER_TILE);
 
   DBIE_TRY(ensure(b.probs, sizeof(ProbDesc) * nprob));
   DBIE_TRY(ensure(b.ppos, sizeof(float4) * N));
@@ -1387,25 +1400,20 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   }
   if (cert) {
     DBIE_TRY(ensure(b.msc, sizeof(double) * 18 * N));
-    DBIE_TRY(ensure(b.fout, sizeof(double) * fitems_cap * 12 * kf.qper));
-    DBIE_TRY(ensure(b.fq_cnt_pass, sizeof(int32_t) * nprob));
-    DBIE_TRY(ensure(b.fitem_off, sizeof(int32_t) * (nprob + 1)));
+    DBIE_TRY(ensure(b.fout, sizeof(double) * std::max(12 * reeval_items(2 * N, grid_re),
+                                                      3 * reeval_items(N, grid_v))));
     for (int sd = 0; sd < 2; ++sd) {
       DBIE_TRY(ensure(b.fpos[sd], sizeof(float4) * 2 * N));
       DBIE_TRY(ensure(b.flam[sd], sizeof(Lam4) * 2 * N));
-      DBIE_TRY(ensure(b.fq_cnt[sd], sizeof(int32_t) * nprob));
       DBIE_TRY(ensure(b.ref[sd], sizeof(int32_t) * N));
     }
   }
   if (dif_on) {
-    DBIE_TRY(ensure(b.dout, sizeof(double) * ditems_cap * 12 * kd.qper));
-    DBIE_TRY(ensure(b.dq_cnt_pass, sizeof(int32_t) * nprob));
-    DBIE_TRY(ensure(b.ditem_off, sizeof(int32_t) * (nprob + 1)));
+    DBIE_TRY(ensure(b.dout, sizeof(double) * 12 * reeval_items(2 * N, grid_re)));
     for (int sd = 0; sd < 2; ++sd) {
       DBIE_TRY(ensure(b.dpos[sd], sizeof(float4) * 2 * N));
       DBIE_TRY(ensure(b.dlam[sd], sizeof(Lam4) * 2 * N));
       DBIE_TRY(ensure(b.dlam0[sd], sizeof(Lam4) * 2 * N));
-      DBIE_TRY(ensure(b.dq_cnt[sd], sizeof(int32_t) * nprob));
     }
   }
   bool any_init = false;
@@ -1432,7 +1440,6 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     pd.near_z = (!fp64 && op.near_z > 0) ? op.near_z : 0.0;
     pd.pxe_z = pxe_on(cp, op) ? op.near_z : 0.0;
     pd.q_off = (int64_t)(dim + 1) * pt_off[p];
-    pd.qff_off = 2 * pt_off[p];
     pd.pt_off = pt_off[p];
     pd.npts = n[p];
   }
@@ -1472,11 +1479,6 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   }
   for (int sd = 0; sd < 2; ++sd) CUDA_TRY(cudaMemsetAsync(b.q_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
   if (cert) {
-    for (int sd = 0; sd < 2; ++sd)
-      CUDA_TRY(cudaMemsetAsync(b.fq_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
-    if (dif_on)
-      for (int sd = 0; sd < 2; ++sd)
-        CUDA_TRY(cudaMemsetAsync(b.dq_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
     // the error bounds' lambda-independent absolute-value sums of every point
     launch_msc(b.probs.as<ProbDesc>(), N, b.ppos.as<float4>(), b.msc.as<double>(),
                b.msc.as<double>() + 15 * N,
@@ -1517,15 +1519,15 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     a.cur = RoundBuf{b.qpos[cur].as<float4>(), b.qlam[cur].as<Lam4>(), b.q_cnt[cur].as<int32_t>(),
                      b.act[cur].as<int32_t>(), &ctrl->act_cnt[cur], b.near[cur].as<int32_t>(),
                      &ctrl->near_cnt[cur], b.fpos[cur].as<float4>(), b.flam[cur].as<Lam4>(),
-                     b.fq_cnt[cur].as<int32_t>(), b.ref[cur].as<int32_t>(), &ctrl->ref_cnt[cur],
+                     &ctrl->f_cnt[cur], b.ref[cur].as<int32_t>(), &ctrl->ref_cnt[cur],
                      b.dpos[cur].as<float4>(), b.dlam[cur].as<Lam4>(), b.dlam0[cur].as<Lam4>(),
-                     b.dq_cnt[cur].as<int32_t>()};
+                     &ctrl->d_cnt[cur]};
     a.nxt = RoundBuf{b.qpos[nx_].as<float4>(), b.qlam[nx_].as<Lam4>(), b.q_cnt[nx_].as<int32_t>(),
                      b.act[nx_].as<int32_t>(), &ctrl->act_cnt[nx_], b.near[nx_].as<int32_t>(),
                      &ctrl->near_cnt[nx_], b.fpos[nx_].as<float4>(), b.flam[nx_].as<Lam4>(),
-                     b.fq_cnt[nx_].as<int32_t>(), b.ref[nx_].as<int32_t>(), &ctrl->ref_cnt[nx_],
+                     &ctrl->f_cnt[nx_], b.ref[nx_].as<int32_t>(), &ctrl->ref_cnt[nx_],
                      b.dpos[nx_].as<float4>(), b.dlam[nx_].as<Lam4>(), b.dlam0[nx_].as<Lam4>(),
-                     b.dq_cnt[nx_].as<int32_t>()};
+                     &ctrl->d_cnt[nx_]};
     a.out = b.out.as<double>();
     a.plan = &ctrl->plan;
     a.item_off = b.item_off.as<int32_t>();
@@ -1546,14 +1548,13 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
       a.msc = b.msc.as<double>();
       a.fout = b.fout.as<double>();
       a.fplan = &ctrl->fplan;
-      a.fitem_off = b.fitem_off.as<int32_t>();
+      a.rework = ctrl->rework;
       a.stat_ties = &ctrl->stat_ties;
       a.msc0 = b.msc.as<double>() + 15 * N;
     }
     if (dif_on) {
       a.dout = b.dout.as<double>();
       a.dplan = &ctrl->dplan;
-      a.ditem_off = b.ditem_off.as<int32_t>();
       a.stat_difs = &ctrl->stat_difs;
     }
   }
@@ -1564,44 +1565,21 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
                     (int)std::min<int64_t>((N + 255) / 256, 8LL * c->sm_count), s);
   CUDA_TRY(cudaGetLastError());
 
-  // One re-evaluation pass of a round (float-float, or differences when lam0 is given): plan
-  // the queued values, run the pair sums, with profiling events ev_at and ev_at + 1 around it.
-  auto record_reeval = [&](cudaStream_t cs, const KernelRef& kr, int grid_r, int target_r,
-                           const DBuf& cnt, const DBuf& cnt_pass, const DBuf& item_off_r,
-                           PlanHdr* plan_r, int32_t* work_r, double* stat_pairs_r,
-                           const DBuf& qpos_r, const DBuf& qlam_r, const DBuf* qlam0_r,
-                           const DBuf& out_r, int ev_at) -> dbie_status {
-    PlanArgs pp{};
-    pp.probs = b.probs.as<ProbDesc>();
-    pp.nprob = nprob;
-    pp.qper = kr.qper;
-    pp.target_items = target_r;
-    pp.nsplit_cap = 1 << 20;
-    pp.q_cnt_cur = cnt.as<int32_t>();
-    pp.q_cnt_pass = cnt_pass.as<int32_t>();
-    pp.item_off = item_off_r.as<int32_t>();
-    pp.plan = plan_r;
-    pp.work = work_r;
-    pp.stat_pairs = stat_pairs_r;
-    launch_plan_round(pp, cs);
-    G1Args ga{};
-    ga.probs = b.probs.as<ProbDesc>();
-    ga.nprob = nprob;
-    ga.plan = plan_r;
-    ga.item_off = item_off_r.as<int32_t>();
-    ga.q_cnt = cnt_pass.as<int32_t>();
-    ga.work = work_r;
-    ga.qpos = qpos_r.as<float4>();
-    ga.qlam = qlam_r.as<Lam4>();
-    ga.qlam0 = qlam0_r ? qlam0_r->as<Lam4>() : nullptr;
-    ga.out = out_r.as<double>();
-    ga.err = c->err.as<unsigned>();
-    if (c->profiling)
-      CUDA_TRY(cudaEventRecordWithFlags(b.ev[ev_at], cs, cudaEventRecordExternal));
-    DBIE_TRY(launch_kernel(kr, grid_r, &ga, cs));
-    if (c->profiling)
-      CUDA_TRY(cudaEventRecordWithFlags(b.ev[ev_at + 1], cs, cudaEventRecordExternal));
-    return DBIE_OK;
+  // Arguments of the re-evaluation pass of a round (side cur).
+  auto reeval_args = [&](int cur) {
+    ReArgs ra{};
+    ra.probs = b.probs.as<ProbDesc>();
+    ra.f = ReList{&ctrl->f_cnt[cur], b.fpos[cur].as<float4>(), b.flam[cur].as<Lam4>(), nullptr,
+                  b.fout.as<double>(), &ctrl->fplan};
+    ra.d = ReList{dif_on ? &ctrl->d_cnt[cur] : &ctrl->zero, b.dpos[cur].as<float4>(),
+                  b.dlam[cur].as<Lam4>(), b.dlam0[cur].as<Lam4>(), b.dout.as<double>(),
+                  &ctrl->dplan};
+    ra.work = &ctrl->rework[0];
+    ra.sctab = c->sctab.as<float4>();
+    ra.stat_ff_pairs = &ctrl->stat_ff_pairs;
+    ra.stat_dif_pairs = &ctrl->stat_dif_pairs;
+    ra.rows = max_rows;
+    return ra;
   };
   // One simplex round = plan, pair sums (objective variant), near-field correction, step.
   constexpr int K = 4;  // rounds per graph launch (even: the ping-pong side returns to 0)
@@ -1623,10 +1601,10 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
       pa.act_cnt_nxt = &ctrl->act_cnt[cur ^ 1];
       pa.near_cnt_nxt = &ctrl->near_cnt[cur ^ 1];
       if (cert) {
-        pa.fq_cnt_nxt = b.fq_cnt[cur ^ 1].as<int32_t>();
+        pa.fq_cnt_nxt = &ctrl->f_cnt[cur ^ 1];
         pa.ref_cnt_nxt = &ctrl->ref_cnt[cur ^ 1];
       }
-      if (dif_on) pa.dq_cnt_nxt = b.dq_cnt[cur ^ 1].as<int32_t>();
+      if (dif_on) pa.dq_cnt_nxt = &ctrl->d_cnt[cur ^ 1];
       pa.round_ctr = &ctrl->round;
       pa.stat_queries = &ctrl->stat_queries;
       pa.stat_pairs = &ctrl->stat_pairs;
@@ -1657,13 +1635,25 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
       if (cert) {
         // the near-tied values of this round in float-float, then those queued as differences
         // from the points' references, then the waiting steps again
-        DBIE_TRY(record_reeval(cs, kf, grid_ff, target_ff, b.fq_cnt[cur], b.fq_cnt_pass,
-                               b.fitem_off, &ctrl->fplan, &ctrl->fwork, &ctrl->stat_ff_pairs,
-                               b.fpos[cur], b.flam[cur], nullptr, b.fout, 6 * r + 2));
-        if (dif_on)
-          DBIE_TRY(record_reeval(cs, kd, grid_dif, target_dif, b.dq_cnt[cur], b.dq_cnt_pass,
-                                 b.ditem_off, &ctrl->dplan, &ctrl->dwork, &ctrl->stat_dif_pairs,
-                                 b.dpos[cur], b.dlam[cur], &b.dlam0[cur], b.dout, 6 * r + 4));
+        ReArgs ra = reeval_args(cur);
+        if (!c->profiling) {
+          DBIE_TRY(launch_kernel(kr, grid_re, &ra, cs));
+        } else {   // the two kinds as launches of their own, to time each
+          ReArgs rf = ra;
+          rf.d.cnt = &ctrl->zero;
+          ra.f.cnt = &ctrl->zero;
+          ra.f.plan = &ctrl->noplan;
+          rf.d.plan = &ctrl->noplan;
+          ra.work = &ctrl->rework[1];
+          CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 2], cs, cudaEventRecordExternal));
+          DBIE_TRY(launch_kernel(kr, grid_re, &rf, cs));
+          CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 3], cs, cudaEventRecordExternal));
+          if (dif_on) {
+            CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 4], cs, cudaEventRecordExternal));
+            DBIE_TRY(launch_kernel(kr, grid_re, &ra, cs));
+            CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 5], cs, cudaEventRecordExternal));
+          }
+        }
         launch_nm_refine(sa[cur], nm_grid, cs);
       }
     }
@@ -1676,12 +1666,13 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     for (auto& e : b.ev) CUDA_TRY(cudaEventCreate(&e));
   }
   // Capture (or reuse) the graph of K rounds; the key is every launch argument.
-  std::vector<unsigned char> key(sizeof sa + sizeof(KernelRef) + 3 * sizeof(int));
+  std::vector<unsigned char> key(sizeof sa + sizeof(KernelRef) + 4 * sizeof(int));
   {
     unsigned char* kp = key.data();
     std::memcpy(kp, sa, sizeof sa);
     std::memcpy(kp + sizeof sa, &k, sizeof k);
-    const int extra[3] = {grid, nm_grid, (c->profiling ? 1 : 0) | (qn ? 2 : 0) | (cert ? 4 : 0)};
+    const int extra[4] = {grid, nm_grid, (c->profiling ? 1 : 0) | (qn ? 2 : 0) | (cert ? 4 : 0),
+                          max_rows};
     std::memcpy(kp + sizeof sa + sizeof k, extra, sizeof extra);
   }
   if (!b.exec || b.key != key) {
@@ -1748,34 +1739,13 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   // relative (the cancellation-dominated points) again, in float-float at lambda* (side 0 is the
   // current side after an even number of rounds).
   if (cert) {
-    const KernelRef kv = g1_ref_ff(VAR_V, tied);
-    CUDA_TRY(cudaMemsetAsync(b.fq_cnt[0].p, 0, sizeof(int32_t) * nprob, s));
+    CUDA_TRY(cudaMemsetAsync(&ctrl->f_cnt[0], 0, sizeof(int32_t), s));
     CUDA_TRY(cudaMemsetAsync(&ctrl->ref_cnt[0], 0, sizeof(int32_t), s));
+    CUDA_TRY(cudaMemsetAsync(&ctrl->rework[0], 0, sizeof(int32_t), s));
     launch_certb_flag(sa[0], 1e-5, (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count), s);
-    PlanArgs pf{};
-    pf.probs = b.probs.as<ProbDesc>();
-    pf.nprob = nprob;
-    pf.qper = kv.qper;
-    pf.target_items = std::max(1, 2 * persistent_grid(kv, c->device));
-    pf.nsplit_cap = 1 << 20;
-    pf.q_cnt_cur = b.fq_cnt[0].as<int32_t>();
-    pf.q_cnt_pass = b.fq_cnt_pass.as<int32_t>();
-    pf.item_off = b.fitem_off.as<int32_t>();
-    pf.plan = &ctrl->fplan;
-    pf.work = &ctrl->fwork;
-    launch_plan_round(pf, s);
-    G1Args gf{};
-    gf.probs = b.probs.as<ProbDesc>();
-    gf.nprob = nprob;
-    gf.plan = &ctrl->fplan;
-    gf.item_off = b.fitem_off.as<int32_t>();
-    gf.q_cnt = b.fq_cnt_pass.as<int32_t>();
-    gf.work = &ctrl->fwork;
-    gf.qpos = b.fpos[0].as<float4>();
-    gf.qlam = b.flam[0].as<Lam4>();
-    gf.out = b.fout.as<double>();
-    gf.err = c->err.as<unsigned>();
-    DBIE_TRY(launch_kernel(kv, persistent_grid(kv, c->device), &gf, s));
+    ReArgs rv = reeval_args(0);
+    rv.stat_ff_pairs = nullptr;
+    DBIE_TRY(launch_kernel(kv, grid_v, &rv, s));
     launch_certb_apply(sa[0], nm_grid, s);
     CUDA_TRY(cudaGetLastError());
     DBIE_TRY(check_device_error(c, s));

@@ -93,7 +93,6 @@ struct ProbDesc {
   double pxe_z;             // pixel-exact near field for z <= pxe_z (0: off)
   double area;              // pixel area of the midpoint weights (dA; usually hx hy)
   int64_t q_off;            // first query slot of this problem
-  int64_t qff_off;          // first float-float re-evaluation slot (2 per point)
   int64_t pt_off;           // first global point index
   int64_t npts;
 };
@@ -120,7 +119,6 @@ struct G1Args {
   double* out;              // per work item a chunk of nsum * qper partial sums (see out_index)
   unsigned* err;
   unsigned long long* trace; // DBIE_TRACE_ITEMS builds: per item start, end (ns) and SM (or null)
-  const Lam4* qlam0;        // [slot] difference sums only: the reference lambda of each query
 };
 
 // Position of partial sum s of the query with local index j (within its problem) for split

@@ -35,9 +35,34 @@ struct KernelRef {
 // rows: every aligned group of 4 quadrature points lies on one row (row length % 4 == 0)
 KernelRef g1_ref_f32(int var, bool tied, int cfg, bool rows);   // pairsum_f32_*.cu
 KernelRef g1_ref_f64(int var, bool tied);            // pairsum_f64.cu
-KernelRef g1_ref_ff(int var, bool tied);             // pairsum_ff.cu (VAR_V, VAR_OBJ)
-KernelRef g1_ref_dif(bool tied);                     // pairsum_dif.cu (objective sums)
+
+// pairsum_re.cu: float-float sums (VAR_V, VAR_OBJ) and difference sums (objective) of queued
+// queries, one CTA per query and row range.
+struct ReList {
+  const int32_t* cnt;       // queries
+  const float4* pos;        // [slot] x, y, z, problem index (int bits)
+  const Lam4* lam;          // [slot] lambda
+  const Lam4* lam0;         // [slot] reference lambda (differences)
+  double* out;              // [slot][split][sums]
+  PlanHdr* plan;            // written by the kernel: the split count (items of one query each)
+};
+struct ReArgs {
+  const ProbDesc* probs;
+  ReList f, d;              // float-float queries, difference queries
+  int32_t* work;            // item counter, zero before the launch
+  const float4* sctab;      // sine and cosine table (launch_fill_sincos)
+  double* stat_ff_pairs;    // pairs of this pass are added (or null)
+  double* stat_dif_pairs;
+  int32_t rows;             // rows of 128 pixels of the largest problem
+  int32_t pad0;
+};
+constexpr int RE_ROWS_PER_TILE = TILE / 128;
+constexpr int SINCOS_TABLE = 52;   // ff::SC_TABLE
+KernelRef reeval_ref(int var, bool tied, bool dif);
+// items that a launch of `grid` CTAs writes at most for up to this many queries
+int64_t reeval_items(int64_t queries, int grid);
 void launch_stage_ff(const double* t64, int ntiles, float* tff, cudaStream_t s);
+void launch_fill_sincos(float4* tab, cudaStream_t s);   // ff::SC_TABLE entries
 KernelRef vjp_ref(bool fp64, bool tied, int cfg);    // vjp.cu
 KernelRef vjp7_ref(bool fp64, bool tied);            // vjp.cu (seven-weight adjoint)
 // FP32 form over element Gauss points with float-pair positions (pairsum_f32_split.cu)
@@ -126,8 +151,8 @@ void launch_nm_step(const SolveArgs& a, int grid, cudaStream_t s);
 void launch_nm_refine(const SolveArgs& a, int grid, cudaStream_t s);
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
                 int grid, cudaStream_t s);
-void launch_dif_debug(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
-                      const Lam4* qlam, const Lam4* qlam0, const double* msc, const double* msc0,
+void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const Lam4* qlam,
+                      const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s);
 void launch_certb_flag(const SolveArgs& a, double rel, int grid, cudaStream_t s);
 void launch_certb_apply(const SolveArgs& a, int grid, cudaStream_t s);

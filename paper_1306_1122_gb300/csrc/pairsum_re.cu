@@ -1,0 +1,392 @@
+// pairsum_re.cu -- the accurate pair sums: float-float sums, and difference sums between two
+// lambdas of a point.
+//
+// Float-float sums.  Every pair term of Eq. 16 (and of the fixed-lambda derivatives of Eq. 13) is
+// carried as hi + lo float pairs (ff_math.cuh): the point-pixel offsets, r and 1/r from the SFU
+// reciprocal square root with Newton corrections, sin and cos of lambda r by a Cody-Waite
+// reduction and a table, the products of the terms and the running sums.  The result agrees with
+// the FP64 sums to about 1e-13 of the absolute-value sum, at the FP32 pipe's issue rate: on GB300
+// about ten times faster than the same sweep in native FP64.
+//
+// Difference sums: the change of the objective sums between lambda_0 and lambda_a of one point,
+// from FP32 terms whose error is proportional to the change.  Per pixel and component, with
+// theta = lambda r, sigma = (lambda_a + lambda_0) r / 2 and delta = (lambda_a - lambda_0) r / 2,
+//   cos(theta_a) - cos(theta_0)                     = -2 sin(sigma) sin(delta)
+//   theta_a sin(theta_a) - theta_0 sin(theta_0)     =  2 [delta sin(sigma) cos(delta)
+//                                                         + sigma cos(sigma) sin(delta)]
+//   lambda_a^2 cos(theta_a) - lambda_0^2 cos(theta_0) = (lambda_a^2 - lambda_0^2) cos(sigma) cos(delta)
+//                                                     - (lambda_a^2 + lambda_0^2) sin(sigma) sin(delta)
+// so the change of u = theta sin(theta) + cos(theta) and of w = lambda^2 cos(theta) - 3 u / r^2
+// is a sum of products that each carry a factor delta (or lambda_a - lambda_0).  Evaluated in FP32
+// (SFU sine and cosine of sigma; sin and cos of delta by their Taylor polynomials for |delta| <= 1),
+// every rounding and every SFU error is relative to that factor: the error of a difference sum is
+// a bound times |lambda_a - lambda_0|, where the error of the plain FP32 sums is a bound times 1.
+// Added to float-float sums at lambda_0, the differences give the sums at lambda_a with an error
+// that shrinks with the distance between the two lambdas.
+//
+// The lambda search re-evaluates with both the queries whose simplex decision the FP32-term sums
+// cannot certify; dbie_eval offers the float-float sums as DBIE_PREC_FLOAT_FLOAT and
+// dbie_eval_difference the difference sums.
+//
+// Work distribution.  Both are bound by FP32 issue (824 and 153 instructions per pair), and their
+// queries are few and scattered: a search round queues tens to thousands of them, over all
+// problems.  So the lanes of a CTA take pixels, not queries: an item is one query and a range of
+// rows of 128 pixels, one pixel per thread, and no lane idles whatever the number of queries
+// (a block of one query per thread kept 128 lanes for the last few queries of every problem, and
+// one thread's 256 dependent pixels of a tile were the length of a round's pass: on a
+// 32 x 32-pixel search of 2,048 points 166 us float-float and 53 us differences per round).
+// Measured against that layout: 4,096 queries over 128 x 128 pixels, float-float, 2.06 -> 1.71 ms
+// (3.3e10 -> 3.9e10 pairs/s); the whole search above 45.6 -> 24.4 ms; 16 magnetograms of 32 to
+// 128 pixels with up to 300 points each, searched in one call, 237 -> 59 ms.
+// Queries of all problems share one queue; one launch takes the float-float items first and the
+// cheaper difference items after them, which fill its tail.  Terms need 40 bytes of tile data
+// per 153 or more instructions, which plain coalesced loads through L1 sustain; nothing is staged.
+#include <type_traits>
+
+#include "ff_math.cuh"
+#include "kernels.h"
+
+namespace dbie {
+
+using ff::ds;
+
+constexpr int RE_NT = 128;           // threads per CTA = pixels per row of an item
+constexpr int RE_NF = 2 * NFIELD;    // floats per pixel in a float-float tile
+constexpr int RE_MAX_SPLIT = 64;     // row ranges per query: the reader adds them one by one
+constexpr int RE_WAVES = 8;          // items per CTA at most (the tail is then 1/8 of a pass)
+constexpr int DIF_BLK = 8;           // pixels per FP32 block sum of the differences
+static_assert(TILE / RE_NT == RE_ROWS_PER_TILE && TILE % RE_NT == 0, "rows tile the tile");
+
+// Float-float tiles: per field (x, y, bx, by, bz) TILE hi parts, then TILE lo parts.
+__global__ void stage_ff_kernel(const double* __restrict__ t64, int ntiles,
+                                float* __restrict__ tff) {
+  const int64_t total = (int64_t)ntiles * TILE;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < total;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t tile = k / TILE;
+    const int e = (int)(k % TILE);
+    for (int f = 0; f < NFIELD; ++f) {
+      const ds d = ff::from_double(t64[tile * (NFIELD * TILE) + f * TILE + e]);
+      float* dst = tff + tile * (int64_t)(RE_NF * TILE) + f * 2 * TILE + e;
+      dst[0] = d.hi;
+      dst[TILE] = d.lo;
+    }
+  }
+}
+
+void launch_stage_ff(const double* t64, int ntiles, float* tff, cudaStream_t s) {
+  const int64_t total = (int64_t)ntiles * TILE;
+  const int grid = (int)((total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192);
+  stage_ff_kernel<<<grid, 256, 0, s>>>(t64, ntiles, tff);
+}
+
+__global__ void fill_sincos_kernel(float4* tab) { ff::fill_sincos_table(tab, threadIdx.x); }
+
+void launch_fill_sincos(float4* tab, cudaStream_t s) {
+  static_assert(ff::SC_TABLE == SINCOS_TABLE && SINCOS_TABLE <= 64, "one thread per table entry");
+  fill_sincos_kernel<<<1, 64, 0, s>>>(tab);
+}
+
+// Row ranges per query.  While a pass is short (at most 4 rows for every CTA) one wave of items
+// spreads it over the chip; a longer pass takes up to RE_WAVES items per CTA, so that the uneven
+// end is a fraction of it.  Rounded down: an item too many would be a wave of its own.
+__device__ __forceinline__ int re_split(int cnt, int rows, int ctas) {
+  if (cnt <= 0) return 1;
+  const int64_t waves = (int64_t)cnt * rows / (4 * (int64_t)ctas);
+  const int64_t target = (int64_t)ctas * (waves < 1 ? 1 : (waves > RE_WAVES ? RE_WAVES : waves));
+  const int most = rows < RE_MAX_SPLIT ? rows : RE_MAX_SPLIT;
+  const int64_t ns = target / cnt;
+  return ns < 1 ? 1 : (ns > most ? most : (int)ns);
+}
+
+// Sums over the CTA's threads: within a warp by halving (each step hands half of the sums to the
+// partner lane, so 16 pair additions reduce 12 sums instead of 60), then the warps' sums in FP64.
+// `red` holds 4 * NSUM doubles.  Writes NSUM values to dst; callers synchronise before red is
+// written again.
+template <int NSUM>
+__device__ __forceinline__ void reduce_store(const ds (&acc)[NSUM], double* red, double* dst) {
+  constexpr int NP = NSUM > 8 ? 16 : 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto plus = [](ds a, ds b) {
+    const ds s = ff::two_sum(a.hi, b.hi);
+    return ds{s.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), s.lo)};
+  };
+  ds v[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) v[i] = i < NSUM ? acc[i < NSUM ? i : 0] : ds{0.f, 0.f};
+  int off = 16;
+#pragma unroll
+  for (int half = NP / 2; half >= 1; half >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const ds give = up ? v[i] : v[i + half];
+      const ds keep = up ? v[i + half] : v[i];
+      v[i] = plus(keep, ds{__shfl_xor_sync(0xffffffffu, give.hi, off),
+                           __shfl_xor_sync(0xffffffffu, give.lo, off)});
+    }
+  }
+  for (; off >= 1; off >>= 1)
+    v[0] = plus(v[0], ds{__shfl_xor_sync(0xffffffffu, v[0].hi, off),
+                         __shfl_xor_sync(0xffffffffu, v[0].lo, off)});
+  constexpr int GL = 32 / NP;   // lanes that hold the same sum
+  if (lane % GL == 0 && lane / GL < NSUM) red[warp * NSUM + lane / GL] = ff::to_double(v[0]);
+  __syncthreads();
+  if (threadIdx.x < NSUM) {
+    double t = red[threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < RE_NT / 32; ++w) t += red[w * NSUM + threadIdx.x];
+    dst[threadIdx.x] = t;
+  }
+}
+
+// The query of an item, prepared by the CTA's first threads (FP64 issues at 1/64 of the FP32
+// rate here: once per CTA, not once per thread).
+struct ReQuery {
+  float x, y, z;
+  int pidx;
+  float lh[3], ll[3];      // lambda (hi, lo)
+  float hs[3], hd[3], pq[3], qq[3];   // differences: (la + l0) / 2, (la - l0) / 2, la^2 -+ l0^2
+  int slow;                // lambda r may leave the range of the float-float reduction
+};
+
+__device__ __forceinline__ float re_load(const float* tile, int f, int part, int e) {
+  return __ldg(tile + f * 2 * TILE + part * TILE + e);
+}
+
+// Float-float sums of the CTA's pixel of each row in [r0, r1).
+template <int VAR, bool TIED, bool ANY>
+__device__ __forceinline__ void ff_rows(const float* tiles, int r0, int r1, const ReQuery& q,
+                                        const float4* tab, ds (&acc)[3 * nsum_per_comp(VAR)]) {
+  using D = ds;
+  constexpr int NS = nsum_per_comp(VAR);
+  constexpr int NL = TIED ? 1 : 3;
+  const D xq = D{q.x, 0.f}, yq = D{q.y, 0.f};
+  const D z2 = ff::two_prod(q.z, q.z);
+  D lam[NL], lam2[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    lam[l] = D{q.lh[l], q.ll[l]};
+    lam2[l] = ff::mul(lam[l], lam[l]);
+  }
+#pragma unroll 1
+  for (int row = r0; row < r1; ++row) {
+    const float* T = tiles + (int64_t)(row / (TILE / RE_NT)) * (RE_NF * TILE);
+    const int e = (row % (TILE / RE_NT)) * RE_NT + threadIdx.x;
+    const D X = D{re_load(T, 0, 0, e), re_load(T, 0, 1, e)};
+    const D Y = D{re_load(T, 1, 0, e), re_load(T, 1, 1, e)};
+    const D dx = ff::sub(xq, X);
+    const D dy = ff::sub(yq, Y);
+    // (products that feed a further float-float operation stay unnormalised: mul_nr)
+    const D r2 = ff::add(ff::add(ff::mul_nr(dx, dx), ff::mul_nr(dy, dy)), z2);
+    D r, ri;
+    ff::sqrt_rsqrt(r2, r, ri);
+    const D ri2 = ff::mul_nr(ri, ri);
+    const D ri3 = ff::mul_nr(ri2, ri);
+    D u[NL], c[NL];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      const D th = ff::mul_nr(lam[l], r);
+      D s;
+      if constexpr (ANY) ff::sincos_ds_any(th, tab, s, c[l]);
+      else ff::sincos_ds<float>(th, tab, s, c[l]);
+      u[l] = ff::add(ff::mul_nr(th, s), c[l]);
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const int lp = TIED ? 0 : p;
+      const D rb = ff::mul_nr(ri3, D{re_load(T, 2 + p, 0, e), re_load(T, 2 + p, 1, e)});
+      ff::acc_add(acc[p * NS], ff::mul_nr(u[lp], rb));
+      if constexpr (has_grad(VAR)) {
+        // psi b = (lambda^2 cos(lambda r) - 3 u / r^2) b / r^3
+        const D w = ff::sub(ff::mul_nr(lam2[lp], c[lp]),
+                            ff::mul_f_nr(ff::mul_nr(u[lp], ri2), 3.0f));
+        const D t1 = ff::mul_nr(w, rb);
+        ff::acc_add(acc[p * NS + 1], t1);
+        ff::acc_add(acc[p * NS + 2], ff::mul_nr(t1, dx));
+        ff::acc_add(acc[p * NS + 3], ff::mul_nr(t1, dy));
+      }
+    }
+  }
+}
+
+// sin(d), cos(d): Taylor polynomials through d^9 and d^10 for |d| <= 1 (truncation below 3e-8
+// relative), the SFU beyond.
+__device__ __forceinline__ void sincos_delta(float d, float& s, float& c) {
+  if (fabsf(d) <= 1.0f) {
+    const float d2 = d * d;
+    s = d * fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, 1.0f / 362880.0f, -1.0f / 5040.0f),
+                                   1.0f / 120.0f), -1.0f / 6.0f), 1.0f);
+    c = fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, -1.0f / 3628800.0f, 1.0f / 40320.0f),
+                                        -1.0f / 720.0f), 1.0f / 24.0f), -0.5f), 1.0f);
+  } else {
+    s = sin_mufu(d);
+    c = cos_mufu(d);
+  }
+}
+
+// Difference sums: FP32 over blocks of DIF_BLK pixels of a thread, the block sums in float-float.
+template <bool TIED>
+__device__ __forceinline__ void dif_rows(const float* tiles, int r0, int r1, const ReQuery& q,
+                                         ds (&acc)[12]) {
+  constexpr int NL = TIED ? 1 : 3;
+  const float z2 = q.z * q.z;
+#pragma unroll 1
+  for (int b0 = r0; b0 < r1; b0 += DIF_BLK) {
+    float bs[12];
+#pragma unroll
+    for (int s = 0; s < 12; ++s) bs[s] = 0.f;
+    const int b1 = b0 + DIF_BLK < r1 ? b0 + DIF_BLK : r1;
+#pragma unroll 2
+    for (int row = b0; row < b1; ++row) {
+      const float* T = tiles + (int64_t)(row / (TILE / RE_NT)) * (RE_NF * TILE);
+      const int e = (row % (TILE / RE_NT)) * RE_NT + threadIdx.x;
+      const float dx = (q.x - re_load(T, 0, 0, e)) - re_load(T, 0, 1, e);
+      const float dy = (q.y - re_load(T, 1, 0, e)) - re_load(T, 1, 1, e);
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, z2));
+      const float ri = rsqrt_mufu(r2);
+      const float r = r2 * ri;
+      const float ri2 = ri * ri;
+      const float ri3 = ri2 * ri;
+      float du[NL], dw[NL];
+#pragma unroll
+      for (int l = 0; l < NL; ++l) {
+        const float sg = q.hs[l] * r, dl = q.hd[l] * r;
+        const float ss = sin_mufu(sg), cs = cos_mufu(sg);
+        float sd, cd;
+        sincos_delta(dl, sd, cd);
+        const float cs_sd = cs * sd, ss_sd = ss * sd;
+        du[l] = 2.0f * (fmaf(dl, ss * cd, sg * cs_sd) - ss_sd);
+        dw[l] = fmaf(q.pq[l], cs * cd, fmaf(-q.qq[l], ss_sd, -3.0f * du[l] * ri2));
+      }
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const int lp = TIED ? 0 : p;
+        const float rb = ri3 * re_load(T, 2 + p, 0, e);
+        const float t1 = dw[lp] * rb;
+        bs[4 * p + 0] = fmaf(du[lp], rb, bs[4 * p + 0]);
+        bs[4 * p + 1] += t1;
+        bs[4 * p + 2] = fmaf(t1, dx, bs[4 * p + 2]);
+        bs[4 * p + 3] = fmaf(t1, dy, bs[4 * p + 3]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 12; ++s) {
+      const ds t = ff::two_sum(acc[s].hi, bs[s]);
+      acc[s] = ds{t.hi, __fadd_rn(acc[s].lo, t.lo)};
+    }
+  }
+}
+
+// Float-float sums of a.f and, with DIF, difference sums of a.d (objective sums).
+template <int VAR, bool TIED, bool DIF>
+__global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
+  static_assert(VAR == VAR_V || VAR == VAR_OBJ, "float-float form: value and objective sums");
+  static_assert(!DIF || VAR == VAR_OBJ, "differences: objective sums");
+  constexpr int NSUM = 3 * nsum_per_comp(VAR);
+  __shared__ float4 s_tab[ff::SC_TABLE];
+  __shared__ double s_red[RE_NT / 32 * NSUM];
+  __shared__ ReQuery s_q;
+  __shared__ int s_item;
+  const int tid = threadIdx.x;
+  if (tid < ff::SC_TABLE) s_tab[tid] = __ldg(a.sctab + tid);
+  const int nf = *a.f.cnt;
+  const int nd = DIF ? *a.d.cnt : 0;
+  const int fs = re_split(nf, a.rows, gridDim.x);
+  const int dsp = DIF ? re_split(nd, a.rows, gridDim.x) : 1;
+  const int fitems = nf * fs, items = fitems + nd * dsp;
+  if (blockIdx.x == 0 && tid == 0) {
+    *a.f.plan = PlanHdr{fitems, fs, 1, 0};
+    if (DIF) *a.d.plan = PlanHdr{nd * dsp, dsp, 1, 0};
+  }
+  long long pf = 0, pd_ = 0;   // thread 32: pairs of the queries whose first range it set up
+
+  for (;;) {
+    if (tid == 0) s_item = atomicAdd(a.work, 1);
+    __syncthreads();   // (also: the previous item's readers of s_red and s_q are done)
+    const int it = s_item;
+    if (it >= items) break;
+    const bool dif = DIF && it >= fitems;
+    const int ns = dif ? dsp : fs;
+    const int local = dif ? it - fitems : it;
+    const int slot = local / ns, sp = local - slot * ns;
+    const ReList& L = dif ? a.d : a.f;
+    const float4 pos = L.pos[slot];
+    const ProbDesc& pd = a.probs[__float_as_int(pos.w)];
+    if (tid < (TIED ? 1 : 3)) {
+      const Lam4 l4 = L.lam[slot];
+      const double la = tid == 0 ? l4.x : (tid == 1 ? l4.y : l4.z);
+      const ds h = ff::from_double(la);
+      s_q.lh[tid] = h.hi;
+      s_q.ll[tid] = h.lo;
+      if (DIF && dif) {   // formed in FP64
+        const Lam4 r4 = L.lam0[slot];
+        const double l0 = tid == 0 ? r4.x : (tid == 1 ? r4.y : r4.z);
+        s_q.hs[tid] = (float)(0.5 * (la + l0));
+        s_q.hd[tid] = (float)(0.5 * (la - l0));
+        s_q.pq[tid] = (float)((la - l0) * (la + l0));
+        s_q.qq[tid] = (float)(la * la + l0 * l0);
+      }
+    } else if (tid == 32) {
+      s_q.x = pos.x;
+      s_q.y = pos.y;
+      s_q.z = pos.z;
+      // lambda r below the reduction range of sincos_ds for every pixel: |lambda| times the
+      // largest distance to the quadrature grid's box (pixel centres, or Gauss points of elements
+      // two node spacings wide, all inside [x0 - |hx|, x0 + 2 nx |hx|] with nx quadrature points
+      // per row); otherwise (rare: a far-out trial lambda, or not finite) the CTA takes the path
+      // with the FP64 fallback, so the common path stays branch-free
+      const Lam4 l4 = L.lam[slot];
+      const float lmax = TIED ? fabsf((float)l4.x)
+                              : fmaxf(fmaxf(fabsf((float)l4.x), fabsf((float)l4.y)),
+                                      fabsf((float)l4.z));
+      const float x0 = (float)pd.x0, y0 = (float)pd.y0;
+      const float ax = (float)fabs(pd.hx), ay = (float)fabs(pd.hy);
+      const float ex = fmaxf(fabsf(pos.x - (x0 - ax)), fabsf(pos.x - (x0 + 2.0f * pd.nx * ax)));
+      const float ey = fmaxf(fabsf(pos.y - (y0 - ay)), fabsf(pos.y - (y0 + 2.0f * pd.ny * ay)));
+      const float rmax = sqrtf(ex * ex + ey * ey + pos.z * pos.z);
+      s_q.slow = !(lmax * rmax < 0.9f * ff::SC_MAX_ARG);
+      if (sp == 0) {
+        const long long px = (long long)pd.nx * pd.ny;
+        if (dif) pd_ += px;
+        else pf += px;
+      }
+    }
+    __syncthreads();
+    const int rows = pd.ntiles * (TILE / RE_NT);
+    const int r0 = (int)((int64_t)sp * rows / ns), r1 = (int)((int64_t)(sp + 1) * rows / ns);
+    ds acc[NSUM];
+#pragma unroll
+    for (int s = 0; s < NSUM; ++s) acc[s] = ds{0.f, 0.f};
+    if constexpr (DIF) {
+      if (dif) dif_rows<TIED>(pd.tilesff, r0, r1, s_q, acc);
+      else if (s_q.slow) ff_rows<VAR, TIED, true>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+      else ff_rows<VAR, TIED, false>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+    } else {
+      if (s_q.slow) ff_rows<VAR, TIED, true>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+      else ff_rows<VAR, TIED, false>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+    }
+    reduce_store<NSUM>(acc, s_red, L.out + (int64_t)local * NSUM);
+  }
+  if (tid == 32) {
+    if (pf && a.stat_ff_pairs) atomicAdd(a.stat_ff_pairs, (double)pf);
+    if (DIF && pd_ && a.stat_dif_pairs) atomicAdd(a.stat_dif_pairs, (double)pd_);
+  }
+}
+
+template <int VAR, bool TIED, bool DIF>
+static KernelRef re_ref_t() {
+  return KernelRef{(const void*)&reeval_kernel<VAR, TIED, DIF>, RE_NT, 1, 0};
+}
+
+KernelRef reeval_ref(int var, bool tied, bool dif) {
+  if (var == VAR_V) return tied ? re_ref_t<VAR_V, true, false>() : re_ref_t<VAR_V, false, false>();
+  if (!dif) return tied ? re_ref_t<VAR_OBJ, true, false>() : re_ref_t<VAR_OBJ, false, false>();
+  return tied ? re_ref_t<VAR_OBJ, true, true>() : re_ref_t<VAR_OBJ, false, true>();
+}
+
+int64_t reeval_items(int64_t queries, int grid) {
+  return queries > (int64_t)RE_WAVES * grid ? queries : (int64_t)RE_WAVES * grid;
+}
+
+}  // namespace dbie

@@ -48,6 +48,15 @@ __device__ __forceinline__ double gather_sum(const double* out, const PlanHdr& h
   return v;
 }
 
+// The same over the row ranges of re-evaluated query `slot` (one item per query and range).
+__device__ __forceinline__ double gather_slot(const double* out, const PlanHdr& h, int64_t slot,
+                                              int nsum, int s) {
+  const double* p = out + slot * h.nsplit * nsum + s;
+  double v = 0.0;
+  for (int sp = 0; sp < h.nsplit; ++sp) v += p[(int64_t)sp * nsum];
+  return v;
+}
+
 // Pixel-exact near field: add the point's lambda-independent correction of B and grad B
 // (corr: dB_p at p, d(dB_p/dx_j) at 3 + 3 p + j).
 __device__ __forceinline__ void add_corr(const double* corr, double B[3], double G[9]) {
@@ -398,10 +407,9 @@ __device__ __forceinline__ void read_eval_ff(const SolveArgs& a, const PlanHdr& 
                                              int64_t slot, double z, Eval& e, int64_t g,
                                              double S[12]) {
   const ProbDesc& pd = a.probs[pidx];
-  const int64_t j = slot - pd.qff_off;
   double G[9];
 #pragma unroll
-  for (int s = 0; s < 12; ++s) S[s] = gather_sum(a.fout, hf, a.fitem_off, pidx, j, 12, s);
+  for (int s = 0; s < 12; ++s) S[s] = gather_slot(a.fout, hf, slot, 12, s);
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
   e.s = 0.0;
 }
@@ -412,11 +420,10 @@ __device__ __forceinline__ void read_eval_dif(const SolveArgs& a, const PlanHdr&
                                               int64_t slot, double z, Eval& e, int64_t g,
                                               const double lt[3]) {
   const ProbDesc& pd = a.probs[pidx];
-  const int64_t j = slot - pd.qff_off;
   double S[12], G[9];
 #pragma unroll
   for (int s = 0; s < 12; ++s)
-    S[s] = SD(a, D_REFS + s, g) + gather_sum(a.dout, hd, a.ditem_off, pidx, j, 12, s);
+    S[s] = SD(a, D_REFS + s, g) + gather_slot(a.dout, hd, slot, 12, s);
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
   const double l0[3] = {SD(a, D_REFL, g), SD(a, D_REFL + 1, g), SD(a, D_REFL + 2, g)};
   double eb[12];
@@ -483,18 +490,17 @@ __device__ __forceinline__ void emit(const SolveArgs& a, int64_t g, const float4
 // float-float reference at lambda lref.  The value ids go to I_RTGT, one per byte (| RT_DIF for
 // differences), and the first slot of each kind to I_RSLOT, I_DSLOT.
 __device__ __forceinline__ void emit_reeval(const SolveArgs& a, const RoundBuf& sd, int64_t g,
-                                            const float4& pos, int pidx, int k,
+                                            const float4& pos, int k,
                                             const double (&l)[2][3], int id0, int id1,
                                             const bool (&dif)[2], const double lref[3]) {
-  const ProbDesc& pd = a.probs[pidx];
   const int nd = (dif[0] ? 1 : 0) + (k > 1 && dif[1] ? 1 : 0);
   const int nf = k - nd;
   auto lam4 = [&](const double* x) {
     return a.o.dim == 1 ? make_lam4(x[0], x[0], x[0]) : make_lam4(x[0], x[1], x[2]);
   };
   int64_t fs = 0, ds = 0;
-  if (nf > 0) fs = pd.qff_off + atomic_add_warp(sd.fq_cnt + pidx, nf);
-  if (nd > 0) ds = pd.qff_off + atomic_add_warp(sd.dq_cnt + pidx, nd);
+  if (nf > 0) fs = atomic_add_warp(sd.fq_cnt, nf);
+  if (nd > 0) ds = atomic_add_warp(sd.dq_cnt, nd);
   SI(a, I_RSLOT, g) = (int32_t)fs;
   SI(a, I_DSLOT, g) = (int32_t)ds;
   int tg = 0xffff;
@@ -596,6 +602,7 @@ __global__ void nm_step_kernel(const SolveArgs a) {
   constexpr int n = N;
   const PlanHdr h = *a.plan;
   PlanHdr hf{}, hd{};
+  if (!REF && a.rework && blockIdx.x == 0 && threadIdx.x == 0) a.rework[0] = a.rework[1] = 0;
   if (REF) {
     hf = *a.fplan;
     if (a.o.tie_dif > 0.0) hd = *a.dplan;
@@ -859,7 +866,7 @@ __global__ void nm_step_kernel(const SolveArgs a) {
           }
         }
       }
-      emit_reeval(a, REF ? a.nxt : a.cur, g, pos, pidx, k, lt, id0, id1, dif, lref);
+      emit_reeval(a, REF ? a.nxt : a.cur, g, pos, k, lt, id0, id1, dif, lref);
       if (single) store_e(a, g, e);
       if (rdirty) store_r(a, g, R);
       SI(a, I_FLAGS, g) = flags;
@@ -968,18 +975,17 @@ __global__ void plan_round_kernel(const PlanArgs a) {
     h.pad0 = 0;
     *a.plan = h;
     *a.work = 0;
-    // the plan of a float-float re-evaluation pass leaves the next round's counters alone
-    if (a.act_cnt_nxt) *a.act_cnt_nxt = 0;
-    if (a.near_cnt_nxt) *a.near_cnt_nxt = 0;
+    *a.act_cnt_nxt = 0;
+    *a.near_cnt_nxt = 0;
+    if (a.fq_cnt_nxt) *a.fq_cnt_nxt = 0;
+    if (a.dq_cnt_nxt) *a.dq_cnt_nxt = 0;
     if (a.ref_cnt_nxt) *a.ref_cnt_nxt = 0;
-    if (a.round_ctr) *a.round_ctr += 1;
-    if (a.stat_queries) *a.stat_queries += queries;
-    if (a.stat_pairs) *a.stat_pairs += pairs;
+    *a.round_ctr += 1;
+    *a.stat_queries += queries;
+    *a.stat_pairs += pairs;
   }
   for (int p = threadIdx.x; p < a.nprob; p += blockDim.x) {
     if (a.q_cnt_nxt) a.q_cnt_nxt[p] = 0;
-    if (a.fq_cnt_nxt) a.fq_cnt_nxt[p] = 0;
-    if (a.dq_cnt_nxt) a.dq_cnt_nxt[p] = 0;
   }
 }
 
@@ -1041,7 +1047,6 @@ void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* ms
 
 // Difference sums of n queries of one problem (slots 0..n-1) and their bounds (debug entry).
 __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
-                                 const int32_t* __restrict__ item_off,
                                  const double* __restrict__ out, const Lam4* __restrict__ qlam,
                                  const Lam4* __restrict__ qlam0, const double* __restrict__ msc,
                                  const double* __restrict__ msc0, int dim, double* dS,
@@ -1049,7 +1054,7 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   const PlanHdr h = *plan;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    for (int s = 0; s < 12; ++s) dS[12 * i + s] = gather_sum(out, h, item_off, 0, i, 12, s);
+    for (int s = 0; s < 12; ++s) dS[12 * i + s] = gather_slot(out, h, i, 12, s);
     if (dS_bound) {
       const double la[3] = {qlam[i].x, qlam[i].y, qlam[i].z};
       const double l0[3] = {qlam0[i].x, qlam0[i].y, qlam0[i].z};
@@ -1060,13 +1065,13 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   }
 }
 
-void launch_dif_debug(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
-                      const Lam4* qlam, const Lam4* qlam0, const double* msc, const double* msc0,
+void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const Lam4* qlam,
+                      const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s) {
   const int64_t nb = (n + 127) / 128;
   if (n > 0)
     dif_debug_kernel<<<(int)(nb < 1024 ? nb : 1024), 128, 0, s>>>(
-        n, plan, item_off, out, qlam, qlam0, msc, msc0, dim, dS, dS_bound);
+        n, plan, out, qlam, qlam0, msc, msc0, dim, dS, dS_bound);
 }
 
 // ------------------------------------------------------------------ certified B ----
@@ -1092,14 +1097,11 @@ __global__ void certb_flag_kernel(const SolveArgs a, double rel) {
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < a.N;
        g += (int64_t)gridDim.x * blockDim.x) {
     const float4 pos = a.ppos[g];
-    const int pidx = __float_as_int(pos.w);
     const double lam[3] = {a.res_lam[3 * g], a.res_lam[3 * g + 1], a.res_lam[3 * g + 2]};
     const double* B = a.res_B + 3 * g;
     const double nB = sqrt(B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
     if (!(mixed_b_bound(a.msc + 15 * g, lam, a.o.dim, (double)pos.z) > rel * nB)) continue;
-    const ProbDesc& pd = a.probs[pidx];
-    const int base = atomic_add_warp(a.cur.fq_cnt + pidx, 1);
-    const int64_t slot = pd.qff_off + base;
+    const int64_t slot = atomic_add_warp(a.cur.fq_cnt, 1);
     a.cur.fpos[slot] = pos;
     a.cur.flam[slot] = make_lam4(lam[0], lam[1], lam[2]);
     SI(a, I_RSLOT, g) = (int32_t)slot;
@@ -1117,11 +1119,10 @@ __global__ void certb_apply_kernel(const SolveArgs a) {
     const int pidx = __float_as_int(pos.w);
     const ProbDesc& pd = a.probs[pidx];
     const double z = (double)pos.z;
-    const int64_t j = (int64_t)SI(a, I_RSLOT, g) - pd.qff_off;
+    const int64_t slot = SI(a, I_RSLOT, g);
     const double* corr = corr_of(a, pd, g, z);
     for (int p = 0; p < 3; ++p)
-      a.res_B[3 * g + p] = z * gather_sum(a.fout, hf, a.fitem_off, pidx, j, 3, p) +
-                           (corr ? corr[p] : 0.0);
+      a.res_B[3 * g + p] = z * gather_slot(a.fout, hf, slot, 3, p) + (corr ? corr[p] : 0.0);
   }
 }
 

@@ -68,16 +68,16 @@ struct RoundBuf {
   int32_t* near;       // near-field query slots
   int32_t* near_cnt;   // [1]
   // certified decisions: float-float re-evaluation queries and the points that wait for them
-  float4* fpos;        // [2 N] slots (problem p from its qff_off)
+  float4* fpos;        // [2 N] slots, all problems in one queue
   Lam4* flam;
-  int32_t* fq_cnt;     // [nprob]
+  int32_t* fq_cnt;     // [1]
   int32_t* ref;        // waiting points
   int32_t* ref_cnt;    // [1]
-  // difference re-evaluation queries (value lambda, reference lambda; slots as fpos)
+  // difference re-evaluation queries (value lambda, reference lambda; a queue of the same kind)
   float4* dpos;
   Lam4* dlam;
   Lam4* dlam0;
-  int32_t* dq_cnt;     // [nprob]
+  int32_t* dq_cnt;     // [1]
 };
 
 struct SolveArgs {
@@ -109,12 +109,11 @@ struct SolveArgs {
   // certified decisions
   const double* msc;         // [N * 15] sum_k |b_pk| / r^j, j = 1..5, per component (or null)
   const double* msc0;        // [N * 3] sum_k |b_pk| per component (difference level)
-  const double* fout;        // float-float pass partial sums of the current round
+  const double* fout;        // float-float sums of the current round, [slot][split][12]
   const PlanHdr* fplan;
-  const int32_t* fitem_off;
-  const double* dout;        // difference pass partial sums of the current round
+  const double* dout;        // difference sums of the current round
   const PlanHdr* dplan;
-  const int32_t* ditem_off;
+  int32_t* rework;           // item counters (2) of the re-evaluation pass, zeroed by each step
   unsigned long long* stat_ties;   // near-tie decisions sent to re-evaluation (or null)
   unsigned long long* stat_difs;   // values re-evaluated by difference (or null)
 };
@@ -133,8 +132,8 @@ struct PlanArgs {
   int32_t* q_cnt_nxt;        // zeroed
   int32_t* act_cnt_nxt;
   int32_t* near_cnt_nxt;
-  int32_t* fq_cnt_nxt;       // zeroed (certified decisions; may be null)
-  int32_t* dq_cnt_nxt;       // zeroed (difference level; may be null)
+  int32_t* fq_cnt_nxt;       // [1] zeroed (certified decisions; may be null)
+  int32_t* dq_cnt_nxt;       // [1] zeroed (difference level; may be null)
   int32_t* ref_cnt_nxt;
   int32_t* round_ctr;        // incremented per round
   unsigned long long* stat_queries;
