@@ -1383,8 +1383,9 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
 
   DBIE_TRY(ensure(b.probs, sizeof(ProbDesc) * nprob));
   DBIE_TRY(ensure(b.ppos, sizeof(float4) * N));
-  DBIE_TRY(ensure(b.sd, sizeof(double) * D_NFIELDS * N));
-  DBIE_TRY(ensure(b.si, sizeof(int32_t) * I_NFIELDS * N));
+  const int64_t N32 = (N + 31) / 32 * 32;
+  DBIE_TRY(ensure(b.sd, sizeof(double) * D_NFIELDS * N32));
+  DBIE_TRY(ensure(b.si, sizeof(int32_t) * I_NFIELDS * N32));
   DBIE_TRY(ensure(b.q_cnt_pass, sizeof(int32_t) * nprob));
   DBIE_TRY(ensure(b.item_off, sizeof(int32_t) * (nprob + 1)));
   DBIE_TRY(ensure(b.ctrl, sizeof(SolveCtrl)));
@@ -1511,6 +1512,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     a = SolveArgs{};
     a.probs = b.probs.as<ProbDesc>();
     a.nprob = nprob;
+    a.nsm = c->sm_count;
     a.N = N;
     a.ppos = b.ppos.as<float4>();
     a.sd = b.sd.as<double>();
@@ -1560,7 +1562,9 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   }
   // Initial simplex and its queries go to side 0.
   SolveArgs a0 = sa[1];  // "next" of the side-1 round is side 0
-  const int nm_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
+  // step kernels: CTAs of one warp, full residency at their register count
+  const int nm_grid = (int)std::min<int64_t>(N, 8LL * c->sm_count);
+  const int apply_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
   (qn ? launch_bfgs_init : launch_solve_init)(a0, any_init ? b.lam0.as<double>() : nullptr,
                     (int)std::min<int64_t>((N + 255) / 256, 8LL * c->sm_count), s);
   CUDA_TRY(cudaGetLastError());
@@ -1746,7 +1750,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     ReArgs rv = reeval_args(0);
     rv.stat_ff_pairs = nullptr;
     DBIE_TRY(launch_kernel(kv, grid_v, &rv, s));
-    launch_certb_apply(sa[0], nm_grid, s);
+    launch_certb_apply(sa[0], apply_grid, s);
     CUDA_TRY(cudaGetLastError());
     DBIE_TRY(check_device_error(c, s));
   }

@@ -155,83 +155,40 @@ void launch_finalize_eval(int var, int64_t n, const PlanHdr* plan, const int32_t
 }
 
 // ------------------------------------------------------------------ simplex state ----
-// A vertex (or the reflected or trial point) of one point's simplex: lambda, the field and
-// objective there, the error bound s of its Phi (0 after a float-float re-evaluation) and its
-// identity in the state the step started from (0..n vertex, VID_R reflected, VID_E trial).
-struct Vert {
-  double l[3];
-  double B[3];
-  double f, g, phi;
-  double s;
-  int id;
-};
-
+// (blocks of 32 points: coalesced over neighbouring points, and every field of a point is at a
+// constant offset from its first, so an access needs no address arithmetic)
 __device__ __forceinline__ double& SD(const SolveArgs& a, int f, int64_t g) {
-  return a.sd[(int64_t)f * a.N + g];
+  return a.sd[(g >> 5) * (int64_t)(D_NFIELDS * 32) + (g & 31) + f * 32];
 }
 __device__ __forceinline__ int32_t& SI(const SolveArgs& a, int f, int64_t g) {
-  return a.si[(int64_t)f * a.N + g];
+  return a.si[(g >> 5) * (int64_t)(I_NFIELDS * 32) + (g & 31) + f * 32];
 }
 
-__device__ __forceinline__ void load_vert(const SolveArgs& a, int64_t g, int v, Vert& x) {
-  for (int d = 0; d < 3; ++d) x.l[d] = SD(a, D_VL + v * 3 + d, g);
-  for (int p = 0; p < 3; ++p) x.B[p] = SD(a, D_VB + v * 3 + p, g);
-  x.f = SD(a, D_VF + v, g);
-  x.g = SD(a, D_VG + v, g);
-  x.phi = SD(a, D_VPHI + v, g);
-  x.s = SD(a, D_VS + v, g);
-  x.id = v;
+// Field f of value record id (vertex slot, VID_R, VID_E) of point g.
+__device__ __forceinline__ double& SV(const SolveArgs& a, int id, int f, int64_t g) {
+  return SD(a, id * VREC + f, g);
 }
-__device__ __forceinline__ void store_vert(const SolveArgs& a, int64_t g, int v, const Vert& x) {
-  for (int d = 0; d < 3; ++d) SD(a, D_VL + v * 3 + d, g) = x.l[d];
-  for (int p = 0; p < 3; ++p) SD(a, D_VB + v * 3 + p, g) = x.B[p];
-  SD(a, D_VF + v, g) = x.f;
-  SD(a, D_VG + v, g) = x.g;
-  SD(a, D_VPHI + v, g) = x.phi;
-  SD(a, D_VS + v, g) = x.s;
+__device__ __forceinline__ void store_value(const SolveArgs& a, int id, int64_t g, const Eval& e) {
+  for (int p = 0; p < 3; ++p) SV(a, id, V_B + p, g) = e.B[p];
+  SV(a, id, V_F, g) = e.f;
+  SV(a, id, V_G, g) = e.g;
+  SV(a, id, V_PHI, g) = e.phi;
+  SV(a, id, V_S, g) = e.s;
 }
-// The reflected point (lambda at D_RL, value at D_RB..D_RPHI, bound at D_RS).
-__device__ __forceinline__ void load_r(const SolveArgs& a, int64_t g, Vert& x) {
-  for (int d = 0; d < 3; ++d) x.l[d] = SD(a, D_RL + d, g);
-  for (int p = 0; p < 3; ++p) x.B[p] = SD(a, D_RB + p, g);
-  x.f = SD(a, D_RF, g);
-  x.g = SD(a, D_RG, g);
-  x.phi = SD(a, D_RPHI, g);
-  x.s = SD(a, D_RS, g);
-  x.id = VID_R;
+__device__ __forceinline__ void copy_value(const SolveArgs& a, int from, int to, int64_t g) {
+  double v[VREC];
+#pragma unroll
+  for (int f = 0; f < VREC; ++f) v[f] = SV(a, from, f, g);
+#pragma unroll
+  for (int f = 0; f < VREC; ++f) SV(a, to, f, g) = v[f];
 }
-__device__ __forceinline__ void store_r(const SolveArgs& a, int64_t g, const Vert& x) {
-  for (int d = 0; d < 3; ++d) SD(a, D_RL + d, g) = x.l[d];
-  for (int p = 0; p < 3; ++p) SD(a, D_RB + p, g) = x.B[p];
-  SD(a, D_RF, g) = x.f;
-  SD(a, D_RG, g) = x.g;
-  SD(a, D_RPHI, g) = x.phi;
-  SD(a, D_RS, g) = x.s;
-}
-// The evaluated single trial point (lambda at D_TL, value at D_EB..D_ES).
-__device__ __forceinline__ void load_e(const SolveArgs& a, int64_t g, Vert& x) {
-  for (int d = 0; d < 3; ++d) x.l[d] = SD(a, D_TL + d, g);
-  for (int p = 0; p < 3; ++p) x.B[p] = SD(a, D_EB + p, g);
-  x.f = SD(a, D_EF, g);
-  x.g = SD(a, D_EG, g);
-  x.phi = SD(a, D_EPHI, g);
-  x.s = SD(a, D_ES, g);
-  x.id = VID_E;
-}
-__device__ __forceinline__ void store_e(const SolveArgs& a, int64_t g, const Vert& x) {
-  for (int p = 0; p < 3; ++p) SD(a, D_EB + p, g) = x.B[p];
-  SD(a, D_EF, g) = x.f;
-  SD(a, D_EG, g) = x.g;
-  SD(a, D_EPHI, g) = x.phi;
-  SD(a, D_ES, g) = x.s;
-}
-__device__ __forceinline__ void set_value(Vert& x, const Eval& e) {
-  for (int p = 0; p < 3; ++p) x.B[p] = e.B[p];
-  x.f = e.f;
-  x.g = e.g;
-  x.phi = e.phi;
-  x.s = e.s;
-}
+
+// What a step compares: Phi, its error bound s, the vertex's storage slot and the record that
+// holds the value (the slot, or VID_R / VID_E for a value that is about to take the slot's place).
+struct Vert {
+  double phi, s;
+  int slot, id;
+};
 
 // The pixel-exact correction of point g, or null (none, or the point is above its height).
 __device__ __forceinline__ const double* corr_of(const SolveArgs& a, const ProbDesc& pd,
@@ -392,44 +349,42 @@ __device__ __forceinline__ void read_eval(const SolveArgs& a, const PlanHdr& h, 
                                           int64_t slot, double z, Eval& e, int64_t g,
                                           const double lam[3]) {
   const ProbDesc& pd = a.probs[pidx];
-  const int64_t j = slot - pd.q_off;
   double S[12], G[9];
 #pragma unroll
-  for (int s = 0; s < 12; ++s) S[s] = gather_sum(a.out, h, a.item_off, pidx, j, 12, s);
+  for (int s = 0; s < 12; ++s)
+    S[s] = gather_sum(a.out, h, a.item_off, pidx, slot - pd.q_off, 12, s);
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
   e.s = (a.o.tie > 0.0 && a.msc)
             ? mixed_phi_bound(a.msc + 15 * g, lam, a.o.dim, z, e.B, G, e.g, pd.g_scale, a.o.w_g)
             : 0.0;
 }
 
-// Objective of a float-float re-evaluation slot of point g (bound 0) and its 12 sums.
-__device__ __forceinline__ void read_eval_ff(const SolveArgs& a, const PlanHdr& hf, int pidx,
-                                             int64_t slot, double z, Eval& e, int64_t g,
-                                             double S[12]) {
+// Objective of a re-evaluated value of point g at lambda lt and its 12 sums: float-float sums
+// (bound 0), or (dif) the point's float-float reference sums plus difference sums, with the bound
+// stored negated (a difference value).  One site for both kinds: lanes of a warp whose values
+// are of different kinds run the FP64 objective together.
+__device__ __forceinline__ void read_reeval(const SolveArgs& a, bool dif, int pidx, int64_t slot,
+                                            double z, Eval& e, int64_t g, const double lt[3],
+                                            double S[12]) {
   const ProbDesc& pd = a.probs[pidx];
+  const double* out = dif ? a.dout : a.fout;
+  const PlanHdr h = dif ? *a.dplan : *a.fplan;
   double G[9];
 #pragma unroll
-  for (int s = 0; s < 12; ++s) S[s] = gather_slot(a.fout, hf, slot, 12, s);
+  for (int s = 0; s < 12; ++s) S[s] = gather_slot(out, h, slot, 12, s);
+  if (dif) {
+#pragma unroll
+    for (int s = 0; s < 12; ++s) S[s] = SD(a, D_REFS + s, g) + S[s];
+  }
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
   e.s = 0.0;
-}
-
-// Objective of a difference re-evaluation slot of point g at lambda lt: the point's float-float
-// reference sums plus the difference sums; its bound is stored negated (a difference value).
-__device__ __forceinline__ void read_eval_dif(const SolveArgs& a, const PlanHdr& hd, int pidx,
-                                              int64_t slot, double z, Eval& e, int64_t g,
-                                              const double lt[3]) {
-  const ProbDesc& pd = a.probs[pidx];
-  double S[12], G[9];
-#pragma unroll
-  for (int s = 0; s < 12; ++s)
-    S[s] = SD(a, D_REFS + s, g) + gather_slot(a.dout, hd, slot, 12, s);
-  assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
-  const double l0[3] = {SD(a, D_REFL, g), SD(a, D_REFL + 1, g), SD(a, D_REFL + 2, g)};
-  double eb[12];
-  dif_sum_bounds(a.msc + 15 * g, a.msc0 + 3 * g, lt, l0, a.o.dim, eb);
-  const double sd = dif_phi_bound(eb, z, e.B, G, e.g, pd.g_scale, a.o.w_g);
-  e.s = -(sd > 0.0 ? sd : 1e-300);
+  if (dif) {
+    const double l0[3] = {SD(a, D_REFL, g), SD(a, D_REFL + 1, g), SD(a, D_REFL + 2, g)};
+    double eb[12];
+    dif_sum_bounds(a.msc + 15 * g, a.msc0 + 3 * g, lt, l0, a.o.dim, eb);
+    const double sd = dif_phi_bound(eb, z, e.B, G, e.g, pd.g_scale, a.o.w_g);
+    e.s = -(sd > 0.0 ? sd : 1e-300);
+  }
 }
 
 // atomicAdd(ctr, v) for the lanes of a warp that reach it together (whatever branch they are
@@ -503,10 +458,11 @@ __device__ __forceinline__ void emit_reeval(const SolveArgs& a, const RoundBuf& 
   if (nd > 0) ds = atomic_add_warp(sd.dq_cnt, nd);
   SI(a, I_RSLOT, g) = (int32_t)fs;
   SI(a, I_DSLOT, g) = (int32_t)ds;
-  int tg = 0xffff;
+  int tg = 0xffff, nt = 0;
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    if (j >= k) break;
+  for (int it = 0; it < 4; ++it) {   // differences first
+    const int j = it & 1;
+    if (j >= k || dif[j] != (it < 2)) continue;
     const int id = j == 0 ? id0 : id1;
     if (dif[j]) {
       sd.dpos[ds] = pos;
@@ -518,7 +474,8 @@ __device__ __forceinline__ void emit_reeval(const SolveArgs& a, const RoundBuf& 
       sd.flam[fs] = lam4(l[j]);
       ++fs;
     }
-    tg = (tg & ~(0xff << (8 * j))) | (((id | (dif[j] ? RT_DIF : 0)) & 0xff) << (8 * j));
+    const int sh = 8 * nt++;
+    tg = (tg & ~(0xff << sh)) | (((id | (dif[j] ? RT_DIF : 0)) & 0xff) << sh);
   }
   SI(a, I_RTGT, g) = tg;
   sd.ref[atomic_add_warp(sd.ref_cnt, 1)] = (int32_t)g;
@@ -545,12 +502,12 @@ __global__ void solve_init_kernel(const SolveArgs a, const double* __restrict__ 
 #pragma unroll
     for (int v = 0; v <= n; ++v)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) SD(a, D_VL + v * 3 + d, g) = lam[v][d];
+      for (int d = 0; d < 3; ++d) SV(a, v, V_L + d, g) = lam[v][d];
     SI(a, I_STAGE, g) = ST_INIT;
     SI(a, I_ITERS, g) = 0;
     SI(a, I_NFEV, g) = 0;
     SI(a, I_STATUS, g) = PT_RUNNING;
-    SI(a, I_FLAGS, g) = 0;
+    SI(a, I_ORDER, g) = 0x3210;
     if (a.o.tie_dif > 0.0) SD(a, D_REFS, g) = __longlong_as_double(0x7ff8000000000000LL);  // NaN
     emit<N + 1>(a, g, pos, pidx, lam);
   }
@@ -562,7 +519,7 @@ void launch_solve_init(const SolveArgs& a, const double* lam_init, int grid, cud
 }
 
 // Stable insertion sort of the N+1 vertices by Phi (ties keep their order), unrolled into
-// adjacent compare-exchanges so the vertices stay in registers.  Without the early exit of the
+// adjacent compare-exchanges so their keys stay in registers.  Without the early exit of the
 // textbook loop the result is the same: after inserting each vertex no adjacent pair of the
 // sorted prefix is out of order (v[j].phi < v[j-1].phi false), so the comparisons below the
 // insertion point never swap.  The insertion's own comparisons (those down to the insertion
@@ -586,150 +543,156 @@ __device__ __forceinline__ void sort_verts(Vert* v, TieLog& tl) {
   }
 }
 
+// Points of one warp of a step kernel (CTAs of one warp).  The steps are FP64: an SM's FP64 pipe
+// takes 16 cycles per warp instruction, so a few points are spread over all SMs, one warp each,
+// with as few lanes (fewer of them in different stages) as that needs; full warps come when there
+// are more than 32 points per SM.
+__device__ __forceinline__ int points_per_warp(int n, int nsm) {
+  const int p = (n + nsm - 1) / nsm;
+  return p < 1 ? 1 : (p > 32 ? 32 : p);
+}
+
 // One simplex step per waiting point.  REF = false: the points whose queries the mixed pass of
 // this round evaluated (their results are read and their bounds computed); REF = true: the
-// points whose near-tied values the float-float pass of this round re-evaluated (the values are
-// replaced, bound 0, and the step is decided again).  A step is taken only when none of its
-// comparisons is a near tie (TieLog); otherwise the step's inputs stay in the state and the
-// near-tied values are queued for float-float re-evaluation, so every decision is the one that
-// sums accurate to the float-float level would take.  With a.o.tie == 0 every step is taken as
-// evaluated.
+// points whose near-tied values this round's re-evaluation pass computed (the values are
+// replaced, and the step is decided again).  A step is taken only when none of its comparisons is
+// a near tie (TieLog); otherwise the near-tied values are queued for re-evaluation and the state
+// stays as it is, so every decision is the one that sums accurate to the float-float level would
+// take.  With a.o.tie == 0 every step is taken as evaluated.
+//
+// What bounds it: the latency of one warp's instructions (about 11 cycles each; the FP64 pipe is
+// less than a quarter busy), so the time is the instruction count of the longest warp.  Hence two
+// phases.  First the lanes share out the values to compute, one FP64 objective and bound per lane
+// whatever the points' stages (a shrink has 3, the start 4; taken in turn by the point's own lane
+// they set the length for the whole warp).  Then each lane decides its point's step on Phi and
+// bound alone; vertices stay in their slots, and a step writes one record, not four.  On 2,048
+// points a step took 63 us (the waiting points' 112 us) with one lane per point evaluating and
+// sorting whole vertices, in CTAs of 128 threads.
 template <int N, bool REF>
-__global__ void nm_step_kernel(const SolveArgs a) {
+__global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
   const double rho = 1.0, chi = 2.0, psi = 0.5, sigma = 0.5;
+  const unsigned FULL = 0xffffffffu;
   const int nact = REF ? *a.cur.ref_cnt : *a.cur.act_cnt;
   const int32_t* list = REF ? a.cur.ref : a.cur.act;
   constexpr int n = N;
   const PlanHdr h = *a.plan;
-  PlanHdr hf{}, hd{};
   if (!REF && a.rework && blockIdx.x == 0 && threadIdx.x == 0) a.rework[0] = a.rework[1] = 0;
-  if (REF) {
-    hf = *a.fplan;
-    if (a.o.tie_dif > 0.0) hd = *a.dplan;
-  }
-  for (int ia = blockIdx.x * blockDim.x + threadIdx.x; ia < nact; ia += gridDim.x * blockDim.x) {
-    const int64_t g = list[ia];
+  const int ppw = points_per_warp(nact, a.nsm);
+  const int lane = threadIdx.x;
+  for (int base = blockIdx.x * ppw; base < nact; base += gridDim.x * ppw) {
+    const bool on = lane < ppw && base + lane < nact;
+    const int gi = on ? list[base + lane] : 0;
+    const int64_t g = gi;
+    int stage = ST_DONE, order = 0, targets = 0xffff, nev = 0;
+    int slot0 = 0, slot1 = 0;   // first query slot (REF: float-float and difference slot)
+    if (on) {
+      stage = SI(a, I_STAGE, g);
+      order = SI(a, I_ORDER, g);
+      if (REF) {
+        targets = SI(a, I_RTGT, g);
+        slot0 = SI(a, I_RSLOT, g);
+        slot1 = SI(a, I_DSLOT, g);
+        nev = (targets >> 8) == 0xff ? 1 : 2;
+      } else {
+        slot0 = SI(a, I_QSLOT, g);
+        nev = stage == ST_INIT ? n + 1 : (stage == ST_SHRINK ? n : 1);
+      }
+    }
+
+    // ---- phase 1: value q of the warp's points, by lane q
+    int incl = nev;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(FULL, incl, off);
+      if (lane >= off) incl += t;
+    }
+    const int total = __shfl_sync(FULL, incl, 31);
+    for (int q0 = 0; q0 < total; q0 += 32) {
+      const int q = q0 + lane;
+      int o = 0;   // the point (lane) that owns value q: the first with incl > q
+#pragma unroll
+      for (int st = 16; st > 0; st >>= 1)
+        if (__shfl_sync(FULL, incl, o + st - 1) <= q) o += st;
+      const int k = q - (__shfl_sync(FULL, incl, o) - __shfl_sync(FULL, nev, o));
+      const int64_t og = __shfl_sync(FULL, gi, o);
+      const int ostage = __shfl_sync(FULL, stage, o), oorder = __shfl_sync(FULL, order, o);
+      const int otg = __shfl_sync(FULL, targets, o);
+      const int os0 = __shfl_sync(FULL, slot0, o), os1 = __shfl_sync(FULL, slot1, o);
+      double S[12];
+      bool newref = false;
+      if (q < total) {
+        const float4 pos = a.ppos[og];
+        const int pidx = __float_as_int(pos.w);
+        Eval ev;
+        int id;
+        bool dif = false;
+        if (REF) {
+          const int code = (otg >> (8 * k)) & 0xff;
+          dif = (code & RT_DIF) != 0;
+          id = code & ~RT_DIF;
+        } else {
+          id = ostage == ST_INIT ? k : (ostage == ST_SHRINK ? (oorder >> (4 * (k + 1))) & 15 : VID_E);
+        }
+        const double lq[3] = {SV(a, id, V_L, og), SV(a, id, V_L + 1, og), SV(a, id, V_L + 2, og)};
+        if (REF) {
+          // (targets: differences first, each kind in consecutive slots)
+          const int nd = ((otg & RT_DIF) ? 1 : 0) + ((otg >> 8) != 0xff && (otg & (RT_DIF << 8)) ? 1 : 0);
+          read_reeval(a, dif, pidx, dif ? os1 + k : os0 + (k - nd), (double)pos.z, ev, og, lq, S);
+          // the last float-float value becomes the point's reference
+          newref = !dif && a.o.tie_dif > 0.0 && (k == 1 || (otg >> 8) == 0xff);
+        } else {
+          read_eval(a, h, pidx, os0 + k, (double)pos.z, ev, og, lq);
+        }
+        store_value(a, id, og, ev);
+        if (newref)
+          for (int d = 0; d < 3; ++d) SD(a, D_REFL + d, og) = lq[d];
+      }
+      __syncwarp();   // the differences have read the old reference sums
+      if (newref)
+        for (int s = 0; s < 12; ++s) SD(a, D_REFS + s, og) = S[s];
+    }
+    __syncwarp();     // values are in the state
+    if (!on) continue;
+
+    // ---- phase 2: the step of the lane's point
     const float4 pos = a.ppos[g];
     const int pidx = __float_as_int(pos.w);
-    const double z = (double)pos.z;
-    int stage = SI(a, I_STAGE, g);
     int iters = SI(a, I_ITERS, g);
-    int nfev = SI(a, I_NFEV, g);
-    int flags = SI(a, I_FLAGS, g);
+    int nfev = SI(a, I_NFEV, g) + (REF ? 0 : nev);
     const bool single = stage != ST_INIT && stage != ST_SHRINK;
-
-    Vert v[N + 1];
+    Vert w[N + 1], e{0.0, 0.0, 0, VID_E}, R{0.0, 0.0, 0, VID_R};
 #pragma unroll
-    for (int k = 0; k <= n; ++k) load_vert(a, g, k, v[k]);
-    Vert e, R;
-    e.id = VID_E;
-    R.id = VID_R;
-    bool vdirty = false, rdirty = false;
-
-    if (!(flags & F_EVAL)) {
-      // The pending queries' objectives, evaluated at one site for every stage: a warp whose
-      // lanes are in different stages runs the FP64 objective once per query index instead of
-      // once per stage.  The initial simplex (n + 1 queries into vertices 0..n) and a shrink
-      // (n queries into vertices 1..n) fill vertices by shifting each result in at the top (no
-      // run-time vertex index, so they stay in registers); the other stages read one trial point.
-      const int64_t slot = SI(a, I_QSLOT, g);
-      const int nev = stage == ST_INIT ? n + 1 : (stage == ST_SHRINK ? n : 1);
-      const int first = stage == ST_SHRINK ? 1 : 0;
-      for (int d = 0; d < 3; ++d) e.l[d] = single ? SD(a, D_TL + d, g) : 0.0;
-#pragma unroll 1
-      for (int k = 0; k < nev; ++k) {
-        double lq[3];   // the query's lambda (read back from the state: a register-array
-                        // index that depends on k would move the vertices to local memory)
-        for (int d = 0; d < 3; ++d)
-          lq[d] = single ? e.l[d] : SD(a, D_VL + 3 * (first + k) + d, g);
-        Eval ev;
-        read_eval(a, h, pidx, slot + k, z, ev, g, lq);
-        if (!single) {
-#pragma unroll
-          for (int m = 0; m < n; ++m)
-            if (m >= first) {
-              for (int p = 0; p < 3; ++p) v[m].B[p] = v[m + 1].B[p];
-              v[m].f = v[m + 1].f; v[m].g = v[m + 1].g; v[m].phi = v[m + 1].phi;
-              v[m].s = v[m + 1].s;
-            }
-          set_value(v[n], ev);
-        } else {
-          set_value(e, ev);
-        }
-      }
-      nfev += nev;
-      vdirty = !single;
-      flags |= F_EVAL;
-    } else if (single) {
-      load_e(a, g, e);
+    for (int k = 0; k <= n; ++k) {
+      const int sl = (order >> (4 * k)) & 15;
+      w[k] = Vert{SV(a, sl, V_PHI, g), SV(a, sl, V_S, g), sl, sl};
     }
-    if (stage == ST_EXPAND || stage == ST_OCONTRACT) load_r(a, g, R);
-    if (REF) {
-      // apply the re-evaluated values of this point's targets: the differences first (they
-      // were queued against the current reference), then the float-float values, each of which
-      // becomes the point's reference
-      const int tg = SI(a, I_RTGT, g);
-      int64_t slot[2] = {SI(a, I_RSLOT, g), SI(a, I_DSLOT, g)};
-#pragma unroll 1
-      for (int it = 0; it < 4; ++it) {
-        const int t = it & 1;
-        const int code = (tg >> (8 * t)) & 0xff;
-        if (code == 0xff) continue;
-        const bool dif = (code & RT_DIF) != 0;
-        if (dif != (it < 2)) continue;
-        const int id = code & ~RT_DIF;
-        Eval ev;
-        double lt[3];
-        for (int d = 0; d < 3; ++d)
-          lt[d] = id == VID_E ? e.l[d] : (id == VID_R ? R.l[d] : SD(a, D_VL + 3 * id + d, g));
-        if (dif) {
-          read_eval_dif(a, hd, pidx, slot[1]++, z, ev, g, lt);
-        } else {
-          double S[12];
-          read_eval_ff(a, hf, pidx, slot[0]++, z, ev, g, S);
-          if (a.o.tie_dif > 0.0) {
-            for (int d = 0; d < 3; ++d) SD(a, D_REFL + d, g) = lt[d];
-            for (int s = 0; s < 12; ++s) SD(a, D_REFS + s, g) = S[s];
-          }
-        }
-        if (id == VID_E) {
-          set_value(e, ev);
-        } else if (id == VID_R) {
-          set_value(R, ev);
-          rdirty = true;
-        } else {
-#pragma unroll
-          for (int k = 0; k <= n; ++k)
-            if (k == id) set_value(v[k], ev);
-          vdirty = true;
-        }
-      }
+    if (single) {
+      e.phi = SV(a, VID_E, V_PHI, g);
+      e.s = SV(a, VID_E, V_S, g);
     }
-
-    // ---- the step.  With certified decisions the vertices the step starts from are in memory
-    // first (the step may turn out to wait), and nothing else is written until the step is
-    // known to be certain.
+    if (stage == ST_EXPAND || stage == ST_OCONTRACT) {
+      R.phi = SV(a, VID_R, V_PHI, g);
+      R.s = SV(a, VID_R, V_S, g);
+    }
     TieLog tl{a.o.tie, a.o.tie_dif, -1, -1};
-    if (vdirty && a.o.tie > 0.0)
-#pragma unroll
-      for (int m = 0; m <= n; ++m) store_vert(a, g, m, v[m]);
-    Vert (&w)[N + 1] = v;
-    bool to_check = false, accepted = false, store_R = false, emit_shrink = false;
-    bool emit_trial = false, mirror = false;
+    bool to_check = false, store_R = false, emit_shrink = false, emit_trial = false;
+    bool mirror = false;
     int next_stage = stage;
-    double xt[3] = {0.0, 0.0, 0.0};
+    int taken = -1;                      // record that takes the worst vertex's slot
+    double coef_c = 0.0, coef_w = 0.0;   // next trial point: coef_c centroid + coef_w worst
     char code = 0;
     int fin = -1;
-    auto trial = [&](double coef_c, double coef_w, double out[3]) {  // coef_c c + coef_w w[n]
-      double c[3];
-#pragma unroll
-      for (int d = 0; d < n; ++d) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < n; ++k) s += w[k].l[d];
-        c[d] = s / n;
-      }
-      for (int d = 0; d < 3; ++d) out[d] = (d < n) ? coef_c * c[d] + coef_w * w[n].l[d] : 0.0;
+    auto trial = [&](double cc, double cw) {
+      coef_c = cc;
+      coef_w = cw;
+      emit_trial = true;
+    };
+    auto take = [&](const Vert& x, char c) {
+      w[n].phi = x.phi;
+      w[n].s = x.s;
+      w[n].id = taken = x.id;
+      code = c;
+      to_check = true;
     };
 
     if (stage == ST_INIT) {
@@ -737,46 +700,26 @@ __global__ void nm_step_kernel(const SolveArgs a) {
     } else if (stage == ST_REFLECT) {
       if (tl.lt(e, w[0])) {
         store_R = true;
-        trial(1.0 + rho * chi, -(rho * chi), xt);
+        trial(1.0 + rho * chi, -(rho * chi));
         next_stage = ST_EXPAND;
-        emit_trial = true;
       } else if (tl.lt(e, w[n - 1])) {
-        w[n] = e;
-        accepted = true;
-        code = 'R';
-        to_check = true;
+        take(e, 'R');
       } else if (tl.lt(e, w[n])) {
         store_R = true;
-        trial(1.0 + psi * rho, -(psi * rho), xt);
+        trial(1.0 + psi * rho, -(psi * rho));
         next_stage = ST_OCONTRACT;
-        emit_trial = true;
       } else {
-        trial(1.0 - psi, psi, xt);
+        trial(1.0 - psi, psi);
         next_stage = ST_ICONTRACT;
-        emit_trial = true;
       }
     } else if (stage == ST_EXPAND) {
-      if (tl.lt(e, R)) {
-        w[n] = e;
-        code = 'E';
-      } else {
-        w[n] = R;
-        code = 'R';
-      }
-      accepted = true;
-      to_check = true;
+      if (tl.lt(e, R)) take(e, 'E');
+      else take(R, 'R');
     } else if (stage == ST_OCONTRACT || stage == ST_ICONTRACT) {
       const bool ok = (stage == ST_OCONTRACT) ? tl.le(e, R) : tl.lt(e, w[n]);
       if (ok) {
-        w[n] = e;
-        accepted = true;
-        code = (stage == ST_OCONTRACT) ? 'O' : 'I';
-        to_check = true;
+        take(e, (stage == ST_OCONTRACT) ? 'O' : 'I');
       } else {
-#pragma unroll
-        for (int k = 1; k <= n; ++k)
-          for (int d = 0; d < 3; ++d)
-            w[k].l[d] = (d < n) ? w[0].l[d] + sigma * (w[k].l[d] - w[0].l[d]) : 0.0;
         next_stage = ST_SHRINK;
         emit_shrink = true;
       }
@@ -787,9 +730,10 @@ __global__ void nm_step_kernel(const SolveArgs a) {
     if (to_check) {
       sort_verts<N>(w, tl);
       // Eq. 12 at the best vertex, then the value spread, then the iteration count
-      tl.note(w[0].id, w[0].s, -1, 0.0, w[0].f - a.o.eps_f);
-      if (w[0].f <= a.o.eps_f) tl.note(w[0].id, w[0].s, -1, 0.0, w[0].g - a.o.eps_g);
-      if (w[0].f <= a.o.eps_f && w[0].g <= a.o.eps_g) {
+      const double f0 = SV(a, w[0].id, V_F, g), g0 = SV(a, w[0].id, V_G, g);
+      tl.note(w[0].id, w[0].s, -1, 0.0, f0 - a.o.eps_f);
+      if (f0 <= a.o.eps_f) tl.note(w[0].id, w[0].s, -1, 0.0, g0 - a.o.eps_g);
+      if (f0 <= a.o.eps_f && g0 <= a.o.eps_g) {
         fin = PT_CONVERGED;
       } else {
         tl.note(w[n].id, w[n].s, w[0].id, w[0].s, w[n].phi - w[0].phi - a.o.tol);
@@ -797,35 +741,32 @@ __global__ void nm_step_kernel(const SolveArgs a) {
         else if (iters >= a.o.max_iter) fin = PT_MAXITER;
       }
       if (fin < 0) {
-        if (n == 1 && w[0].l[0] == 0.0) {
+        if (n == 1 && SV(a, w[0].id, V_L, g) == 0.0) {
           // Mirror step: with the best vertex at lambda = 0 the reflection is -w[1], where Phi
           // (even in lambda, Eq. 6) takes w[1]'s value exactly.  Its comparisons are settled
           // (not below w[0], by the sort just done; not below w[1], by equality), so the step
           // goes straight to the inside contraction, and the reflection is counted as the
           // evaluation the search makes.  Every form then decides these exact ties as exact
           // arithmetic does, instead of by the rounding of two sums.
-          trial(1.0 - psi, psi, xt);
+          trial(1.0 - psi, psi);
           next_stage = ST_ICONTRACT;
           mirror = true;
         } else {
-          trial(1.0 + rho, -rho, xt);
+          trial(1.0 + rho, -rho);
           next_stage = ST_REFLECT;
         }
-        emit_trial = true;
       }
     }
 
     if (tl.a >= 0) {
-      // near tie: keep the step's inputs and re-evaluate the near-tied values in float-float
-      // (tl.a >= 0 always; tl.b >= 0 when both values carry a bound).  A vertex target's lambda
-      // comes from the stored state the step started from.
+      // near tie: keep the state and re-evaluate the near-tied values (tl.a >= 0 always;
+      // tl.b >= 0 when both values carry a bound)
       double lt[2][3];
       const int ida = tl.a, idb = tl.b;
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        lt[0][d] = ida == VID_E ? e.l[d] : (ida == VID_R ? R.l[d] : SD(a, D_VL + 3 * ida + d, g));
-        lt[1][d] = idb < 0 ? 0.0 : idb == VID_E ? e.l[d]
-                 : (idb == VID_R ? R.l[d] : SD(a, D_VL + 3 * idb + d, g));
+        lt[0][d] = SV(a, ida, V_L + d, g);
+        lt[1][d] = idb < 0 ? 0.0 : SV(a, idb, V_L + d, g);
       }
       // A value goes to the difference pass when the point has a float-float reference, the
       // value still carries its mixed-form bound and it lies near the reference (the difference
@@ -839,24 +780,21 @@ __global__ void nm_step_kernel(const SolveArgs a) {
       bool dif[2] = {false, false};
       double lref[3] = {0.0, 0.0, 0.0};
       if (a.o.tie_dif > 0.0) {
-        const double sv[2] = {
-            ida == VID_E ? e.s : (ida == VID_R ? R.s : SD(a, D_VS + ida, g)),
-            idb < 0 ? 0.0 : idb == VID_E ? e.s : (idb == VID_R ? R.s : SD(a, D_VS + idb, g))};
+        const double sv[2] = {SV(a, ida, V_S, g), idb < 0 ? 0.0 : SV(a, idb, V_S, g)};
         if (!isnan(SD(a, D_REFS, g))) {
 #pragma unroll
           for (int d = 0; d < 3; ++d) lref[d] = SD(a, D_REFL + d, g);
+          bool near[2] = {sv[0] > 0.0, k > 1 && sv[1] > 0.0};
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            bool near = j < k && sv[j] > 0.0;
+          for (int p = 0; p < 3; ++p) {
+            const int q = n == 1 ? 0 : p;
+            const double m1 = a.msc[15 * g + 5 * p];
+            const double reach = m1 > 0.0 ? a.msc0[3 * g + p] / m1 : 0.0;
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {
-              const int q = n == 1 ? 0 : p;
-              const double m1 = a.msc[15 * g + 5 * p];
-              const double reach = m1 > 0.0 ? a.msc0[3 * g + p] / m1 : 0.0;
-              near = near && fabs(lt[j][q] - lref[q]) * reach < 0.25;
-            }
-            dif[j] = near;
+            for (int j = 0; j < 2; ++j) near[j] = near[j] && fabs(lt[j][q] - lref[q]) * reach < 0.25;
           }
+          dif[0] = near[0];
+          dif[1] = near[1];
         } else if (k == 2 && sv[0] > 0.0 && sv[1] > 0.0) {
           k = 1;
           if (sv[1] > sv[0]) {
@@ -867,67 +805,86 @@ __global__ void nm_step_kernel(const SolveArgs a) {
         }
       }
       emit_reeval(a, REF ? a.nxt : a.cur, g, pos, k, lt, id0, id1, dif, lref);
-      if (single) store_e(a, g, e);
-      if (rdirty) store_r(a, g, R);
-      SI(a, I_FLAGS, g) = flags;
       SI(a, I_NFEV, g) = nfev;
       continue;
     }
 
     // ---- the step is certain: take it
-    if (rdirty && !store_R) store_r(a, g, R);
-    if (store_R) {
-      Vert r = e;
-      store_r(a, g, r);
-    }
     if (code && a.codes && iters >= 1 && iters <= a.codes_stride)
       a.codes[g * a.codes_stride + (iters - 1)] = code;
     if (fin >= 0) {
       for (int p = 0; p < 3; ++p) {
-        a.res_B[3 * g + p] = w[0].B[p];
-        a.res_lam[3 * g + p] = fabs(n == 1 ? w[0].l[0] : w[0].l[p]);
+        a.res_B[3 * g + p] = SV(a, w[0].id, V_B + p, g);
+        a.res_lam[3 * g + p] = fabs(SV(a, w[0].id, V_L + (n == 1 ? 0 : p), g));
       }
-      a.res_f[g] = w[0].f;
-      a.res_g[g] = w[0].g;
+      a.res_f[g] = SV(a, w[0].id, V_F, g);
+      a.res_g[g] = SV(a, w[0].id, V_G, g);
       a.res_iters[g] = iters;
       a.res_status[g] = fin;
       a.res_nfev[g] = nfev;
       stage = ST_DONE;
       SI(a, I_STATUS, g) = fin;
     } else {
-      if (to_check) iters += 1;
+      if (store_R || taken >= 0) {
+        int to = VID_R;
+        if (taken >= 0) {
+#pragma unroll
+          for (int k = 0; k <= n; ++k)
+            if (w[k].id == taken) to = w[k].slot;
+        }
+        copy_value(a, taken >= 0 ? taken : VID_E, to, g);
+      }
+      if (to_check) {
+        iters += 1;
+        int ord = 0;
+#pragma unroll
+        for (int k = 0; k <= n; ++k) ord |= w[k].slot << (4 * k);
+        SI(a, I_ORDER, g) = ord;
+      }
       if (mirror) nfev += 1;
       if (emit_trial) {
-        double rows[1][3] = {{xt[0], xt[1], xt[2]}};
-        for (int d = 0; d < 3; ++d) SD(a, D_TL + d, g) = xt[d];
+        // one site for every kind of step: its divisions are run once per warp
+        double rows[1][3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          double s = 0.0;
+          if (d < n) {
+#pragma unroll
+            for (int k = 0; k < n; ++k) s += SV(a, w[k].slot, V_L + d, g);
+            rows[0][d] = coef_c * (s / n) + coef_w * SV(a, w[n].slot, V_L + d, g);
+          } else {
+            rows[0][d] = 0.0;
+          }
+        }
+        for (int d = 0; d < 3; ++d) SV(a, VID_E, V_L + d, g) = rows[0][d];
         emit<1>(a, g, pos, pidx, rows);
       } else if (emit_shrink) {
-        double rows[N][3];
+        double rows[N][3], l0[3];
+        for (int d = 0; d < 3; ++d) l0[d] = SV(a, w[0].slot, V_L + d, g);
 #pragma unroll
         for (int k = 1; k <= n; ++k)
-          for (int d = 0; d < 3; ++d) rows[k - 1][d] = w[k].l[d];
+          for (int d = 0; d < 3; ++d) {
+            const double l = SV(a, w[k].slot, V_L + d, g);
+            rows[k - 1][d] = (d < n) ? l0[d] + sigma * (l - l0[d]) : 0.0;
+            SV(a, w[k].slot, V_L + d, g) = rows[k - 1][d];
+          }
         emit<N>(a, g, pos, pidx, rows);
       }
       stage = next_stage;
-      // a finished point's vertices are not read again; otherwise store what changed
-      if (vdirty || to_check || accepted || emit_shrink)
-#pragma unroll
-        for (int k = 0; k <= n; ++k) store_vert(a, g, k, w[k]);
     }
     SI(a, I_STAGE, g) = stage;
     SI(a, I_ITERS, g) = iters;
     SI(a, I_NFEV, g) = nfev;
-    SI(a, I_FLAGS, g) = 0;
   }
 }
 
 void launch_nm_step(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) nm_step_kernel<1, false><<<grid, 128, 0, s>>>(a);
-  else nm_step_kernel<3, false><<<grid, 128, 0, s>>>(a);
+  if (a.o.dim == 1) nm_step_kernel<1, false><<<grid, 32, 0, s>>>(a);
+  else nm_step_kernel<3, false><<<grid, 32, 0, s>>>(a);
 }
 void launch_nm_refine(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) nm_step_kernel<1, true><<<grid, 128, 0, s>>>(a);
-  else nm_step_kernel<3, true><<<grid, 128, 0, s>>>(a);
+  if (a.o.dim == 1) nm_step_kernel<1, true><<<grid, 32, 0, s>>>(a);
+  else nm_step_kernel<3, true><<<grid, 32, 0, s>>>(a);
 }
 
 // --------------------------------------------------------------- per-round plan ----
@@ -1269,7 +1226,9 @@ __global__ void bfgs_step_kernel(const SolveArgs a) {
   const int nact = *a.cur.act_cnt;
   constexpr int n = N;
   const PlanHdr h = *a.plan;
-  for (int ia = blockIdx.x * blockDim.x + threadIdx.x; ia < nact; ia += gridDim.x * blockDim.x) {
+  const int ppw = points_per_warp(nact, a.nsm);
+  if ((int)threadIdx.x >= ppw) return;
+  for (int ia = blockIdx.x * ppw + threadIdx.x; ia < nact; ia += gridDim.x * ppw) {
     const int64_t g = a.cur.act[ia];
     const float4 pos = a.ppos[g];
     const int pidx = __float_as_int(pos.w);
@@ -1422,8 +1381,8 @@ __global__ void bfgs_step_kernel(const SolveArgs a) {
 }
 
 void launch_bfgs_step(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) bfgs_step_kernel<1><<<grid, 128, 0, s>>>(a);
-  else bfgs_step_kernel<3><<<grid, 128, 0, s>>>(a);
+  if (a.o.dim == 1) bfgs_step_kernel<1><<<grid, 32, 0, s>>>(a);
+  else bfgs_step_kernel<3><<<grid, 32, 0, s>>>(a);
 }
 
 }  // namespace dbie

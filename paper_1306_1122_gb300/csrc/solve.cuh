@@ -4,32 +4,23 @@
 
 namespace dbie {
 
-// Per-point simplex state, structure-of-arrays: field f of point g is at [f * N + g].
+// Per-point simplex state: field f of point g is at [g / 32][f][g % 32].  Six value
+// records of VREC fields: the vertices (storage slots 0..3; I_ORDER holds their order by Phi, so
+// a step moves no vertex), the reflected point (VID_R) and the pending trial point (VID_E).
+constexpr int VREC = 10;
+enum RField {
+  V_L = 0,      // lambda (3)
+  V_B = 3,      // field B (3)
+  V_F = 6, V_G = 7, V_PHI = 8,
+  V_S = 9       // certified decisions: the value's error bound (0 once re-evaluated in float-float)
+};
+constexpr int VID_R = 4, VID_E = 5;
 enum DField {
-  D_VL = 0,      // vertex lambda: D_VL + v * 3 + d   (v = 0..3, d = 0..2)
-  D_VB = 12,     // vertex field B: D_VB + v * 3 + p
-  D_VF = 24,     // vertex f: D_VF + v
-  D_VG = 28,     // vertex g
-  D_VPHI = 32,   // vertex Phi
-  D_RL = 36,     // reflected point: lambda (3), B (3), f, g, Phi
-  D_RB = 39,
-  D_RF = 42,
-  D_RG = 43,
-  D_RPHI = 44,
-  D_TL = 45,     // pending single trial point lambda (3)
-  // certified decisions: the error bound of each value (0 once re-evaluated in float-float)
-  D_VS = 48,     // vertex bounds: D_VS + v
-  D_RS = 52,     // reflected point's bound
-  D_EB = 53,     // evaluated single trial point: B (3), f, g, Phi, bound (kept while its step
-  D_EF = 56,     // waits for a float-float re-evaluation)
-  D_EG = 57,
-  D_EPHI = 58,
-  D_ES = 59,
   // certified decisions, difference level: the point's float-float reference value, lambda (3)
   // and its 12 sums (D_REFS = NaN: no reference yet)
-  D_REFL = 60,
-  D_REFS = 63,
-  D_NFIELDS = 75
+  D_REFL = 6 * VREC,
+  D_REFS = D_REFL + 3,
+  D_NFIELDS = D_REFS + 12
 };
 // Quasi-Newton state (same arrays, other meaning): x, grad Phi, inverse Hessian H (3 x 3),
 // direction d, B, f, g, Phi at x, line-search step alpha, grad . d, |grad|.
@@ -37,16 +28,13 @@ enum BField {
   B_X = 0, B_GR = 3, B_H = 6, B_D = 15, B_B = 18, B_F = 21, B_G = 22, B_PHI = 23, B_ALPHA = 24,
   B_GD = 25, B_GN = 26
 };
-// I_FLAGS bit F_EVAL: this step's evaluations are in the state (the step waits for a
-// re-evaluation); I_RSLOT, I_DSLOT: first float-float and first difference query slot of the
-// point's pending re-evaluation; I_RTGT: its targets, one per byte: value id (0..3 vertex,
-// 4 reflected point, 5 trial point) | RT_DIF when the value goes to the difference pass,
-// 0xff = none.
-enum IField { I_STAGE = 0, I_ITERS = 1, I_NFEV = 2, I_STATUS = 3, I_QSLOT = 4, I_FLAGS = 5,
+// I_ORDER: storage slots of the vertices by ascending Phi, 4 bits each; I_RSLOT, I_DSLOT: first
+// float-float and first difference query slot of the point's pending re-evaluation; I_RTGT: its
+// targets, one per byte, differences first: value id (0..3 vertex slot, VID_R, VID_E) | RT_DIF
+// when the value goes to the difference pass, 0xff = none.
+enum IField { I_STAGE = 0, I_ITERS = 1, I_NFEV = 2, I_STATUS = 3, I_QSLOT = 4, I_ORDER = 5,
               I_RSLOT = 6, I_RTGT = 7, I_DSLOT = 8, I_NFIELDS = 9 };
-constexpr int F_EVAL = 1;
 constexpr int RT_DIF = 0x40;
-constexpr int VID_R = 4, VID_E = 5;
 enum PtStatus { PT_RUNNING = -1, PT_CONVERGED = 0, PT_MAXITER = 1 };
 enum Stage { ST_INIT = 0, ST_REFLECT = 1, ST_EXPAND = 2, ST_OCONTRACT = 3, ST_ICONTRACT = 4,
              ST_SHRINK = 5, ST_DONE = 6, ST_BF_INIT = 10, ST_BF_LS = 11 };
@@ -83,11 +71,11 @@ struct RoundBuf {
 struct SolveArgs {
   const ProbDesc* probs;
   int32_t nprob;
-  int32_t pad0;
+  int32_t nsm;               // SMs of the device
   int64_t N;                 // total points
   const float4* ppos;        // [N] x, y, z, problem (int bits)
-  double* sd;                // [D_NFIELDS * N]
-  int32_t* si;               // [I_NFIELDS * N]
+  double* sd;                // [ceil(N / 32)][D_NFIELDS][32]
+  int32_t* si;               // [ceil(N / 32)][I_NFIELDS][32]
   RoundBuf cur, nxt;
   const double* out;         // pair-sum partials of the current round (item chunks)
   const PlanHdr* plan;       // plan of the current round
