@@ -188,8 +188,9 @@ void launch_plan_single(PlanHdr* plan, int32_t* item_off, int32_t* q_cnt, int32_
 // Near-field correction (mixed precision, points with z <= near_z): over the (2W+1)^2 pixels
 // around the point, replace the FP32 pair terms that the pair-sum kernel added by FP64 ones.
 // The FP32 terms are recomputed with the same explicitly rounded code (pair_terms32), so the
-// correction sum_k (t64 - t32) removes exactly what was added.  Eight lanes per query; the
-// correction is added in place to the query's split-0 partial sums (run after the pair sums).
+// correction sum_k (t64 - t32) removes exactly what was added.  The correction is added in place
+// to the query's split-0 partial sums (a dense pass: run after the pair sums) or is the query's
+// last record (a pass of few queries: in any order with it).
 // Index (along one axis) of the quadrature point nearest to coordinate x: the pixel for the
 // midpoint rule; for nine-node elements of width 2h with g Gauss points, element e and the
 // nearest abscissa a give e * g + a.
@@ -210,25 +211,15 @@ __device__ __forceinline__ long near_index(double x, double x0, double h, int nq
   return e * g + best;
 }
 
-template <int VAR, bool TIED>
-__global__ void nearfield_kernel(const ProbDesc* __restrict__ probs,
-                                 const int32_t* __restrict__ near_list,
-                                 const int32_t* __restrict__ near_cnt,
-                                 const float4* __restrict__ qpos, const Lam4* __restrict__ qlam,
-                                 const PlanHdr* __restrict__ plan,
-                                 const int32_t* __restrict__ item_off, double* __restrict__ out) {
+// GL lanes per query (a divisor of 32).
+template <int VAR, bool TIED, int GL>
+__device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const PlanHdr& h,
+                                             const float4* s_tab) {
   constexpr int NS = nsum_per_comp(VAR);
   constexpr int NSUM = 3 * NS;
-  // Eight lanes per query, four queries per warp: a 7 x 7 window takes 7 passes of 8 lanes
-  // (49 of 56 lane slots busy) instead of 2 of 32 (49 of 64).  The loop runs warp-uniformly so
-  // the shuffles see every lane.
-  constexpr int GL = 8;
   // sin and cos of lambda r in float-float on the FP32 pipe (absolute error ~1e-13 + 5e-15 |lambda
   // r|, far below the FP32 terms' error that the correction removes) instead of FP64 sincos,
   // which cost most of this kernel's FP64-pipe time
-  __shared__ float4 s_tab[ff::SC_TABLE];
-  ff::fill_sincos_table(s_tab, threadIdx.x);
-  __syncthreads();
   auto sincos_ff = [&](double th, double& s, double& c) {
     ff::ds S, C;
     ff::sincos_ds_any(ff::from_double(th), s_tab, S, C);
@@ -236,17 +227,16 @@ __global__ void nearfield_kernel(const ProbDesc* __restrict__ probs,
     c = ff::to_double(C);
   };
   const int lane = threadIdx.x & 31, sub = lane & (GL - 1), grp = lane / GL;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int cnt = *near_cnt;
-  for (int64_t wb = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * (32 / GL); wb < cnt;
-       wb += nwarps * (32 / GL)) {
+  // (the loop runs warp-uniformly so the shuffles see every lane)
+  for (int64_t wb = blockIdx.x * (int64_t)(32 / GL); wb < cnt; wb += gridDim.x * (int64_t)(32 / GL)) {
     const int64_t w = wb + grp;
-    const bool valid = w < cnt;
-    const int64_t slot = near_list[valid ? w : wb];
-    const float4 pos = qpos[slot];
-    const Lam4 lam = qlam[slot];
+    const bool listed = w < cnt;
+    const int64_t wq = listed ? w : wb;
+    const int64_t slot = a.list ? a.list[wq] : wq;
+    const float4 pos = a.qpos[slot];
+    const Lam4 lam = a.qlam[slot];
     const int pidx = __float_as_int(pos.w);
-    const ProbDesc& pd = probs[pidx];
+    const ProbDesc& pd = a.probs[pidx];
     const Query<float, TIED> q32 = make_query<float, TIED>(pos, lam);
     const Query<double, TIED> q64 = make_query<double, TIED>(pos, lam);
     const int W = pd.near_w > 0 ? pd.near_w : NEAR_W;
@@ -260,6 +250,7 @@ __global__ void nearfield_kernel(const ProbDesc* __restrict__ probs,
     double c[NSUM];
 #pragma unroll
     for (int s = 0; s < NSUM; ++s) c[s] = 0.0;
+    const bool valid = listed && (a.list || (double)pos.z <= a.near_z);
     if (valid && wi > 0 && wj > 0 && wi <= 2 * W + 1 && wj <= 2 * W + 1) {
       const int nwin = (int)(wi * wj);
       for (int e = sub; e < nwin; e += GL) {
@@ -310,23 +301,43 @@ __global__ void nearfield_kernel(const ProbDesc* __restrict__ probs,
         }
       }
     }
-    const PlanHdr h = *plan;
 #pragma unroll
     for (int s = 0; s < NSUM; ++s) {
       double v = c[s];
       for (int off = GL / 2; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (sub == 0 && valid) out[out_index(h, item_off, pidx, slot - pd.q_off, 0, s, NSUM)] += v;
+      if (sub == 0 && valid) {
+        if (a.warps > 0) a.out[(slot * h.nsplit + h.nsplit - 1) * NSUM + s] = v;
+        else a.out[out_index(h, a.item_off, pidx, slot - pd.q_off, 0, s, NSUM)] += v;
+      }
     }
   }
 }
 
-void launch_nearfield(int var, bool tied, const ProbDesc* probs, const int32_t* near_list,
-                      const int32_t* near_cnt, const float4* qpos, const Lam4* qlam,
-                      const PlanHdr* plan, const int32_t* item_off, double* out, int grid,
-                      cudaStream_t s) {
-#define NF(V, T)                                                                            \
-  nearfield_kernel<V, T><<<grid, 256, 0, s>>>(probs, near_list, near_cnt, qpos, qlam, plan, \
-                                              item_off, out)
+// CTAs of one warp.  Eight lanes per query, four queries per warp: a 7 x 7 window takes 7 passes
+// of 8 lanes (49 of 56 lane slots busy) instead of 2 of 32 (49 of 64).  With no more queries than
+// CTAs a query takes a whole warp instead: the two passes then set the kernel's length, which is
+// latency (about 500 instructions a pass), not FP64 throughput.  512 near queries of 2,048: 71 us
+// in CTAs of 256 threads (16 SMs busy), 50 us as one-warp CTAs of four queries.
+template <int VAR, bool TIED>
+__global__ void __launch_bounds__(32) nearfield_kernel(const NearArgs a) {
+  __shared__ float4 s_tab[ff::SC_TABLE];
+  const int cnt = a.list ? *a.cnt : a.n;
+  if (blockIdx.x >= cnt) return;
+  for (int i = threadIdx.x; i < ff::SC_TABLE; i += 32) {
+    if (a.sctab) s_tab[i] = __ldg(a.sctab + i);
+    else ff::fill_sincos_table(s_tab, i);
+  }
+  __syncwarp();
+  PlanHdr h{0, 1, 1, 0};
+  if (a.warps > 0) h.nsplit = few_split(a.q_cnt ? *a.q_cnt : a.n, a.strips, a.warps) + 1;
+  else h = *a.plan;
+  if (cnt <= (int)gridDim.x) near_queries<VAR, TIED, 32>(a, cnt, h, s_tab);
+  else near_queries<VAR, TIED, 8>(a, cnt, h, s_tab);
+}
+
+void launch_nearfield(int var, bool tied, const NearArgs& a, int sm_count, cudaStream_t s) {
+  const int grid = 16 * sm_count;   // resident at the kernel's register count
+#define NF(V, T) nearfield_kernel<V, T><<<grid, 32, 0, s>>>(a)
   if (tied) {
     switch (var) {
       case VAR_V: NF(VAR_V, true); break;

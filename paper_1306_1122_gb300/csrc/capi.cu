@@ -77,6 +77,7 @@ struct Misc {
   int32_t zero;             // an empty queue's count
   int32_t pad;
   PlanHdr plan2;            // an empty queue's plan
+  float4 sctab[SINCOS_TABLE];   // sine and cosine table of the float-float kernels
 };
 
 struct SolveBufs {
@@ -169,7 +170,6 @@ struct dbie_ctx {
   DBuf st_in, st_out, st_aux;     // host-memory staging
   DBuf qpos, qlam, near_list, out, ptiles;
   DBuf qlam0, dmsc;                // dbie_eval_difference: reference lambdas, bound sums
-  DBuf sctab;                     // sine and cosine table of the float-float kernels
   DBuf trace;                     // DBIE_TRACE_ITEMS builds: item timeline of the last pass
   int64_t trace_items = 0;
   DBuf tv32, tv64, probv;         // noise-variance tiles and their problem descriptor
@@ -184,7 +184,9 @@ struct dbie_ctx {
   SolveBufs sb;
   int cfg[NVAR][2] = {};   // tuned launch configuration per variant / tied
   int vjp_cfg = 0;
-  cudaStream_t cap_stream = nullptr;  // stream used only to capture graphs
+  cudaStream_t cap_stream = nullptr;  // streams and events used only to capture graphs
+  cudaStream_t cap_side = nullptr;
+  cudaEvent_t cap_ev[2] = {};
   int32_t* pinned = nullptr;          // pinned host words for polling
   bool profiling = false;
   dbie_stats stats{};
@@ -370,11 +372,33 @@ dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float*
   a.f = dif ? none : list;
   a.d = dif ? list : none;
   a.work = &m->work;
-  a.sctab = c->sctab.as<float4>();
+  a.sctab = c->misc.as<Misc>()->sctab;
   a.rows = c->ntiles * RE_ROWS_PER_TILE;
   DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
   CUDA_TRY(cudaGetLastError());
   return DBIE_OK;
+}
+
+// Fault injection for tests of the bounded waits: the CTA that takes work item 0 never issues its
+// tile copies, its waits expire after their time limit and the call reports DBIE_ETIMEOUT.  (Of
+// the dense kernels: the others wait for nothing.)
+int fault_injection() {
+  const char* fi = std::getenv("DBIE_FAULT_INJECT");
+  return fi && std::atoi(fi) == 1 ? 1 : 0;
+}
+
+// Whether a pass runs on the kernel for few queries (pairsum_few.cu): the forms it has, and n
+// queries over npix quadrature points (a search: its points and largest problem).  The dense
+// kernel needs blocks of 128 queries enough to fill the chip; where it does it is 10-17 % faster
+// (measured from 32 x 32 to 512 x 256 pixels; us per call of B, dense against few: 1,024 pixels
+// 70 / 30 at 1,000 points, 88 / 60 at 8,000, 95 / 103 at 16,000; 9,030 pixels 95 / 33 at 300,
+// 103 / 64 at 2,000, 105 / 107 at 4,000; 131,072 pixels 250 / 106 at 300, 516 / 509 at 2,000,
+// 932 / 1,002 at 4,000).  A search's later rounds have fewer queries than its points: it stays
+// with few up to 12,000 (128 x 128 pixels, ms: 62.3 / 57.6 at 8,000 points, 173 / 182 at 32,000).
+bool use_few(int var, bool tied, bool fp64, int64_t n, double npix, bool search) {
+  if (fp64 || var == VAR_HESS || var == VAR_NV) return false;
+  if (tied && var != VAR_OBJ && var != VAR_OBJN) return false;
+  return n <= (search ? 12000 : 2500) || (!search && n <= 6000 && (double)n * npix <= 7e7);
 }
 
 // One pair-sum pass over n queries of this context (single problem): pack, plan, sweep,
@@ -388,6 +412,42 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   if (ffp) return pass_reeval(c, var, tied, n, d_xyz, d_lamf, nullptr, nullptr, s);
   // (the noise variance sums positive terms: FP32 is accurate there without a near field)
   const bool near_on = !fp64 && o.near_z > 0 && var != VAR_NV;
+  const int fault = fault_injection();
+  NearArgs na{};
+  na.probs = c->prob.as<ProbDesc>();
+  na.qpos = c->qpos.as<float4>();
+  na.qlam = c->qlam.as<Lam4>();
+  na.sctab = c->misc.as<Misc>()->sctab;
+  if (use_few(var, tied, fp64, n, (double)c->nquad, false) && !fault) {
+    const KernelRef k = few_ref(var, tied, c->quad_g != 0);
+    const int grid = persistent_grid(k, c->device);
+    const int nsum = 3 * nsum_per_comp(var);
+    DBIE_TRY(ensure(c->out, sizeof(double) * few_records(n, grid) * nsum));
+    FewArgs a{};
+    a.probs = c->prob.as<ProbDesc>();
+    a.n = (int32_t)n;
+    a.near_on = near_on ? 1 : 0;
+    a.near_z = o.near_z;
+    a.qpos = c->qpos.as<float4>();
+    a.qlam = c->qlam.as<Lam4>();
+    a.xyz = d_xyz;
+    a.lam_f = d_lamf;
+    a.lam_d = d_lamd;
+    a.out = c->out.as<double>();
+    a.plan = &m->plan;
+    a.strips = c->ntiles * FEW_STRIPS_PER_TILE;
+    DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
+    if (near_on) {
+      na.n = (int32_t)n;
+      na.warps = grid * (k.nt / 32);
+      na.strips = a.strips;
+      na.near_z = o.near_z;
+      na.out = c->out.as<double>();
+      launch_nearfield(var, tied, na, c->sm_count, s);
+    }
+    CUDA_TRY(cudaGetLastError());
+    return DBIE_OK;
+  }
   if (near_on) DBIE_TRY(ensure(c->near_list, sizeof(int32_t) * n));
   CUDA_TRY(cudaMemsetAsync(&m->near_cnt, 0, sizeof(int32_t), s));
   launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(),
@@ -407,9 +467,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   G1Args a{};
   a.probs = var == VAR_NV ? c->probv.as<ProbDesc>() : c->prob.as<ProbDesc>();
   a.nprob = 1;
-  // Fault injection for tests of the bounded waits: the CTA that takes work item 0 never issues
-  // its tile copies, its waits expire after their time limit and the call reports DBIE_ETIMEOUT.
-  if (const char* fi = std::getenv("DBIE_FAULT_INJECT")) a.fault = std::atoi(fi) == 1 ? 1 : 0;
+  a.fault = fault;
   a.plan = &m->plan;
   a.item_off = m->item_off;
   a.q_cnt = m->q_cnt;
@@ -425,10 +483,14 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   c->trace_items = nitems;
 #endif
   DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
-  if (near_on)
-    launch_nearfield(var, tied, c->prob.as<ProbDesc>(), c->near_list.as<int32_t>(), &m->near_cnt,
-                     c->qpos.as<float4>(), c->qlam.as<Lam4>(), &m->plan, m->item_off,
-                     c->out.as<double>(), 2 * c->sm_count, s);
+  if (near_on) {
+    na.list = c->near_list.as<int32_t>();
+    na.cnt = &m->near_cnt;
+    na.plan = &m->plan;
+    na.item_off = m->item_off;
+    na.out = c->out.as<double>();
+    launch_nearfield(var, tied, na, c->sm_count, s);
+  }
   CUDA_TRY(cudaGetLastError());
   return DBIE_OK;
 }
@@ -552,7 +614,7 @@ void dbie_destroy(dbie_ctx* c) {
                   &c->st_aux, &c->qpos, &c->qlam, &c->near_list, &c->out, &c->ptiles, &c->tv32,
                   &c->tv64, &c->probv, &c->b0raw, &c->vtmp, &c->pxe_corr, &c->pxe_pos,
                   &c->pxe_list, &c->pxe_w, &c->pxe_part, &c->pxe_bins, &c->trace, &c->qlam0,
-                  &c->dmsc, &c->sctab})
+                  &c->dmsc})
     b->release();
   c->sb.release();
   for (auto& pr : c->pending) {
@@ -561,6 +623,9 @@ void dbie_destroy(dbie_ctx* c) {
   }
   for (cudaEvent_t e : c->free_events) cudaEventDestroy(e);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+  if (c->cap_side) cudaStreamDestroy(c->cap_side);
+  for (cudaEvent_t e : c->cap_ev)
+    if (e) cudaEventDestroy(e);
   if (c->pinned) cudaFreeHost(c->pinned);
   cudaSetDevice(prev);
   delete c;
@@ -712,13 +777,12 @@ dbie_status dbie_create(dbie_ctx** out, int32_t nx, int32_t ny, double x0, doubl
   if ((st = ensure(c->prob, sizeof(ProbDesc))) != DBIE_OK) return bail(st);
   if ((st = ensure(c->err, sizeof(unsigned))) != DBIE_OK) return bail(st);
   if ((st = ensure(c->misc, sizeof(Misc))) != DBIE_OK) return bail(st);
-  if ((st = ensure(c->sctab, sizeof(float4) * SINCOS_TABLE)) != DBIE_OK) return bail(st);
-  launch_fill_sincos(c->sctab.as<float4>(), s);
   if (cudaMemsetAsync(c->err.p, 0, sizeof(unsigned), s) != cudaSuccess ||
       cudaMemsetAsync(c->misc.p, 0, sizeof(Misc), s) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaHostAlloc((void**)&c->pinned, 64, cudaHostAllocDefault) != cudaSuccess)
     return bail(fail(DBIE_ECUDA, "context set-up failed"));
+  launch_fill_sincos(c->misc.as<Misc>()->sctab, s);
   const ProbDesc pd = desc_of(c);
   if (cudaMemcpyAsync(c->prob.p, &pd, sizeof pd, cudaMemcpyHostToDevice, s) != cudaSuccess)
     return bail(fail(DBIE_ECUDA, "copy of the problem descriptor failed"));
@@ -1389,7 +1453,12 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   DBIE_TRY(ensure(b.q_cnt_pass, sizeof(int32_t) * nprob));
   DBIE_TRY(ensure(b.item_off, sizeof(int32_t) * (nprob + 1)));
   DBIE_TRY(ensure(b.ctrl, sizeof(SolveCtrl)));
-  DBIE_TRY(ensure(b.out, sizeof(double) * items_cap * nsum * k.qper));
+  // passes of few queries: the lanes of a warp take pixels, all problems share one queue
+  const bool few = use_few(var, tied, fp64, N, (double)max_rows * (TILE / RE_ROWS_PER_TILE), true);
+  const KernelRef kw = few_ref(var, tied, c->quad_g != 0);
+  const int grid_few = few ? persistent_grid(kw, c->device) : 0;
+  DBIE_TRY(ensure(b.out, sizeof(double) * nsum *
+                             (few ? few_records(Qcap, grid_few) : items_cap * k.qper)));
   DBIE_TRY(ensure(b.res, align256(sizeof(double) * 8 * N) + align256(sizeof(int32_t) * 3 * N)));
   if (codes_stride) DBIE_TRY(ensure(b.codes, (size_t)codes_stride * N));
   for (int sd = 0; sd < 2; ++sd) {
@@ -1544,6 +1613,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     a.res_nfev = res_i + 2 * N;
     a.codes = codes_stride ? b.codes.as<char>() : nullptr;
     a.codes_stride = codes_stride;
+    a.one_queue = few ? 1 : 0;
     a.err = c->err.as<unsigned>();
     a.corr = pxe_any ? b.corr.as<double>() : nullptr;
     if (cert) {
@@ -1579,7 +1649,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
                   b.dlam[cur].as<Lam4>(), b.dlam0[cur].as<Lam4>(), b.dout.as<double>(),
                   &ctrl->dplan};
     ra.work = &ctrl->rework[0];
-    ra.sctab = c->sctab.as<float4>();
+    ra.sctab = c->misc.as<Misc>()->sctab;
     ra.stat_ff_pairs = &ctrl->stat_ff_pairs;
     ra.stat_dif_pairs = &ctrl->stat_dif_pairs;
     ra.rows = max_rows;
@@ -1587,54 +1657,106 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   };
   // One simplex round = plan, pair sums (objective variant), near-field correction, step.
   constexpr int K = 4;  // rounds per graph launch (even: the ping-pong side returns to 0)
+  // The near field of a round's queries; in a pass of few queries beside the pair sums.
+  auto near_args = [&](int cur) {
+    NearArgs na{};
+    na.probs = b.probs.as<ProbDesc>();
+    na.list = b.near[cur].as<int32_t>();
+    na.cnt = &ctrl->near_cnt[cur];
+    na.qpos = b.qpos[cur].as<float4>();
+    na.qlam = b.qlam[cur].as<Lam4>();
+    na.plan = &ctrl->plan;
+    na.item_off = b.item_off.as<int32_t>();
+    na.sctab = c->misc.as<Misc>()->sctab;
+    na.out = b.out.as<double>();
+    if (few) {
+      na.warps = grid_few * (kw.nt / 32);
+      na.strips = max_rows;
+      na.q_cnt = b.q_cnt[cur].as<int32_t>();
+    }
+    return na;
+  };
+  static_assert(FEW_STRIPS_PER_TILE == RE_ROWS_PER_TILE, "max_rows counts both");
+  auto record_few = [&](cudaStream_t cs, int r) -> dbie_status {
+    const int cur = r & 1;
+    if (near_on) {
+      CUDA_TRY(cudaEventRecord(c->cap_ev[0], cs));
+      CUDA_TRY(cudaStreamWaitEvent(c->cap_side, c->cap_ev[0], 0));
+      launch_nearfield(var, tied, near_args(cur), c->sm_count, c->cap_side);
+      CUDA_TRY(cudaEventRecord(c->cap_ev[1], c->cap_side));
+    }
+    FewArgs fa{};
+    fa.probs = b.probs.as<ProbDesc>();
+    fa.cnt = b.q_cnt[cur].as<int32_t>();
+    fa.near_on = near_on ? 1 : 0;
+    fa.near_z = -1.0;
+    fa.qpos = b.qpos[cur].as<float4>();
+    fa.qlam = b.qlam[cur].as<Lam4>();
+    fa.out = b.out.as<double>();
+    fa.plan = &ctrl->plan;
+    fa.strips = max_rows;
+    fa.next = NextSide{b.q_cnt[cur ^ 1].as<int32_t>(), &ctrl->act_cnt[cur ^ 1],
+                       &ctrl->near_cnt[cur ^ 1], &ctrl->f_cnt[cur ^ 1], &ctrl->d_cnt[cur ^ 1],
+                       &ctrl->ref_cnt[cur ^ 1]};
+    fa.round_ctr = &ctrl->round;
+    fa.stat_queries = &ctrl->stat_queries;
+    fa.stat_pairs = &ctrl->stat_pairs;
+    if (c->profiling) CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r], cs, cudaEventRecordExternal));
+    DBIE_TRY(launch_kernel(kw, grid_few, &fa, cs));
+    if (c->profiling)
+      CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 1], cs, cudaEventRecordExternal));
+    if (near_on) CUDA_TRY(cudaStreamWaitEvent(cs, c->cap_ev[1], 0));
+    return DBIE_OK;
+  };
+  auto record_dense = [&](cudaStream_t cs, int r) -> dbie_status {
+    const int cur = r & 1;
+    PlanArgs pa{};
+    pa.probs = b.probs.as<ProbDesc>();
+    pa.nprob = nprob;
+    pa.qper = k.qper;
+    pa.target_items = target;
+    pa.nsplit_cap = 1 << 20;
+    pa.q_cnt_cur = b.q_cnt[cur].as<int32_t>();
+    pa.q_cnt_pass = b.q_cnt_pass.as<int32_t>();
+    pa.item_off = b.item_off.as<int32_t>();
+    pa.plan = &ctrl->plan;
+    pa.work = &ctrl->work;
+    pa.q_cnt_nxt = b.q_cnt[cur ^ 1].as<int32_t>();
+    pa.act_cnt_nxt = &ctrl->act_cnt[cur ^ 1];
+    pa.near_cnt_nxt = &ctrl->near_cnt[cur ^ 1];
+    if (cert) {
+      pa.fq_cnt_nxt = &ctrl->f_cnt[cur ^ 1];
+      pa.ref_cnt_nxt = &ctrl->ref_cnt[cur ^ 1];
+    }
+    if (dif_on) pa.dq_cnt_nxt = &ctrl->d_cnt[cur ^ 1];
+    pa.round_ctr = &ctrl->round;
+    pa.stat_queries = &ctrl->stat_queries;
+    pa.stat_pairs = &ctrl->stat_pairs;
+    launch_plan_round(pa, cs);
+    G1Args ga{};
+    ga.probs = b.probs.as<ProbDesc>();
+    ga.nprob = nprob;
+    ga.plan = &ctrl->plan;
+    ga.item_off = b.item_off.as<int32_t>();
+    ga.q_cnt = b.q_cnt_pass.as<int32_t>();
+    ga.work = &ctrl->work;
+    ga.qpos = b.qpos[cur].as<float4>();
+    ga.qlam = b.qlam[cur].as<Lam4>();
+    ga.out = b.out.as<double>();
+    ga.err = c->err.as<unsigned>();
+    // External event records become event-record nodes of the graph (plain records inside a
+    // capture only order work and are never timestamped).
+    if (c->profiling) CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r], cs, cudaEventRecordExternal));
+    DBIE_TRY(launch_kernel(k, grid, &ga, cs));
+    if (c->profiling)
+      CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 1], cs, cudaEventRecordExternal));
+    if (near_on) launch_nearfield(var, tied, near_args(cur), c->sm_count, cs);
+    return DBIE_OK;
+  };
   auto record_rounds = [&](cudaStream_t cs) -> dbie_status {
     for (int r = 0; r < K; ++r) {
       const int cur = r & 1;
-      PlanArgs pa{};
-      pa.probs = b.probs.as<ProbDesc>();
-      pa.nprob = nprob;
-      pa.qper = k.qper;
-      pa.target_items = target;
-      pa.nsplit_cap = 1 << 20;
-      pa.q_cnt_cur = b.q_cnt[cur].as<int32_t>();
-      pa.q_cnt_pass = b.q_cnt_pass.as<int32_t>();
-      pa.item_off = b.item_off.as<int32_t>();
-      pa.plan = &ctrl->plan;
-      pa.work = &ctrl->work;
-      pa.q_cnt_nxt = b.q_cnt[cur ^ 1].as<int32_t>();
-      pa.act_cnt_nxt = &ctrl->act_cnt[cur ^ 1];
-      pa.near_cnt_nxt = &ctrl->near_cnt[cur ^ 1];
-      if (cert) {
-        pa.fq_cnt_nxt = &ctrl->f_cnt[cur ^ 1];
-        pa.ref_cnt_nxt = &ctrl->ref_cnt[cur ^ 1];
-      }
-      if (dif_on) pa.dq_cnt_nxt = &ctrl->d_cnt[cur ^ 1];
-      pa.round_ctr = &ctrl->round;
-      pa.stat_queries = &ctrl->stat_queries;
-      pa.stat_pairs = &ctrl->stat_pairs;
-      launch_plan_round(pa, cs);
-      G1Args ga{};
-      ga.probs = b.probs.as<ProbDesc>();
-      ga.nprob = nprob;
-      ga.plan = &ctrl->plan;
-      ga.item_off = b.item_off.as<int32_t>();
-      ga.q_cnt = b.q_cnt_pass.as<int32_t>();
-      ga.work = &ctrl->work;
-      ga.qpos = b.qpos[cur].as<float4>();
-      ga.qlam = b.qlam[cur].as<Lam4>();
-      ga.out = b.out.as<double>();
-      ga.err = c->err.as<unsigned>();
-      // External event records become event-record nodes of the graph (plain records inside a
-      // capture only order work and are never timestamped).
-      if (c->profiling) CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r], cs, cudaEventRecordExternal));
-      DBIE_TRY(launch_kernel(k, grid, &ga, cs));
-      if (c->profiling)
-        CUDA_TRY(cudaEventRecordWithFlags(b.ev[6 * r + 1], cs, cudaEventRecordExternal));
-      if (near_on)
-        launch_nearfield(var, tied, b.probs.as<ProbDesc>(), b.near[cur].as<int32_t>(),
-                         &ctrl->near_cnt[cur], b.qpos[cur].as<float4>(), b.qlam[cur].as<Lam4>(),
-                         &ctrl->plan, b.item_off.as<int32_t>(), b.out.as<double>(),
-                         2 * c->sm_count, cs);
+      DBIE_TRY(few ? record_few(cs, r) : record_dense(cs, r));
       (qn ? launch_bfgs_step : launch_nm_step)(sa[cur], nm_grid, cs);
       if (cert) {
         // the near-tied values of this round in float-float, then those queued as differences
@@ -1675,13 +1797,18 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     unsigned char* kp = key.data();
     std::memcpy(kp, sa, sizeof sa);
     std::memcpy(kp + sizeof sa, &k, sizeof k);
-    const int extra[4] = {grid, nm_grid, (c->profiling ? 1 : 0) | (qn ? 2 : 0) | (cert ? 4 : 0),
-                          max_rows};
+    const int extra[4] = {grid, nm_grid, (c->profiling ? 1 : 0) | (qn ? 2 : 0) | (cert ? 4 : 0) |
+                          (few ? 8 : 0), max_rows};
     std::memcpy(kp + sizeof sa + sizeof k, extra, sizeof extra);
   }
   if (!b.exec || b.key != key) {
     if (b.exec) cudaGraphExecDestroy(b.exec);
     b.exec = nullptr;
+    if (few && near_on && !c->cap_side) {   // (not while capturing)
+      CUDA_TRY(cudaStreamCreateWithFlags(&c->cap_side, cudaStreamNonBlocking));
+      for (cudaEvent_t& e : c->cap_ev)
+        CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     dbie_status st = record_rounds(c->cap_stream);
     cudaGraph_t graph = nullptr;

@@ -124,12 +124,31 @@ struct G1Args {
 // Position of partial sum s of the query with local index j (within its problem) for split
 // `sp`: work item = item_off[problem] + (j / qper) * nsplit + sp owns a dense chunk of
 // nsum * qper values, so the buffer size is bounded by the number of items, not by nsplit.
+// Passes of one query per item (qper == 1) number the queries of all problems in one queue and
+// need no item_off.
 __host__ __device__ inline int64_t out_index(const PlanHdr& h, const int32_t* item_off, int pidx,
                                              int64_t j, int sp, int s, int nsum) {
-  const int64_t blk = j / h.qper;
+  if (h.qper == 1) return (j * h.nsplit + sp) * nsum + s;
+  const int64_t blk = (int64_t)((uint32_t)j / (uint32_t)h.qper);
   const int64_t r = j - blk * h.qper;
   const int64_t item = (int64_t)item_off[pidx] + blk * h.nsplit + sp;
   return (item * nsum + s) * h.qper + r;
+}
+
+// S[0..NSUM): the query's sums over its splits, added in order.
+template <int NSUM>
+__device__ __forceinline__ void gather_sums(const double* __restrict__ out, const PlanHdr& h,
+                                            const int32_t* item_off, int pidx, int64_t j,
+                                            double* S) {
+  const double* p = out + out_index(h, item_off, pidx, j, 0, 0, NSUM);
+  const int64_t step = (int64_t)NSUM * h.qper;
+#pragma unroll
+  for (int s = 0; s < NSUM; ++s) S[s] = p[(int64_t)s * h.qper];
+  for (int sp = 1; sp < h.nsplit; ++sp) {
+    p += step;
+#pragma unroll
+    for (int s = 0; s < NSUM; ++s) S[s] += p[(int64_t)s * h.qper];
+  }
 }
 
 // Point tiles for the adjoint: per tile TILE x, y, z^2, lambda_x, lambda_y, lambda_z and the

@@ -36,6 +36,49 @@ struct KernelRef {
 KernelRef g1_ref_f32(int var, bool tied, int cfg, bool rows);   // pairsum_f32_*.cu
 KernelRef g1_ref_f64(int var, bool tied);            // pairsum_f64.cu
 
+// pairsum_few.cu: FP32 sums of few queries, the lanes of a warp taking pixels.
+constexpr int FEW_STRIPS_PER_TILE = TILE / 128;   // strips: 128 pixels, 4 per lane
+// Counters of the next side that a search round's pass clears (null outside a search).
+struct NextSide {
+  int32_t *q_cnt, *act_cnt, *near_cnt, *fq_cnt, *dq_cnt, *ref_cnt;   // the last three nullable
+};
+struct FewArgs {
+  const ProbDesc* probs;
+  const int32_t* cnt;       // queries (device), or null: n
+  int32_t n;
+  int32_t near_on;          // a record per query for the near field (after the ranges)
+  double near_z;            // near field for z <= near_z (< 0: the problem's own near_z)
+  float4* qpos;             // [slot] x, y, z, problem
+  Lam4* qlam;               // [slot] lambda
+  const float* xyz;         // a call's points (n, 3) and lambda (float or double), packed into
+  const float* lam_f;       // qpos, qlam by the kernel; null: qpos, qlam hold the queries
+  const double* lam_d;
+  double* out;              // [slot][record][sums]
+  PlanHdr* plan;            // written by the kernel: records per query (items of one query)
+  int32_t strips;           // strips of the largest problem
+  int32_t pad0;
+  NextSide next;
+  int32_t* round_ctr;       // statistics of a search (or null)
+  unsigned long long* stat_queries;
+  double* stat_pairs;
+};
+KernelRef few_ref(int var, bool tied, bool split);
+// records that a launch of `grid` CTAs writes at most for up to this many queries
+int64_t few_records(int64_t queries, int grid);
+
+// Strip ranges per query of a pass of nq queries on `warps` warps.  Short passes are one wave
+// (rounded down: an item too many would be a wave of its own); with more than 32 strips for every
+// warp about four items each even out the end, of at least 8 strips, which pay for their
+// combination.  At most 32 ranges: a thread adds them up.
+__host__ __device__ inline int few_split(int nq, int strips, int warps) {
+  if (nq <= 0) return 1;
+  const bool large = (int64_t)nq * strips > (int64_t)32 * warps;
+  const int64_t ns = large ? (4 * (int64_t)warps + nq - 1) / nq : warps / nq;
+  int64_t most = large ? strips / 8 : strips;
+  most = most > 32 ? 32 : most;
+  return (int)(ns > most ? (most < 1 ? 1 : most) : (ns < 1 ? 1 : ns));
+}
+
 // pairsum_re.cu: float-float sums (VAR_V, VAR_OBJ) and difference sums (objective) of queued
 // queries, one CTA per query and row range.
 struct ReList {
@@ -89,10 +132,24 @@ void launch_pack_eval(int64_t n, const float* xyz, const float* lam_f, const dou
                       int near_on, double near_z, cudaStream_t s);
 void launch_plan_single(PlanHdr* plan, int32_t* item_off, int32_t* q_cnt, int32_t* work,
                         int nitems, int nsplit, int qper, int qcount, cudaStream_t s);
-void launch_nearfield(int var, bool tied, const ProbDesc* probs, const int32_t* near_list,
-                      const int32_t* near_cnt, const float4* qpos, const Lam4* qlam,
-                      const PlanHdr* plan, const int32_t* item_off, double* out, int grid,
-                      cudaStream_t s);
+// Near-field correction of the queries of a pass: added to the partial sums of a dense pass
+// (plan, item_off), or written as the last record of a pass of few queries (warps > 0).
+struct NearArgs {
+  const ProbDesc* probs;
+  const int32_t* list;      // near query slots; null: all of n queries, those with z <= near_z
+  const int32_t* cnt;       // entries of list (device)
+  int32_t n;
+  int32_t warps, strips;    // the pass of few queries: its warps and strips (0: a dense pass)
+  const int32_t* q_cnt;     // and its query count (device), or null: n
+  double near_z;
+  const float4* qpos;
+  const Lam4* qlam;
+  const PlanHdr* plan;      // dense pass
+  const int32_t* item_off;
+  const float4* sctab;      // sine and cosine table, or null: made by every CTA
+  double* out;
+};
+void launch_nearfield(int var, bool tied, const NearArgs& a, int sm_count, cudaStream_t s);
 void launch_pack_vjp(int64_t n, const float* xyz, const double* lam, const double* gB, int tied,
                      int nptiles, float* p32, double* p64, int fp64, cudaStream_t s);
 void launch_finalize_vjp(int64_t npix, const PlanHdr* plan, const double* out, double scale,

@@ -175,8 +175,16 @@ extern "C" dbie_status dbie_eval_noalloc(int32_t nx, int32_t ny, double x0, doub
   if (e != cudaSuccess) return err(DBIE_ECUDA, std::string("launch: ") + cudaGetErrorString(e));
   int sms = 1;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  launch_nearfield(VAR_V, false, prob, near, &ctl->near_cnt, qpos, qlam, &ctl->plan,
-                   ctl->item_off, out, 2 * sms, s);
+  NearArgs na{};
+  na.probs = prob;
+  na.list = near;
+  na.cnt = &ctl->near_cnt;
+  na.qpos = qpos;
+  na.qlam = qlam;
+  na.plan = &ctl->plan;
+  na.item_off = ctl->item_off;
+  na.out = out;
+  launch_nearfield(VAR_V, false, na, sms, s);
   launch_finalize_eval(VAR_V, n, &ctl->plan, ctl->item_off, out, qpos, qlam, hx / 6.0, 1.0, B,
                        nullptr, nullptr, nullptr, nullptr, nullptr, s);
   e = cudaGetLastError();

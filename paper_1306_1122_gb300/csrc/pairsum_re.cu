@@ -45,6 +45,7 @@
 
 #include "ff_math.cuh"
 #include "kernels.h"
+#include "warp_sums.cuh"
 
 namespace dbie {
 
@@ -99,38 +100,15 @@ __device__ __forceinline__ int re_split(int cnt, int rows, int ctas) {
   return ns < 1 ? 1 : (ns > most ? most : (int)ns);
 }
 
-// Sums over the CTA's threads: within a warp by halving (each step hands half of the sums to the
-// partner lane, so 16 pair additions reduce 12 sums instead of 60), then the warps' sums in FP64.
+// Sums over the CTA's threads: over the lanes of each warp, then the warps' sums in FP64.
 // `red` holds 4 * NSUM doubles.  Writes NSUM values to dst; callers synchronise before red is
 // written again.
 template <int NSUM>
 __device__ __forceinline__ void reduce_store(const ds (&acc)[NSUM], double* red, double* dst) {
-  constexpr int NP = NSUM > 8 ? 16 : 4;
+  constexpr int GL = WarpSums<NSUM>::GL;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto plus = [](ds a, ds b) {
-    const ds s = ff::two_sum(a.hi, b.hi);
-    return ds{s.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), s.lo)};
-  };
-  ds v[NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) v[i] = i < NSUM ? acc[i < NSUM ? i : 0] : ds{0.f, 0.f};
-  int off = 16;
-#pragma unroll
-  for (int half = NP / 2; half >= 1; half >>= 1, off >>= 1) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const ds give = up ? v[i] : v[i + half];
-      const ds keep = up ? v[i + half] : v[i];
-      v[i] = plus(keep, ds{__shfl_xor_sync(0xffffffffu, give.hi, off),
-                           __shfl_xor_sync(0xffffffffu, give.lo, off)});
-    }
-  }
-  for (; off >= 1; off >>= 1)
-    v[0] = plus(v[0], ds{__shfl_xor_sync(0xffffffffu, v[0].hi, off),
-                         __shfl_xor_sync(0xffffffffu, v[0].lo, off)});
-  constexpr int GL = 32 / NP;   // lanes that hold the same sum
-  if (lane % GL == 0 && lane / GL < NSUM) red[warp * NSUM + lane / GL] = ff::to_double(v[0]);
+  const ds r = WarpSums<NSUM>::reduce(acc, lane);
+  if (lane % GL == 0 && lane / GL < NSUM) red[warp * NSUM + lane / GL] = ff::to_double(r);
   __syncthreads();
   if (threadIdx.x < NSUM) {
     double t = red[threadIdx.x];

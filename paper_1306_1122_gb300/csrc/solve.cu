@@ -38,25 +38,6 @@ __device__ __forceinline__ void objective(const double B[3], const double G[9], 
   phi = f + w_g * g;
 }
 
-// Sum over the split partials of sum s of the query with local index j in problem pidx
-// (near-field corrections were already added to split 0).
-__device__ __forceinline__ double gather_sum(const double* out, const PlanHdr& h,
-                                             const int32_t* item_off, int pidx, int64_t j,
-                                             int nsum, int s) {
-  double v = 0.0;
-  for (int sp = 0; sp < h.nsplit; ++sp) v += out[out_index(h, item_off, pidx, j, sp, s, nsum)];
-  return v;
-}
-
-// The same over the row ranges of re-evaluated query `slot` (one item per query and range).
-__device__ __forceinline__ double gather_slot(const double* out, const PlanHdr& h, int64_t slot,
-                                              int nsum, int s) {
-  const double* p = out + slot * h.nsplit * nsum + s;
-  double v = 0.0;
-  for (int sp = 0; sp < h.nsplit; ++sp) v += p[(int64_t)sp * nsum];
-  return v;
-}
-
 // Pixel-exact near field: add the point's lambda-independent correction of B and grad B
 // (corr: dB_p at p, d(dB_p/dx_j) at 3 + 3 p + j).
 __device__ __forceinline__ void add_corr(const double* corr, double B[3], double G[9]) {
@@ -97,7 +78,7 @@ __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan
     const float4 pos = qpos[i];
     const double z = (double)pos.z;
     double S[NSUM];
-    for (int s = 0; s < NSUM; ++s) S[s] = gather_sum(out, h, item_off, 0, i, NSUM, s);
+    gather_sums<NSUM>(out, h, item_off, 0, i, S);
     double Bv[3], G[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int p = 0; p < 3; ++p) Bv[p] = z * S[p * NS];
     if constexpr (has_grad(VAR)) {
@@ -162,6 +143,11 @@ __device__ __forceinline__ double& SD(const SolveArgs& a, int f, int64_t g) {
 }
 __device__ __forceinline__ int32_t& SI(const SolveArgs& a, int f, int64_t g) {
   return a.si[(g >> 5) * (int64_t)(I_NFIELDS * 32) + (g & 31) + f * 32];
+}
+
+// First query slot of a point's problem: the problem's own range, or one queue for all.
+__device__ __forceinline__ int64_t queue_base(const SolveArgs& a, const ProbDesc& pd) {
+  return a.one_queue ? 0 : pd.q_off;
 }
 
 // Field f of value record id (vertex slot, VID_R, VID_E) of point g.
@@ -350,9 +336,7 @@ __device__ __forceinline__ void read_eval(const SolveArgs& a, const PlanHdr& h, 
                                           const double lam[3]) {
   const ProbDesc& pd = a.probs[pidx];
   double S[12], G[9];
-#pragma unroll
-  for (int s = 0; s < 12; ++s)
-    S[s] = gather_sum(a.out, h, a.item_off, pidx, slot - pd.q_off, 12, s);
+  gather_sums<12>(a.out, h, a.item_off, pidx, slot - queue_base(a, pd), S);
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
   e.s = (a.o.tie > 0.0 && a.msc)
             ? mixed_phi_bound(a.msc + 15 * g, lam, a.o.dim, z, e.B, G, e.g, pd.g_scale, a.o.w_g)
@@ -370,8 +354,7 @@ __device__ __forceinline__ void read_reeval(const SolveArgs& a, bool dif, int pi
   const double* out = dif ? a.dout : a.fout;
   const PlanHdr h = dif ? *a.dplan : *a.fplan;
   double G[9];
-#pragma unroll
-  for (int s = 0; s < 12; ++s) S[s] = gather_slot(out, h, slot, 12, s);
+  gather_sums<12>(out, h, nullptr, 0, slot, S);
   if (dif) {
 #pragma unroll
     for (int s = 0; s < 12; ++s) S[s] = SD(a, D_REFS + s, g) + S[s];
@@ -423,8 +406,8 @@ template <int K>
 __device__ __forceinline__ void emit(const SolveArgs& a, int64_t g, const float4& pos, int pidx,
                                      const double (*lam)[3]) {
   const ProbDesc& pd = a.probs[pidx];
-  const int base = atomic_add_warp(a.nxt.q_cnt + pidx, K);
-  const int64_t slot0 = pd.q_off + base;
+  const int base = atomic_add_warp(a.nxt.q_cnt + (a.one_queue ? 0 : pidx), K);
+  const int64_t slot0 = queue_base(a, pd) + base;
 #pragma unroll
   for (int j = 0; j < K; ++j) {
     a.nxt.qpos[slot0 + j] = pos;
@@ -1011,7 +994,7 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   const PlanHdr h = *plan;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    for (int s = 0; s < 12; ++s) dS[12 * i + s] = gather_slot(out, h, i, 12, s);
+    gather_sums<12>(out, h, nullptr, 0, i, dS + 12 * i);
     if (dS_bound) {
       const double la[3] = {qlam[i].x, qlam[i].y, qlam[i].z};
       const double l0[3] = {qlam0[i].x, qlam0[i].y, qlam0[i].z};
@@ -1078,8 +1061,9 @@ __global__ void certb_apply_kernel(const SolveArgs a) {
     const double z = (double)pos.z;
     const int64_t slot = SI(a, I_RSLOT, g);
     const double* corr = corr_of(a, pd, g, z);
-    for (int p = 0; p < 3; ++p)
-      a.res_B[3 * g + p] = z * gather_slot(a.fout, hf, slot, 3, p) + (corr ? corr[p] : 0.0);
+    double S[3];
+    gather_sums<3>(a.fout, hf, nullptr, 0, slot, S);
+    for (int p = 0; p < 3; ++p) a.res_B[3 * g + p] = z * S[p] + (corr ? corr[p] : 0.0);
   }
 }
 
@@ -1161,8 +1145,7 @@ __global__ void finalize_objective_kernel(int64_t n, const PlanHdr* __restrict__
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     double S[21];
-#pragma unroll
-    for (int s = 0; s < 21; ++s) S[s] = gather_sum(out, h, item_off, 0, i, 21, s);
+    gather_sums<21>(out, h, item_off, 0, i, S);
     const Lam4 l = qlam[i];
     const double lam[3] = {l.x, l.y, l.z};
     Eval e;
@@ -1257,9 +1240,7 @@ __global__ void bfgs_step_kernel(const SolveArgs a) {
     }
     const double lamt[3] = {xt[0], n == 1 ? xt[0] : xt[1], n == 1 ? xt[0] : xt[2]};
     double S[21];
-    const int64_t j = (int64_t)SI(a, I_QSLOT, g) - pd.q_off;
-#pragma unroll
-    for (int s = 0; s < 21; ++s) S[s] = gather_sum(a.out, h, a.item_off, pidx, j, 21, s);
+    gather_sums<21>(a.out, h, a.item_off, pidx, (int64_t)SI(a, I_QSLOT, g) - queue_base(a, pd), S);
     Eval e;
     double dp[3], gt[3] = {0, 0, 0};
     objective_grad(S, z, lamt, pd.g_scale, a.o.w_g, e, dp, corr_of(a, pd, g, z));

@@ -91,7 +91,7 @@ struct SolveArgs {
   int32_t* res_nfev;
   char* codes;               // [N * codes_stride] or null
   int32_t codes_stride;
-  int32_t pad1;
+  int32_t one_queue;         // passes of few queries: query slots of all problems in one queue
   unsigned* err;
   const double* corr;        // [N * 12] pixel-exact corrections (dB, d grad B), or null
   // certified decisions
