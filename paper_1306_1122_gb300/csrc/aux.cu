@@ -211,6 +211,8 @@ __device__ __forceinline__ long near_index(double x, double x0, double h, int nq
   return e * g + best;
 }
 
+constexpr int NEAR_NT = 128;   // four independent warps
+
 // GL lanes per query (a divisor of 32).
 template <int VAR, bool TIED, int GL>
 __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const PlanHdr& h,
@@ -227,8 +229,10 @@ __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const P
     c = ff::to_double(C);
   };
   const int lane = threadIdx.x & 31, sub = lane & (GL - 1), grp = lane / GL;
+  const int64_t warp = blockIdx.x * (int64_t)(NEAR_NT / 32) + (threadIdx.x >> 5);
+  const int64_t nwarps = (int64_t)gridDim.x * (NEAR_NT / 32);
   // (the loop runs warp-uniformly so the shuffles see every lane)
-  for (int64_t wb = blockIdx.x * (int64_t)(32 / GL); wb < cnt; wb += gridDim.x * (int64_t)(32 / GL)) {
+  for (int64_t wb = warp * (32 / GL); wb < cnt; wb += nwarps * (32 / GL)) {
     const int64_t w = wb + grp;
     const bool listed = w < cnt;
     const int64_t wq = listed ? w : wb;
@@ -252,9 +256,9 @@ __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const P
     for (int s = 0; s < NSUM; ++s) c[s] = 0.0;
     const bool valid = listed && (a.list || (double)pos.z <= a.near_z);
     if (valid && wi > 0 && wj > 0 && wi <= 2 * W + 1 && wj <= 2 * W + 1) {
-      const int nwin = (int)(wi * wj);
+      const int nwin = (int)(wi * wj), wx = (int)wi;
       for (int e = sub; e < nwin; e += GL) {
-        const int64_t k = (j0 + e / wi) * (int64_t)pd.nx + (i0 + e % wi);
+        const int64_t k = (j0 + e / wx) * (int64_t)pd.nx + (i0 + e % wx);
         const int nf = pd.nf32 > 0 ? pd.nf32 : NFIELD;
         const float b32[3] = {*tile_field(pd.tiles32, k, 2, nf), *tile_field(pd.tiles32, k, 3, nf),
                               *tile_field(pd.tiles32, k, 4, nf)};
@@ -301,43 +305,67 @@ __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const P
         }
       }
     }
+    // the lanes' sums, by halving: each step hands half of the sums to the partner lane (16 FP64
+    // additions for 12 sums over 32 lanes instead of 60)
+    constexpr int NP = NSUM > 16 ? 32 : NSUM > 8 ? 16 : NSUM > 4 ? 8 : 4;
+    constexpr int LEFT = NP / GL > 0 ? NP / GL : 1;   // sums per lane at the end
+    double v[NP];
 #pragma unroll
-    for (int s = 0; s < NSUM; ++s) {
-      double v = c[s];
-      for (int off = GL / 2; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (sub == 0 && valid) {
-        if (a.warps > 0) a.out[(slot * h.nsplit + h.nsplit - 1) * NSUM + s] = v;
-        else a.out[out_index(h, a.item_off, pidx, slot - pd.q_off, 0, s, NSUM)] += v;
+    for (int s = 0; s < NP; ++s) v[s] = s < NSUM ? c[s < NSUM ? s : 0] : 0.0;
+    int half = NP / 2;
+#pragma unroll
+    for (int off = GL / 2; off > 0; off >>= 1, half >>= 1) {
+      if (half >= 1) {
+        const bool up = (sub & off) != 0;
+#pragma unroll
+        for (int s = 0; s < half; ++s) {
+          const double give = up ? v[s] : v[s + half];
+          const double keep = up ? v[s + half] : v[s];
+          v[s] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+      }
+    }
+    constexpr int SAME = NP < GL ? GL / NP : 1;       // lanes that hold the same sums
+    if (valid && sub % SAME == 0) {
+#pragma unroll
+      for (int i = 0; i < LEFT; ++i) {
+        const int s = sub / SAME * LEFT + i;
+        if (s < NSUM) {
+          if (a.warps > 0) a.out[(slot * h.nsplit + h.nsplit - 1) * NSUM + s] = v[i];
+          else a.out[out_index(h, a.item_off, pidx, slot - pd.q_off, 0, s, NSUM)] += v[i];
+        }
       }
     }
   }
 }
 
-// CTAs of one warp.  Eight lanes per query, four queries per warp: a 7 x 7 window takes 7 passes
-// of 8 lanes (49 of 56 lane slots busy) instead of 2 of 32 (49 of 64).  With no more queries than
-// CTAs a query takes a whole warp instead: the two passes then set the kernel's length, which is
-// latency (about 500 instructions a pass), not FP64 throughput.  512 near queries of 2,048: 71 us
-// in CTAs of 256 threads (16 SMs busy), 50 us as one-warp CTAs of four queries.
+// Eight lanes per query, four queries per warp: a 7 x 7 window takes 7 passes of 8 lanes (49 of 56
+// lane slots busy) instead of 2 of 32 (49 of 64).  With no more queries than warps a query takes a
+// whole warp instead: the two passes then set the kernel's length, which is latency (about 400
+// instructions a pass).  CTAs of four independent warps, one per SM sub-partition.  512 near queries of 2,048:
+// 71 us in CTAs of 256 threads and four queries per warp (16 SMs busy).
 template <int VAR, bool TIED>
-__global__ void __launch_bounds__(32) nearfield_kernel(const NearArgs a) {
+__global__ void __launch_bounds__(NEAR_NT) nearfield_kernel(const NearArgs a) {
   __shared__ float4 s_tab[ff::SC_TABLE];
   const int cnt = a.list ? *a.cnt : a.n;
   if (blockIdx.x >= cnt) return;
-  for (int i = threadIdx.x; i < ff::SC_TABLE; i += 32) {
-    if (a.sctab) s_tab[i] = __ldg(a.sctab + i);
-    else ff::fill_sincos_table(s_tab, i);
+  if (threadIdx.x < ff::SC_TABLE) {
+    if (a.sctab) s_tab[threadIdx.x] = __ldg(a.sctab + threadIdx.x);
+    else ff::fill_sincos_table(s_tab, threadIdx.x);
   }
-  __syncwarp();
+  __syncthreads();
   PlanHdr h{0, 1, 1, 0};
   if (a.warps > 0) h.nsplit = few_split(a.q_cnt ? *a.q_cnt : a.n, a.strips, a.warps) + 1;
   else h = *a.plan;
-  if (cnt <= (int)gridDim.x) near_queries<VAR, TIED, 32>(a, cnt, h, s_tab);
+  if (cnt <= (int)gridDim.x * (NEAR_NT / 32)) near_queries<VAR, TIED, 32>(a, cnt, h, s_tab);
   else near_queries<VAR, TIED, 8>(a, cnt, h, s_tab);
 }
 
 void launch_nearfield(int var, bool tied, const NearArgs& a, int sm_count, cudaStream_t s) {
-  const int grid = 16 * sm_count;   // resident at the kernel's register count
-#define NF(V, T) nearfield_kernel<V, T><<<grid, 32, 0, s>>>(a)
+  const int grid = 4 * sm_count;
+#define NF(V, T) nearfield_kernel<V, T><<<grid, NEAR_NT, 0, s>>>(a)
   if (tied) {
     switch (var) {
       case VAR_V: NF(VAR_V, true); break;
@@ -429,8 +457,8 @@ __global__ void finalize_vjp_kernel(int64_t npix, const PlanHdr* __restrict__ pl
 
 void launch_finalize_vjp(int64_t npix, const PlanHdr* plan, const double* out, double scale,
                          double* gB0, int accumulate, cudaStream_t s) {
-  const int grid = (int)((npix + 255) / 256 < 8192 ? (npix + 255) / 256 : 8192);
-  finalize_vjp_kernel<<<grid, 256, 0, s>>>(npix, plan, out, scale, gB0, accumulate);
+  const PerPoint L(npix);
+  finalize_vjp_kernel<<<L.grid, L.nt, 0, s>>>(npix, plan, out, scale, gB0, accumulate);
 }
 
 }  // namespace dbie

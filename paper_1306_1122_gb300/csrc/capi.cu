@@ -953,8 +953,7 @@ dbie_status dbie_eval_difference(dbie_ctx* c, int64_t n, const float* xyz,
   if (dS_bound) {
     DBIE_TRY(ensure(c->dmsc, sizeof(double) * 18 * n));
     msc = c->dmsc.as<double>();
-    launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n,
-               (int)std::min<int64_t>((n + 127) / 128, 32LL * c->sm_count), s);
+    launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n, c->sm_count, s);
   }
   launch_dif_debug(n, &m->plan, c->out.as<double>(), c->qlam.as<Lam4>(),
                    c->qlam0.as<Lam4>(), msc, msc ? msc + 15 * n : nullptr, tied ? 1 : 3, dS,
@@ -1469,7 +1468,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     if (!fp64) DBIE_TRY(ensure(b.near[sd], sizeof(int32_t) * Qcap));
   }
   if (cert) {
-    DBIE_TRY(ensure(b.msc, sizeof(double) * 18 * N));
+    DBIE_TRY(ensure(b.msc, sizeof(float) * 18 * N));
     DBIE_TRY(ensure(b.fout, sizeof(double) * std::max(12 * reeval_items(2 * N, grid_re),
                                                       3 * reeval_items(N, grid_v))));
     for (int sd = 0; sd < 2; ++sd) {
@@ -1550,9 +1549,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   for (int sd = 0; sd < 2; ++sd) CUDA_TRY(cudaMemsetAsync(b.q_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
   if (cert) {
     // the error bounds' lambda-independent absolute-value sums of every point
-    launch_msc(b.probs.as<ProbDesc>(), N, b.ppos.as<float4>(), b.msc.as<double>(),
-               b.msc.as<double>() + 15 * N,
-               (int)std::min<int64_t>((N + 127) / 128, 32LL * c->sm_count), s);
+    launch_msc(b.probs.as<ProbDesc>(), N, b.ppos.as<float4>(), b.msc.as<float>(),
+               b.msc.as<float>() + 15 * N, c->sm_count, s);
     CUDA_TRY(cudaGetLastError());
   }
   if (codes_stride) CUDA_TRY(cudaMemsetAsync(b.codes.p, 0, (size_t)codes_stride * N, s));
@@ -1617,12 +1615,12 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     a.err = c->err.as<unsigned>();
     a.corr = pxe_any ? b.corr.as<double>() : nullptr;
     if (cert) {
-      a.msc = b.msc.as<double>();
+      a.msc = b.msc.as<float>();
       a.fout = b.fout.as<double>();
       a.fplan = &ctrl->fplan;
       a.rework = ctrl->rework;
       a.stat_ties = &ctrl->stat_ties;
-      a.msc0 = b.msc.as<double>() + 15 * N;
+      a.msc0 = b.msc.as<float>() + 15 * N;
     }
     if (dif_on) {
       a.dout = b.dout.as<double>();
@@ -1632,8 +1630,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   }
   // Initial simplex and its queries go to side 0.
   SolveArgs a0 = sa[1];  // "next" of the side-1 round is side 0
-  // step kernels: CTAs of one warp, full residency at their register count
-  const int nm_grid = (int)std::min<int64_t>(N, 8LL * c->sm_count);
+  // step kernels: four warps per CTA, resident at their register count; every point a warp at most
+  const int nm_grid = (int)std::min<int64_t>((N + 3) / 4, 4LL * c->sm_count);
   const int apply_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
   (qn ? launch_bfgs_init : launch_solve_init)(a0, any_init ? b.lam0.as<double>() : nullptr,
                     (int)std::min<int64_t>((N + 255) / 256, 8LL * c->sm_count), s);

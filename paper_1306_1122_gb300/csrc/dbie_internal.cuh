@@ -135,16 +135,16 @@ __host__ __device__ inline int64_t out_index(const PlanHdr& h, const int32_t* it
   return (item * nsum + s) * h.qper + r;
 }
 
-// S[0..NSUM): the query's sums over its splits, added in order.
+// S[0..NSUM): the query's sums over its splits (without the last `skip`), added in order.
 template <int NSUM>
 __device__ __forceinline__ void gather_sums(const double* __restrict__ out, const PlanHdr& h,
                                             const int32_t* item_off, int pidx, int64_t j,
-                                            double* S) {
+                                            double* S, int skip = 0) {
   const double* p = out + out_index(h, item_off, pidx, j, 0, 0, NSUM);
   const int64_t step = (int64_t)NSUM * h.qper;
 #pragma unroll
   for (int s = 0; s < NSUM; ++s) S[s] = p[(int64_t)s * h.qper];
-  for (int sp = 1; sp < h.nsplit; ++sp) {
+  for (int sp = 1; sp < h.nsplit - skip; ++sp) {
     p += step;
 #pragma unroll
     for (int s = 0; s < NSUM; ++s) S[s] += p[(int64_t)s * h.qper];

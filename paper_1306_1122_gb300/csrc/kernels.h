@@ -25,6 +25,19 @@ __host__ __device__ constexpr LaunchCfg cfg_of(int c, int var = -1) {
                 : LaunchCfg{1, 128, var == VAR_HESS ? 4 : 7};
 }
 
+// Launch shape of kernels with one thread per point or pixel (gathering of partial sums, FP64
+// objective): their length is one thread's latency, so few points go to small CTAs on all 152 SMs
+// instead of filling some of them (4,096 points: 66 us in 16 CTAs of 256 threads).
+struct PerPoint {
+  int grid, nt;
+  explicit PerPoint(int64_t n, int nt_many = 256) {
+    const int64_t warps = (n + 32 * 152 - 1) / (32 * 152);   // per SM
+    nt = warps >= nt_many / 32 ? nt_many : (warps < 1 ? 32 : 32 * (int)warps);
+    const int64_t g = (n + nt - 1) / nt;
+    grid = (int)(g < 1 ? 1 : (g < 4096 ? g : 4096));
+  }
+};
+
 struct KernelRef {
   const void* fn;     // __global__ function
   int nt;             // threads per CTA
@@ -206,8 +219,10 @@ void launch_solve_init(const SolveArgs& a, const double* lam_init, int grid, cud
 void launch_plan_round(const PlanArgs& a, cudaStream_t s);
 void launch_nm_step(const SolveArgs& a, int grid, cudaStream_t s);
 void launch_nm_refine(const SolveArgs& a, int grid, cudaStream_t s);
+void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, float* msc, float* msc0,
+                int sm_count, cudaStream_t s);
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
-                int grid, cudaStream_t s);
+                int sm_count, cudaStream_t s);
 void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const Lam4* qlam,
                       const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s);

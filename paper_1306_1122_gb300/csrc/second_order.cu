@@ -443,9 +443,9 @@ void launch_finalize_hessian(int64_t n, const PlanHdr* plan, const int32_t* item
                              double g_scale, double w_g, double* phi, double* grad, double* hess,
                              const double* corr, cudaStream_t s) {
   if (n <= 0) return;
-  finalize_hessian_kernel<<<grid_for(n, 4096), 256, 0, s>>>(n, plan, item_off, out, qpos, qlam,
-                                                            dim, g_scale, w_g, phi, grad, hess,
-                                                            corr);
+  const PerPoint L(n);
+  finalize_hessian_kernel<<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, qlam, dim, g_scale,
+                                                  w_g, phi, grad, hess, corr);
 }
 
 void launch_implicit_weights(int64_t n, int nptiles, const PlanHdr* plan, const int32_t* item_off,
@@ -455,7 +455,8 @@ void launch_implicit_weights(int64_t n, int nptiles, const PlanHdr* plan, const 
                              const double* corr, double* pxe_w, cudaStream_t s) {
   const int64_t total = (int64_t)nptiles * TILE;
   if (total <= 0) return;
-  implicit_weights_kernel<<<grid_for(total, 4096), 128, 0, s>>>(
+  const PerPoint L(total, 128);
+  implicit_weights_kernel<<<L.grid, L.nt, 0, s>>>(
       n, nptiles, plan, item_off, out, qpos, qlam, gB, dim, g_scale, w_g, p32, p64, fp64, v_out,
       flags, corr, pxe_w);
 }
@@ -463,7 +464,8 @@ void launch_implicit_weights(int64_t n, int nptiles, const PlanHdr* plan, const 
 void launch_finalize_nv(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
                         const float4* qpos, double* var, cudaStream_t s) {
   if (n <= 0) return;
-  finalize_nv_kernel<<<grid_for(n, 4096), 256, 0, s>>>(n, plan, item_off, out, qpos, var);
+  const PerPoint L(n);
+  finalize_nv_kernel<<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, var);
 }
 
 void launch_stage_variance(const float* sx, const float* sy, const float* sz, double sigma0,

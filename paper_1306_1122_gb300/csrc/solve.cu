@@ -12,17 +12,20 @@
 //    trial points of all active points in one pair-sum pass.
 #include "kernels.h"
 #include "solve.cuh"
+#include "warp_sums.cuh"
 
 namespace dbie {
 
 struct Eval {
   double B[3];
   double f, g, phi;
-  double s;   // error bound of phi (certified decisions; 0 when not computed)
+  double nJ, nB;   // |J|, |B|
+  float s;         // signed tie radius of phi (certified decisions; see TieLog)
 };
 
 __device__ __forceinline__ void objective(const double B[3], const double G[9], double g_scale,
-                                          double w_g, double& f, double& g, double& phi) {
+                                          double w_g, double& f, double& g, double& phi,
+                                          double* norms = nullptr) {
   const double Jx = G[3 * 2 + 1] - G[3 * 1 + 2];
   const double Jy = G[3 * 0 + 2] - G[3 * 2 + 0];
   const double Jz = G[3 * 1 + 0] - G[3 * 0 + 1];
@@ -36,6 +39,10 @@ __device__ __forceinline__ void objective(const double B[3], const double G[9], 
   f = (nJ * nB > 0.0) ? nC / (nJ * nB) : 0.0;
   g = (nB > 0.0) ? fabs(div) * g_scale / nB : 0.0;
   phi = f + w_g * g;
+  if (norms) {
+    norms[0] = nJ;
+    norms[1] = nB;
+  }
 }
 
 // Pixel-exact near field: add the point's lambda-independent correction of B and grad B
@@ -58,7 +65,10 @@ __device__ __forceinline__ void assemble_obj(const double S[12], double z, doubl
     G[3 * p + 2] = S0 + z * z * S1;
   }
   add_corr(corr, e.B, G);
-  objective(e.B, G, g_scale, w_g, e.f, e.g, e.phi);
+  double norms[2];
+  objective(e.B, G, g_scale, w_g, e.f, e.g, e.phi, norms);
+  e.nJ = norms[0];
+  e.nB = norms[1];
 }
 
 // ----------------------------------------------------------------- eval finalize ----
@@ -122,10 +132,10 @@ void launch_finalize_eval(int var, int64_t n, const PlanHdr* plan, const int32_t
                           double w_g, double* B, double* gradB, double* dBdl, const double* gB,
                           double* fgphi, const double* corr, cudaStream_t s) {
   if (n <= 0) return;
-  const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-#define FIN(V)                                                                              \
-  finalize_eval_kernel<V><<<grid, 256, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale, \
-                                               w_g, B, gradB, dBdl, gB, fgphi, corr)
+  const PerPoint L(n);
+#define FIN(V)                                                                                \
+  finalize_eval_kernel<V><<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale, \
+                                                  w_g, B, gradB, dBdl, gB, fgphi, corr)
   switch (var) {
     case VAR_V: FIN(VAR_V); break;
     case VAR_VL: FIN(VAR_VL); break;
@@ -154,12 +164,19 @@ __device__ __forceinline__ int64_t queue_base(const SolveArgs& a, const ProbDesc
 __device__ __forceinline__ double& SV(const SolveArgs& a, int id, int f, int64_t g) {
   return SD(a, id * VREC + f, g);
 }
+// A float as a double, without a conversion (which would run at the FP64 rate); subnormals to 0.
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  const unsigned hi = e == 0u ? 0u : (e == 255u ? 0x7ff00000u : (e + 896u) << 20);
+  const unsigned m = e == 0u ? 0u : b & 0x7fffffu;
+  return __hiloint2double((int)((b & 0x80000000u) | hi | (m >> 3)), (int)(m << 29));
+}
 __device__ __forceinline__ void store_value(const SolveArgs& a, int id, int64_t g, const Eval& e) {
   for (int p = 0; p < 3; ++p) SV(a, id, V_B + p, g) = e.B[p];
   SV(a, id, V_F, g) = e.f;
   SV(a, id, V_G, g) = e.g;
   SV(a, id, V_PHI, g) = e.phi;
-  SV(a, id, V_S, g) = e.s;
+  SV(a, id, V_S, g) = f64_of(e.s);
 }
 __device__ __forceinline__ void copy_value(const SolveArgs& a, int from, int to, int64_t g) {
   double v[VREC];
@@ -169,10 +186,11 @@ __device__ __forceinline__ void copy_value(const SolveArgs& a, int from, int to,
   for (int f = 0; f < VREC; ++f) SV(a, to, f, g) = v[f];
 }
 
-// What a step compares: Phi, its error bound s, the vertex's storage slot and the record that
+// What a step compares: Phi, its signed tie radius, the vertex's storage slot and the record that
 // holds the value (the slot, or VID_R / VID_E for a value that is about to take the slot's place).
 struct Vert {
-  double phi, s;
+  double phi;
+  float s;
   int slot, id;
 };
 
@@ -201,43 +219,64 @@ __device__ __forceinline__ const double* corr_of(const SolveArgs& a, const ProbD
 constexpr double BND_A0 = 9.5e-7, BND_A1 = 1.06e-6, BND_A2 = 1.1e-7, BND_A3 = 1.45e-6,
                  BND_A4 = 1.56e-6;
 
-// First-order bound of Phi's error from the bounds dB (3) and dG (9) of B and grad B.
-__device__ __forceinline__ double propagate_bound(const double dB[3], const double dG[9],
-                                                  const double B[3], const double G[9],
-                                                  double g, double g_scale, double w_g) {
-  const double Jx = G[7] - G[5], Jy = G[2] - G[6], Jz = G[3] - G[1];
-  const double nJ = sqrt(Jx * Jx + Jy * Jy + Jz * Jz);
-  const double nB = sqrt(B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
-  const double dJx = dG[7] + dG[5], dJy = dG[2] + dG[6], dJz = dG[3] + dG[1];
-  const double ndJ = sqrt(dJx * dJx + dJy * dJy + dJz * dJz);
-  const double ndB = sqrt(dB[0] * dB[0] + dB[1] * dB[1] + dB[2] * dB[2]);
-  if (!(nB > 0.0)) return 2.0;
-  double sf = nJ > 0.0 ? ndJ / nJ + ndB / nB : 1.0;
-  if (sf > 1.0) sf = 1.0;
-  const double sg = g_scale * (dG[0] + dG[4] + dG[8]) / nB + g * ndB / nB;
-  return sf + w_g * sg;
+// The bounds are evaluated in FP32: a dependent FP64 instruction takes 70 cycles and more here, the
+// bound took two thirds of a value's time, and a worst case whose coefficients have two or three
+// digits (and M_j, summed from FP32 terms) does not need more.
+// A double's value in FP32, truncated (FP64 conversions run at the FP64 rate).
+__device__ __forceinline__ float f32_of(double x) {
+  const int hi = __double2hiint(x);
+  const int e = ((hi >> 20) & 0x7ff) - 896;   // FP32 exponent field
+  const unsigned m = ((unsigned)hi << 3 & 0x7fffffu) | ((unsigned)__double2loint(x) >> 29);
+  const unsigned sg = (unsigned)hi & 0x80000000u;
+  if (e <= 0) return __uint_as_float(sg);                              // below FP32's range: 0
+  if (e >= 255) return __uint_as_float(sg | 0x7f800000u | (e == 1151 ? m : 0u));   // inf, NaN
+  return __uint_as_float(sg | (unsigned)e << 23 | m);
+}
+// Norm without overflow or underflow of the squares.
+__device__ __forceinline__ float norm3f(float x, float y, float z) {
+  const float m = fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)));
+  if (!(m > 0.f)) return m;
+  const float i = 1.0f / m;
+  x *= i;
+  y *= i;
+  z *= i;
+  return m * sqrtf(x * x + y * y + z * z);
 }
 
-__device__ __forceinline__ double mixed_phi_bound(const double* M, const double lam[3], int dim,
-                                                   double z, const double B[3], const double G[9],
-                                                   double g, double g_scale, double w_g) {
-  double dB[3], dG[9];
+// First-order bound of Phi's error from the bounds dB (3) and dG (9) of B and grad B.
+__device__ __forceinline__ float propagate_bound(const float dB[3], const float dG[9],
+                                                 const Eval& e, double g_scale, double w_g) {
+  const float nJ = f32_of(e.nJ), nB = f32_of(e.nB);
+  if (!(e.nB > 0.0)) return 2.0f;
+  const float ndJ = norm3f(dG[7] + dG[5], dG[2] + dG[6], dG[3] + dG[1]);
+  const float rB = norm3f(dB[0], dB[1], dB[2]) / nB;
+  float sf = nJ > 0.f ? ndJ / nJ + rB : 1.0f;
+  if (sf > 1.0f) sf = 1.0f;
+  const float sg = f32_of(g_scale) * (dG[0] + dG[4] + dG[8]) / nB + f32_of(e.g) * rB;
+  return sf + f32_of(w_g) * sg;
+}
+
+__device__ __forceinline__ float mixed_phi_bound(const float* M, const double lam[3], int dim,
+                                                 float z, const Eval& e, double g_scale,
+                                                 double w_g) {
+  constexpr float A0 = BND_A0, A1 = BND_A1, A2 = BND_A2, A3 = BND_A3, A4 = BND_A4;
+  float dB[3], dG[9];
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    const double L = fabs(dim == 1 ? lam[0] : lam[p]);
-    const double* m = M + 5 * p;
-    const double L2 = L * L, L3 = L2 * L;
-    const double s0 = BND_A0 * m[2] + BND_A1 * L * m[1] + BND_A2 * L2 * m[0];
-    const double sx = BND_A0 * L2 * m[1] + BND_A2 * L3 * m[0] +
-                      3.0 * (BND_A3 * m[3] + BND_A4 * L * m[2] + BND_A2 * L2 * m[1]);
-    const double s1 = BND_A0 * L2 * m[2] + BND_A2 * L3 * m[1] +
-                      3.0 * (BND_A3 * m[4] + BND_A4 * L * m[3] + BND_A2 * L2 * m[2]);
+    const float L = fabsf(f32_of(dim == 1 ? lam[0] : lam[p]));
+    const float* m = M + 5 * p;
+    const float L2 = L * L, L3 = L2 * L;
+    const float s0 = A0 * m[2] + A1 * L * m[1] + A2 * L2 * m[0];
+    const float sx = A0 * L2 * m[1] + A2 * L3 * m[0] +
+                     3.0f * (A3 * m[3] + A4 * L * m[2] + A2 * L2 * m[1]);
+    const float s1 = A0 * L2 * m[2] + A2 * L3 * m[1] +
+                     3.0f * (A3 * m[4] + A4 * L * m[3] + A2 * L2 * m[2]);
     dB[p] = z * s0;
     dG[3 * p + 0] = z * sx;
     dG[3 * p + 1] = z * sx;
     dG[3 * p + 2] = s0 + z * z * s1;
   }
-  return propagate_bound(dB, dG, B, G, g, g_scale, w_g);
+  return propagate_bound(dB, dG, e, g_scale, w_g);
 }
 
 // Error bounds of the difference sums (pairsum_dif.cu) that take a point's float-float
@@ -257,26 +296,25 @@ constexpr double DIF_C00 = 4.2e-6, DIF_C01 = 5.2e-6, DIF_C02 = 2.2e-7;
 constexpr double DIF_C10 = 1.3e-5, DIF_C11 = 2.4e-5, DIF_C12 = 5.2e-6, DIF_C13 = 2.2e-7;
 constexpr double DIF_FF = 1e-12;
 
-// e[4 p + s]: bounds of S0, S1, Sx, Sy of component p (M: M_1..M_5 per component, M0: M_0).
-__device__ __forceinline__ void dif_sum_bounds(const double* M, const double* M0,
-                                               const double la[3], const double l0[3], int dim,
-                                               double e[12]) {
+// e[4 p + s]: bounds of S0, S1, Sx, Sy of component p (M: M_1..M_5 per component, M0: M_0; per free
+// lambda, dl = |lambda_a - lambda_0|, L = |lambda_a| + |lambda_0| and R = |lambda_0|).
+template <typename T>
+__device__ __forceinline__ void dif_sum_bounds(const T* M, const T* M0, const T dl_[3],
+                                               const T L_[3], const T R_[3], int dim, T e[12]) {
+  constexpr T C00 = DIF_C00, C01 = DIF_C01, C02 = DIF_C02, C10 = DIF_C10, C11 = DIF_C11,
+              C12 = DIF_C12, C13 = DIF_C13, FF = DIF_FF;
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
     const int q = dim == 1 ? 0 : p;
-    const double dl = fabs(la[q] - l0[q]);
-    const double L = fabs(la[q]) + fabs(l0[q]), L2 = L * L, L3 = L2 * L;
-    const double R = fabs(l0[q]), R2 = R * R;
-    const double* m = M + 5 * p;   // m[j - 1] = M_j
-    const double m0 = M0[p];
-    const double e0 = dl * (DIF_C00 * m[1] + DIF_C01 * L * m[0] + DIF_C02 * L2 * m0) +
-                      DIF_FF * (m[2] + R * m[1]);
-    const double e1 = dl * (DIF_C10 * m[3] + DIF_C11 * L * m[2] + DIF_C12 * L2 * m[1] +
-                            DIF_C13 * L3 * m[0]) +
-                      DIF_FF * (3.0 * m[4] + 3.0 * R * m[3] + R2 * m[2]);
-    const double ex = dl * (DIF_C10 * m[2] + DIF_C11 * L * m[1] + DIF_C12 * L2 * m[0] +
-                            DIF_C13 * L3 * m0) +
-                      DIF_FF * (3.0 * m[3] + 3.0 * R * m[2] + R2 * m[1]);
+    const T dl = dl_[q], L = L_[q], L2 = L * L, L3 = L2 * L;
+    const T R = R_[q], R2 = R * R;
+    const T* m = M + 5 * p;   // m[j - 1] = M_j
+    const T m0 = M0[p];
+    const T e0 = dl * (C00 * m[1] + C01 * L * m[0] + C02 * L2 * m0) + FF * (m[2] + R * m[1]);
+    const T e1 = dl * (C10 * m[3] + C11 * L * m[2] + C12 * L2 * m[1] + C13 * L3 * m[0]) +
+                 FF * (T(3) * m[4] + T(3) * R * m[3] + R2 * m[2]);
+    const T ex = dl * (C10 * m[2] + C11 * L * m[1] + C12 * L2 * m[0] + C13 * L3 * m0) +
+                 FF * (T(3) * m[3] + T(3) * R * m[2] + R2 * m[1]);
     e[4 * p + 0] = e0;
     e[4 * p + 1] = e1;
     e[4 * p + 2] = ex;
@@ -284,49 +322,69 @@ __device__ __forceinline__ void dif_sum_bounds(const double* M, const double* M0
   }
 }
 
-// Phi bound of a value assembled from reference plus difference sums with sum bounds e.
-__device__ __forceinline__ double dif_phi_bound(const double e[12], double z, const double B[3],
-                                                const double G[9], double g, double g_scale,
-                                                double w_g) {
-  double dB[3], dG[9];
+// Phi bound of a value assembled from reference plus difference sums with sum bounds eb.
+__device__ __forceinline__ float dif_phi_bound(const float eb[12], float z, const Eval& e,
+                                               double g_scale, double w_g) {
+  float dB[3], dG[9];
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    dB[p] = z * e[4 * p];
-    dG[3 * p + 0] = z * e[4 * p + 2];
-    dG[3 * p + 1] = z * e[4 * p + 3];
-    dG[3 * p + 2] = e[4 * p] + z * z * e[4 * p + 1];
+    dB[p] = z * eb[4 * p];
+    dG[3 * p + 0] = z * eb[4 * p + 2];
+    dG[3 * p + 1] = z * eb[4 * p + 3];
+    dG[3 * p + 2] = eb[4 * p] + z * z * eb[4 * p + 1];
   }
-  return propagate_bound(dB, dG, B, G, g, g_scale, w_g);
+  return propagate_bound(dB, dG, e, g_scale, w_g);
+}
+
+// Comparisons of doubles on the integer pipe, with the results of <, <= on doubles (NaN false).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return (b << 1) == 0 ? 0 : b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ bool not_nan(double x) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffll) <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool less(double x, double y) {
+  return not_nan(x) && not_nan(y) && order_key(x) < order_key(y);
+}
+__device__ __forceinline__ bool less_eq(double x, double y) {
+  return not_nan(x) && not_nan(y) && order_key(x) <= order_key(y);
+}
+
+// Tie radius of a value: `band` times its bound (never 0, which marks a value without one).
+__device__ __forceinline__ float radius_of(double band, float bound) {
+  const float r = f32_of(band) * bound;
+  return r < 1e-37f ? 1e-37f : r;
 }
 
 // The first near tie of a step: a comparison whose two values differ by no more than the sum of
-// their tie radii.  A value's radius is `band` times its bound for a mixed-form value (bound
-// s > 0), `band_d` times it for a value re-evaluated by difference (stored as -s), and 0 for a
-// value re-evaluated in float-float.
+// their tie radii.  A mixed-form value carries the radius band x bound (certify), a value
+// re-evaluated by difference certify_ref x bound, stored negated, and one re-evaluated in
+// float-float 0.  (No value carries one when decisions are not certified.)
 struct TieLog {
-  double band;     // 0: decisions are not certified
-  double band_d;
   int a, b;        // ids of the first near-tied values (-1: none)
-  __device__ __forceinline__ double radius(double s) const {
-    return s > 0.0 ? band * s : band_d * (-s);
-  }
-  __device__ __forceinline__ void note(int ia, double sa, int ib, double sb, double gap) {
-    if (band > 0.0 && a < 0) {
-      const double r = radius(sa) + radius(sb);
-      if (r > 0.0 && fabs(gap) <= r) {
-        a = sa != 0.0 ? ia : -1;
-        b = sb != 0.0 ? ib : -1;
+  // values ia, ib with signed radii ra, rb
+  __device__ __forceinline__ void note(int ia, float ra, int ib, float rb, double gap) {
+    if (a < 0 && (ra != 0.f || rb != 0.f)) {
+      const float r = fabsf(ra) + fabsf(rb);
+      if (less_eq(fabs(gap), f64_of(r))) {
+        a = ra != 0.f ? ia : -1;
+        b = rb != 0.f ? ib : -1;
         if (a < 0) { a = b; b = -1; }
       }
     }
   }
+  __device__ __forceinline__ void note(const Vert& x, double gap) { note(x.id, x.s, -1, 0.f, gap); }
+  __device__ __forceinline__ void note(const Vert& x, const Vert& y, double gap) {
+    note(x.id, x.s, y.id, y.s, gap);
+  }
   __device__ __forceinline__ bool lt(const Vert& x, const Vert& y) {
-    note(x.id, x.s, y.id, y.s, x.phi - y.phi);
-    return x.phi < y.phi;
+    note(x, y, x.phi - y.phi);
+    return less(x.phi, y.phi);
   }
   __device__ __forceinline__ bool le(const Vert& x, const Vert& y) {
-    note(x.id, x.s, y.id, y.s, x.phi - y.phi);
-    return x.phi <= y.phi;
+    note(x, y, x.phi - y.phi);
+    return less_eq(x.phi, y.phi);
   }
 };
 
@@ -336,11 +394,14 @@ __device__ __forceinline__ void read_eval(const SolveArgs& a, const PlanHdr& h, 
                                           const double lam[3]) {
   const ProbDesc& pd = a.probs[pidx];
   double S[12], G[9];
-  gather_sums<12>(a.out, h, a.item_off, pidx, slot - queue_base(a, pd), S);
+  // (of a pass of few queries the last record is the near field's: zero above near_z)
+  const int skip = a.one_queue && a.o.near_on && !less_eq(z, pd.near_z) ? 1 : 0;
+  gather_sums<12>(a.out, h, a.item_off, pidx, slot - queue_base(a, pd), S, skip);
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
-  e.s = (a.o.tie > 0.0 && a.msc)
-            ? mixed_phi_bound(a.msc + 15 * g, lam, a.o.dim, z, e.B, G, e.g, pd.g_scale, a.o.w_g)
-            : 0.0;
+  e.s = 0.f;
+  if (a.o.tie > 0.0 && a.msc)
+    e.s = radius_of(a.o.tie, mixed_phi_bound(a.msc + 15 * g, lam, a.o.dim, (float)z, e, pd.g_scale,
+                                             a.o.w_g));
 }
 
 // Objective of a re-evaluated value of point g at lambda lt and its 12 sums: float-float sums
@@ -360,13 +421,18 @@ __device__ __forceinline__ void read_reeval(const SolveArgs& a, bool dif, int pi
     for (int s = 0; s < 12; ++s) S[s] = SD(a, D_REFS + s, g) + S[s];
   }
   assemble_obj(S, z, pd.g_scale, a.o.w_g, e, G, corr_of(a, pd, g, z));
-  e.s = 0.0;
+  e.s = 0.f;
   if (dif) {
-    const double l0[3] = {SD(a, D_REFL, g), SD(a, D_REFL + 1, g), SD(a, D_REFL + 2, g)};
-    double eb[12];
-    dif_sum_bounds(a.msc + 15 * g, a.msc0 + 3 * g, lt, l0, a.o.dim, eb);
-    const double sd = dif_phi_bound(eb, z, e.B, G, e.g, pd.g_scale, a.o.w_g);
-    e.s = -(sd > 0.0 ? sd : 1e-300);
+    float dl[3], L[3], R[3], eb[12];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double l0 = SD(a, D_REFL + d, g);
+      dl[d] = fabsf(f32_of(lt[d] - l0));
+      R[d] = fabsf(f32_of(l0));
+      L[d] = fabsf(f32_of(lt[d])) + R[d];
+    }
+    dif_sum_bounds<float>(a.msc + 15 * g, a.msc0 + 3 * g, dl, L, R, a.o.dim, eb);
+    e.s = -radius_of(a.o.tie_dif, dif_phi_bound(eb, (float)z, e, pd.g_scale, a.o.w_g));
   }
 }
 
@@ -526,13 +592,28 @@ __device__ __forceinline__ void sort_verts(Vert* v, TieLog& tl) {
   }
 }
 
-// Points of one warp of a step kernel (CTAs of one warp).  The steps are FP64: an SM's FP64 pipe
-// takes 16 cycles per warp instruction, so a few points are spread over all SMs, one warp each,
-// with as few lanes (fewer of them in different stages) as that needs; full warps come when there
-// are more than 32 points per SM.
+// Points of one warp of a step kernel.  A warp's time is its chain of dependent FP64 instructions
+// (70 to 150 cycles each), not the FP64 rate, so a few points are spread over all SMs and their
+// sub-partitions, one warp each, with as few lanes (fewer of them in different stages) as that
+// needs; full warps come when there are more than 128 points per SM.  (2,048 points in warps of
+// 14, 7, 4 and 2: 8.6, 8.2, 8.0 and 8.2 ms per search.)
+constexpr int STEP_NT = 128;
 __device__ __forceinline__ int points_per_warp(int n, int nsm) {
-  const int p = (n + nsm - 1) / nsm;
+  const int p = (n + 4 * nsm - 1) / (4 * nsm);
   return p < 1 ? 1 : (p > 32 ? 32 : p);
+}
+
+// x / n, correctly rounded.  x / 3 in two operations: with zh + zl = 1/3 to 107 bits, x zh + x zl
+// is x / 3 to about 2^-105, and x / 3 is never nearer than 1/6 ulp to the middle between two
+// doubles (a third of an integer is no nearer than 1/6 to a half-integer), so rounding the one sum
+// in fma rounds x / 3.  (Away from underflow of x zl.)
+template <int n>
+__device__ __forceinline__ double over(double x) {
+  static_assert(n == 1 || n == 3, "simplex of one or three lambdas");
+  if (n == 1) return x;
+  const double zh = 0x1.5555555555555p-2, zl = 0x1.5555555555555p-56;
+  if (!less(fabs(x), 1e-250)) return __fma_rn(x, zh, __dmul_rn(x, zl));
+  return x / 3.0;
 }
 
 // One simplex step per waiting point.  REF = false: the points whose queries the mixed pass of
@@ -543,8 +624,9 @@ __device__ __forceinline__ int points_per_warp(int n, int nsm) {
 // stays as it is, so every decision is the one that sums accurate to the float-float level would
 // take.  With a.o.tie == 0 every step is taken as evaluated.
 //
-// What bounds it: the latency of one warp's instructions (about 11 cycles each; the FP64 pipe is
-// less than a quarter busy), so the time is the instruction count of the longest warp.  Hence two
+// What bounds it: one warp's chain of instructions, its FP64 instructions above all (70 to 150
+// cycles each), so the time is the instruction count of the longest warp.  Hence FP64 only where the
+// values and lambdas are formed (comparisons on the integer pipe, bounds in FP32), and two
 // phases.  First the lanes share out the values to compute, one FP64 objective and bound per lane
 // whatever the points' stages (a shrink has 3, the start 4; taken in turn by the point's own lane
 // they set the length for the whole warp).  Then each lane decides its point's step on Phi and
@@ -552,7 +634,7 @@ __device__ __forceinline__ int points_per_warp(int n, int nsm) {
 // points a step took 63 us (the waiting points' 112 us) with one lane per point evaluating and
 // sorting whole vertices, in CTAs of 128 threads.
 template <int N, bool REF>
-__global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
+__global__ void __launch_bounds__(STEP_NT) nm_step_kernel(const SolveArgs a) {
   const double rho = 1.0, chi = 2.0, psi = 0.5, sigma = 0.5;
   const unsigned FULL = 0xffffffffu;
   const int nact = REF ? *a.cur.ref_cnt : *a.cur.act_cnt;
@@ -561,8 +643,10 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
   const PlanHdr h = *a.plan;
   if (!REF && a.rework && blockIdx.x == 0 && threadIdx.x == 0) a.rework[0] = a.rework[1] = 0;
   const int ppw = points_per_warp(nact, a.nsm);
-  const int lane = threadIdx.x;
-  for (int base = blockIdx.x * ppw; base < nact; base += gridDim.x * ppw) {
+  const int lane = threadIdx.x & 31;
+  const int warp = blockIdx.x * (STEP_NT / 32) + (threadIdx.x >> 5);
+  const int nwarps = gridDim.x * (STEP_NT / 32);
+  for (int base = warp * ppw; base < nact; base += nwarps * ppw) {
     const bool on = lane < ppw && base + lane < nact;
     const int gi = on ? list[base + lane] : 0;
     const int64_t g = gi;
@@ -643,21 +727,18 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
     int iters = SI(a, I_ITERS, g);
     int nfev = SI(a, I_NFEV, g) + (REF ? 0 : nev);
     const bool single = stage != ST_INIT && stage != ST_SHRINK;
-    Vert w[N + 1], e{0.0, 0.0, 0, VID_E}, R{0.0, 0.0, 0, VID_R};
+    TieLog tl{-1, -1};
+    auto vert = [&](int id, int slot) {
+      return Vert{SV(a, id, V_PHI, g), f32_of(SV(a, id, V_S, g)), slot, id};
+    };
+    Vert w[N + 1], e{}, R{};
 #pragma unroll
     for (int k = 0; k <= n; ++k) {
       const int sl = (order >> (4 * k)) & 15;
-      w[k] = Vert{SV(a, sl, V_PHI, g), SV(a, sl, V_S, g), sl, sl};
+      w[k] = vert(sl, sl);
     }
-    if (single) {
-      e.phi = SV(a, VID_E, V_PHI, g);
-      e.s = SV(a, VID_E, V_S, g);
-    }
-    if (stage == ST_EXPAND || stage == ST_OCONTRACT) {
-      R.phi = SV(a, VID_R, V_PHI, g);
-      R.s = SV(a, VID_R, V_S, g);
-    }
-    TieLog tl{a.o.tie, a.o.tie_dif, -1, -1};
+    if (single) e = vert(VID_E, 0);
+    if (stage == ST_EXPAND || stage == ST_OCONTRACT) R = vert(VID_R, 0);
     bool to_check = false, store_R = false, emit_shrink = false, emit_trial = false;
     bool mirror = false;
     int next_stage = stage;
@@ -714,13 +795,15 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
       sort_verts<N>(w, tl);
       // Eq. 12 at the best vertex, then the value spread, then the iteration count
       const double f0 = SV(a, w[0].id, V_F, g), g0 = SV(a, w[0].id, V_G, g);
-      tl.note(w[0].id, w[0].s, -1, 0.0, f0 - a.o.eps_f);
-      if (f0 <= a.o.eps_f) tl.note(w[0].id, w[0].s, -1, 0.0, g0 - a.o.eps_g);
-      if (f0 <= a.o.eps_f && g0 <= a.o.eps_g) {
+      const bool f_met = less_eq(f0, a.o.eps_f), g_met = less_eq(g0, a.o.eps_g);
+      tl.note(w[0], f0 - a.o.eps_f);
+      if (f_met) tl.note(w[0], g0 - a.o.eps_g);
+      if (f_met && g_met) {
         fin = PT_CONVERGED;
       } else {
-        tl.note(w[n].id, w[n].s, w[0].id, w[0].s, w[n].phi - w[0].phi - a.o.tol);
-        if (w[n].phi - w[0].phi <= a.o.tol) fin = PT_CONVERGED;
+        const double spread = w[n].phi - w[0].phi;
+        tl.note(w[n], w[0], spread - a.o.tol);
+        if (less_eq(spread, a.o.tol)) fin = PT_CONVERGED;
         else if (iters >= a.o.max_iter) fin = PT_MAXITER;
       }
       if (fin < 0) {
@@ -763,22 +846,23 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
       bool dif[2] = {false, false};
       double lref[3] = {0.0, 0.0, 0.0};
       if (a.o.tie_dif > 0.0) {
-        const double sv[2] = {SV(a, ida, V_S, g), idb < 0 ? 0.0 : SV(a, idb, V_S, g)};
+        const float sv[2] = {f32_of(SV(a, ida, V_S, g)), idb < 0 ? 0.f : f32_of(SV(a, idb, V_S, g))};
         if (!isnan(SD(a, D_REFS, g))) {
 #pragma unroll
           for (int d = 0; d < 3; ++d) lref[d] = SD(a, D_REFL + d, g);
-          bool near[2] = {sv[0] > 0.0, k > 1 && sv[1] > 0.0};
+          bool near[2] = {sv[0] > 0.f, k > 1 && sv[1] > 0.f};
 #pragma unroll
           for (int p = 0; p < 3; ++p) {
             const int q = n == 1 ? 0 : p;
-            const double m1 = a.msc[15 * g + 5 * p];
-            const double reach = m1 > 0.0 ? a.msc0[3 * g + p] / m1 : 0.0;
+            const float m1 = a.msc[15 * g + 5 * p];
+            const float reach = m1 > 0.f ? a.msc0[3 * g + p] / m1 : 0.f;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) near[j] = near[j] && fabs(lt[j][q] - lref[q]) * reach < 0.25;
+            for (int j = 0; j < 2; ++j)
+              near[j] = near[j] && fabsf(f32_of(lt[j][q] - lref[q])) * reach < 0.25f;
           }
           dif[0] = near[0];
           dif[1] = near[1];
-        } else if (k == 2 && sv[0] > 0.0 && sv[1] > 0.0) {
+        } else if (k == 2 && sv[0] > 0.f && sv[1] > 0.f) {
           k = 1;
           if (sv[1] > sv[0]) {
             id0 = idb;
@@ -834,7 +918,8 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
           if (d < n) {
 #pragma unroll
             for (int k = 0; k < n; ++k) s += SV(a, w[k].slot, V_L + d, g);
-            rows[0][d] = coef_c * (s / n) + coef_w * SV(a, w[n].slot, V_L + d, g);
+            // (coef_w is a power of two: its product is exact, the fma rounds as the sum does)
+            rows[0][d] = __fma_rn(coef_w, SV(a, w[n].slot, V_L + d, g), coef_c * over<n>(s));
           } else {
             rows[0][d] = 0.0;
           }
@@ -862,12 +947,12 @@ __global__ void __launch_bounds__(32) nm_step_kernel(const SolveArgs a) {
 }
 
 void launch_nm_step(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) nm_step_kernel<1, false><<<grid, 32, 0, s>>>(a);
-  else nm_step_kernel<3, false><<<grid, 32, 0, s>>>(a);
+  if (a.o.dim == 1) nm_step_kernel<1, false><<<grid, STEP_NT, 0, s>>>(a);
+  else nm_step_kernel<3, false><<<grid, STEP_NT, 0, s>>>(a);
 }
 void launch_nm_refine(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) nm_step_kernel<1, true><<<grid, 32, 0, s>>>(a);
-  else nm_step_kernel<3, true><<<grid, 32, 0, s>>>(a);
+  if (a.o.dim == 1) nm_step_kernel<1, true><<<grid, STEP_NT, 0, s>>>(a);
+  else nm_step_kernel<3, true><<<grid, STEP_NT, 0, s>>>(a);
 }
 
 // --------------------------------------------------------------- per-round plan ----
@@ -932,57 +1017,86 @@ __global__ void plan_round_kernel(const PlanArgs a) {
 void launch_plan_round(const PlanArgs& a, cudaStream_t s) { plan_round_kernel<<<1, 256, 0, s>>>(a); }
 
 // The lambda-independent absolute-value sums of every point, the coefficients of the mixed
-// form's error bound: msc[15 g + 5 p + j - 1] = sum_k |b_pk| / r_gk^j, j = 1..5, over the
-// quadrature points of the point's problem.  FP32 terms summed per tile, tiles summed in FP64
-// (relative error below 1e-4: a scale, not a result).
-__global__ void msc_kernel(const ProbDesc* __restrict__ probs, int64_t N,
-                           const float4* __restrict__ ppos, double* __restrict__ msc,
-                           double* __restrict__ msc0) {
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N;
-       g += (int64_t)gridDim.x * blockDim.x) {
+// form's error bound: msc[15 g + 5 p + j - 1] = sum_k |b_pk| / r_gk^j, j = 1..5, and msc0[3 g + p] =
+// sum_k |b_pk|, over the quadrature points of the point's problem.  FP32 terms summed per 256
+// pixels of a thread, those in float pairs (relative error below 1e-4: a scale, not a result).
+// FP32 issue bounds it (about 30 instructions per pair); a point per CTA, its lanes taking four
+// pixels each, keeps a search of few points from walking the boundary pixel by pixel (2,048 points
+// over 32 x 32 pixels: 100 us with a thread per point).
+constexpr int MSC_NT = 128;
+template <typename T>
+__global__ void __launch_bounds__(MSC_NT) msc_kernel(const ProbDesc* __restrict__ probs, int64_t N,
+                                                     const float4* __restrict__ ppos,
+                                                     T* __restrict__ msc, T* __restrict__ msc0) {
+  constexpr int NSUM = 18;
+  __shared__ double s_red[MSC_NT / 32][NSUM];
+  const int lane = threadIdx.x & 31;
+  for (int64_t g = blockIdx.x; g < N; g += gridDim.x) {
     const float4 pos = ppos[g];
     const ProbDesc& pd = probs[__float_as_int(pos.w)];
     const float z2 = __fmul_rn(pos.z, pos.z);
-    double tot[15], tot0[3] = {0.0, 0.0, 0.0};
+    const int groups = pd.ntiles * (TILE / 4);
+    ff::ds tot[NSUM];
 #pragma unroll
-    for (int i = 0; i < 15; ++i) tot[i] = 0.0;
-    for (int t = 0; t < pd.ntiles; ++t) {
-      const float* T = pd.tiles32 + (int64_t)t * pd.nf32 * TILE;
-      float acc[15], acc0[3] = {0.f, 0.f, 0.f};
+    for (int i = 0; i < NSUM; ++i) tot[i] = ff::ds{0.f, 0.f};
+    for (int q0 = threadIdx.x; q0 < groups; q0 += 64 * MSC_NT) {
+      float acc[NSUM];
 #pragma unroll
-      for (int i = 0; i < 15; ++i) acc[i] = 0.f;
-#pragma unroll 2
-      for (int e = 0; e < TILE; ++e) {
-        const float dx = pos.x - __ldg(T + e), dy = pos.y - __ldg(T + TILE + e);
-        const float ri = rsqrtf(dx * dx + dy * dy + z2);
-        const float b[3] = {fabsf(__ldg(T + 2 * TILE + e)), fabsf(__ldg(T + 3 * TILE + e)),
-                            fabsf(__ldg(T + 4 * TILE + e))};
+      for (int i = 0; i < NSUM; ++i) acc[i] = 0.f;
+      const int q1 = q0 + 64 * MSC_NT < groups ? q0 + 64 * MSC_NT : groups;
+      for (int q = q0; q < q1; q += MSC_NT) {
+        const float* T32 = pd.tiles32 + (int64_t)(q / (TILE / 4)) * pd.nf32 * TILE +
+                           (q % (TILE / 4)) * 4;
+        auto ld = [&](int f) { return __ldg(reinterpret_cast<const float4*>(T32 + f * TILE)); };
+        const float4 X = ld(0), Y = ld(1), B[3] = {ld(2), ld(3), ld(4)};
+        const float x[4] = {X.x, X.y, X.z, X.w}, y[4] = {Y.x, Y.y, Y.z, Y.w};
+        const float b[3][4] = {{B[0].x, B[0].y, B[0].z, B[0].w},
+                               {B[1].x, B[1].y, B[1].z, B[1].w},
+                               {B[2].x, B[2].y, B[2].z, B[2].w}};
 #pragma unroll
-        for (int p = 0; p < 3; ++p) acc0[p] += b[p];
-        float wj = ri;
+        for (int e = 0; e < 4; ++e) {
+          const float dx = pos.x - x[e], dy = pos.y - y[e];
+          const float ri = rsqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, z2)));
+          float wj = 1.f;
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+          for (int j = 0; j < 6; ++j) {   // acc[3 j + p]: M_j of component p
 #pragma unroll
-          for (int p = 0; p < 3; ++p) acc[5 * p + j] += b[p] * wj;
-          wj *= ri;
+            for (int p = 0; p < 3; ++p) acc[3 * j + p] = __fmaf_rn(fabsf(b[p][e]), wj, acc[3 * j + p]);
+            wj *= ri;
+          }
         }
       }
 #pragma unroll
-      for (int i = 0; i < 15; ++i) tot[i] += (double)acc[i];
-#pragma unroll
-      for (int p = 0; p < 3; ++p) tot0[p] += (double)acc0[p];
+      for (int i = 0; i < NSUM; ++i) ff::acc_add(tot[i], ff::ds{acc[i], 0.f});
     }
+    const ff::ds r = WarpSums<NSUM>::reduce(tot, lane);
+    __syncthreads();   // the previous point's sums are read
+    if (lane < NSUM) s_red[threadIdx.x >> 5][lane] = ff::to_double(r);
+    __syncthreads();
+    if (threadIdx.x < NSUM) {
+      double t = s_red[0][threadIdx.x];
 #pragma unroll
-    for (int i = 0; i < 15; ++i) msc[15 * g + i] = tot[i];
-    if (msc0)
-#pragma unroll
-      for (int p = 0; p < 3; ++p) msc0[3 * g + p] = tot0[p];
+      for (int w = 1; w < MSC_NT / 32; ++w) t += s_red[w][threadIdx.x];
+      const int j = threadIdx.x / 3, p = threadIdx.x % 3;
+      if (j > 0) msc[15 * g + 5 * p + j - 1] = (T)t;
+      else msc0[3 * g + p] = (T)t;
+    }
   }
 }
 
+template <typename T>
+static void launch_msc_t(const ProbDesc* probs, int64_t N, const float4* ppos, T* msc, T* msc0,
+                         int sm_count, cudaStream_t s) {
+  const int64_t most = 16LL * sm_count;
+  if (N > 0) msc_kernel<T><<<(int)(N < most ? N : most), MSC_NT, 0, s>>>(probs, N, ppos, msc, msc0);
+}
+void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, float* msc, float* msc0,
+                int sm_count, cudaStream_t s) {
+  launch_msc_t(probs, N, ppos, msc, msc0, sm_count, s);
+}
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
-                int grid, cudaStream_t s) {
-  if (N > 0) msc_kernel<<<grid, 128, 0, s>>>(probs, N, ppos, msc, msc0);
+                int sm_count, cudaStream_t s) {
+  launch_msc_t(probs, N, ppos, msc, msc0, sm_count, s);
 }
 
 // Difference sums of n queries of one problem (slots 0..n-1) and their bounds (debug entry).
@@ -998,8 +1112,13 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
     if (dS_bound) {
       const double la[3] = {qlam[i].x, qlam[i].y, qlam[i].z};
       const double l0[3] = {qlam0[i].x, qlam0[i].y, qlam0[i].z};
-      double e[12];
-      dif_sum_bounds(msc + 15 * i, msc0 + 3 * i, la, l0, dim, e);
+      double dl[3], L[3], R[3], e[12];
+      for (int d = 0; d < 3; ++d) {
+        dl[d] = fabs(la[d] - l0[d]);
+        R[d] = fabs(l0[d]);
+        L[d] = fabs(la[d]) + R[d];
+      }
+      dif_sum_bounds<double>(msc + 15 * i, msc0 + 3 * i, dl, L, R, dim, e);
       for (int s = 0; s < 12; ++s) dS_bound[12 * i + s] = e[s];
     }
   }
@@ -1017,13 +1136,13 @@ void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const L
 // ------------------------------------------------------------------ certified B ----
 // Worst-case error of the mixed form's B at lambda (the B part of mixed_phi_bound): per
 // component z (A0 M3 + A1 |lambda| M2 + A2 lambda^2 M1); returns the Euclidean norm.
-__device__ __forceinline__ double mixed_b_bound(const double* M, const double lam[3], int dim,
+__device__ __forceinline__ double mixed_b_bound(const float* M, const double lam[3], int dim,
                                                 double z) {
   double s = 0.0;
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
     const double L = fabs(dim == 1 ? lam[0] : lam[p]);
-    const double* m = M + 5 * p;
+    const float* m = M + 5 * p;
     const double d = z * (BND_A0 * m[2] + BND_A1 * L * m[1] + BND_A2 * L * L * m[0]);
     s += d * d;
   }
@@ -1168,9 +1287,9 @@ void launch_finalize_objective(int64_t n, const PlanHdr* plan, const int32_t* it
                                double g_scale, double w_g, double* fgphi, double* dphi, double* B,
                                const double* corr, cudaStream_t s) {
   if (n <= 0) return;
-  const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  finalize_objective_kernel<<<grid, 256, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale,
-                                                 w_g, fgphi, dphi, B, corr);
+  const PerPoint L(n);
+  finalize_objective_kernel<<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale,
+                                                    w_g, fgphi, dphi, B, corr);
 }
 
 // ----------------------------------------------------------------------- quasi-Newton ----
@@ -1210,8 +1329,11 @@ __global__ void bfgs_step_kernel(const SolveArgs a) {
   constexpr int n = N;
   const PlanHdr h = *a.plan;
   const int ppw = points_per_warp(nact, a.nsm);
-  if ((int)threadIdx.x >= ppw) return;
-  for (int ia = blockIdx.x * ppw + threadIdx.x; ia < nact; ia += gridDim.x * ppw) {
+  const int lane = threadIdx.x & 31;
+  if (lane >= ppw) return;
+  const int warp = blockIdx.x * (STEP_NT / 32) + (threadIdx.x >> 5);
+  const int nwarps = gridDim.x * (STEP_NT / 32);
+  for (int ia = warp * ppw + lane; ia < nact; ia += nwarps * ppw) {
     const int64_t g = a.cur.act[ia];
     const float4 pos = a.ppos[g];
     const int pidx = __float_as_int(pos.w);
@@ -1362,8 +1484,8 @@ __global__ void bfgs_step_kernel(const SolveArgs a) {
 }
 
 void launch_bfgs_step(const SolveArgs& a, int grid, cudaStream_t s) {
-  if (a.o.dim == 1) bfgs_step_kernel<1><<<grid, 32, 0, s>>>(a);
-  else bfgs_step_kernel<3><<<grid, 32, 0, s>>>(a);
+  if (a.o.dim == 1) bfgs_step_kernel<1><<<grid, STEP_NT, 0, s>>>(a);
+  else bfgs_step_kernel<3><<<grid, STEP_NT, 0, s>>>(a);
 }
 
 }  // namespace dbie

@@ -12,7 +12,8 @@ enum RField {
   V_L = 0,      // lambda (3)
   V_B = 3,      // field B (3)
   V_F = 6, V_G = 7, V_PHI = 8,
-  V_S = 9       // certified decisions: the value's error bound (0 once re-evaluated in float-float)
+  V_S = 9       // certified decisions: the value's tie radius (negated for a value re-evaluated by
+                // difference, 0 for one re-evaluated in float-float)
 };
 constexpr int VID_R = 4, VID_E = 5;
 enum DField {
@@ -95,8 +96,8 @@ struct SolveArgs {
   unsigned* err;
   const double* corr;        // [N * 12] pixel-exact corrections (dB, d grad B), or null
   // certified decisions
-  const double* msc;         // [N * 15] sum_k |b_pk| / r^j, j = 1..5, per component (or null)
-  const double* msc0;        // [N * 3] sum_k |b_pk| per component (difference level)
+  const float* msc;          // [N * 15] sum_k |b_pk| / r^j, j = 1..5, per component (or null)
+  const float* msc0;         // [N * 3] sum_k |b_pk| per component (difference level)
   const double* fout;        // float-float sums of the current round, [slot][split][12]
   const PlanHdr* fplan;
   const double* dout;        // difference sums of the current round
