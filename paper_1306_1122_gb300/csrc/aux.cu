@@ -1,6 +1,7 @@
 // aux.cu -- staging, packing, near-field correction and adjoint finalisation kernels.
 #include "ff_math.cuh"
 #include "kernels.h"
+#include "nearfield.cuh"
 
 namespace dbie {
 
@@ -185,49 +186,14 @@ void launch_plan_single(PlanHdr* plan, int32_t* item_off, int32_t* q_cnt, int32_
   plan_single_kernel<<<1, 1, 0, s>>>(plan, item_off, q_cnt, work, nitems, nsplit, qper, qcount);
 }
 
-// Near-field correction (mixed precision, points with z <= near_z): over the (2W+1)^2 pixels
-// around the point, replace the FP32 pair terms that the pair-sum kernel added by FP64 ones.
-// The FP32 terms are recomputed with the same explicitly rounded code (pair_terms32), so the
-// correction sum_k (t64 - t32) removes exactly what was added.  The correction is added in place
-// to the query's split-0 partial sums (a dense pass: run after the pair sums) or is the query's
-// last record (a pass of few queries: in any order with it).
-// Index (along one axis) of the quadrature point nearest to coordinate x: the pixel for the
-// midpoint rule; for nine-node elements of width 2h with g Gauss points, element e and the
-// nearest abscissa a give e * g + a.
-__device__ __forceinline__ long near_index(double x, double x0, double h, int nq,
-                                           const ProbDesc& pd) {
-  if (pd.quad_g == 0) return lrint((x - x0) / h);
-  const int g = pd.quad_g;
-  const long ne = nq / g;
-  long e = (long)floor((x - x0) / (2.0 * h));
-  e = e < 0 ? 0 : (e > ne - 1 ? ne - 1 : e);
-  const double xi = (x - x0) / h - (double)(2 * e + 1);
-  int best = 0;
-  double bd = fabs(xi - pd.gx[0]);
-  for (int a = 1; a < g; ++a) {
-    const double d = fabs(xi - pd.gx[a]);
-    if (d < bd) { bd = d; best = a; }
-  }
-  return e * g + best;
-}
-
 constexpr int NEAR_NT = 128;   // four independent warps
 
 // GL lanes per query (a divisor of 32).
 template <int VAR, bool TIED, int GL>
 __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const PlanHdr& h,
                                              const float4* s_tab) {
-  constexpr int NS = nsum_per_comp(VAR);
-  constexpr int NSUM = 3 * NS;
-  // sin and cos of lambda r in float-float on the FP32 pipe (absolute error ~1e-13 + 5e-15 |lambda
-  // r|, far below the FP32 terms' error that the correction removes) instead of FP64 sincos,
-  // which cost most of this kernel's FP64-pipe time
-  auto sincos_ff = [&](double th, double& s, double& c) {
-    ff::ds S, C;
-    ff::sincos_ds_any(ff::from_double(th), s_tab, S, C);
-    s = ff::to_double(S);
-    c = ff::to_double(C);
-  };
+  constexpr int NSUM = 3 * nsum_per_comp(VAR);
+  using Lanes = NearLanes<NSUM, GL>;
   const int lane = threadIdx.x & 31, sub = lane & (GL - 1), grp = lane / GL;
   const int64_t warp = blockIdx.x * (int64_t)(NEAR_NT / 32) + (threadIdx.x >> 5);
   const int64_t nwarps = (int64_t)gridDim.x * (NEAR_NT / 32);
@@ -238,100 +204,15 @@ __device__ __forceinline__ void near_queries(const NearArgs& a, int cnt, const P
     const int64_t wq = listed ? w : wb;
     const int64_t slot = a.list ? a.list[wq] : wq;
     const float4 pos = a.qpos[slot];
-    const Lam4 lam = a.qlam[slot];
     const int pidx = __float_as_int(pos.w);
     const ProbDesc& pd = a.probs[pidx];
-    const Query<float, TIED> q32 = make_query<float, TIED>(pos, lam);
-    const Query<double, TIED> q64 = make_query<double, TIED>(pos, lam);
-    const int W = pd.near_w > 0 ? pd.near_w : NEAR_W;
-    const long ix = near_index((double)pos.x, pd.x0, pd.hx, pd.nx, pd);
-    const long iy = near_index((double)pos.y, pd.y0, pd.hy, pd.ny, pd);
-    const long i0 = ix - W < 0 ? 0 : ix - W;
-    const long i1 = ix + W > pd.nx - 1 ? pd.nx - 1 : ix + W;
-    const long j0 = iy - W < 0 ? 0 : iy - W;
-    const long j1 = iy + W > pd.ny - 1 ? pd.ny - 1 : iy + W;
-    const long wi = i1 - i0 + 1, wj = j1 - j0 + 1;
-    double c[NSUM];
-#pragma unroll
-    for (int s = 0; s < NSUM; ++s) c[s] = 0.0;
     const bool valid = listed && (a.list || (double)pos.z <= a.near_z);
-    if (valid && wi > 0 && wj > 0 && wi <= 2 * W + 1 && wj <= 2 * W + 1) {
-      const int nwin = (int)(wi * wj), wx = (int)wi;
-      for (int e = sub; e < nwin; e += GL) {
-        const int64_t k = (j0 + e / wx) * (int64_t)pd.nx + (i0 + e % wx);
-        const int nf = pd.nf32 > 0 ? pd.nf32 : NFIELD;
-        const float b32[3] = {*tile_field(pd.tiles32, k, 2, nf), *tile_field(pd.tiles32, k, 3, nf),
-                              *tile_field(pd.tiles32, k, 4, nf)};
-        const double b64[3] = {*tile_field(pd.tiles64, k, 2), *tile_field(pd.tiles64, k, 3),
-                               *tile_field(pd.tiles64, k, 4)};
-        Terms32<VAR, TIED> t32;
-        Terms64<VAR, TIED> t64;
-        if (nf == NFIELD_SPLIT)
-          pair_terms32_split<VAR, TIED>(q32, *tile_field(pd.tiles32, k, 0, nf),
-                                        *tile_field(pd.tiles32, k, 1, nf),
-                                        *tile_field(pd.tiles32, k, 5, nf),
-                                        *tile_field(pd.tiles32, k, 6, nf), b32, t32);
-        else
-          pair_terms32<VAR, TIED>(q32, *tile_field(pd.tiles32, k, 0), *tile_field(pd.tiles32, k, 1),
-                                  b32, t32);
-        pair_terms64_sc<VAR, TIED>(q64, *tile_field(pd.tiles64, k, 0),
-                                   *tile_field(pd.tiles64, k, 1), b64, t64, sincos_ff);
+    double v[Lanes::NP];
+    near_window<VAR, TIED, GL>(pd, pos, a.qlam[slot], valid, s_tab, sub, v);
+    if (valid && sub % Lanes::SAME == 0) {
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-          const int lp = TIED ? 0 : p;
-          // FP32 contributions as the scalar FP32 code computes them (products of two FP32
-          // factors, exact in FP64; the packed kernel's can differ by a rounding of a factor),
-          // replaced by the FP64 terms.
-          if constexpr (has_hess(VAR)) c[p * NS] += t64.t0[p] - (double)t32.t0[p];
-          else c[p * NS] += t64.t0[p] - (double)t32.u[lp] * (double)t32.rb[p];
-          if constexpr (has_grad(VAR)) {
-            c[p * NS + 1] += t64.t1[p] - (double)t32.t1[p];
-            c[p * NS + 2] += t64.t1[p] * t64.dx - (double)t32.t1[p] * (double)t32.dx;
-            c[p * NS + 3] += t64.t1[p] * t64.dy - (double)t32.t1[p] * (double)t32.dy;
-          }
-          if constexpr (has_hess(VAR))
-            c[p * NS + idx_sl(VAR)] += t64.tl[p] - (double)t32.tl[p];
-          else if constexpr (has_dlam(VAR))
-            c[p * NS + idx_sl(VAR)] += t64.tl[p] - (double)t32.cr[lp] * (double)b32[p];
-          if constexpr (has_newton(VAR)) {
-            c[p * NS + IDX_TX] += t64.t0[p] * t64.dx - (double)t32.t0[p] * (double)t32.dx;
-            c[p * NS + IDX_TY] += t64.t0[p] * t64.dy - (double)t32.t0[p] * (double)t32.dy;
-          }
-          if constexpr (has_hess(VAR)) {
-            c[p * NS + IDX_Q] += t64.tq[p] - (double)t32.sn[lp] * (double)b32[p];
-            c[p * NS + IDX_UX] += t64.tl[p] * t64.dx - (double)t32.tl[p] * (double)t32.dx;
-            c[p * NS + IDX_UY] += t64.tl[p] * t64.dy - (double)t32.tl[p] * (double)t32.dy;
-          }
-        }
-      }
-    }
-    // the lanes' sums, by halving: each step hands half of the sums to the partner lane (16 FP64
-    // additions for 12 sums over 32 lanes instead of 60)
-    constexpr int NP = NSUM > 16 ? 32 : NSUM > 8 ? 16 : NSUM > 4 ? 8 : 4;
-    constexpr int LEFT = NP / GL > 0 ? NP / GL : 1;   // sums per lane at the end
-    double v[NP];
-#pragma unroll
-    for (int s = 0; s < NP; ++s) v[s] = s < NSUM ? c[s < NSUM ? s : 0] : 0.0;
-    int half = NP / 2;
-#pragma unroll
-    for (int off = GL / 2; off > 0; off >>= 1, half >>= 1) {
-      if (half >= 1) {
-        const bool up = (sub & off) != 0;
-#pragma unroll
-        for (int s = 0; s < half; ++s) {
-          const double give = up ? v[s] : v[s + half];
-          const double keep = up ? v[s + half] : v[s];
-          v[s] = keep + __shfl_xor_sync(0xffffffffu, give, off);
-        }
-      } else {
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
-      }
-    }
-    constexpr int SAME = NP < GL ? GL / NP : 1;       // lanes that hold the same sums
-    if (valid && sub % SAME == 0) {
-#pragma unroll
-      for (int i = 0; i < LEFT; ++i) {
-        const int s = sub / SAME * LEFT + i;
+      for (int i = 0; i < Lanes::LEFT; ++i) {
+        const int s = sub / Lanes::SAME * Lanes::LEFT + i;
         if (s < NSUM) {
           if (a.warps > 0) a.out[(slot * h.nsplit + h.nsplit - 1) * NSUM + s] = v[i];
           else a.out[out_index(h, a.item_off, pidx, slot - pd.q_off, 0, s, NSUM)] += v[i];

@@ -43,8 +43,7 @@
 // per 153 or more instructions, which plain coalesced loads through L1 sustain; nothing is staged.
 #include <type_traits>
 
-#include "ff_math.cuh"
-#include "kernels.h"
+#include "re_rows.cuh"
 #include "warp_sums.cuh"
 
 namespace dbie {
@@ -52,10 +51,8 @@ namespace dbie {
 using ff::ds;
 
 constexpr int RE_NT = 128;           // threads per CTA = pixels per row of an item
-constexpr int RE_NF = 2 * NFIELD;    // floats per pixel in a float-float tile
 constexpr int RE_MAX_SPLIT = 64;     // row ranges per query: the reader adds them one by one
 constexpr int RE_WAVES = 8;          // items per CTA at most (the tail is then 1/8 of a pass)
-constexpr int DIF_BLK = 8;           // pixels per FP32 block sum of the differences
 static_assert(TILE / RE_NT == RE_ROWS_PER_TILE && TILE % RE_NT == 0, "rows tile the tile");
 
 // Float-float tiles: per field (x, y, bx, by, bz) TILE hi parts, then TILE lo parts.
@@ -118,144 +115,6 @@ __device__ __forceinline__ void reduce_store(const ds (&acc)[NSUM], double* red,
   }
 }
 
-// The query of an item, prepared by the CTA's first threads (FP64 issues at 1/64 of the FP32
-// rate here: once per CTA, not once per thread).
-struct ReQuery {
-  float x, y, z;
-  int pidx;
-  float lh[3], ll[3];      // lambda (hi, lo)
-  float hs[3], hd[3], pq[3], qq[3];   // differences: (la + l0) / 2, (la - l0) / 2, la^2 -+ l0^2
-  int slow;                // lambda r may leave the range of the float-float reduction
-};
-
-__device__ __forceinline__ float re_load(const float* tile, int f, int part, int e) {
-  return __ldg(tile + f * 2 * TILE + part * TILE + e);
-}
-
-// Float-float sums of the CTA's pixel of each row in [r0, r1).
-template <int VAR, bool TIED, bool ANY>
-__device__ __forceinline__ void ff_rows(const float* tiles, int r0, int r1, const ReQuery& q,
-                                        const float4* tab, ds (&acc)[3 * nsum_per_comp(VAR)]) {
-  using D = ds;
-  constexpr int NS = nsum_per_comp(VAR);
-  constexpr int NL = TIED ? 1 : 3;
-  const D xq = D{q.x, 0.f}, yq = D{q.y, 0.f};
-  const D z2 = ff::two_prod(q.z, q.z);
-  D lam[NL], lam2[NL];
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    lam[l] = D{q.lh[l], q.ll[l]};
-    lam2[l] = ff::mul(lam[l], lam[l]);
-  }
-#pragma unroll 1
-  for (int row = r0; row < r1; ++row) {
-    const float* T = tiles + (int64_t)(row / (TILE / RE_NT)) * (RE_NF * TILE);
-    const int e = (row % (TILE / RE_NT)) * RE_NT + threadIdx.x;
-    const D X = D{re_load(T, 0, 0, e), re_load(T, 0, 1, e)};
-    const D Y = D{re_load(T, 1, 0, e), re_load(T, 1, 1, e)};
-    const D dx = ff::sub(xq, X);
-    const D dy = ff::sub(yq, Y);
-    // (products that feed a further float-float operation stay unnormalised: mul_nr)
-    const D r2 = ff::add(ff::add(ff::mul_nr(dx, dx), ff::mul_nr(dy, dy)), z2);
-    D r, ri;
-    ff::sqrt_rsqrt(r2, r, ri);
-    const D ri2 = ff::mul_nr(ri, ri);
-    const D ri3 = ff::mul_nr(ri2, ri);
-    D u[NL], c[NL];
-#pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      const D th = ff::mul_nr(lam[l], r);
-      D s;
-      if constexpr (ANY) ff::sincos_ds_any(th, tab, s, c[l]);
-      else ff::sincos_ds<float>(th, tab, s, c[l]);
-      u[l] = ff::add(ff::mul_nr(th, s), c[l]);
-    }
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-      const int lp = TIED ? 0 : p;
-      const D rb = ff::mul_nr(ri3, D{re_load(T, 2 + p, 0, e), re_load(T, 2 + p, 1, e)});
-      ff::acc_add(acc[p * NS], ff::mul_nr(u[lp], rb));
-      if constexpr (has_grad(VAR)) {
-        // psi b = (lambda^2 cos(lambda r) - 3 u / r^2) b / r^3
-        const D w = ff::sub(ff::mul_nr(lam2[lp], c[lp]),
-                            ff::mul_f_nr(ff::mul_nr(u[lp], ri2), 3.0f));
-        const D t1 = ff::mul_nr(w, rb);
-        ff::acc_add(acc[p * NS + 1], t1);
-        ff::acc_add(acc[p * NS + 2], ff::mul_nr(t1, dx));
-        ff::acc_add(acc[p * NS + 3], ff::mul_nr(t1, dy));
-      }
-    }
-  }
-}
-
-// sin(d), cos(d): Taylor polynomials through d^9 and d^10 for |d| <= 1 (truncation below 3e-8
-// relative), the SFU beyond.
-__device__ __forceinline__ void sincos_delta(float d, float& s, float& c) {
-  if (fabsf(d) <= 1.0f) {
-    const float d2 = d * d;
-    s = d * fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, 1.0f / 362880.0f, -1.0f / 5040.0f),
-                                   1.0f / 120.0f), -1.0f / 6.0f), 1.0f);
-    c = fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, fmaf(d2, -1.0f / 3628800.0f, 1.0f / 40320.0f),
-                                        -1.0f / 720.0f), 1.0f / 24.0f), -0.5f), 1.0f);
-  } else {
-    s = sin_mufu(d);
-    c = cos_mufu(d);
-  }
-}
-
-// Difference sums: FP32 over blocks of DIF_BLK pixels of a thread, the block sums in float-float.
-template <bool TIED>
-__device__ __forceinline__ void dif_rows(const float* tiles, int r0, int r1, const ReQuery& q,
-                                         ds (&acc)[12]) {
-  constexpr int NL = TIED ? 1 : 3;
-  const float z2 = q.z * q.z;
-#pragma unroll 1
-  for (int b0 = r0; b0 < r1; b0 += DIF_BLK) {
-    float bs[12];
-#pragma unroll
-    for (int s = 0; s < 12; ++s) bs[s] = 0.f;
-    const int b1 = b0 + DIF_BLK < r1 ? b0 + DIF_BLK : r1;
-#pragma unroll 2
-    for (int row = b0; row < b1; ++row) {
-      const float* T = tiles + (int64_t)(row / (TILE / RE_NT)) * (RE_NF * TILE);
-      const int e = (row % (TILE / RE_NT)) * RE_NT + threadIdx.x;
-      const float dx = (q.x - re_load(T, 0, 0, e)) - re_load(T, 0, 1, e);
-      const float dy = (q.y - re_load(T, 1, 0, e)) - re_load(T, 1, 1, e);
-      const float r2 = fmaf(dx, dx, fmaf(dy, dy, z2));
-      const float ri = rsqrt_mufu(r2);
-      const float r = r2 * ri;
-      const float ri2 = ri * ri;
-      const float ri3 = ri2 * ri;
-      float du[NL], dw[NL];
-#pragma unroll
-      for (int l = 0; l < NL; ++l) {
-        const float sg = q.hs[l] * r, dl = q.hd[l] * r;
-        const float ss = sin_mufu(sg), cs = cos_mufu(sg);
-        float sd, cd;
-        sincos_delta(dl, sd, cd);
-        const float cs_sd = cs * sd, ss_sd = ss * sd;
-        du[l] = 2.0f * (fmaf(dl, ss * cd, sg * cs_sd) - ss_sd);
-        dw[l] = fmaf(q.pq[l], cs * cd, fmaf(-q.qq[l], ss_sd, -3.0f * du[l] * ri2));
-      }
-#pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        const int lp = TIED ? 0 : p;
-        const float rb = ri3 * re_load(T, 2 + p, 0, e);
-        const float t1 = dw[lp] * rb;
-        bs[4 * p + 0] = fmaf(du[lp], rb, bs[4 * p + 0]);
-        bs[4 * p + 1] += t1;
-        bs[4 * p + 2] = fmaf(t1, dx, bs[4 * p + 2]);
-        bs[4 * p + 3] = fmaf(t1, dy, bs[4 * p + 3]);
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < 12; ++s) {
-      const ds t = ff::two_sum(acc[s].hi, bs[s]);
-      acc[s] = ds{t.hi, __fadd_rn(acc[s].lo, t.lo)};
-    }
-  }
-}
-
 // Float-float sums of a.f and, with DIF, difference sums of a.d (objective sums).
 template <int VAR, bool TIED, bool DIF>
 __global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
@@ -294,36 +153,19 @@ __global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
     if (tid < (TIED ? 1 : 3)) {
       const Lam4 l4 = L.lam[slot];
       const double la = tid == 0 ? l4.x : (tid == 1 ? l4.y : l4.z);
-      const ds h = ff::from_double(la);
-      s_q.lh[tid] = h.hi;
-      s_q.ll[tid] = h.lo;
-      if (DIF && dif) {   // formed in FP64
+      set_lambda(s_q, tid, la);
+      if (DIF && dif) {
         const Lam4 r4 = L.lam0[slot];
-        const double l0 = tid == 0 ? r4.x : (tid == 1 ? r4.y : r4.z);
-        s_q.hs[tid] = (float)(0.5 * (la + l0));
-        s_q.hd[tid] = (float)(0.5 * (la - l0));
-        s_q.pq[tid] = (float)((la - l0) * (la + l0));
-        s_q.qq[tid] = (float)(la * la + l0 * l0);
+        set_difference(s_q, tid, la, tid == 0 ? r4.x : (tid == 1 ? r4.y : r4.z));
       }
     } else if (tid == 32) {
       s_q.x = pos.x;
       s_q.y = pos.y;
       s_q.z = pos.z;
-      // lambda r below the reduction range of sincos_ds for every pixel: |lambda| times the
-      // largest distance to the quadrature grid's box (pixel centres, or Gauss points of elements
-      // two node spacings wide, all inside [x0 - |hx|, x0 + 2 nx |hx|] with nx quadrature points
-      // per row); otherwise (rare: a far-out trial lambda, or not finite) the CTA takes the path
-      // with the FP64 fallback, so the common path stays branch-free
       const Lam4 l4 = L.lam[slot];
-      const float lmax = TIED ? fabsf((float)l4.x)
-                              : fmaxf(fmaxf(fabsf((float)l4.x), fabsf((float)l4.y)),
-                                      fabsf((float)l4.z));
-      const float x0 = (float)pd.x0, y0 = (float)pd.y0;
-      const float ax = (float)fabs(pd.hx), ay = (float)fabs(pd.hy);
-      const float ex = fmaxf(fabsf(pos.x - (x0 - ax)), fabsf(pos.x - (x0 + 2.0f * pd.nx * ax)));
-      const float ey = fmaxf(fabsf(pos.y - (y0 - ay)), fabsf(pos.y - (y0 + 2.0f * pd.ny * ay)));
-      const float rmax = sqrtf(ex * ex + ey * ey + pos.z * pos.z);
-      s_q.slow = !(lmax * rmax < 0.9f * ff::SC_MAX_ARG);
+      const float lx = fabsf((float)l4.x);
+      s_q.slow = beyond_reduction(pd, pos, TIED ? lx : fmaxf(fmaxf(lx, fabsf((float)l4.y)),
+                                                             fabsf((float)l4.z)));
       if (sp == 0) {
         const long long px = (long long)pd.nx * pd.ny;
         if (dif) pd_ += px;
@@ -337,12 +179,12 @@ __global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
 #pragma unroll
     for (int s = 0; s < NSUM; ++s) acc[s] = ds{0.f, 0.f};
     if constexpr (DIF) {
-      if (dif) dif_rows<TIED>(pd.tilesff, r0, r1, s_q, acc);
-      else if (s_q.slow) ff_rows<VAR, TIED, true>(pd.tilesff, r0, r1, s_q, s_tab, acc);
-      else ff_rows<VAR, TIED, false>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+      if (dif) dif_rows<TIED, RE_NT>(pd.tilesff, r0, r1, tid, s_q, acc);
+      else if (s_q.slow) ff_rows<VAR, TIED, true, RE_NT>(pd.tilesff, r0, r1, tid, s_q, s_tab, acc);
+      else ff_rows<VAR, TIED, false, RE_NT>(pd.tilesff, r0, r1, tid, s_q, s_tab, acc);
     } else {
-      if (s_q.slow) ff_rows<VAR, TIED, true>(pd.tilesff, r0, r1, s_q, s_tab, acc);
-      else ff_rows<VAR, TIED, false>(pd.tilesff, r0, r1, s_q, s_tab, acc);
+      if (s_q.slow) ff_rows<VAR, TIED, true, RE_NT>(pd.tilesff, r0, r1, tid, s_q, s_tab, acc);
+      else ff_rows<VAR, TIED, false, RE_NT>(pd.tilesff, r0, r1, tid, s_q, s_tab, acc);
     }
     reduce_store<NSUM>(acc, s_red, L.out + (int64_t)local * NSUM);
   }
