@@ -23,6 +23,7 @@ UNITS = {
     "capi.cu": [],
     "aux.cu": [],
     "solve.cu": ["-fmad=false"],
+    "search.cu": ["-fmad=false"],
     "second_order.cu": ["-fmad=false"],
     "pairsum_f32_val.cu": [],
     "pairsum_f32_obj.cu": [],

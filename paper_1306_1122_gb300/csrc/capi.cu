@@ -111,7 +111,7 @@ struct SolveCtrl {
   int32_t act_cnt[2];
   int32_t near_cnt[2];
   int32_t bad;
-  int32_t pad;
+  int32_t next;             // a resident search's queue position
   unsigned long long stat_queries;
   double stat_pairs;
   // certified decisions: the re-evaluation pass of each round (float-float and differences)
@@ -400,6 +400,15 @@ bool use_few(int var, bool tied, bool fp64, int64_t n, double npix, bool search)
   if (tied && var != VAR_OBJ && var != VAR_OBJN) return false;
   return n <= (search ? 12000 : 2500) || (!search && n <= 6000 && (double)n * npix <= 7e7);
 }
+
+// Whether a search of few points runs whole in one kernel (search.cu) instead of rounds by
+// launches: few points on few strips of 128 pixels, so that a CTA's share of a round is short.
+// Measured (ms, launches / one kernel; 10 iterations, then to convergence): 50 points over 32 x 32
+// pixels 1.39 / 0.97, 6.1 / 3.5; 200 there 1.71 / 0.99, 6.7 / 3.7; 1,000 there 1.98 / 1.28, 8.5 / 7.2;
+// 200 over 64 x 64 1.66 / 1.10, 7.5 / 5.2; 50 over 128 x 128 1.39 / 1.17, 7.1 / 5.5; but 2,000 over
+// 32 x 32 2.08 / 1.64, 9.1 / 10.3, 1,000 over 64 x 64 2.39 / 2.33, 8.8 / 8.2, 200 over 128 x 128
+// 2.30 / 3.07, 8.1 / 6.3 and 200 over 256 x 200 3.4 / 8.0, 11.4 / 13.3.
+bool use_resident(int64_t N, int strips) { return N <= 1200 && N * strips <= 10000; }
 
 // One pair-sum pass over n queries of this context (single problem): pack, plan, sweep,
 // near-field correction.  Results are in c->out as item chunks described by c->misc.
@@ -1454,13 +1463,16 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   DBIE_TRY(ensure(b.ctrl, sizeof(SolveCtrl)));
   // passes of few queries: the lanes of a warp take pixels, all problems share one queue
   const bool few = use_few(var, tied, fp64, N, (double)max_rows * (TILE / RE_ROWS_PER_TILE), true);
+  // or the whole search in one kernel (no launches to time while profiling)
+  const bool resident = few && !qn && !c->profiling && use_resident(N, max_rows);
   const KernelRef kw = few_ref(var, tied, c->quad_g != 0);
-  const int grid_few = few ? persistent_grid(kw, c->device) : 0;
-  DBIE_TRY(ensure(b.out, sizeof(double) * nsum *
-                             (few ? few_records(Qcap, grid_few) : items_cap * k.qper)));
+  const int grid_few = few && !resident ? persistent_grid(kw, c->device) : 0;
+  if (!resident)
+    DBIE_TRY(ensure(b.out, sizeof(double) * nsum *
+                               (few ? few_records(Qcap, grid_few) : items_cap * k.qper)));
   DBIE_TRY(ensure(b.res, align256(sizeof(double) * 8 * N) + align256(sizeof(int32_t) * 3 * N)));
   if (codes_stride) DBIE_TRY(ensure(b.codes, (size_t)codes_stride * N));
-  for (int sd = 0; sd < 2; ++sd) {
+  for (int sd = 0; sd < 2 && !resident; ++sd) {
     DBIE_TRY(ensure(b.qpos[sd], sizeof(float4) * Qcap));
     DBIE_TRY(ensure(b.qlam[sd], sizeof(Lam4) * Qcap));
     DBIE_TRY(ensure(b.q_cnt[sd], sizeof(int32_t) * nprob));
@@ -1471,13 +1483,13 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     DBIE_TRY(ensure(b.msc, sizeof(float) * 18 * N));
     DBIE_TRY(ensure(b.fout, sizeof(double) * std::max(12 * reeval_items(2 * N, grid_re),
                                                       3 * reeval_items(N, grid_v))));
-    for (int sd = 0; sd < 2; ++sd) {
+    for (int sd = 0; sd < (resident ? 1 : 2); ++sd) {
       DBIE_TRY(ensure(b.fpos[sd], sizeof(float4) * 2 * N));
       DBIE_TRY(ensure(b.flam[sd], sizeof(Lam4) * 2 * N));
       DBIE_TRY(ensure(b.ref[sd], sizeof(int32_t) * N));
     }
   }
-  if (dif_on) {
+  if (dif_on && !resident) {
     DBIE_TRY(ensure(b.dout, sizeof(double) * 12 * reeval_items(2 * N, grid_re)));
     for (int sd = 0; sd < 2; ++sd) {
       DBIE_TRY(ensure(b.dpos[sd], sizeof(float4) * 2 * N));
@@ -1546,7 +1558,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     CUDA_TRY(cudaStreamSynchronize(s));
     if (c->pinned[0]) return fail(DBIE_EINVAL, "a point is not finite or has z <= 0");
   }
-  for (int sd = 0; sd < 2; ++sd) CUDA_TRY(cudaMemsetAsync(b.q_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
+  for (int sd = 0; sd < 2 && !resident; ++sd)
+    CUDA_TRY(cudaMemsetAsync(b.q_cnt[sd].p, 0, sizeof(int32_t) * nprob, s));
   if (cert) {
     // the error bounds' lambda-independent absolute-value sums of every point
     launch_msc(b.probs.as<ProbDesc>(), N, b.ppos.as<float4>(), b.msc.as<float>(),
@@ -1628,15 +1641,12 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
       a.stat_difs = &ctrl->stat_difs;
     }
   }
-  // Initial simplex and its queries go to side 0.
-  SolveArgs a0 = sa[1];  // "next" of the side-1 round is side 0
-  // step kernels: four warps per CTA, resident at their register count; every point a warp at most
-  const int nm_grid = (int)std::min<int64_t>((N + 3) / 4, 4LL * c->sm_count);
-  const int apply_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
-  (qn ? launch_bfgs_init : launch_solve_init)(a0, any_init ? b.lam0.as<double>() : nullptr,
-                    (int)std::min<int64_t>((N + 255) / 256, 8LL * c->sm_count), s);
-  CUDA_TRY(cudaGetLastError());
-
+  // Rounds a point can take: the simplex spends at most 3 per iteration; the quasi-Newton search
+  // at most 31 line-search trials (alpha = 1 ... 2^-30) per accepted step.
+  // A certified step waits at most once per value it compares (4 vertices, the trial and the
+  // reflected point), each re-evaluation removing one bound; twice with the difference level
+  // (a difference value that ties again goes to float-float).
+  const int max_rounds = (qn ? 31 : (dif_on ? 39 : (cert ? 21 : 3))) * o.max_iter + (cert ? 26 : 8);
   // Arguments of the re-evaluation pass of a round (side cur).
   auto reeval_args = [&](int cur) {
     ReArgs ra{};
@@ -1653,6 +1663,34 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     ra.rows = max_rows;
     return ra;
   };
+  const int apply_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
+  if (resident) {
+    const KernelRef ks = search_ref(tied, c->quad_g != 0);
+    const int grid_s = (int)std::min<int64_t>(N, persistent_grid(ks, c->device));
+    ResidentArgs ra{};
+    ra.a = sa[0];
+    ra.lam_init = any_init ? b.lam0.as<double>() : nullptr;
+    ra.sctab = c->misc.as<Misc>()->sctab;
+    ra.next = &ctrl->next;
+    ra.points = (int32_t)std::min<int64_t>(ks.qper, (N + grid_s - 1) / grid_s);
+    ra.strips = max_rows;
+    ra.max_rounds = max_rounds;
+    ra.rounds = &ctrl->round;
+    ra.stat_queries = &ctrl->stat_queries;
+    ra.stat_pairs = &ctrl->stat_pairs;
+    ra.stat_ff_pairs = &ctrl->stat_ff_pairs;
+    ra.stat_dif_pairs = &ctrl->stat_dif_pairs;
+    DBIE_TRY(launch_kernel(ks, grid_s, &ra, s));
+    DBIE_TRY(check_device_error(c, s));
+  } else {
+  // Initial simplex and its queries go to side 0.
+  SolveArgs a0 = sa[1];  // "next" of the side-1 round is side 0
+  // step kernels: four warps per CTA, resident at their register count; every point a warp at most
+  const int nm_grid = (int)std::min<int64_t>((N + 3) / 4, 4LL * c->sm_count);
+  (qn ? launch_bfgs_init : launch_solve_init)(a0, any_init ? b.lam0.as<double>() : nullptr,
+                    (int)std::min<int64_t>((N + 255) / 256, 8LL * c->sm_count), s);
+  CUDA_TRY(cudaGetLastError());
+
   // One simplex round = plan, pair sums (objective variant), near-field correction, step.
   constexpr int K = 4;  // rounds per graph launch (even: the ping-pong side returns to 0)
   // The near field of a round's queries; in a pass of few queries beside the pair sums.
@@ -1821,12 +1859,6 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     if (ce != cudaSuccess) return fail(DBIE_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
     b.key = key;
   }
-  // Rounds a point can take: the simplex spends at most 3 per iteration; the quasi-Newton search
-  // at most 31 line-search trials (alpha = 1 ... 2^-30) per accepted step.
-  // A certified step waits at most once per value it compares (4 vertices, the trial and the
-  // reflected point), each re-evaluation removing one bound; twice with the difference level
-  // (a difference value that ties again goes to float-float).
-  const int max_rounds = (qn ? 31 : (dif_on ? 39 : (cert ? 21 : 3))) * o.max_iter + (cert ? 26 : 8);
   const int max_launches = max_rounds / K + 2;
   int launches = 0;
   for (;;) {
@@ -1863,6 +1895,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     DBIE_TRY(check_device_error(c, s));
     if (c->pinned[0] == 0 && c->pinned[1] == 0) break;
     if (launches >= max_launches) return fail(DBIE_EINTERNAL, "lambda-search rounds did not terminate");
+  }
   }
   // Certified B: the final field of every point whose error bound does not certify 1e-5
   // relative (the cancellation-dominated points) again, in float-float at lambda* (side 0 is the

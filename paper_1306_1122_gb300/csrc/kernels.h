@@ -92,6 +92,22 @@ __host__ __device__ inline int few_split(int nq, int strips, int warps) {
   return (int)(ns > most ? (most < 1 ? 1 : most) : (ns < 1 ? 1 : ns));
 }
 
+// search.cu: the simplex search of few points, whole in one kernel.
+struct ResidentArgs {
+  SolveArgs a;              // state, results and options (its round buffers are not used)
+  const double* lam_init;   // (N, 3) or null
+  const float4* sctab;
+  int32_t* next;            // queue position, zero before the launch
+  int32_t points;           // points of a CTA at a time, at most KernelRef::qper
+  int32_t strips;           // strips of 128 pixels of the largest problem
+  int32_t max_rounds;       // rounds a point can take
+  int32_t pad0;
+  int32_t* rounds;          // statistics
+  unsigned long long* stat_queries;
+  double *stat_pairs, *stat_ff_pairs, *stat_dif_pairs;
+};
+KernelRef search_ref(bool tied, bool split);
+
 // pairsum_re.cu: float-float sums (VAR_V, VAR_OBJ) and difference sums (objective) of queued
 // queries, one CTA per query and row range.
 struct ReList {

@@ -640,13 +640,14 @@ __device__ __forceinline__ double over(double x) {
 //
 // What bounds it: one warp's chain of instructions, its FP64 instructions above all (64 cycles
 // each), so the time is the instruction count of the longest warp.  Hence FP64 only where the
-// values and lambdas are formed (comparisons on the integer pipe, bounds in FP32), and two
+// values and lambdas are formed (comparisons on the integer pipe, bounds in FP32), and three
 // phases.  First the lanes share out the values to compute, whatever the points' stages (a shrink
 // has 3, the start 4; taken in turn by the point's own lane they set the length for the whole
-// warp): one FP64 objective and bound per lane, or per four lanes where the warp has few points.  Then each lane decides its point's step on Phi and
-// bound alone; vertices stay in their slots, and a step writes one record, not four.  On 2,048
-// points a step took 63 us (the waiting points' 112 us) with one lane per point evaluating and
-// sorting whole vertices, in CTAs of 128 threads.
+// warp): one FP64 objective and bound per lane, or per four lanes where the warp has few points.
+// Then each lane decides its point's step on Phi and tie radius alone; vertices stay in their slots,
+// and a step writes one record, not four.  Then the lanes share out the trial points' lambdas.  On
+// 2,048 points a step took 63 us and the waiting points' 112 us with one lane per point evaluating
+// and sorting whole vertices, in CTAs of 128 threads; now 28 and 15.
 // Warp `warp` of `nwarps` takes ppw points at a time.
 template <int N, bool REF>
 __device__ __forceinline__ void step_points(const SolveArgs& a, int warp, int nwarps, int ppw) {
