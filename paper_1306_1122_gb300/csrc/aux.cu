@@ -261,6 +261,7 @@ void launch_nearfield(int var, bool tied, const NearArgs& a, int sm_count, cudaS
     switch (var) {
       case VAR_V: NF(VAR_V, false); break;
       case VAR_VL: NF(VAR_VL, false); break;
+      case VAR_L: NF(VAR_L, false); break;
       case VAR_OBJ: NF(VAR_OBJ, false); break;
       case VAR_OBJL: NF(VAR_OBJL, false); break;
       case VAR_OBJN: NF(VAR_OBJN, false); break;

@@ -338,7 +338,7 @@ KernelRef g1_ref(dbie_ctx* c, int var, bool tied, bool fp64, int rows = -1) {
   if (fp64) return g1_ref_f64(var, tied);
   const bool r = rows < 0 ? (c->qnx % 4 == 0) : rows != 0;
   if (c->quad_g != 0) return g1_ref_f32_split(var, tied, r);   // element Gauss points
-  return g1_ref_f32(var, tied, c->cfg[var][tied ? 1 : 0], r);
+  return g1_ref_f32(var, tied, c->cfg[cfg_var(var)][tied ? 1 : 0], r);
 }
 
 // Float-float sums of n queries of this context, or with lam_ref (float64, as lam) the
@@ -1129,9 +1129,9 @@ dbie_status dbie_vjp(dbie_ctx* c, int64_t n, const float* xyz, const double* lam
       DBIE_TRY(pxe_adjoint(c, n, c->pxe_pos.as<float4>(), d_gB, false, fp64, o, d_gB0, s));
     }
     if (d_glam) {
-      // dL/dlambda_p = gB_p * z lambda_p Sl_p, from a value + dB/dlambda pass.
-      DBIE_TRY(pass_single(c, VAR_VL, fp64, o, n, d_xyz, nullptr, d_lam, s));
-      launch_finalize_eval(VAR_VL, n, &m->plan, m->item_off, c->out.as<double>(),
+      // dL/dlambda_p = gB_p * z lambda_p Sl_p
+      DBIE_TRY(pass_single(c, VAR_L, fp64, o, n, d_xyz, nullptr, d_lam, s));
+      launch_finalize_eval(VAR_L, n, &m->plan, m->item_off, c->out.as<double>(),
                            c->qpos.as<float4>(), c->qlam.as<Lam4>(), o.g_scale, o.w_g, nullptr,
                            nullptr, d_glam, d_gB, nullptr, nullptr, s);
       CUDA_TRY(cudaGetLastError());

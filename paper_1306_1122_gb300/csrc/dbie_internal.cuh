@@ -41,21 +41,25 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // 2 s per wait
 // dS1/dlambda = -lambda S0, dSx/dlambda = -lambda Tx, dSy/dlambda = -lambda Ty.
 // VAR_HESS adds Q = sum sin(lambda r) b, Ux = sum cos(lambda r) (x_i - x_k) b / r and Uy, the
 // second derivatives: dSl/dlambda = -Q, dTx/dlambda = lambda Ux, dTy/dlambda = lambda Uy.
+// VAR_L sums Sl alone (dL/dlambda): cosines without sines, four SFU operations per pair instead of
+// seven.  Its launch configuration is VAR_VL's.
 // VAR_NV (noise variance) sums phi^2 s over a boundary whose "b" fields hold
 // s = sigma^2 (dA / 2 pi)^2, so that Var B_p = z^2 S0 (B is linear in B0, Eq. 16).
 enum Variant {
-  VAR_V = 0, VAR_VL = 1, VAR_OBJ = 2, VAR_OBJL = 3, VAR_OBJN = 4, VAR_HESS = 5, VAR_NV = 6
+  VAR_V = 0, VAR_VL = 1, VAR_OBJ = 2, VAR_OBJL = 3, VAR_OBJN = 4, VAR_HESS = 5, VAR_NV = 6, VAR_L = 7
 };
-constexpr int NVAR = 7;
+constexpr int NVAR = 7;   // variants with a launch configuration of their own
+__host__ __device__ constexpr int cfg_var(int var) { return var == VAR_L ? VAR_VL : var; }
 __host__ __device__ constexpr int nsum_per_comp(int var) {
   return var == VAR_V ? 1 : var == VAR_VL ? 2 : var == VAR_OBJ ? 4 : var == VAR_OBJL ? 5
        : var == VAR_OBJN ? 7 : var == VAR_HESS ? 10 : 1;
 }
+__host__ __device__ constexpr bool has_value(int var) { return var != VAR_L; }
 __host__ __device__ constexpr bool has_grad(int var) {
   return var == VAR_OBJ || var == VAR_OBJL || var == VAR_OBJN || var == VAR_HESS;
 }
 __host__ __device__ constexpr bool has_dlam(int var) {
-  return var == VAR_VL || var == VAR_OBJL || var == VAR_OBJN || var == VAR_HESS;
+  return var == VAR_VL || var == VAR_OBJL || var == VAR_OBJN || var == VAR_HESS || var == VAR_L;
 }
 __host__ __device__ constexpr bool has_newton(int var) {
   return var == VAR_OBJN || var == VAR_HESS;
@@ -65,7 +69,9 @@ __host__ __device__ constexpr bool is_nv(int var) { return var == VAR_NV; }
 // indices of Tx, Ty (VAR_OBJN, VAR_HESS) and of Q, Ux, Uy (VAR_HESS) within a component's block
 constexpr int IDX_TX = 5, IDX_TY = 6, IDX_Q = 7, IDX_UX = 8, IDX_UY = 9;
 // index of the Sl sum within a component's block
-__host__ __device__ constexpr int idx_sl(int var) { return var == VAR_VL ? 1 : 4; }
+__host__ __device__ constexpr int idx_sl(int var) {
+  return var == VAR_L ? 0 : (var == VAR_VL ? 1 : 4);
+}
 
 // Lambda triple of a query (FP64; the mixed form rounds it to FP32 when loading).
 struct __align__(32) Lam4 {
@@ -437,6 +443,11 @@ __device__ __forceinline__ void pair_angularv(const Query<V, TIED>& q, const Geo
                                               const V b[3], TermsV<V, VAR, TIED>& t) {
   t.dx = g.dx;
   t.dy = g.dy;
+  if constexpr (!has_value(VAR)) {
+#pragma unroll
+    for (int p = 0; p < (TIED ? 1 : 3); ++p) t.cr[p] = vmul(vcos(vmul(q.l[p], g.r)), g.ri);
+    return;
+  }
 #pragma unroll
   for (int p = 0; p < 3; ++p) t.rb[p] = vmul(g.ri3, b[p]);
 #pragma unroll

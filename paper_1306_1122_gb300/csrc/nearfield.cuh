@@ -98,7 +98,7 @@ __device__ __forceinline__ void near_window(
         // factors, exact in FP64; the packed kernel's can differ by a rounding of a factor),
         // replaced by the FP64 terms.
         if constexpr (has_hess(VAR)) c[p * NS] += t64.t0[p] - (double)t32.t0[p];
-        else c[p * NS] += t64.t0[p] - (double)t32.u[lp] * (double)t32.rb[p];
+        else if constexpr (has_value(VAR)) c[p * NS] += t64.t0[p] - (double)t32.u[lp] * (double)t32.rb[p];
         if constexpr (has_grad(VAR)) {
           c[p * NS + 1] += t64.t1[p] - (double)t32.t1[p];
           c[p * NS + 2] += t64.t1[p] * t64.dx - (double)t32.t1[p] * (double)t32.dx;

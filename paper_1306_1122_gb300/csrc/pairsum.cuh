@@ -138,7 +138,8 @@ __device__ __forceinline__ void accumulatev(V* acc, const TermsV<V, VAR, TIED>& 
     const int lp = TIED ? 0 : p;
     // (the Hessian pass adds the rounded products phi b and cos(lambda r) b / r, which its
     // row-group form sums in pairs; the near-field correction subtracts the same values)
-    if constexpr (is_nv(VAR)) acc[p * NS + 0] = vfma(t.ph[lp], t.t0[p], acc[p * NS + 0]);
+    if constexpr (!has_value(VAR)) (void)lp;
+    else if constexpr (is_nv(VAR)) acc[p * NS + 0] = vfma(t.ph[lp], t.t0[p], acc[p * NS + 0]);
     else if constexpr (has_hess(VAR)) acc[p * NS + 0] = vadd(acc[p * NS + 0], t.t0[p]);
     else acc[p * NS + 0] = vfma(t.u[lp], t.rb[p], acc[p * NS + 0]);
     if constexpr (has_grad(VAR)) {
@@ -200,7 +201,7 @@ __device__ __forceinline__ void accumulate64(double* acc, const Terms64<VAR, TIE
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
     if constexpr (is_nv(VAR)) acc[p * NS + 0] += t.ph[p] * t.t0[p];
-    else acc[p * NS + 0] += t.t0[p];
+    else if constexpr (has_value(VAR)) acc[p * NS + 0] += t.t0[p];
     if constexpr (has_grad(VAR)) {
       acc[p * NS + 1] += t.t1[p];
       acc[p * NS + 2] += t.t1[p] * t.dx;

@@ -18,6 +18,7 @@ KernelRef split_ref(bool rows) {
 KernelRef g1_ref_f32_split(int var, bool tied, bool rows) {
   switch (var) {
     case VAR_V: return tied ? split_ref<VAR_V, true>(rows) : split_ref<VAR_V, false>(rows);
+    case VAR_L: return split_ref<VAR_L, false>(rows);
     case VAR_VL: return tied ? split_ref<VAR_VL, true>(rows) : split_ref<VAR_VL, false>(rows);
     case VAR_OBJ: return tied ? split_ref<VAR_OBJ, true>(rows) : split_ref<VAR_OBJ, false>(rows);
     case VAR_OBJL: return tied ? split_ref<VAR_OBJL, true>(rows) : split_ref<VAR_OBJL, false>(rows);

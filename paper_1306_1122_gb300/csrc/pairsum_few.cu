@@ -89,6 +89,7 @@ KernelRef few_ref(int var, bool tied, bool split) {
   switch (var) {
     case VAR_V: return few_ref_t<VAR_V, false>(split);
     case VAR_VL: return few_ref_t<VAR_VL, false>(split);
+    case VAR_L: return few_ref_t<VAR_L, false>(split);
     case VAR_OBJ: return tied ? few_ref_t<VAR_OBJ, true>(split) : few_ref_t<VAR_OBJ, false>(split);
     case VAR_OBJL: return few_ref_t<VAR_OBJL, false>(split);
     default: return tied ? few_ref_t<VAR_OBJN, true>(split) : few_ref_t<VAR_OBJN, false>(split);

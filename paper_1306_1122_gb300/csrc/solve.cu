@@ -35,7 +35,7 @@ __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan
     double S[NSUM];
     gather_sums<NSUM>(out, h, item_off, 0, i, S);
     double Bv[3], G[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int p = 0; p < 3; ++p) Bv[p] = z * S[p * NS];
+    for (int p = 0; p < 3; ++p) Bv[p] = has_value(VAR) ? z * S[p * NS] : 0.0;
     if constexpr (has_grad(VAR)) {
       for (int p = 0; p < 3; ++p) {
         G[3 * p + 0] = z * S[p * NS + 2];
@@ -84,6 +84,7 @@ void launch_finalize_eval(int var, int64_t n, const PlanHdr* plan, const int32_t
   switch (var) {
     case VAR_V: FIN(VAR_V); break;
     case VAR_VL: FIN(VAR_VL); break;
+    case VAR_L: FIN(VAR_L); break;
     case VAR_OBJ: FIN(VAR_OBJ); break;
     default: FIN(VAR_OBJL); break;
   }
