@@ -17,7 +17,7 @@
 using namespace dbie;
 
 #ifndef DBIE_SPLIT_TARGET_PCT
-#define DBIE_SPLIT_TARGET_PCT 200
+#define DBIE_SPLIT_TARGET_PCT 400
 #endif
 
 namespace {
@@ -182,7 +182,11 @@ struct dbie_ctx {
   int64_t nquad = 0;              // quadrature points: npix, or (elements x g)^2
   int32_t qnx = 0, qny = 0;       // quadrature-point grid
   SolveBufs sb;
-  int cfg[NVAR][2] = {};   // tuned launch configuration per variant / tied
+  // Launch configuration per variant / tied until dbie_autotune picks one: uncapped, but the
+  // objective variants at six CTAs of 128 threads per SM (80 registers), which keep the SFU busier.
+  // (B, gradient, f and g at 20,000 points over 300 x 300 pixels 3.51 -> 3.16 ms, with dB/dlambda
+  // 3.67 -> 3.40; ten search iterations of 131,072 points over 128 x 128 94 -> 87 ms.)
+  int cfg[NVAR][2] = {{0, 0}, {0, 0}, {3, 0}, {3, 0}, {0, 0}, {0, 0}, {0, 0}};
   int vjp_cfg = 0;
   cudaStream_t cap_stream = nullptr;  // streams and events used only to capture graphs
   cudaStream_t cap_side = nullptr;
@@ -329,6 +333,12 @@ dbie_status timed_launch(dbie_ctx* c, const KernelRef& k, int grid, void* args, 
   return DBIE_OK;
 }
 
+// Work items that a pass of few blocks is split into over tile ranges, in percent of the persistent
+// grid.  Four items per CTA even out the last wave (items of two per CTA ended in a third wave a few
+// per cent full): B at 20,000 points over 300 x 300 pixels 2.93 -> 2.82 ms, with gradient 3.48 -> 3.27,
+// 15,000 points over 257 x 200 pixels 1.32 -> 1.26.
+int split_pct(int var) { return var == VAR_HESS || var == VAR_NV ? 200 : DBIE_SPLIT_TARGET_PCT; }
+
 int var_of(bool grad, bool dlam) {
   return grad ? (dlam ? VAR_OBJL : VAR_OBJ) : (dlam ? VAR_VL : VAR_V);
 }
@@ -464,7 +474,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   const KernelRef k = g1_ref(c, var, tied, fp64);
   const int grid = persistent_grid(k, c->device);
   const int64_t nblk = (n + k.qper - 1) / k.qper;
-  const int64_t target = std::max<int64_t>(1, (int64_t)grid * DBIE_SPLIT_TARGET_PCT / 100);
+  const int64_t target = std::max<int64_t>(1, (int64_t)grid * split_pct(var) / 100);
   int64_t nsplit = 1;
   if (nblk < target) nsplit = std::min<int64_t>((target + nblk - 1) / nblk, c->ntiles);
   const int64_t nitems = nblk * nsplit;
@@ -1440,7 +1450,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   const int grid = persistent_grid(k, c->device);
   // Split a round's queries over tile ranges until the items cover this many CTAs (percent of
   // the persistent grid): more items balance the queue, fewer items mean fewer partial sums.
-  const int target = (int)((int64_t)grid * DBIE_SPLIT_TARGET_PCT / 100);
+  const int target = (int)((int64_t)grid * split_pct(var) / 100);
   const int64_t items_cap = std::max<int64_t>((Qcap + k.qper - 1) / k.qper + nprob, 2LL * target) + 1;
   // re-evaluation pass (at most 2 float-float and 2 difference queries per point and round); the
   // difference level re-evaluates values near the point's float-float reference
