@@ -476,7 +476,8 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   const int64_t nblk = (n + k.qper - 1) / k.qper;
   const int64_t target = std::max<int64_t>(1, (int64_t)grid * split_pct(var) / 100);
   int64_t nsplit = 1;
-  if (nblk < target) nsplit = std::min<int64_t>((target + nblk - 1) / nblk, c->ntiles);
+  if (nblk < target)
+    nsplit = std::min<int64_t>((target + nblk - 1) / nblk, (int64_t)c->ntiles * (fp64 ? F64_PARTS : 1));
   const int64_t nitems = nblk * nsplit;
   if (nitems > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
   const int nsum = 3 * nsum_per_comp(var);
@@ -1761,7 +1762,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     pa.nprob = nprob;
     pa.qper = k.qper;
     pa.target_items = target;
-    pa.nsplit_cap = 1 << 20;
+    pa.parts = fp64 ? F64_PARTS : 1;
     pa.q_cnt_cur = b.q_cnt[cur].as<int32_t>();
     pa.q_cnt_pass = b.q_cnt_pass.as<int32_t>();
     pa.item_off = b.item_off.as<int32_t>();

@@ -14,6 +14,7 @@ namespace dbie {
 
 constexpr int TILE = 256;            // pixels (or points, for the adjoint) per tile
 constexpr int NFIELD = 5;            // x, y, bx, by, bz
+constexpr int F64_PARTS = 4;         // ranges of the FP64 form are in quarters of a tile
 // FP32 tiles of element Gauss points (Eq. 15) carry their positions as float pairs (hi + lo):
 // x, y, bx, by, bz, x_lo, y_lo.  The pair sums form x_i - x_k as (x_i - x_hi) - x_lo, so the
 // FP32 rounding of an irrational Gauss abscissa does not enter the kernel.

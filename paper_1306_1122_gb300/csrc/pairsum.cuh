@@ -9,7 +9,9 @@
 //
 //  * Work: persistent CTAs take items (problem, register block, tile range) from a device
 //    counter, so many magnetograms of uneven size share one launch and small sets can be split
-//    over tile ranges; each item writes FP64 partial sums for its split.
+//    over tile ranges; each item writes FP64 partial sums for its split.  A CTA's first item is its
+//    own number: consecutive CTAs start on different SMs, where the counter let the CTAs that
+//    share an SM take all of a small pass (256 items: up to six on one SM and none on others).
 //  * Staging: one elected thread moves each tile with one cp.async.bulk (TMA bulk copy, no
 //    multicast) into an NSTAGE-deep ring of shared-memory buffers guarded by mbarriers (full:
 //    transaction bytes; empty: one arrival per warp).  Every wait is bounded in time.
@@ -232,6 +234,15 @@ __device__ __forceinline__ void fold2(V& hi, V& a) {
   a = e;
 }
 
+// Thread 0: the CTA's next work item (its own number first, then the counter's).
+__device__ __forceinline__ int next_item(int32_t* work, bool& first) {
+  if (first) {
+    first = false;
+    return blockIdx.x;
+  }
+  return gridDim.x + atomicAdd(work, 1);
+}
+
 // Locate the problem owning work item `it` (item_off is a prefix array of length nprob + 1).
 __device__ __forceinline__ int find_problem(const int32_t* item_off, int nprob, int it) {
   int lo = 0, hi = nprob - 1;
@@ -272,10 +283,11 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
   }
   __syncthreads();
   const PlanHdr plan = *a.plan;
+  bool first = true;
 
   for (;;) {
     // Thread 0 alone decides whether to stop, so the decision is uniform across the CTA.
-    if (tid == 0) s_item = s_abort ? plan.nitems : atomicAdd(a.work, 1);
+    if (tid == 0) s_item = s_abort ? plan.nitems : next_item(a.work, first);
     __syncthreads();
     const int it = s_item;
     __syncthreads();  // every thread has read s_item before it can be overwritten
@@ -292,8 +304,15 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
     const int blk = local / plan.nsplit;
     const int sp = local - blk * plan.nsplit;
     const int qtotal = __ldg(a.q_cnt + pidx);
-    const int t0 = (int)(((int64_t)sp * pd.ntiles) / plan.nsplit);
-    const int t1 = (int)(((int64_t)(sp + 1) * pd.ntiles) / plan.nsplit);
+    // Tile range.  FP64 form: a range of quarters of a tile, since one item of 128 queries by a
+    // tile takes ~1.5 ms there (an FP64 instruction holds its SM sub-partition for 64 cycles, a
+    // pair needs ~115), so whole tiles leave most of the chip idle behind the last items.
+    // 2,048 queries x 4,096 pixels: 5.0 -> 1.57 ms (with the first-item rule above).
+    constexpr int PARTS = F32 ? 1 : F64_PARTS;
+    const int u0 = (int)(((int64_t)sp * pd.ntiles * PARTS) / plan.nsplit);
+    const int u1 = (int)(((int64_t)(sp + 1) * pd.ntiles * PARTS) / plan.nsplit);
+    const int t0 = u0 / PARTS, t1 = (u1 + PARTS - 1) / PARTS;
+    int kt = u0 * (TILE / PARTS) - t0 * TILE, kleft = (u1 - u0) * (TILE / PARTS);
     const Real* tiles = F32 ? reinterpret_cast<const Real*>(pd.tiles32)
                             : reinterpret_cast<const Real*>(pd.tiles64);
 
@@ -482,8 +501,9 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
             for (int s = 0; s < NSUM; ++s) fold2(hi[u][s], acc[u][s]);
         }
       } else {
+        const int k1 = kt + kleft < TILE ? kt + kleft : TILE;
 #pragma unroll 2
-        for (int k = 0; k < TILE; ++k) {
+        for (int k = kt; k < k1; ++k) {
           const double b[3] = {sx[2 * TILE + k], sx[3 * TILE + k], sx[4 * TILE + k]};
           const double px = sx[k], py = sx[TILE + k];
 #pragma unroll
@@ -493,6 +513,8 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
             accumulate64<VAR, TIED, NS>(acc[u], tm);
           }
         }
+        kleft -= k1 - kt;
+        kt = 0;
       }
     });
 
@@ -559,9 +581,10 @@ __device__ __forceinline__ void vjp_body(const VjpArgs& a) {
                            : reinterpret_cast<const Real*>(a.ptiles64);
   const Real* btiles = F32 ? reinterpret_cast<const Real*>(a.btiles32)
                            : reinterpret_cast<const Real*>(a.btiles64);
+  bool first = true;
 
   for (;;) {
-    if (tid == 0) s_item = s_abort ? plan.nitems : atomicAdd(a.work, 1);
+    if (tid == 0) s_item = s_abort ? plan.nitems : next_item(a.work, first);
     __syncthreads();
     const int it = s_item;
     __syncthreads();
@@ -713,9 +736,10 @@ __device__ __forceinline__ void vjp7_body(const VjpArgs& a) {
                            : reinterpret_cast<const Real*>(a.ptiles64);
   const Real* btiles = F32 ? reinterpret_cast<const Real*>(a.btiles32)
                            : reinterpret_cast<const Real*>(a.btiles64);
+  bool first = true;
 
   for (;;) {
-    if (tid == 0) s_item = s_abort ? plan.nitems : atomicAdd(a.work, 1);
+    if (tid == 0) s_item = s_abort ? plan.nitems : next_item(a.work, first);
     __syncthreads();
     const int it = s_item;
     __syncthreads();

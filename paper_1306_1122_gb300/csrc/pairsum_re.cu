@@ -136,10 +136,12 @@ __global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
     *a.f.plan = PlanHdr{fitems, fs, 1, 0};
     if (DIF) *a.d.plan = PlanHdr{nd * dsp, dsp, 1, 0};
   }
+  bool first = true;   // (a CTA's first item is its own number: see pairsum.cuh)
   long long pf = 0, pd_ = 0;   // thread 32: pairs of the queries whose first range it set up
 
   for (;;) {
-    if (tid == 0) s_item = atomicAdd(a.work, 1);
+    if (tid == 0) s_item = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(a.work, 1);
+    first = false;
     __syncthreads();   // (also: the previous item's readers of s_red and s_q are done)
     const int it = s_item;
     if (it >= items) break;

@@ -155,8 +155,7 @@ __global__ void plan_round_kernel(const PlanArgs a) {
     int nsplit = 1;
     if (blocks > 0 && blocks < a.target_items) {
       nsplit = (int)((a.target_items + blocks - 1) / blocks);
-      if (nsplit > a.nsplit_cap) nsplit = a.nsplit_cap;
-      if (nsplit > s_minTiles) nsplit = s_minTiles;
+      if (nsplit > s_minTiles * a.parts) nsplit = s_minTiles * a.parts;
       if (nsplit < 1) nsplit = 1;
     }
     int acc = 0;

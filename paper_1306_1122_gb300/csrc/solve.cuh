@@ -112,7 +112,7 @@ struct PlanArgs {
   int32_t nprob;
   int32_t qper;              // queries per item
   int32_t target_items;
-  int32_t nsplit_cap;
+  int32_t parts;             // ranges per tile (F64_PARTS for the FP64 form, else 1)
   const int32_t* q_cnt_cur;
   int32_t* q_cnt_pass;       // copy of the current counts read by the pair-sum pass
   int32_t* item_off;         // [nprob + 1]
