@@ -352,6 +352,55 @@ __device__ __forceinline__ V vconst(float a) {
   if constexpr (sizeof(V) == 4) return a;
   else return pack2(a, a);
 }
+// f * f, at most 1
+__device__ __forceinline__ float vsqr_sat(float f) {
+  float y;
+  asm("mul.rn.sat.f32 %0, %1, %1;" : "=f"(y) : "f"(f));
+  return y;
+}
+__device__ __forceinline__ f32x2 vsqr_sat(f32x2 x) {
+  float a, b;
+  unpack2(x, a, b);
+  return pack2(vsqr_sat(a), vsqr_sat(b));
+}
+// x with its sign changed where the whole number held in the low bits of `k` is odd
+__device__ __forceinline__ float vflip(float x, float k) {
+  return __uint_as_float(__float_as_uint(x) ^ (__float_as_uint(k) << 31));
+}
+__device__ __forceinline__ f32x2 vflip(f32x2 x, f32x2 k) {
+  float a, b, ka, kb;
+  unpack2(x, a, b);
+  unpack2(k, ka, kb);
+  return pack2(vflip(a, ka), vflip(b, kb));
+}
+
+// sin and cos of an angle on the FMA pipe: theta = pi (k + f) with k whole and |f| <= 1/2, and
+// minimax polynomials (own exchange fit, 5e-8 and 8e-9) of sin and cos of pi f; both results still
+// want the sign (-1)^k, which vflip applies to a factor that they share.  `vk` returns 1.5 2^23 + k,
+// whose lowest bit is k's.  Errors on [-60, 60]: at most 1.3e-7 (sin) and 2.4e-7 (cos).  Past 1e7
+// rad f grows with theta's rounding; the saturated square keeps the polynomials bounded there.
+template <typename V>
+__device__ __forceinline__ V half_turns(V th, V& vk) {
+  const V ip = vconst<V>(0.31830987334251404f);
+  const V big = vconst<V>(12582912.f);
+  vk = vfma(th, ip, big);
+  const V f = vfma(th, ip, vsub(big, vk));
+  return vfma(th, vconst<V>(1.2841276486597053e-08f), f);
+}
+template <typename V>
+__device__ __forceinline__ V cos_half_turns(V f2) {
+  V c = vfma(vconst<V>(0.22008005f), f2, vconst<V>(-1.3320936f));
+  c = vfma(c, f2, vconst<V>(4.0584513f));
+  c = vfma(c, f2, vconst<V>(-4.9347955f));
+  return vfma(c, f2, vconst<V>(1.f));
+}
+template <typename V>
+__device__ __forceinline__ V sin_half_turns(V f, V f2) {
+  V s = vfma(vconst<V>(0.078012043f), f2, vconst<V>(-0.59851248f));
+  s = vfma(s, f2, vconst<V>(2.5501251f));
+  s = vfma(s, f2, vconst<V>(-5.1677141f));
+  return vmul(vfma(s, f2, vconst<V>(3.14159274f)), f);
+}
 
 // A query with every member in both lanes.
 template <bool TIED>
@@ -438,15 +487,44 @@ __device__ __forceinline__ Geom32 pair_geom32_split(const Query<float, TIED>& q,
                              __fsub_rn(__fsub_rn(q.y, py), pyl));
 }
 
+// Index of a pixel pair within its group of four pixels, as a type.
+template <int H>
+struct Half {
+  static constexpr int value = H;
+};
+
+// Components (bit p) whose sine and cosine the FP32 sums take from the FMA pipe, for even (h = 0)
+// and odd pixel pairs.  The SFU gives 16 results a clock per SM, seven per pair of the field sums
+// (1/r and three sines and cosines) against ~20 operations on the FMA pipe's 128 lanes, so it
+// alone set their time; one component of three on the FMA pipe leaves five SFU results and ~34
+// operations (SFU 85 % busy, FMA pipe 72 %).  Points by pixels 20,000 x 131,072: B 3.98 -> 3.17 ms
+// (one pair of two 3.48, one and two components by turns 3.57), adjoint 4.05 -> 3.38, cosine sums
+// alone, four SFU results per pair, 2.31 -> 2.12 with one component of every second pair (of every
+// pair 2.35).  The gradient sums have ~40 operations per pair already and lose (4.43 -> 4.68 ms at
+// one pair of two), and so do pairs of one tied lambda, which need three SFU results.
+__host__ __device__ constexpr int fma_sincos(int var, bool tied, int h) {
+  return tied ? 0 : var == VAR_V || var == VAR_VL ? 4 : var == VAR_L ? (h ? 0 : 4) : 0;
+}
+
 // Angular part: sin, cos of lambda r (SFU) and the factors of the sums.
-template <typename V, int VAR, bool TIED>
+template <typename V, int VAR, bool TIED, int H = 0>
 __device__ __forceinline__ void pair_angularv(const Query<V, TIED>& q, const GeomV<V>& g,
                                               const V b[3], TermsV<V, VAR, TIED>& t) {
+  constexpr int FMA_SC = fma_sincos(VAR, TIED, H);
   t.dx = g.dx;
   t.dy = g.dy;
   if constexpr (!has_value(VAR)) {
 #pragma unroll
-    for (int p = 0; p < (TIED ? 1 : 3); ++p) t.cr[p] = vmul(vcos(vmul(q.l[p], g.r)), g.ri);
+    for (int p = 0; p < (TIED ? 1 : 3); ++p) {
+      const V th = vmul(q.l[p], g.r);
+      if (FMA_SC >> p & 1) {
+        V k;
+        const V f = half_turns(th, k);
+        t.cr[p] = vflip(vmul(cos_half_turns(vsqr_sat(f)), g.ri), k);
+      } else {
+        t.cr[p] = vmul(vcos(th), g.ri);
+      }
+    }
     return;
   }
 #pragma unroll
@@ -454,7 +532,19 @@ __device__ __forceinline__ void pair_angularv(const Query<V, TIED>& q, const Geo
 #pragma unroll
   for (int p = 0; p < (TIED ? 1 : 3); ++p) {
     const V th = vmul(q.l[p], g.r);
-    const V s = vsin(th), c = vcos(th);
+    V s, c;
+    if (FMA_SC >> p & 1) {   // (the sign goes to b / r^3, and below to cos(lambda r) / r)
+      V k;
+      const V f = half_turns(th, k), f2 = vsqr_sat(f);
+      s = sin_half_turns(f, f2);
+      c = cos_half_turns(f2);
+      t.rb[p] = vflip(t.rb[p], k);
+      if constexpr (has_dlam(VAR)) t.cr[p] = vmul(c, vflip(g.ri, k));
+    } else {
+      s = vsin(th);
+      c = vcos(th);
+      if constexpr (has_dlam(VAR)) t.cr[p] = vmul(c, g.ri);
+    }
     t.u[p] = vfma(th, s, c);
     if constexpr (is_nv(VAR)) t.ph[p] = vmul(t.u[p], g.ri3);
     if constexpr (has_hess(VAR)) t.sn[p] = s;
@@ -476,7 +566,6 @@ __device__ __forceinline__ void pair_angularv(const Query<V, TIED>& q, const Geo
         t.t1[p] = vmul(w, t.rb[p]);
       }
     }
-    if constexpr (has_dlam(VAR)) t.cr[p] = vmul(c, g.ri);
     if constexpr (has_hess(VAR)) {
       if constexpr (TIED) {
 #pragma unroll
@@ -487,22 +576,25 @@ __device__ __forceinline__ void pair_angularv(const Query<V, TIED>& q, const Geo
     }
   }
 }
+// (`odd`: of an odd pixel pair of its tile)
 template <int VAR, bool TIED>
 __device__ __forceinline__ void pair_angular32(const Query<float, TIED>& q, const Geom32& g,
-                                               const float b[3], Terms32<VAR, TIED>& t) {
-  pair_angularv<float, VAR, TIED>(q, g, b, t);
+                                               const float b[3], bool odd, Terms32<VAR, TIED>& t) {
+  if (fma_sincos(VAR, TIED, 0) != fma_sincos(VAR, TIED, 1) && odd)
+    pair_angularv<float, VAR, TIED, 1>(q, g, b, t);
+  else pair_angularv<float, VAR, TIED, 0>(q, g, b, t);
 }
 
 template <int VAR, bool TIED>
 __device__ __forceinline__ void pair_terms32(const Query<float, TIED>& q, float px, float py,
-                                             const float b[3], Terms32<VAR, TIED>& t) {
-  pair_angular32<VAR, TIED>(q, pair_geom32<TIED>(q, px, py), b, t);
+                                             const float b[3], bool odd, Terms32<VAR, TIED>& t) {
+  pair_angular32<VAR, TIED>(q, pair_geom32<TIED>(q, px, py), b, odd, t);
 }
 template <int VAR, bool TIED>
 __device__ __forceinline__ void pair_terms32_split(const Query<float, TIED>& q, float px, float py,
-                                                   float pxl, float pyl, const float b[3],
+                                                   float pxl, float pyl, const float b[3], bool odd,
                                                    Terms32<VAR, TIED>& t) {
-  pair_angular32<VAR, TIED>(q, pair_geom32_split<TIED>(q, px, py, pxl, pyl), b, t);
+  pair_angular32<VAR, TIED>(q, pair_geom32_split<TIED>(q, px, py, pxl, pyl), b, odd, t);
 }
 
 // FP64 terms (used by the FP64 form and by the near-field correction).

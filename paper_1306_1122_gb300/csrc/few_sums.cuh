@@ -24,17 +24,19 @@ __device__ __forceinline__ void strip_step(const float* T, int k, const Query<f3
   const f32x2 py2[2] = {pack2(Y.x, Y.y), pack2(Y.z, Y.w)};
   const f32x2 b2[2][3] = {{pack2(BX.x, BX.y), pack2(BY.x, BY.y), pack2(BZ.x, BZ.y)},
                           {pack2(BX.z, BX.w), pack2(BY.z, BY.w), pack2(BZ.z, BZ.w)}};
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  auto pair = [&](auto half) {
+    constexpr int h = decltype(half)::value;
     f32x2 dx = vsub(q2.x, px2[h]), dy = vsub(q2.y, py2[h]);
     if constexpr (SPLIT) {
       dx = vsub(dx, h == 0 ? pack2(XL.x, XL.y) : pack2(XL.z, XL.w));
       dy = vsub(dy, h == 0 ? pack2(YL.x, YL.y) : pack2(YL.z, YL.w));
     }
     TermsV<f32x2, VAR, TIED> tm;
-    pair_angularv<f32x2, VAR, TIED>(q2, pair_geomv_d<f32x2, TIED>(q2, dx, dy), b2[h], tm);
+    pair_angularv<f32x2, VAR, TIED, h>(q2, pair_geomv_d<f32x2, TIED>(q2, dx, dy), b2[h], tm);
     accumulatev<f32x2, VAR, TIED, NS>(acc2, tm, b2[h]);
-  }
+  };
+  pair(Half<0>{});
+  pair(Half<1>{});
 }
 
 // Sums of a query over strips [s0, s1) of its problem; lane l returns sum l / WarpSums<NSUM>::GL.

@@ -85,10 +85,10 @@ __device__ __forceinline__ void near_window(
         pair_terms32_split<VAR, TIED>(q32, *tile_field(pd.tiles32, k, 0, nf),
                                       *tile_field(pd.tiles32, k, 1, nf),
                                       *tile_field(pd.tiles32, k, 5, nf),
-                                      *tile_field(pd.tiles32, k, 6, nf), b32, t32);
+                                      *tile_field(pd.tiles32, k, 6, nf), b32, k & 2, t32);
       else
         pair_terms32<VAR, TIED>(q32, *tile_field(pd.tiles32, k, 0), *tile_field(pd.tiles32, k, 1),
-                                b32, t32);
+                                b32, k & 2, t32);
       pair_terms64_sc<VAR, TIED>(q64, *tile_field(pd.tiles64, k, 0),
                                  *tile_field(pd.tiles64, k, 1), b64, t64, sincos_ff);
 #pragma unroll

@@ -42,6 +42,7 @@ constexpr int SUB = DBIE_FOLD_PIXELS;  // pixels summed in plain FP32 before a c
 constexpr int SUB1 = 32;  // elements per fold where one accumulator takes every element (adjoints,
                           // the unpacked FP32 form): the per-accumulator length of the packed form
 constexpr int GROUP_UNROLL = DBIE_GROUP_UNROLL;  // 4-pixel groups unrolled within a block
+constexpr int VJP_GROUPS = 8;                    // the same in the adjoint (4 points)
 static_assert(TILE % SUB == 0 && SUB % 4 == 0, "fold blocks must tile the 256-pixel tile");
 // The Hessian pass folds its 30 sums every 128 pixels (64 terms per lane): with ten sums per
 // component the fold is ~8 % of its FP32 work at 64.  (The objective kernels keep SUB: the error
@@ -399,8 +400,8 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
                 accumulate_hess_row<f32x2, TIED, NS>(acc2[u], tm[0], tm[1], b2[0], b2[1], dy2[u]);
               }
             } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            auto pair = [&](auto half) {
+              constexpr int h = decltype(half)::value;
 #pragma unroll
               for (int u = 0; u < P; ++u) {
                 f32x2 dx = vsub(q2[u].x, px2[h]);
@@ -414,10 +415,12 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
                   g = pair_geomv_d<f32x2, TIED>(q2[u], dx, dy);
                 }
                 TermsV<f32x2, VAR, TIED> tm;
-                pair_angularv<f32x2, VAR, TIED>(q2[u], g, b2[h], tm);
+                pair_angularv<f32x2, VAR, TIED, h>(q2[u], g, b2[h], tm);
                 accumulatev<f32x2, VAR, TIED, NS>(acc2[u], tm, b2[h]);
               }
-            }
+            };
+            pair(Half<0>{});
+            pair(Half<1>{});
             }
           }
 #pragma unroll
@@ -462,7 +465,7 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
 #pragma unroll
               for (int u = 0; u < P; ++u) {
                 Terms32<VAR, TIED> tm;
-                pair_angular32<VAR, TIED>(q[u], gm[e][u], b, tm);
+                pair_angular32<VAR, TIED>(q[u], gm[e][u], b, e & 2, tm);
                 accumulate32<VAR, TIED, NS>(acc[u], tm, b);
               }
             }
@@ -484,11 +487,12 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
                 if constexpr (ROWS) {
                   const float dx = SPLIT ? __fsub_rn(__fsub_rn(q[u].x, px[e]), pxl[e])
                                          : __fsub_rn(q[u].x, px[e]);
-                  pair_angular32<VAR, TIED>(q[u], pair_geom32_dz<TIED>(dx, dyg[u], dyzg[u]), b, tm);
+                  pair_angular32<VAR, TIED>(q[u], pair_geom32_dz<TIED>(dx, dyg[u], dyzg[u]), b, e & 2,
+                                            tm);
                 } else if constexpr (SPLIT) {
-                  pair_terms32_split<VAR, TIED>(q[u], px[e], py[e], pxl[e], pyl[e], b, tm);
+                  pair_terms32_split<VAR, TIED>(q[u], px[e], py[e], pxl[e], pyl[e], b, e & 2, tm);
                 } else {
-                  pair_terms32<VAR, TIED>(q[u], px[e], py[e], b, tm);
+                  pair_terms32<VAR, TIED>(q[u], px[e], py[e], b, e & 2, tm);
                 }
                 accumulate32<VAR, TIED, NS>(acc[u], tm, b);
               }
@@ -607,15 +611,27 @@ __device__ __forceinline__ void vjp_body(const VjpArgs& a) {
       pxl[u] = SPLIT ? *tile_field(btiles, k, 5, NF) : Real(0);
       pyl[u] = SPLIT ? *tile_field(btiles, k, 6, NF) : Real(0);
     }
-    Real acc[P][3];
-    float hi[F32 ? P : 1][3];
+    // FP64 form: one accumulator per pixel and component.  FP32 form: two points per f32x2
+    // (adjacent in shared memory), the thread's pixels in both lanes.
+    Real acc[F32 ? 1 : P][3];
+    f32x2 acc2[F32 ? P : 1][3], hi2[F32 ? P : 1][3];
+    f32x2 px2[F32 ? P : 1], py2[F32 ? P : 1], pxl2[F32 ? P : 1], pyl2[F32 ? P : 1];
+    if constexpr (F32) {
 #pragma unroll
-    for (int u = 0; u < P; ++u)
+      for (int u = 0; u < P; ++u) {
+        px2[u] = pack2(px[u], px[u]);
+        py2[u] = pack2(py[u], py[u]);
+        pxl2[u] = pack2(pxl[u], pxl[u]);
+        pyl2[u] = pack2(pyl[u], pyl[u]);
 #pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        acc[u][p] = Real(0);
-        if constexpr (F32) hi[u][p] = 0.f;
+        for (int p = 0; p < 3; ++p) acc2[u][p] = hi2[u][p] = vconst<f32x2>(0.f);
       }
+    } else {
+#pragma unroll
+      for (int u = 0; u < P; ++u)
+#pragma unroll
+        for (int p = 0; p < 3; ++p) acc[u][p] = Real(0);
+    }
 
     sweep_tiles(ring, ptiles, t0, t1, tid, [&](const Real* sx) {
       const Real* X = sx;
@@ -624,45 +640,64 @@ __device__ __forceinline__ void vjp_body(const VjpArgs& a) {
       const Real* L = sx + 3 * TILE;
       const Real* W = sx + 6 * TILE;
       if constexpr (F32) {
-#pragma unroll 1
-        for (int k0 = 0; k0 < TILE; k0 += SUB1) {
-#pragma unroll 4
-          for (int k = k0; k < k0 + SUB1; ++k) {
-            const float xi = X[k], yi = Y[k], z2 = Z2[k];
-            float lam[NL];
+        // the terms of two points (x2 .. w2: pairs of their fields)
+        constexpr int FMA_SC = fma_sincos(VAR_V, TIED, 0);
+        auto two = [&](const float* x2, const float* y2, const float* z22, const float* l2,
+                       const float* w2) {
+          const f32x2 xi = pack2(x2[0], x2[1]), yi = pack2(y2[0], y2[1]);
+          const f32x2 z2 = pack2(z22[0], z22[1]);
 #pragma unroll
-            for (int l = 0; l < NL; ++l) lam[l] = L[l * TILE + k];
-            const float w[3] = {W[k], W[TILE + k], W[2 * TILE + k]};
+          for (int u = 0; u < P; ++u) {
+            f32x2 dx = vsub(px2[u], xi), dy = vsub(py2[u], yi);
+            if constexpr (SPLIT) {
+              dx = vadd(dx, pxl2[u]);
+              dy = vadd(dy, pyl2[u]);
+            }
+            const f32x2 r2 = vfma(dx, dx, vfma(dy, dy, z2));
+            const f32x2 ri = vrsqrt(r2);
+            const f32x2 r = vmul(r2, ri);
+            const f32x2 ri3 = vmul(vmul(ri, ri), ri);
+            f32x2 phi;
 #pragma unroll
-            for (int u = 0; u < P; ++u) {
-              float dx = __fsub_rn(px[u], xi), dy = __fsub_rn(py[u], yi);
-              if constexpr (SPLIT) {
-                dx = __fadd_rn(dx, pxl[u]);
-                dy = __fadd_rn(dy, pyl[u]);
-              }
-              const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, z2));
-              const float ri = rsqrt_mufu(r2);
-              const float r = __fmul_rn(r2, ri);
-              const float ri3 = __fmul_rn(__fmul_rn(ri, ri), ri);
-              if constexpr (TIED) {
-                const float th = __fmul_rn(lam[0], r);
-                const float phi = __fmul_rn(__fmaf_rn(th, sin_mufu(th), cos_mufu(th)), ri3);
-#pragma unroll
-                for (int p = 0; p < 3; ++p) acc[u][p] = __fmaf_rn(phi, w[p], acc[u][p]);
-              } else {
-#pragma unroll
-                for (int p = 0; p < 3; ++p) {
-                  const float th = __fmul_rn(lam[p], r);
-                  const float phi = __fmul_rn(__fmaf_rn(th, sin_mufu(th), cos_mufu(th)), ri3);
-                  acc[u][p] = __fmaf_rn(phi, w[p], acc[u][p]);
+            for (int p = 0; p < 3; ++p) {
+              if (!TIED || p == 0) {
+                const f32x2 th = vmul(pack2(l2[4 * p], l2[4 * p + 1]), r);
+                if (FMA_SC >> p & 1) {
+                  f32x2 k;
+                  const f32x2 f = half_turns(th, k), f2 = vsqr_sat(f);
+                  phi = vmul(vfma(th, sin_half_turns(f, f2), cos_half_turns(f2)), vflip(ri3, k));
+                } else {
+                  phi = vmul(vfma(th, vsin(th), vcos(th)), ri3);
                 }
               }
+              acc2[u][p] = vfma(phi, pack2(w2[4 * p], w2[4 * p + 1]), acc2[u][p]);
             }
+          }
+        };
+#pragma unroll 1
+        for (int k0 = 0; k0 < TILE; k0 += SUB) {
+#pragma unroll VJP_GROUPS
+          for (int k = k0; k < k0 + SUB; k += 4) {
+            // fields of four points, one 128-bit load each
+            float x[4], y[4], z2[4], l[4 * NL], w[12];
+            auto ld = [&](float* d, const Real* s4) {
+              const float4 v = *reinterpret_cast<const float4*>(s4);
+              d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+            };
+            ld(x, X + k);
+            ld(y, Y + k);
+            ld(z2, Z2 + k);
+#pragma unroll
+            for (int p = 0; p < NL; ++p) ld(l + 4 * p, L + p * TILE + k);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) ld(w + 4 * p, W + p * TILE + k);
+            two(x, y, z2, l, w);
+            two(x + 2, y + 2, z2 + 2, l + 2, w + 2);
           }
 #pragma unroll
           for (int u = 0; u < P; ++u)
 #pragma unroll
-            for (int p = 0; p < 3; ++p) fold2(hi[u][p], acc[u][p]);
+            for (int p = 0; p < 3; ++p) fold2(hi2[u][p], acc2[u][p]);
         }
       } else {
 #pragma unroll 2
@@ -693,8 +728,14 @@ __device__ __forceinline__ void vjp_body(const VjpArgs& a) {
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
         double v;
-        if constexpr (F32) v = (double)hi[u][p] + (double)acc[u][p];
-        else v = (double)acc[u][p];
+        if constexpr (F32) {
+          float h0, h1, a0, a1;
+          unpack2(hi2[u][p], h0, h1);
+          unpack2(acc2[u][p], a0, a1);
+          v = ((double)h0 + (double)h1) + ((double)a0 + (double)a1);
+        } else {
+          v = (double)acc[u][p];
+        }
         a.out[((int64_t)it * 3 + p) * Q + (tid + u * NT)] = v;
       }
     }
