@@ -47,19 +47,35 @@ class Options:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the current stream's handle alone: torch.cuda.current_stream() builds a Stream object, 5 us
+    # of the ~33 a call of few points spends on the host
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _dev(x, device, dtype):
+    """x on the device, contiguous, in dtype.  A plain tensor that is so already is returned as it
+    is, without the three no-op calls (2 us)."""
+    if (type(x) is torch.Tensor and x.dtype is dtype and x.is_cuda and x.is_contiguous()
+            and device.type == "cuda" and x.get_device() ==
+            (torch.cuda.current_device() if device.index is None else device.index)):
+        return x
+    return torch.as_tensor(x).to(device=device, dtype=dtype).contiguous()
 
 
 def _dev_f32(x, device):
-    return torch.as_tensor(x).to(device=device, dtype=torch.float32).contiguous()
+    return _dev(x, device, torch.float32)
 
 
 def _dev_f64(x, device):
-    return torch.as_tensor(x).to(device=device, dtype=torch.float64).contiguous()
+    return _dev(x, device, torch.float64)
+
+
+def _rows3(x):
+    return x if x.dim() == 2 and x.shape[1] == 3 else x.reshape(-1, 3)
 
 
 class DBIEField:
@@ -103,8 +119,8 @@ class DBIEField:
         self._keep = comps  # kept alive until the asynchronous staging has run
 
     def eval(self, xyz, lam, grad=False, dlam=False, objective=False, options: Options | None = None):
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f32(lam, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f32(lam, self.device))
         n = xyz.shape[0]
         kw = dict(device=self.device, dtype=torch.float64)
         B = torch.empty((n, 3), **kw)
@@ -124,8 +140,8 @@ class DBIEField:
 
     def objective(self, xyz, lam, options: Options | None = None):
         """f, g, Phi and dPhi/dlambda (n, 3) at fixed lambda."""
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f32(lam, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f32(lam, self.device))
         n = xyz.shape[0]
         F = torch.empty((n, 3), device=self.device, dtype=torch.float64)
         D = torch.empty((n, 3), device=self.device, dtype=torch.float64)
@@ -136,8 +152,8 @@ class DBIEField:
     def eval_difference(self, xyz, lam, lam_ref, tied=False, bound=True):
         """Change of the 12 objective sums between lam_ref and lam (n, 12 float64; per component
         S0, S1, Sx, Sy) and, with bound, the worst-case bound of each entry's error."""
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f64(lam, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f64(lam, self.device))
         lam_ref = _dev_f64(lam_ref, self.device).reshape(-1, 3)
         n = xyz.shape[0]
         dS = torch.empty((n, 12), device=self.device, dtype=torch.float64)
@@ -165,7 +181,7 @@ class DBIEField:
         return r, so
 
     def solve(self, xyz, options: Options | None = None, lambda_init=None, codes: int = 0):
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
         n = xyz.shape[0]
         l0 = None if lambda_init is None else _dev_f64(lambda_init, self.device).reshape(-1, 3)
         r, so = self._solve_out(n, codes)
@@ -174,9 +190,9 @@ class DBIEField:
         return r
 
     def vjp(self, xyz, lam, gB, glam=True, options: Options | None = None, gB0=None):
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f64(lam, self.device).reshape(-1, 3)
-        gB = _dev_f64(gB, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f64(lam, self.device))
+        gB = _rows3(_dev_f64(gB, self.device))
         n = xyz.shape[0]
         acc = gB0 is not None
         if gB0 is None:
@@ -197,8 +213,8 @@ class DBIEField:
     def hessian(self, xyz, lam, options: Options | None = None):
         """Phi (n,), dPhi/dlambda (n, 3) and the lambda-Hessian (n, 3, 3) at fixed lambda (tied
         mode: the derivatives along the shared lambda in entry 0)."""
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f64(lam, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f64(lam, self.device))
         n = xyz.shape[0]
         kw = dict(device=self.device, dtype=torch.float64)
         P, G, H = torch.empty(n, **kw), torch.empty((n, 3), **kw), torch.empty((n, 3, 3), **kw)
@@ -210,9 +226,9 @@ class DBIEField:
         """dL/dB0 (ny, nx, 3) through the lambda search at a stationary lambda (n, 3), plus the
         adjoint vectors v = H^-1 dL/dlambda (n, 3) and flags (n,) (1: H not positive definite,
         only the fixed-lambda term kept).  gB0 given: accumulated into it."""
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f64(lam, self.device).reshape(-1, 3)
-        gB = _dev_f64(gB, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f64(lam, self.device))
+        gB = _rows3(_dev_f64(gB, self.device))
         n = xyz.shape[0]
         acc = gB0 is not None
         if gB0 is None:
@@ -227,8 +243,8 @@ class DBIEField:
     def noise_var(self, xyz, lam, sigma=None, sigma0: float = 1.0, options: Options | None = None):
         """Var B (n, 3) at fixed lambda for independent pixel noise: sigma None (sigma0 on every
         pixel) or three (ny, nx) standard-deviation maps (entries may be None)."""
-        xyz = _dev_f32(xyz, self.device).reshape(-1, 3)
-        lam = _dev_f64(lam, self.device).reshape(-1, 3)
+        xyz = _rows3(_dev_f32(xyz, self.device))
+        lam = _rows3(_dev_f64(lam, self.device))
         n = xyz.shape[0]
         sg = [None, None, None] if sigma is None else [
             None if a is None else _dev_f32(a, self.device).reshape(self.ny, self.nx) for a in sigma]
