@@ -321,26 +321,35 @@ void launch_pack_vjp(int64_t n, const float* xyz, const double* lam, const doubl
   pack_vjp_kernel<<<grid, 256, 0, s>>>(n, xyz, lam, gB, tied, nptiles, p32, p64, fp64);
 }
 
+template <bool WIDE>
 __global__ void finalize_vjp_kernel(int64_t npix, const PlanHdr* __restrict__ plan,
                                     const double* __restrict__ out, double scale, double* gB0,
                                     int accumulate) {
   const PlanHdr h = *plan;
   const int32_t zero = 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < npix;
-       k += (int64_t)gridDim.x * blockDim.x) {
+  __shared__ double sh[WIDE ? 3 * 32 * GATHER_WARPS : 1];
+  const int per = WIDE ? 32 : blockDim.x;
+  for (int64_t k0 = blockIdx.x * (int64_t)per; k0 < npix; k0 += (int64_t)gridDim.x * per) {
+    const int64_t k = k0 + (WIDE ? threadIdx.x & 31 : threadIdx.x);
+    double S[3];
+    if constexpr (WIDE) gather_by_warps<3>(out, h, &zero, k, k < npix, S, sh);
+    if (k >= npix || (WIDE && threadIdx.x >= 32)) continue;
+    if constexpr (!WIDE) gather_sums<3>(out, h, &zero, 0, k, S);
     for (int p = 0; p < 3; ++p) {
-      double v = 0.0;
-      for (int sp = 0; sp < h.nsplit; ++sp) v += out[out_index(h, &zero, 0, k, sp, p, 3)];
-      v *= scale;
+      const double v = S[p] * scale;
       gB0[3 * k + p] = accumulate ? gB0[3 * k + p] + v : v;
     }
   }
 }
 
 void launch_finalize_vjp(int64_t npix, const PlanHdr* plan, const double* out, double scale,
-                         double* gB0, int accumulate, cudaStream_t s) {
+                         double* gB0, int accumulate, int64_t nsplit, cudaStream_t s) {
   const PerPoint L(npix);
-  finalize_vjp_kernel<<<L.grid, L.nt, 0, s>>>(npix, plan, out, scale, gB0, accumulate);
+  if (gather_wide(npix, nsplit))
+    finalize_vjp_kernel<true><<<gather_grid(npix), 32 * GATHER_WARPS, 0, s>>>(npix, plan, out, scale,
+                                                                              gB0, accumulate);
+  else
+    finalize_vjp_kernel<false><<<L.grid, L.nt, 0, s>>>(npix, plan, out, scale, gB0, accumulate);
 }
 
 }  // namespace dbie

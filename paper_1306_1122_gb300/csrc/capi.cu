@@ -165,6 +165,7 @@ struct dbie_ctx {
   double x0 = 0, y0 = 0, hx = 1, hy = 1, dA = 1;
   int64_t npix = 0;
   int32_t ntiles = 0;
+  int64_t pass_splits = 1;   // splits per query of the last pass_single
   int sm_count = 1;
   DBuf t32, t64, tff, prob, err, misc;
   DBuf st_in, st_out, st_aux;     // host-memory staging
@@ -368,6 +369,7 @@ dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float*
   const int grid = persistent_grid(k, c->device);
   const int64_t items = reeval_items(n, grid);
   if (items > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
+  c->pass_splits = items / n;
   const int nsum = 3 * nsum_per_comp(var);
   DBIE_TRY(ensure(c->out, sizeof(double) * items * nsum));
   launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, 0, 1, 1, (int)n, s);
@@ -455,6 +457,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
     a.out = c->out.as<double>();
     a.plan = &m->plan;
     a.strips = c->ntiles * FEW_STRIPS_PER_TILE;
+    c->pass_splits = few_split((int)n, a.strips, grid * (k.nt / 32));
     DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
     if (near_on) {
       na.n = (int32_t)n;
@@ -480,6 +483,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
     nsplit = std::min<int64_t>((target + nblk - 1) / nblk, (int64_t)c->ntiles * (fp64 ? F64_PARTS : 1));
   const int64_t nitems = nblk * nsplit;
   if (nitems > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
+  c->pass_splits = nsplit;
   const int nsum = 3 * nsum_per_comp(var);
   DBIE_TRY(ensure(c->out, sizeof(double) * nitems * nsum * k.qper));
   launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, (int)nitems, (int)nsplit, k.qper,
@@ -941,7 +945,7 @@ dbie_status dbie_eval(dbie_ctx* c, int64_t n, const float* xyz, const float* lam
   Misc* m = c->misc.as<Misc>();
   launch_finalize_eval(var, n, &m->plan, m->item_off, c->out.as<double>(), c->qpos.as<float4>(),
                        c->qlam.as<Lam4>(), o.g_scale, o.w_g, dB, dG, dL, nullptr, dF,
-                       pxe ? c->pxe_corr.as<double>() : nullptr, s);
+                       pxe ? c->pxe_corr.as<double>() : nullptr, c->pass_splits, s);
   CUDA_TRY(cudaGetLastError());
   if (mem_kind == DBIE_MEM_HOST) {
     CUDA_TRY(cudaMemcpyAsync(B, dB, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s));
@@ -1022,7 +1026,7 @@ dbie_status dbie_objective(dbie_ctx* c, int64_t n, const float* xyz, const float
   Misc* m = c->misc.as<Misc>();
   launch_finalize_objective(n, &m->plan, m->item_off, c->out.as<double>(), c->qpos.as<float4>(),
                             c->qlam.as<Lam4>(), o.g_scale, o.w_g, dF, dD, nullptr,
-                            pxe ? c->pxe_corr.as<double>() : nullptr, s);
+                            pxe ? c->pxe_corr.as<double>() : nullptr, c->pass_splits, s);
   CUDA_TRY(cudaGetLastError());
   if (mem_kind == DBIE_MEM_HOST) {
     if (fgphi) CUDA_TRY(cudaMemcpyAsync(fgphi, dF, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s));
@@ -1034,13 +1038,15 @@ dbie_status dbie_objective(dbie_ctx* c, int64_t n, const float* xyz, const float
 
 // Per-quadrature-point adjoint sums (item chunks of 3 sums) -> dL/dB0 per node: scaled by
 // dA / 2 pi at pixel centres, or gathered through the nine-node shape functions.
-static dbie_status finalize_adjoint(dbie_ctx* c, const PlanHdr* plan, double* gB0, int accumulate,
-                                    cudaStream_t s) {
+static dbie_status finalize_adjoint(dbie_ctx* c, const PlanHdr* plan, int64_t nsplit, double* gB0,
+                                    int accumulate, cudaStream_t s) {
   if (c->quad_g == 0) {
-    launch_finalize_vjp(c->npix, plan, c->out.as<double>(), c->dA / TWO_PI, gB0, accumulate, s);
+    launch_finalize_vjp(c->npix, plan, c->out.as<double>(), c->dA / TWO_PI, gB0, accumulate,
+                        nsplit, s);
   } else {
     DBIE_TRY(ensure(c->vtmp, sizeof(double) * 3 * (size_t)c->nquad));
-    launch_finalize_vjp(c->nquad, plan, c->out.as<double>(), 1.0, c->vtmp.as<double>(), 0, s);
+    launch_finalize_vjp(c->nquad, plan, c->out.as<double>(), 1.0, c->vtmp.as<double>(), 0,
+                        nsplit, s);
     launch_q9_gather(c->vtmp.as<double>(), c->nx, c->ny, c->hx, c->hy, c->qi, gB0, accumulate, s);
   }
   CUDA_TRY(cudaGetLastError());
@@ -1134,7 +1140,7 @@ dbie_status dbie_vjp(dbie_ctx* c, int64_t n, const float* xyz, const double* lam
       c->pending.push_back({e0, e1});
       c->pending_pairs.push_back((double)n * (double)nq);
     }
-    DBIE_TRY(finalize_adjoint(c, &m->plan, d_gB0, accumulate ? 1 : 0, s));
+    DBIE_TRY(finalize_adjoint(c, &m->plan, nsplit, d_gB0, accumulate ? 1 : 0, s));
     if (pxe_on(c, o)) {
       DBIE_TRY(ensure(c->pxe_pos, sizeof(float4) * n));
       launch_pack_points(n, d_xyz, 0, c->pxe_pos.as<float4>(), s);
@@ -1145,7 +1151,7 @@ dbie_status dbie_vjp(dbie_ctx* c, int64_t n, const float* xyz, const double* lam
       DBIE_TRY(pass_single(c, VAR_L, fp64, o, n, d_xyz, nullptr, d_lam, s));
       launch_finalize_eval(VAR_L, n, &m->plan, m->item_off, c->out.as<double>(),
                            c->qpos.as<float4>(), c->qlam.as<Lam4>(), o.g_scale, o.w_g, nullptr,
-                           nullptr, d_glam, d_gB, nullptr, nullptr, s);
+                           nullptr, d_glam, d_gB, nullptr, nullptr, c->pass_splits, s);
       CUDA_TRY(cudaGetLastError());
     }
   }
@@ -1332,7 +1338,7 @@ dbie_status dbie_vjp_implicit(dbie_ctx* c, int64_t n, const float* xyz, const do
       c->pending.push_back({e0, e1});
       c->pending_pairs.push_back((double)n * (double)nq);
     }
-    DBIE_TRY(finalize_adjoint(c, &m->plan, d_gB0, accumulate ? 1 : 0, s));
+    DBIE_TRY(finalize_adjoint(c, &m->plan, nsplit, d_gB0, accumulate ? 1 : 0, s));
     if (pxe)
       DBIE_TRY(pxe_adjoint(c, n, c->qpos.as<float4>(), c->pxe_w.as<double>(), true, fp64, o,
                            d_gB0, s));

@@ -158,6 +158,38 @@ __device__ __forceinline__ void gather_sums(const double* __restrict__ out, cons
   }
 }
 
+// The same by the warps of a CTA whose lanes have one query each (`on`: lane has one): warp w adds
+// every W-th split from w on, and the CTA's first warp ends with the sums.  Every thread of the CTA
+// calls it; sh: NSUM * blockDim.x values of shared memory.
+template <int NSUM>
+__device__ __forceinline__ void gather_by_warps(const double* __restrict__ out, const PlanHdr& h,
+                                                const int32_t* item_off, int64_t j, bool on,
+                                                double* S, double* sh) {
+  const int w = threadIdx.x >> 5, W = blockDim.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < NSUM; ++s) S[s] = 0.0;
+  if (on) {
+    const double* p = out + out_index(h, item_off, 0, j, w, 0, NSUM);
+    const int64_t step = (int64_t)NSUM * h.qper;
+    for (int sp = w; sp < h.nsplit; sp += W, p += step * W)
+#pragma unroll
+      for (int s = 0; s < NSUM; ++s) S[s] += p[(int64_t)s * h.qper];
+  }
+  __syncthreads();   // (the last query's sums have been read)
+#pragma unroll
+  for (int s = 0; s < NSUM; ++s) sh[(w * NSUM + s) * 32 + lane] = S[s];
+  __syncthreads();
+  for (int s = w; s < NSUM; s += W) {
+    double v = sh[s * 32 + lane];
+    for (int k = 1; k < W; ++k) v += sh[(k * NSUM + s) * 32 + lane];
+    sh[s * 32 + lane] = v;
+  }
+  __syncthreads();
+  if (w == 0)
+#pragma unroll
+    for (int s = 0; s < NSUM; ++s) S[s] = sh[s * 32 + lane];
+}
+
 // Point tiles for the adjoint: per tile TILE x, y, z^2, lambda_x, lambda_y, lambda_z and the
 // weights w_p = gB_p * z (padding points carry w = 0).
 struct VjpArgs {

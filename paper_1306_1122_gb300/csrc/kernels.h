@@ -38,6 +38,24 @@ struct PerPoint {
   }
 };
 
+// Launch shape of those kernels where a query has many splits, gathered by the eight warps of a CTA
+// (gather_by_warps; otherwise one thread's serial chain of loads and FP64 additions: a call with
+// 4,096 points over 36,864 quadrature points, 76 splits, 466 -> 399 us).  Fewer than eight
+// splits are not worth the exchange, nor are many points, whose threads fill the chip (us per
+// call, thread / warps, at 32 x 32 pixels and at most four splits: field and gradient of 20,000
+// points 100 / 103, 65,536 points 200 / 215; adjoint of 65,536 points, 53 splits, 159 / 120; at 300 x
+// 300 pixels the same of 4,096 points 777 / 712, B of 64 points 48 / 41).  `most`: the points up to
+// which it pays; the objective's gradient, long after its sums are there, runs on one warp in eight
+// (20,000 points over 128 x 128 pixels 897 / 926, 4,096 points over 300 x 300 1,020 / 978).
+constexpr int GATHER_WARPS = 8;
+inline bool gather_wide(int64_t n, int64_t nsplit, int64_t most = 65536) {
+  return nsplit >= GATHER_WARPS && n <= most;
+}
+inline int gather_grid(int64_t n) {
+  const int64_t g = (n + 31) / 32;
+  return (int)(g < 8192 ? g : 8192);
+}
+
 struct KernelRef {
   const void* fn;     // __global__ function
   int nt;             // threads per CTA
@@ -182,7 +200,7 @@ void launch_nearfield(int var, bool tied, const NearArgs& a, int sm_count, cudaS
 void launch_pack_vjp(int64_t n, const float* xyz, const double* lam, const double* gB, int tied,
                      int nptiles, float* p32, double* p64, int fp64, cudaStream_t s);
 void launch_finalize_vjp(int64_t npix, const PlanHdr* plan, const double* out, double scale,
-                         double* gB0, int accumulate, cudaStream_t s);
+                         double* gB0, int accumulate, int64_t nsplit, cudaStream_t s);
 
 // pxe.cu (pixel-exact near field)
 void launch_pxe_corr(bool fp64, const ProbDesc* probs, int64_t n, const float4* pos, double zmax,
@@ -206,11 +224,11 @@ void launch_finalize_eval(int var, int64_t n, const PlanHdr* plan, const int32_t
                           const double* out, const float4* qpos, const Lam4* qlam, double g_scale,
                           double w_g, double* B, double* gradB, double* dBdl,
                           const double* gB_for_glam, double* fgphi, const double* corr,
-                          cudaStream_t s);
+                          int64_t nsplit, cudaStream_t s);
 void launch_finalize_objective(int64_t n, const PlanHdr* plan, const int32_t* item_off,
                                const double* out, const float4* qpos, const Lam4* qlam,
                                double g_scale, double w_g, double* fgphi, double* dphi, double* B,
-                               const double* corr, cudaStream_t s);
+                               const double* corr, int64_t nsplit, cudaStream_t s);
 // second_order.cu
 void launch_finalize_hessian(int64_t n, const PlanHdr* plan, const int32_t* item_off,
                              const double* out, const float4* qpos, const Lam4* qlam, int dim,

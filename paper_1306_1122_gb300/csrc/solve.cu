@@ -17,7 +17,8 @@
 namespace dbie {
 
 // ----------------------------------------------------------------- eval finalize ----
-template <int VAR>
+// WIDE: CTAs of GATHER_WARPS warps, 32 points each; else a thread per point.
+template <int VAR, bool WIDE>
 __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan,
                                      const int32_t* __restrict__ item_off,
                                      const double* __restrict__ out,
@@ -27,13 +28,17 @@ __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan
                                      double* fgphi, const double* corr) {
   constexpr int NS = nsum_per_comp(VAR);
   constexpr int NSUM = 3 * NS;
+  __shared__ double sh[WIDE ? NSUM * 32 * GATHER_WARPS : 1];
   const PlanHdr h = *plan;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  const int per = WIDE ? 32 : blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)per; i0 < n; i0 += (int64_t)gridDim.x * per) {
+    const int64_t i = i0 + (WIDE ? threadIdx.x & 31 : threadIdx.x);
+    double S[NSUM];
+    if constexpr (WIDE) gather_by_warps<NSUM>(out, h, item_off, i, i < n, S, sh);
+    if (i >= n || (WIDE && threadIdx.x >= 32)) continue;
     const float4 pos = qpos[i];
     const double z = (double)pos.z;
-    double S[NSUM];
-    gather_sums<NSUM>(out, h, item_off, 0, i, S);
+    if constexpr (!WIDE) gather_sums<NSUM>(out, h, item_off, 0, i, S);
     double Bv[3], G[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int p = 0; p < 3; ++p) Bv[p] = has_value(VAR) ? z * S[p * NS] : 0.0;
     if constexpr (has_grad(VAR)) {
@@ -75,12 +80,16 @@ __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan
 void launch_finalize_eval(int var, int64_t n, const PlanHdr* plan, const int32_t* item_off,
                           const double* out, const float4* qpos, const Lam4* qlam, double g_scale,
                           double w_g, double* B, double* gradB, double* dBdl, const double* gB,
-                          double* fgphi, const double* corr, cudaStream_t s) {
+                          double* fgphi, const double* corr, int64_t nsplit, cudaStream_t s) {
   if (n <= 0) return;
   const PerPoint L(n);
-#define FIN(V)                                                                                \
-  finalize_eval_kernel<V><<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale, \
-                                                  w_g, B, gradB, dBdl, gB, fgphi, corr)
+#define FIN(V)                                                                                  \
+  if (gather_wide(n, nsplit))                                                                           \
+    finalize_eval_kernel<V, true><<<gather_grid(n), 32 * GATHER_WARPS, 0, s>>>(                 \
+        n, plan, item_off, out, qpos, qlam, g_scale, w_g, B, gradB, dBdl, gB, fgphi, corr);     \
+  else                                                                                          \
+    finalize_eval_kernel<V, false><<<L.grid, L.nt, 0, s>>>(                                     \
+        n, plan, item_off, out, qpos, qlam, g_scale, w_g, B, gradB, dBdl, gB, fgphi, corr)
   switch (var) {
     case VAR_V: FIN(VAR_V); break;
     case VAR_VL: FIN(VAR_VL); break;
@@ -429,6 +438,7 @@ __device__ void objective_grad(const double* S, double z, const double lam[3], d
   }
 }
 
+template <bool WIDE>
 __global__ void finalize_objective_kernel(int64_t n, const PlanHdr* __restrict__ plan,
                                           const int32_t* __restrict__ item_off,
                                           const double* __restrict__ out,
@@ -436,11 +446,15 @@ __global__ void finalize_objective_kernel(int64_t n, const PlanHdr* __restrict__
                                           const Lam4* __restrict__ qlam, double g_scale,
                                           double w_g, double* fgphi, double* dphi, double* B,
                                           const double* corr) {
+  __shared__ double sh[WIDE ? 21 * 32 * GATHER_WARPS : 1];
   const PlanHdr h = *plan;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+  const int per = WIDE ? 32 : blockDim.x;
+  for (int64_t i0 = blockIdx.x * (int64_t)per; i0 < n; i0 += (int64_t)gridDim.x * per) {
+    const int64_t i = i0 + (WIDE ? threadIdx.x & 31 : threadIdx.x);
     double S[21];
-    gather_sums<21>(out, h, item_off, 0, i, S);
+    if constexpr (WIDE) gather_by_warps<21>(out, h, item_off, i, i < n, S, sh);
+    if (i >= n || (WIDE && threadIdx.x >= 32)) continue;
+    if constexpr (!WIDE) gather_sums<21>(out, h, item_off, 0, i, S);
     const Lam4 l = qlam[i];
     const double lam[3] = {l.x, l.y, l.z};
     Eval e;
@@ -461,11 +475,15 @@ __global__ void finalize_objective_kernel(int64_t n, const PlanHdr* __restrict__
 void launch_finalize_objective(int64_t n, const PlanHdr* plan, const int32_t* item_off,
                                const double* out, const float4* qpos, const Lam4* qlam,
                                double g_scale, double w_g, double* fgphi, double* dphi, double* B,
-                               const double* corr, cudaStream_t s) {
+                               const double* corr, int64_t nsplit, cudaStream_t s) {
   if (n <= 0) return;
   const PerPoint L(n);
-  finalize_objective_kernel<<<L.grid, L.nt, 0, s>>>(n, plan, item_off, out, qpos, qlam, g_scale,
-                                                    w_g, fgphi, dphi, B, corr);
+  if (gather_wide(n, nsplit, 8192))
+    finalize_objective_kernel<true><<<gather_grid(n), 32 * GATHER_WARPS, 0, s>>>(
+        n, plan, item_off, out, qpos, qlam, g_scale, w_g, fgphi, dphi, B, corr);
+  else
+    finalize_objective_kernel<false><<<L.grid, L.nt, 0, s>>>(
+        n, plan, item_off, out, qpos, qlam, g_scale, w_g, fgphi, dphi, B, corr);
 }
 
 // ----------------------------------------------------------------------- quasi-Newton ----
