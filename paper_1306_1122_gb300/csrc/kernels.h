@@ -100,7 +100,7 @@ int64_t few_records(int64_t queries, int grid);
 // Strip ranges per query of a pass of nq queries on `warps` warps.  Short passes are one wave
 // (rounded down: an item too many would be a wave of its own); with more than 32 strips for every
 // warp about four items each even out the end, of at least 8 strips, which pay for their
-// combination.  At most 32 ranges: a thread adds them up.
+// combination.  At most 32 ranges: a thread of a step kernel adds them up.
 __host__ __device__ inline int few_split(int nq, int strips, int warps) {
   if (nq <= 0) return 1;
   const bool large = (int64_t)nq * strips > (int64_t)32 * warps;

@@ -969,9 +969,9 @@ __global__ void __launch_bounds__(NT) g1_kernel(const G1Args a) {
   g1_body<Real, VAR, TIED, P, NT, NSTAGE, SPLIT, ROWS>(a);
 }
 template <typename Real, int VAR, bool TIED, int P, int NT, int NSTAGE, int MINB,
-          bool ROWS = false>
+          bool ROWS = false, bool SPLIT = false>
 __global__ void __launch_bounds__(NT, MINB) g1_kernel_mb(const G1Args a) {
-  g1_body<Real, VAR, TIED, P, NT, NSTAGE, false, ROWS>(a);
+  g1_body<Real, VAR, TIED, P, NT, NSTAGE, SPLIT, ROWS>(a);
 }
 template <typename Real, bool TIED, int P, int NT, int NSTAGE, bool SPLIT = false>
 __global__ void __launch_bounds__(NT) vjp_kernel(const VjpArgs a) {

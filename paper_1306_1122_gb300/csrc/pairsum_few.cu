@@ -8,11 +8,12 @@
 // four pixels per lane and load (five or seven 128-bit loads, from L1: the warps of an SM work on
 // neighbouring queries of the same range), the arithmetic is the other kernels' (f32x2 pixel
 // pairs, folded every 64 pixels of a lane), and the lanes' sums are combined in the warp.  The SFU
-// bounds it as it does the dense kernels (7 operations per pair); a warp's combination costs about
+// bounds it as it does the dense kernels (5 or 7 operations per pair); a warp's combination costs about
 // as much issue time as 10 pixels per lane, but no SFU time.
 // Measured, dense kernels and their reduction against this one: B at 64 points over 128 x 128
-// pixels 113 -> 50 us per call (the kernels 107 -> about 15 us), B, gradient and objective at 300
-// points over 129 x 70 pixels 167 -> 112 us; a search of 2,048 points over 32 x 32 pixels 20.7 ->
+// pixels 113 -> 50 us per call (the kernels 107 -> about 15 us; 31 us per call since with a shorter
+// front end and gathering by warps), B, gradient and objective at 300 points over 129 x 70 pixels
+// 167 -> 112 us (81 us since); a search of 2,048 points over 32 x 32 pixels 20.7 ->
 // 11.1 ms.
 #include "few_sums.cuh"
 

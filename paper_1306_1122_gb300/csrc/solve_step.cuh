@@ -200,7 +200,7 @@ __device__ __forceinline__ float mixed_phi_bound(const float* M, const double la
   return propagate_bound(dB, dG, e, g_scale, w_g);
 }
 
-// Error bounds of the difference sums (pairsum_dif.cu) that take a point's float-float
+// Error bounds of the difference sums (re_rows.cuh) that take a point's float-float
 // reference sums at lambda_0 to lambda_a, per component p, with dl = |lambda_a - lambda_0| and
 // L = |lambda_a| + |lambda_0|.  Every product of a pixel's difference terms carries a factor
 // |delta| = dl r / 2 (or dl).  With the operation accuracies of mixed_phi_bound (SFU sine and
