@@ -34,9 +34,10 @@ METRIC = ("point×boundary pair evals/s and solve time at ≤1e-5 rel err vs FP6
 WORKLOAD = "ll128: Low&Lou n=1 m=1 l=0.3 Phi=pi/4, 128x128 boundary, 64x64x32 points (131072)"
 SMS, MUFU_PER_SM_CLK, MAX_SM_MHZ = 152, 16, 2070.0
 MUFU_PER_PAIR = 7           # objective variant, one lambda per component: rsqrt + 3 x (sin, cos)
+VALUE_MUFU_PER_PAIR = 5     # value variant: rsqrt + 2 x (sin, cos), the third pair on the FMA pipe
 FP32_PER_SM_CLK = 124       # measured FP32 FMA-pipe rate per SM and clock (of 128 lanes)
 FF_FP32_PER_PAIR = 727      # float-float objective sums: FP32 operations per point-pixel pair
-DIF_INST_PER_PAIR = 153     # difference sums: thread instructions per pair (ncu, all pipes)
+DIF_INST_PER_PAIR = 183     # difference sums: thread instructions per pair (ncu, all pipes)
 ISSUE_PER_SM_CLK = 128      # thread instructions issued per SM and clock (4 schedulers x 32)
 FP32_PER_PAIR = 44
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one objective launch, the first
@@ -300,7 +301,7 @@ def run_ours(args):
                    "launch_configs": tuned},
         "solve_ms": step_ms,
         "roofline_float_float": {
-            "bound": "alu", "pipe": "FP32 (FMA)", "kernel": "g1_ff_kernel (float-float "
+            "bound": "alu", "pipe": "FP32 (FMA)", "kernel": "reeval_kernel (float-float "
             "re-evaluation of near-tied simplex decisions)",
             "achieved": (stats[-1]["ff_pairs"] * FF_FP32_PER_PAIR /
                          (sum(s["ff_ms"] for s in stats) / args.steps / 1e3) / 1e12)
@@ -309,8 +310,8 @@ def run_ours(args):
             "per_pair": {"fp32": FF_FP32_PER_PAIR, "mufu": 1},
             "peak_source": "152 SMs x 124 FP32 ops/clk/SM (measured per-clock rate) x 2070 MHz"},
         "roofline_difference": {
-            "bound": "alu", "pipe": "instruction issue (FP32 FMA 68 %, MUFU 16 % of it)",
-            "kernel": "g1_dif_kernel (difference sums of near-tied values from a float-float "
+            "bound": "alu", "pipe": "instruction issue",
+            "kernel": "reeval_kernel (difference sums of near-tied values from a float-float "
             "reference)",
             "achieved": (stats[-1]["dif_pairs"] * DIF_INST_PER_PAIR /
                          (sum(s["dif_ms"] for s in stats) / args.steps / 1e3) / 1e12)
@@ -752,7 +753,7 @@ def ar1024_block(dev, sub=20000, oracle_points=48):
     f.set_profiling(False)
     t_fwd, t_bwd = e[0].elapsed_time(e[1]) / 1e3, e[1].elapsed_time(e[2]) / 1e3
     pairs = float(n) * m.npix
-    mufu = st["pair_evals"] * 7 / (st["kernel_ms"] / 1e3) / 1e12 if st["kernel_ms"] else None
+    mufu = st["pair_evals"] * VALUE_MUFU_PER_PAIR / (st["kernel_ms"] / 1e3) / 1e12 if st["kernel_ms"] else None
     peak = SMS * MUFU_PER_SM_CLK * MAX_SM_MHZ * 1e6 / 1e12
     rng = np.random.default_rng(5)
     idx = np.sort(rng.choice(n, sub, replace=False))
