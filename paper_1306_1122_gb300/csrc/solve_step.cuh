@@ -966,6 +966,10 @@ __device__ __forceinline__ void step_points(const SolveArgs& a, int warp, int nw
     SI(a, I_NFEV, g) = nfev;
     };
     if (on) decide();
+    // The lanes of phase 3 read vertices that other lanes have just stored (copy_value), and
+    // overwrite the lambdas of trial records that other lanes have just copied from.  (The votes and
+    // shuffles below order no memory.)
+    __syncwarp();
 
     // ---- phase 3: the trial points, a lane per lambda of a point (seven FP64 instructions a pass)
     const unsigned trials = __ballot_sync(FULL, emit_trial);
