@@ -160,6 +160,7 @@ __device__ __noinline__ void rs_refill(const SolveArgs& a, const ResidentArgs& r
   const int lane = threadIdx.x & 31;
   __syncwarp();
   const int want = points - *a.nxt.act_cnt - *a.nxt.ref_cnt;
+  __syncwarp();   // every lane has read the counts that init_point adds to
   int64_t first = 0;
   if (lane == 0 && want > 0) first = atomicAdd(r.next, want);
   first = __shfl_sync(0xffffffffu, first, 0);

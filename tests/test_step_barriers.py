@@ -27,3 +27,9 @@ def test_values_are_visible_to_the_lanes_that_decide():
     # value lanes store their values; then the point's lane reads them
     src = _between(_code("solve_step.cuh"), "SD(a, D_REFS + s, og) = S[s];", "auto decide")
     assert "__syncwarp();" in src
+
+
+def test_counts_are_read_before_points_are_added():
+    # every lane reads the side's counts; then lanes add points to them
+    src = _between(_code("search.cu"), "const int want =", "init_point<N>(")
+    assert "__syncwarp();" in src
