@@ -139,7 +139,10 @@ constexpr double BND_A0 = 9.5e-7, BND_A1 = 1.06e-6, BND_A2 = 1.1e-7, BND_A3 = 1.
 
 // The bounds are evaluated in FP32: an FP64 warp instruction takes 64 cycles here, the bound
 // took two thirds of a value's time, and a worst case whose coefficients have two or three
-// digits (and M_j, summed from FP32 terms) does not need more.
+// digits (and M_j, summed from FP32 terms) does not need more.  Nor does it need more range: the
+// polynomials are nested, so no power of lambda stands alone and a part underflows only where the
+// pair terms that it bounds (FP32 too) have done so, and a bound that overflows counts as infinite:
+// its value ties with every other and is re-evaluated (radius_of).
 // A double's value in FP32, truncated (FP64 conversions run at the FP64 rate).
 __device__ __forceinline__ float f32_of(double x) {
   const int hi = __double2hiint(x);
@@ -150,10 +153,10 @@ __device__ __forceinline__ float f32_of(double x) {
   if (e >= 255) return __uint_as_float(sg | 0x7f800000u | (e == 1151 ? m : 0u));   // inf, NaN
   return __uint_as_float(sg | (unsigned)e << 23 | m);
 }
-// Norm without overflow or underflow of the squares.
+// Norm without overflow or underflow of the squares (of infinite elements infinite, NaN stays).
 __device__ __forceinline__ float norm3f(float x, float y, float z) {
   const float m = fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)));
-  if (!(m > 0.f)) return m;
+  if (!(m > 0.f && m <= 3.4e38f)) return fabsf(x) + fabsf(y) + fabsf(z);   // 0, infinite or NaN
   const float i = 1.0f / m;
   x *= i;
   y *= i;
@@ -169,7 +172,7 @@ __device__ __forceinline__ float propagate_bound(const float dB[3], const float 
   const float ndJ = norm3f(dG[7] + dG[5], dG[2] + dG[6], dG[3] + dG[1]);
   const float rB = norm3f(dB[0], dB[1], dB[2]) / nB;
   float sf = nJ > 0.f ? ndJ / nJ + rB : 1.0f;
-  if (sf > 1.0f) sf = 1.0f;
+  if (!(sf <= 1.0f)) sf = 1.0f;
   const float sg = f32_of(g_scale) * (dG[0] + dG[4] + dG[8]) / nB + f32_of(e.g) * rB;
   return sf + f32_of(w_g) * sg;
 }
@@ -178,10 +181,11 @@ __device__ __forceinline__ float propagate_bound(const float dB[3], const float 
 __device__ __forceinline__ void mixed_component(const float* m, float L, float& s0, float& s1,
                                                 float& sx) {
   constexpr float A0 = BND_A0, A1 = BND_A1, A2 = BND_A2, A3 = BND_A3, A4 = BND_A4;
-  const float L2 = L * L, L3 = L2 * L;
-  s0 = A0 * m[2] + A1 * L * m[1] + A2 * L2 * m[0];
-  sx = A0 * L2 * m[1] + A2 * L3 * m[0] + 3.0f * (A3 * m[3] + A4 * L * m[2] + A2 * L2 * m[1]);
-  s1 = A0 * L2 * m[2] + A2 * L3 * m[1] + 3.0f * (A3 * m[4] + A4 * L * m[3] + A2 * L2 * m[2]);
+  s0 = A0 * m[2] + L * (A1 * m[1] + A2 * (L * m[0]));
+  sx = L * (L * (A0 * m[1] + A2 * (L * m[0]))) +
+       3.0f * (A3 * m[3] + L * (A4 * m[2] + A2 * (L * m[1])));
+  s1 = L * (L * (A0 * m[2] + A2 * (L * m[1]))) +
+       3.0f * (A3 * m[4] + L * (A4 * m[3] + A2 * (L * m[2])));
 }
 
 __device__ __forceinline__ float mixed_phi_bound(const float* M, const double lam[3], int dim,
@@ -223,12 +227,11 @@ template <typename T>
 __device__ __forceinline__ void dif_component(const T* m, T m0, T dl, T L, T R, T& e0, T& e1, T& ex) {
   constexpr T C00 = DIF_C00, C01 = DIF_C01, C02 = DIF_C02, C10 = DIF_C10, C11 = DIF_C11,
               C12 = DIF_C12, C13 = DIF_C13, FF = DIF_FF;
-  const T L2 = L * L, L3 = L2 * L, R2 = R * R;
-  e0 = dl * (C00 * m[1] + C01 * L * m[0] + C02 * L2 * m0) + FF * (m[2] + R * m[1]);
-  e1 = dl * (C10 * m[3] + C11 * L * m[2] + C12 * L2 * m[1] + C13 * L3 * m[0]) +
-       FF * (T(3) * m[4] + T(3) * R * m[3] + R2 * m[2]);
-  ex = dl * (C10 * m[2] + C11 * L * m[1] + C12 * L2 * m[0] + C13 * L3 * m0) +
-       FF * (T(3) * m[3] + T(3) * R * m[2] + R2 * m[1]);
+  e0 = dl * (C00 * m[1] + L * (C01 * m[0] + C02 * (L * m0))) + FF * (m[2] + R * m[1]);
+  e1 = dl * (C10 * m[3] + L * (C11 * m[2] + L * (C12 * m[1] + C13 * (L * m[0])))) +
+       FF * (T(3) * m[4] + R * (T(3) * m[3] + R * m[2]));
+  ex = dl * (C10 * m[2] + L * (C11 * m[1] + L * (C12 * m[0] + C13 * (L * m0)))) +
+       FF * (T(3) * m[3] + R * (T(3) * m[2] + R * m[1]));
 }
 
 // e[4 p + s]: bounds of S0, S1, Sx, Sy of component p (dl, L, R per free lambda).
@@ -272,10 +275,11 @@ __device__ __forceinline__ bool less_eq(double x, double y) {
   return not_nan(x) && not_nan(y) && order_key(x) <= order_key(y);
 }
 
-// Tie radius of a value: `band` times its bound (never 0, which marks a value without one).
+// Tie radius of a value: `band` times its bound (never 0, which marks a value without one; infinite,
+// a tie with any value, where the bound is not a number because its parts overflowed).
 __device__ __forceinline__ float radius_of(double band, float bound) {
   const float r = f32_of(band) * bound;
-  return r < 1e-37f ? 1e-37f : r;
+  return r != r ? __int_as_float(0x7f800000) : (r < 1e-37f ? 1e-37f : r);
 }
 
 // The first near tie of a step: a comparison whose two values differ by no more than the sum of
