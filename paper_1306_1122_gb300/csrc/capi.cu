@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "dbie.h"
+#include "grid_cache.h"
 #include "kernels.h"
 
 using namespace dbie;
@@ -133,28 +134,19 @@ int device_sm_count(int dev) {
   return n > 0 ? n : 1;
 }
 
-// Persistent grid size of a kernel: resident CTAs per SM times SMs.
-struct GridCache {
-  std::mutex mu;
-  std::vector<std::pair<const void*, int>> entries;
-};
 GridCache g_grids;
 
-int persistent_grid(const KernelRef& k, int dev) {
-  {
-    std::lock_guard<std::mutex> lk(g_grids.mu);
-    for (auto& e : g_grids.entries)
-      if (e.first == k.fn) return e.second;
-  }
+// Persistent grid size of a kernel on device dev (the current one): resident CTAs per SM times SMs.
+dbie_status persistent_grid(const KernelRef& k, int dev, int* grid) {
+  *grid = g_grids.find(k.fn, dev);
+  if (*grid > 0) return DBIE_OK;
   if (k.smem > 48 * 1024)
-    cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    CUDA_TRY(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.nt, k.smem);
-  if (per_sm < 1) per_sm = 1;
-  const int g = per_sm * device_sm_count(dev);
-  std::lock_guard<std::mutex> lk(g_grids.mu);
-  g_grids.entries.push_back({k.fn, g});
-  return g;
+  CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.nt, k.smem));
+  *grid = std::max(per_sm, 1) * device_sm_count(dev);
+  g_grids.put(k.fn, dev, *grid);
+  return DBIE_OK;
 }
 
 }  // namespace
@@ -366,7 +358,8 @@ dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float*
   launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(), nullptr,
                    nullptr, 0, 0.0, s);
   const KernelRef k = reeval_ref(var, tied, dif);
-  const int grid = persistent_grid(k, c->device);
+  int grid = 0;
+  DBIE_TRY(persistent_grid(k, c->device, &grid));
   const int64_t items = reeval_items(n, grid);
   if (items > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
   c->pass_splits = items / n;
@@ -441,7 +434,8 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   na.sctab = c->misc.as<Misc>()->sctab;
   if (use_few(var, tied, fp64, n, (double)c->nquad, false) && !fault) {
     const KernelRef k = few_ref(var, tied, c->quad_g != 0);
-    const int grid = persistent_grid(k, c->device);
+    int grid = 0;
+    DBIE_TRY(persistent_grid(k, c->device, &grid));
     const int nsum = 3 * nsum_per_comp(var);
     DBIE_TRY(ensure(c->out, sizeof(double) * few_records(n, grid) * nsum));
     FewArgs a{};
@@ -475,7 +469,8 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(),
                    c->near_list.as<int32_t>(), &m->near_cnt, near_on ? 1 : 0, o.near_z, s);
   const KernelRef k = g1_ref(c, var, tied, fp64);
-  const int grid = persistent_grid(k, c->device);
+  int grid = 0;
+  DBIE_TRY(persistent_grid(k, c->device, &grid));
   const int64_t nblk = (n + k.qper - 1) / k.qper;
   // (element objective sums: two even items per CTA, since four make a few thousand points' items of
   // one tile or two: 4,096 points over 36,864 Gauss points 361 -> 340 us, 16,000 over 49,600 833 ->
@@ -1115,7 +1110,8 @@ dbie_status dbie_vjp(dbie_ctx* c, int64_t n, const float* xyz, const double* lam
                     c->ptiles.as<double>(), fp64 ? 1 : 0, s);
     const KernelRef k = (!fp64 && c->quad_g != 0) ? vjp_ref_split(false)
                                                    : vjp_ref(fp64, false, c->vjp_cfg);
-    const int grid = persistent_grid(k, c->device);
+    int grid = 0;
+    DBIE_TRY(persistent_grid(k, c->device, &grid));
     const int64_t nq = c->nquad;   // quadrature points (pixels, or element Gauss points)
     const int64_t nblk = (nq + k.qper - 1) / k.qper;
     // eight items per CTA: 32,768 points x 16,384 pixels 807 -> 768 us against two
@@ -1313,7 +1309,8 @@ dbie_status dbie_vjp_implicit(dbie_ctx* c, int64_t n, const float* xyz, const do
                             pxe ? c->pxe_w.as<double>() : nullptr, s);
     CUDA_TRY(cudaGetLastError());
     const KernelRef k = (!fp64 && c->quad_g != 0) ? vjp7_ref_split(tied) : vjp7_ref(fp64, tied);
-    const int grid = persistent_grid(k, c->device);
+    int grid = 0;
+    DBIE_TRY(persistent_grid(k, c->device, &grid));
     const int64_t nq = c->nquad;   // quadrature points (pixels, or element Gauss points)
     const int64_t nblk = (nq + k.qper - 1) / k.qper;
     const int64_t target = 2LL * grid;
@@ -1465,7 +1462,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   bool rows_all = true;   // one kernel for all problems: rows only if every grid allows it
   for (int p = 0; p < nprob; ++p) rows_all &= ctxs[p]->qnx % 4 == 0;
   const KernelRef k = g1_ref(c, var, tied, fp64, rows_all ? 1 : 0);
-  const int grid = persistent_grid(k, c->device);
+  int grid = 0;
+  DBIE_TRY(persistent_grid(k, c->device, &grid));
   // Split a round's queries over tile ranges until the items cover this many CTAs (percent of
   // the persistent grid): more items balance the queue, fewer items mean fewer partial sums.
   const int target = (int)((int64_t)grid * split_pct(var) / 100);
@@ -1475,8 +1473,11 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   const bool dif_on = cert && o.certify_ref > 0;
   const KernelRef kr = reeval_ref(VAR_OBJ, tied, dif_on);
   const KernelRef kv = reeval_ref(VAR_V, tied, false);   // certified B
-  const int grid_re = cert ? persistent_grid(kr, c->device) : 0;
-  const int grid_v = cert ? persistent_grid(kv, c->device) : 0;
+  int grid_re = 0, grid_v = 0;
+  if (cert) {
+    DBIE_TRY(persistent_grid(kr, c->device, &grid_re));
+    DBIE_TRY(persistent_grid(kv, c->device, &grid_v));
+  }
   int max_rows = 0;
   for (int p = 0; p < nprob; ++p)
     max_rows = std::max(max_rows, ctxs[p]->ntiles * RE_ROWS_PER_TILE);
@@ -1494,7 +1495,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   // or the whole search in one kernel (no launches to time while profiling)
   const bool resident = few && !qn && !c->profiling && use_resident(N, max_rows);
   const KernelRef kw = few_ref(var, tied, c->quad_g != 0);
-  const int grid_few = few && !resident ? persistent_grid(kw, c->device) : 0;
+  int grid_few = 0;
+  if (few && !resident) DBIE_TRY(persistent_grid(kw, c->device, &grid_few));
   if (!resident)
     DBIE_TRY(ensure(b.out, sizeof(double) * nsum *
                                (few ? few_records(Qcap, grid_few) : items_cap * k.qper)));
@@ -1694,7 +1696,9 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   const int apply_grid = (int)std::min<int64_t>((N + 127) / 128, 8LL * c->sm_count);
   if (resident) {
     const KernelRef ks = search_ref(tied, c->quad_g != 0);
-    const int grid_s = (int)std::min<int64_t>(N, persistent_grid(ks, c->device));
+    int grid_s = 0;
+    DBIE_TRY(persistent_grid(ks, c->device, &grid_s));
+    grid_s = (int)std::min<int64_t>(N, grid_s);
     ResidentArgs ra{};
     ra.a = sa[0];
     ra.lam_init = any_init ? b.lam0.as<double>() : nullptr;
