@@ -130,7 +130,9 @@ typedef struct {
   int32_t reserved0;
 } dbie_solve_out;
 
-/* Timing of the pair-sum kernels recorded while profiling is on (see dbie_set_profiling). */
+/* Timing of the pair-sum kernels recorded while profiling is on (see dbie_set_profiling).  A search
+ * of few points over few pixels is one launch that does everything: its time counts as objective_ms
+ * (and kernel_ms), and refine_ms and dif_ms get nothing from it. */
 typedef struct {
   int64_t launches;        /* pair-sum kernel launches timed */
   double kernel_ms;        /* summed CUDA-event time of those launches */

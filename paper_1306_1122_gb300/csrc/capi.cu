@@ -1492,8 +1492,8 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   DBIE_TRY(ensure(b.ctrl, sizeof(SolveCtrl)));
   // passes of few queries: the lanes of a warp take pixels, all problems share one queue
   const bool few = use_few(var, tied, fp64, N, (double)max_rows * (TILE / RE_ROWS_PER_TILE), true);
-  // or the whole search in one kernel (no launches to time while profiling)
-  const bool resident = few && !qn && !c->profiling && use_resident(N, max_rows);
+  // or the whole search in one kernel
+  const bool resident = few && !qn && use_resident(N, max_rows);
   const KernelRef kw = few_ref(var, tied, c->quad_g != 0);
   int grid_few = 0;
   if (few && !resident) DBIE_TRY(persistent_grid(kw, c->device, &grid_few));
@@ -1712,8 +1712,12 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
     ra.stat_pairs = &ctrl->stat_pairs;
     ra.stat_ff_pairs = &ctrl->stat_ff_pairs;
     ra.stat_dif_pairs = &ctrl->stat_dif_pairs;
-    DBIE_TRY(launch_kernel(ks, grid_s, &ra, s));
+    resolve_pending(c);   // (calls before this one)
+    const double before = c->stats.kernel_ms;
+    DBIE_TRY(timed_launch(c, ks, grid_s, &ra, 0.0, s));   // (its pairs are counted on the device)
     DBIE_TRY(check_device_error(c, s));
+    resolve_pending(c);
+    c->stats.objective_ms += c->stats.kernel_ms - before;
   } else {
   // Initial simplex and its queries go to side 0.
   SolveArgs a0 = sa[1];  // "next" of the side-1 round is side 0
