@@ -407,13 +407,23 @@ bool use_few(int var, bool tied, bool fp64, int64_t n, double npix, bool search)
 }
 
 // Whether a search of few points runs whole in one kernel (search.cu) instead of rounds by
-// launches: few points on few strips of 128 pixels, so that a CTA's share of a round is short.
+// launches: few points on few strips of 128 pixels, so that a CTA's share of a round is short.  A
+// CTA sweeps the whole boundary for each of its points, where launches spread one query over the
+// chip, so strips are limited by themselves however few the points.
 // Measured (ms, launches / one kernel; 10 iterations, then to convergence): 50 points over 32 x 32
 // pixels 1.39 / 0.97, 6.1 / 3.5; 200 there 1.71 / 0.99, 6.7 / 3.7; 1,000 there 1.98 / 1.28, 8.5 / 7.2;
-// 200 over 64 x 64 1.66 / 1.10, 7.5 / 5.2; 50 over 128 x 128 1.39 / 1.17, 7.1 / 5.5; but 2,000 over
-// 32 x 32 2.08 / 1.64, 9.1 / 10.3, 1,000 over 64 x 64 2.39 / 2.33, 8.8 / 8.2, 200 over 128 x 128
-// 2.30 / 3.07, 8.1 / 6.3 and 200 over 256 x 200 3.4 / 8.0, 11.4 / 13.3.
-bool use_resident(int64_t N, int strips) { return N <= 1200 && N * strips <= 10000; }
+// 200 over 64 x 64 1.66 / 1.10, 7.5 / 5.2; but 2,000 over 32 x 32 2.08 / 1.64, 9.1 / 10.3, 1,000 over
+// 64 x 64 2.39 / 2.33, 8.8 / 8.2 and 200 over 128 x 128 2.30 / 3.07, 8.1 / 6.3.  By strips, at 1, 4, 16
+// and 64 points:
+//   128 x  64   0.91 / 0.80, 3.6 / 3.1   1.01 / 0.84, 4.4 / 3.3   1.14 / 0.96, 6.2 / 4.0   1.21 / 0.97, 7.0 / 3.9
+//   128 x 128   0.89 / 0.81, 3.9 / 4.0   0.98 / 0.89, 4.0 / 3.7   1.18 / 1.15, 6.2 / 4.8   1.43 / 1.26, 7.4 / 4.9
+//   192 x 192   0.97 / 1.09, 4.0 / 4.5   1.02 / 1.12, 4.6 / 5.7   1.10 / 1.27, 5.2 / 5.9   1.44 / 1.70, 6.9 / 7.9
+//   256 x 256   1.05 / 1.31, 4.4 / 5.8   1.12 / 1.42, 5.2 / 6.9   2.15 / 8.34, 7.1 / 13    1.80 / 3.27, 8.0 / 10
+//   512 x 256   1.16 / 1.94, 3.4 / 18    1.38 / 2.89, 6.4 / 17    1.92 / 4.58, 8.6 / 28    2.47 / 10.1, 11 / 24
+//  1024 x 512   2.70 / 15.8, 5.6 / 44    3.77 / 19.8, 15 / 104    4.71 / 35.6, 17 / 63     8.49 / 67.1, 27 / 101
+bool use_resident(int64_t N, int strips) {
+  return N <= 1200 && strips <= 128 && N * strips <= 10000;
+}
 
 // One pair-sum pass over n queries of this context (single problem): pack, plan, sweep,
 // near-field correction.  Results are in c->out as item chunks described by c->misc.

@@ -107,3 +107,21 @@ def test_field_without_certification(dbie, n):
         w = P[:, 2:] / d ** 3 * (mag.dA / (2 * np.pi))
         err = w * (1.5e-6 * (1 + th) + 4e-7 * th ** 2) @ abs(b)
         assert (abs(r["B"][:, p].cpu().numpy() - w * (th * np.sin(th) + np.cos(th)) @ b) <= err).all()
+
+
+@pytest.mark.parametrize("nx,ny,n,route", [(128, 128, 4, one), (129, 128, 1, many), (150, 131, 3, many),
+                                           (256, 256, 2, many)])
+def test_few_points_over_many_pixels(dbie, nx, ny, n, route):
+    """Past 128 strips of 128 pixels even one point's search goes by launches; the decisions are the
+    FP64 form's, and B is certified to 1e-5."""
+    mag = random_mag(nx, ny, 770 + nx)
+    xyz, _ = random_points(mag, n, 771, zlo=0.5, zhi=12.0)
+    f = dbie.DBIEField.from_magnetogram(mag)
+    X = torch.from_numpy(xyz).cuda()
+    r = profiled(f, lambda: f.solve(X, dbie.Options(max_iter=12), codes=12), route)
+    d = f.solve(X, dbie.Options(max_iter=12, precision=1), codes=12)
+    f.close()
+    for k in ("iters", "nfev", "status", "codes"):
+        assert torch.equal(r[k], d[k]), k
+    assert torch.allclose(r["lam"], d["lam"], rtol=1e-9, atol=1e-12)
+    assert ((r["B"] - d["B"]).norm(dim=1) <= 1e-5 * d["B"].norm(dim=1)).all()
