@@ -255,13 +255,6 @@ __device__ bool chol3(int m, const double* H, const double* r, double* v) {
   return true;
 }
 
-__device__ __forceinline__ double gsum(const double* out, const PlanHdr& h,
-                                       const int32_t* item_off, int64_t j, int nsum, int s) {
-  double v = 0.0;
-  for (int sp = 0; sp < h.nsplit; ++sp) v += out[out_index(h, item_off, 0, j, sp, s, nsum)];
-  return v;
-}
-
 __global__ void finalize_hessian_kernel(int64_t n, const PlanHdr* __restrict__ plan,
                                         const int32_t* __restrict__ item_off,
                                         const double* __restrict__ out,
@@ -274,7 +267,7 @@ __global__ void finalize_hessian_kernel(int64_t n, const PlanHdr* __restrict__ p
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     double S[NSUM];
-    for (int s = 0; s < NSUM; ++s) S[s] = gsum(out, h, item_off, i, NSUM, s);
+    gather_sums<NSUM>(out, h, item_off, 0, i, S);
     const Lam4 l = qlam[i];
     // one shared lambda: lambda_x for every component, as the tied pair-sum pass used
     const double lam[3] = {l.x, dim == 1 ? l.x : l.y, dim == 1 ? l.x : l.z};
@@ -323,7 +316,7 @@ __global__ void implicit_weights_kernel(int64_t n, int nptiles, const PlanHdr* _
       lam[1] = dim == 1 ? l.x : l.y;
       lam[2] = dim == 1 ? l.x : l.z;
       double S[NSUM];
-      for (int s = 0; s < NSUM; ++s) S[s] = gsum(out, h, item_off, i, NSUM, s);
+      gather_sums<NSUM>(out, h, item_off, 0, i, S);
       double q[12], d1[12], d2[12], phi = 0.0, grad[3], H[9];
       q_derivs(S, z, lam, q, d1, d2);
       if (corr)
@@ -398,7 +391,9 @@ __global__ void finalize_nv_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double z = (double)qpos[i].z;
-    for (int p = 0; p < 3; ++p) var[3 * i + p] = z * z * gsum(out, h, item_off, i, 3, p);
+    double S[3];
+    gather_sums<3>(out, h, item_off, 0, i, S);
+    for (int p = 0; p < 3; ++p) var[3 * i + p] = z * z * S[p];
   }
 }
 
