@@ -517,15 +517,20 @@ __device__ __forceinline__ void g1_body(const G1Args& a) {
         }
       } else {
         const int k1 = kt + kleft < TILE ? kt + kleft : TILE;
+        // (quarters of constant length: the loop over a variable range of pixels cost the Hessian sums
+        // 13 %, 6,000 points over 64 x 64 pixels 7.51 -> 6.59 ms)
+#pragma unroll 1
+        for (int kq = kt; kq < k1; kq += TILE / PARTS) {
 #pragma unroll 2
-        for (int k = kt; k < k1; ++k) {
-          const double b[3] = {sx[2 * TILE + k], sx[3 * TILE + k], sx[4 * TILE + k]};
-          const double px = sx[k], py = sx[TILE + k];
+          for (int k = kq; k < kq + TILE / PARTS; ++k) {
+            const double b[3] = {sx[2 * TILE + k], sx[3 * TILE + k], sx[4 * TILE + k]};
+            const double px = sx[k], py = sx[TILE + k];
 #pragma unroll
-          for (int u = 0; u < P; ++u) {
-            Terms64<VAR, TIED> tm;
-            pair_terms64<VAR, TIED>(q[u], px, py, b, tm);
-            accumulate64<VAR, TIED, NS>(acc[u], tm);
+            for (int u = 0; u < P; ++u) {
+              Terms64<VAR, TIED> tm;
+              pair_terms64<VAR, TIED>(q[u], px, py, b, tm);
+              accumulate64<VAR, TIED, NS>(acc[u], tm);
+            }
           }
         }
         kleft -= k1 - kt;
