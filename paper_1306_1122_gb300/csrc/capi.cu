@@ -330,7 +330,11 @@ dbie_status timed_launch(dbie_ctx* c, const KernelRef& k, int grid, void* args, 
 // grid.  Four items per CTA even out the last wave (items of two per CTA ended in a third wave a few
 // per cent full): B at 20,000 points over 300 x 300 pixels 2.93 -> 2.82 ms, with gradient 3.48 -> 3.27,
 // 15,000 points over 257 x 200 pixels 1.32 -> 1.26.
-int split_pct(int var) { return var == VAR_HESS || var == VAR_NV ? 200 : DBIE_SPLIT_TARGET_PCT; }
+// Not for the tied gradient sums of the quasi-Newton search, whose step reads 21 sums of every split:
+// 100,000 points over 128 x 128 pixels 21.4 ms at four, 18.5 at two, 50,000 over 64 x 48 6.7 and 5.9.
+int split_pct(int var, bool tied) {
+  return var == VAR_HESS || var == VAR_NV || (var == VAR_OBJN && tied) ? 200 : DBIE_SPLIT_TARGET_PCT;
+}
 
 int var_of(bool grad, bool dlam) {
   return grad ? (dlam ? VAR_OBJL : VAR_OBJ) : (dlam ? VAR_VL : VAR_V);
@@ -486,7 +490,7 @@ dbie_status pass_single(dbie_ctx* c, int var, bool fp64, const dbie_options& o, 
   // one tile or two: 4,096 points over 36,864 Gauss points 361 -> 340 us, 16,000 over 49,600 833 ->
   // 799)
   const bool even = c->quad_g != 0 && var == VAR_OBJ && !fp64;
-  const int64_t target = std::max<int64_t>(1, (int64_t)grid * (even ? 200 : split_pct(var)) / 100);
+  const int64_t target = std::max<int64_t>(1, (int64_t)grid * (even ? 200 : split_pct(var, tied)) / 100);
   int64_t nsplit = 1;
   if (nblk < target) {
     const int64_t units = (int64_t)c->ntiles * (fp64 ? F64_PARTS : 1);
@@ -1485,7 +1489,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   DBIE_TRY(persistent_grid(k, c->device, &grid));
   // Split a round's queries over tile ranges until the items cover this many CTAs (percent of
   // the persistent grid): more items balance the queue, fewer items mean fewer partial sums.
-  const int target = (int)((int64_t)grid * split_pct(var) / 100);
+  const int target = (int)((int64_t)grid * split_pct(var, tied) / 100);
   const int64_t items_cap = std::max<int64_t>((Qcap + k.qper - 1) / k.qper + nprob, 2LL * target) + 1;
   // re-evaluation pass (at most 2 float-float and 2 difference queries per point and round); the
   // difference level re-evaluates values near the point's float-float reference
