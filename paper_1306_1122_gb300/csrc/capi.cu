@@ -348,9 +348,30 @@ KernelRef g1_ref(dbie_ctx* c, int var, bool tied, bool fp64, int rows = -1) {
   return g1_ref_f32(var, tied, c->cfg[cfg_var(var)][tied ? 1 : 0], r);
 }
 
+// Fault injection for tests of the bounded waits: the CTA that takes work item 0 never issues its
+// tile copies, its waits expire after their time limit and the call reports DBIE_ETIMEOUT.  (Of
+// the dense kernels: the others wait for nothing.)
+int fault_injection() {
+  const char* fi = std::getenv("DBIE_FAULT_INJECT");
+  return fi && std::atoi(fi) == 1 ? 1 : 0;
+}
+
+// Whether the accurate sums of a call take one query per thread (re_points_kernel) instead of one per
+// CTA and pixel range: where the threads fill the chip, which needs blocks of 128 queries enough, and
+// the other form's items are short.  Measured (ms, the other form / this one), differences: 6,000
+// points over 16 x 16 pixels 0.060 / 0.081, over 128 x 128 0.60 / 0.55; 12,000 there 0.089 / 0.081 and
+// 1.14 / 1.03, over 300 x 257 5.10 / 4.93; 50,000 there 20.7 / 20.6; of one tied lambda 6,000 points
+// 0.053 / 0.052, 0.41 / 0.32 and 1.77 / 1.34.  Float-float terms are five times as long, so only the
+// smallest boundaries gain: B over 16 x 16 pixels, 100,000 points 0.59 / 0.65, 200,000 1.15 / 0.99, over
+// 33 x 20 200,000 2.97 / 3.03, 400,000 5.91 / 5.47, over 64 x 48 200,000 11.2 / 10.9 but with gradient
+// 14.7 / 15.6.
+bool reeval_points(bool dif, bool tied, int64_t n, int ntiles) {
+  if (dif) return n >= (tied ? 6000 : 12000);
+  return ntiles <= 4 && n >= (ntiles == 1 ? 150000 : 300000);
+}
+
 // Float-float sums of n queries of this context, or with lam_ref (float64, as lam) the
-// difference sums between the two lambdas.  Results are in c->out, described by c->misc, as a
-// pass of one query per item.
+// difference sums between the two lambdas.  Results are in c->out, described by c->misc.
 dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float* d_xyz,
                         const float* d_lamf, const double* d_lamd, const double* lam_ref,
                         cudaStream_t s) {
@@ -361,13 +382,42 @@ dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float*
                      nullptr, nullptr, 0, 0.0, s);
   launch_pack_eval(n, d_xyz, d_lamf, d_lamd, c->qpos.as<float4>(), c->qlam.as<Lam4>(), nullptr,
                    nullptr, 0, 0.0, s);
-  const KernelRef k = reeval_ref(var, tied, dif);
+  const int nsum = 3 * nsum_per_comp(var);
+  KernelRef k = reeval_ref(var, tied, dif);
   int grid = 0;
   DBIE_TRY(persistent_grid(k, c->device, &grid));
   const int64_t items = reeval_items(n, grid);
-  if (items > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
+  if (reeval_points(dif, tied, n, c->ntiles) || items > INT32_MAX / 2) {
+    k = re_points_ref(var, tied, dif);
+    DBIE_TRY(persistent_grid(k, c->device, &grid));
+    const int64_t nblk = (n + k.qper - 1) / k.qper;
+    const int64_t target = 2LL * grid;
+    int64_t nsplit = 1;
+    if (nblk < target) nsplit = std::min<int64_t>((target + nblk - 1) / nblk, c->ntiles);
+    const int64_t nitems = nblk * nsplit;
+    if (nitems > INT32_MAX / 2) return fail(DBIE_EINVAL, "too many points for one call");
+    c->pass_splits = nsplit;
+    DBIE_TRY(ensure(c->out, sizeof(double) * nitems * nsum * k.qper));
+    launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, (int)nitems, (int)nsplit, k.qper,
+                       (int)n, s);
+    RePointsArgs a{};
+    a.g.probs = c->prob.as<ProbDesc>();
+    a.g.nprob = 1;
+    a.g.plan = &m->plan;
+    a.g.item_off = m->item_off;
+    a.g.q_cnt = m->q_cnt;
+    a.g.work = &m->work;
+    a.g.qpos = c->qpos.as<float4>();
+    a.g.qlam = c->qlam.as<Lam4>();
+    a.g.out = c->out.as<double>();
+    a.g.err = c->err.as<unsigned>();
+    a.qlam0 = dif ? c->qlam0.as<Lam4>() : nullptr;
+    a.sctab = m->sctab;
+    DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
+    CUDA_TRY(cudaGetLastError());
+    return DBIE_OK;
+  }
   c->pass_splits = items / n;
-  const int nsum = 3 * nsum_per_comp(var);
   DBIE_TRY(ensure(c->out, sizeof(double) * items * nsum));
   launch_plan_single(&m->plan, m->item_off, m->q_cnt, &m->work, 0, 1, 1, (int)n, s);
   CUDA_TRY(cudaMemsetAsync(&m->zero, 0, sizeof(int32_t), s));
@@ -381,19 +431,11 @@ dbie_status pass_reeval(dbie_ctx* c, int var, bool tied, int64_t n, const float*
   a.f = dif ? none : list;
   a.d = dif ? list : none;
   a.work = &m->work;
-  a.sctab = c->misc.as<Misc>()->sctab;
+  a.sctab = m->sctab;
   a.rows = c->ntiles * RE_ROWS_PER_TILE;
   DBIE_TRY(timed_launch(c, k, grid, &a, (double)n * (double)c->nquad, s));
   CUDA_TRY(cudaGetLastError());
   return DBIE_OK;
-}
-
-// Fault injection for tests of the bounded waits: the CTA that takes work item 0 never issues its
-// tile copies, its waits expire after their time limit and the call reports DBIE_ETIMEOUT.  (Of
-// the dense kernels: the others wait for nothing.)
-int fault_injection() {
-  const char* fi = std::getenv("DBIE_FAULT_INJECT");
-  return fi && std::atoi(fi) == 1 ? 1 : 0;
 }
 
 // Whether a pass runs on the kernel for few queries (pairsum_few.cu): the forms it has, and n
@@ -1007,7 +1049,7 @@ dbie_status dbie_eval_difference(dbie_ctx* c, int64_t n, const float* xyz,
     msc = c->dmsc.as<double>();
     launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n, c->sm_count, s);
   }
-  launch_dif_debug(n, &m->plan, c->out.as<double>(), c->qlam.as<Lam4>(),
+  launch_dif_debug(n, &m->plan, m->item_off, c->out.as<double>(), c->qlam.as<Lam4>(),
                    c->qlam0.as<Lam4>(), msc, msc ? msc + 15 * n : nullptr, tied ? 1 : 3, dS,
                    dS_bound, s);
   CUDA_TRY(cudaGetLastError());

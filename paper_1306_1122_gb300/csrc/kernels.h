@@ -149,6 +149,13 @@ struct ReArgs {
 constexpr int RE_ROWS_PER_TILE = TILE / 128;
 constexpr int SINCOS_TABLE = 52;   // ff::SC_TABLE
 KernelRef reeval_ref(int var, bool tied, bool dif);
+// The same of one problem's queries, one per thread (plan, item_off and out as a dense pass).
+struct RePointsArgs {
+  G1Args g;
+  const Lam4* qlam0;        // [slot] reference lambda (differences)
+  const float4* sctab;
+};
+KernelRef re_points_ref(int var, bool tied, bool dif);
 // items that a launch of `grid` CTAs writes at most for up to this many queries
 int64_t reeval_items(int64_t queries, int grid);
 void launch_stage_ff(const double* t64, int ntiles, float* tff, cudaStream_t s);
@@ -257,8 +264,8 @@ void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, float* msc
                 int sm_count, cudaStream_t s);
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
                 int sm_count, cudaStream_t s);
-void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const Lam4* qlam,
-                      const Lam4* qlam0, const double* msc, const double* msc0,
+void launch_dif_debug(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
+                      const Lam4* qlam, const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s);
 void launch_certb_flag(const SolveArgs& a, double rel, int grid, cudaStream_t s);
 void launch_certb_apply(const SolveArgs& a, int grid, cudaStream_t s);

@@ -43,6 +43,7 @@
 // per 153 or more instructions, which plain coalesced loads through L1 sustain; nothing is staged.
 #include <type_traits>
 
+#include "pairsum.cuh"
 #include "re_rows.cuh"
 #include "warp_sums.cuh"
 
@@ -194,6 +195,123 @@ __global__ void __launch_bounds__(RE_NT) reeval_kernel(const ReArgs a) {
     if (pf && a.stat_ff_pairs) atomicAdd(a.stat_ff_pairs, (double)pf);
     if (DIF && pd_ && a.stat_dif_pairs) atomicAdd(a.stat_dif_pairs, (double)pd_);
   }
+}
+
+// The same sums with one query per thread, for calls of many queries on few pixels (reeval_dense in
+// capi.cu): where an item above is a few rows, its set-up and the combination of its threads' sums
+// outweigh the terms.  Items are blocks of 128 queries and a tile range, tiles come through the ring of
+// pairsum.cuh, read by all threads at once.  FP32 issue bounds it as it does the other form.
+// Measured, an item per query and pixel range / this form (ms): differences of 300,000 points over
+// 33 x 20 pixels 2.14 / 1.12, 100,000 over 128 x 128 9.0 / 7.7 (tied 6.1 / 4.1), 30,000 over 300 x 257
+// 12.5 / 11.9; float-float B of 400,000 points over 16 x 16 pixels 2.27 / 1.85.
+template <int VAR, bool TIED, bool DIF>
+__global__ void __launch_bounds__(RE_NT) re_points_kernel(const RePointsArgs a) {
+  constexpr int NSUM = 3 * nsum_per_comp(VAR);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[NSTAGE];
+  __shared__ __align__(8) uint64_t empty_bar[NSTAGE];
+  __shared__ int s_item;
+  __shared__ volatile int s_abort;
+  __shared__ float4 s_tab[ff::SC_TABLE];
+  const int tid = threadIdx.x;
+  TileRing<float, NSTAGE, RE_NT / 32> ring{reinterpret_cast<float*>(smem_raw), full_bar, empty_bar,
+                                           &s_abort, a.g.err, (uint32_t)(RE_NF * TILE), 0u, 0u};
+  if (tid < ff::SC_TABLE) s_tab[tid] = __ldg(a.sctab + tid);
+  if (tid == 0) {
+    ring.init_barriers();
+    s_abort = 0;
+  }
+  __syncthreads();
+  const PlanHdr plan = *a.g.plan;
+  const ProbDesc& pd = a.g.probs[0];
+  const int n = *a.g.q_cnt;
+  // (items by the counter alone: with the first-item rule of pairsum.cuh the difference sums schedule
+  // worse, 30,000 points over 300 x 257 pixels 11.9 -> 13.1 ms)
+  for (;;) {
+    if (tid == 0) s_item = s_abort ? plan.nitems : atomicAdd(a.g.work, 1);
+    __syncthreads();
+    const int it = s_item;
+    __syncthreads();
+    if (it >= plan.nitems) break;
+    const int blk = it / plan.nsplit, sp = it - blk * plan.nsplit;
+    const int t0 = (int)(((int64_t)sp * pd.ntiles) / plan.nsplit);
+    const int t1 = (int)(((int64_t)(sp + 1) * pd.ntiles) / plan.nsplit);
+    const int64_t j = (int64_t)blk * RE_NT + tid;
+    const bool valid = j < n;
+    const float4 pos = valid ? a.g.qpos[j] : make_float4(0.f, 0.f, 1.f, 0.f);
+    const Lam4 l4 = valid ? a.g.qlam[j] : make_lam4(0.0, 0.0, 0.0);
+    ReQuery q;
+    q.x = pos.x;
+    q.y = pos.y;
+    q.z = pos.z;
+    const double la[3] = {l4.x, l4.y, l4.z};
+    if constexpr (DIF) {
+      const Lam4 r4 = valid ? a.qlam0[j] : l4;
+      const double l0[3] = {r4.x, r4.y, r4.z};
+#pragma unroll
+      for (int i = 0; i < (TIED ? 1 : 3); ++i) set_difference(q, i, la[i], l0[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < (TIED ? 1 : 3); ++i) set_lambda(q, i, la[i]);
+    }
+    ds acc[NSUM];
+#pragma unroll
+    for (int s = 0; s < NSUM; ++s) acc[s] = ds{0.f, 0.f};
+    // (a warp without a query only keeps the ring's protocol)
+    const bool busy = __any_sync(0xffffffffu, valid);
+    if constexpr (DIF) {
+      const float z2 = q.z * q.z;
+      sweep_tiles(ring, pd.tilesff, t0, t1, tid, [&](const float* sx) {
+        if (!busy) return;
+#pragma unroll 1
+        for (int k0 = 0; k0 < TILE; k0 += DIF_BLK) {
+          float bs[12];
+#pragma unroll
+          for (int s = 0; s < 12; ++s) bs[s] = 0.f;
+#pragma unroll 2
+          for (int k = k0; k < k0 + DIF_BLK; ++k)
+            dif_pixel<TIED>(q, z2, [&](int f, int part) { return sx[(2 * f + part) * TILE + k]; }, bs);
+          dif_fold(acc, bs);
+        }
+      });
+    } else {
+      const float lx = fabsf(q.lh[0]);
+      const bool slow = __any_sync(
+          0xffffffffu,
+          valid && beyond_reduction(pd, pos, TIED ? lx : fmaxf(fmaxf(lx, fabsf(q.lh[1])),
+                                                               fabsf(q.lh[2]))));
+      const FfQuery<TIED> fq(q);
+      auto tile = [&](const float* sx, auto any) {
+#pragma unroll 1
+        for (int k = 0; k < TILE; ++k)
+          ff_pixel<VAR, TIED, decltype(any)::value>(
+              fq, s_tab, [&](int f, int part) { return sx[(2 * f + part) * TILE + k]; }, acc);
+      };
+      sweep_tiles(ring, pd.tilesff, t0, t1, tid, [&](const float* sx) {
+        if (!busy) return;
+        if (slow) tile(sx, std::true_type{});
+        else tile(sx, std::false_type{});
+      });
+    }
+    if (valid) {
+#pragma unroll
+      for (int s = 0; s < NSUM; ++s)
+        a.g.out[((int64_t)it * NSUM + s) * RE_NT + tid] = ff::to_double(acc[s]);
+    }
+  }
+  if (tid == 0) ring.drain();
+}
+
+template <int VAR, bool TIED, bool DIF>
+static KernelRef re_points_t() {
+  return KernelRef{(const void*)&re_points_kernel<VAR, TIED, DIF>, RE_NT, RE_NT,
+                   (size_t)NSTAGE * RE_NF * TILE * sizeof(float)};
+}
+
+KernelRef re_points_ref(int var, bool tied, bool dif) {
+  if (dif) return tied ? re_points_t<VAR_OBJ, true, true>() : re_points_t<VAR_OBJ, false, true>();
+  if (var == VAR_V) return tied ? re_points_t<VAR_V, true, false>() : re_points_t<VAR_V, false, false>();
+  return tied ? re_points_t<VAR_OBJ, true, false>() : re_points_t<VAR_OBJ, false, false>();
 }
 
 template <int VAR, bool TIED, bool DIF>

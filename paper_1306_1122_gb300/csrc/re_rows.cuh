@@ -49,59 +49,74 @@ __device__ __forceinline__ float re_load(const float* tile, int f, int part, int
   return __ldg(tile + f * 2 * TILE + part * TILE + e);
 }
 
+// A query's float-float factors.
+template <bool TIED>
+struct FfQuery {
+  static constexpr int NL = TIED ? 1 : 3;
+  ff::ds x, y, z2, lam[NL], lam2[NL];
+  __device__ __forceinline__ explicit FfQuery(const ReQuery& q)
+      : x{q.x, 0.f}, y{q.y, 0.f}, z2(ff::two_prod(q.z, q.z)) {
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      lam[l] = ff::ds{q.lh[l], q.ll[l]};
+      lam2[l] = ff::mul(lam[l], lam[l]);
+    }
+  }
+};
+
+// Adds one pixel's float-float terms; ld(f, part): the pixel's field f, part 0 (hi) or 1 (lo).
+template <int VAR, bool TIED, bool ANY, typename Load>
+__device__ __forceinline__ void ff_pixel(const FfQuery<TIED>& q, const float4* tab, Load ld,
+                                         ff::ds (&acc)[3 * nsum_per_comp(VAR)]) {
+  using D = ff::ds;
+  constexpr int NS = nsum_per_comp(VAR);
+  constexpr int NL = FfQuery<TIED>::NL;
+  const D X = D{ld(0, 0), ld(0, 1)};
+  const D Y = D{ld(1, 0), ld(1, 1)};
+  const D dx = ff::sub(q.x, X);
+  const D dy = ff::sub(q.y, Y);
+  // (products that feed a further float-float operation stay unnormalised: mul_nr)
+  const D r2 = ff::add(ff::add(ff::mul_nr(dx, dx), ff::mul_nr(dy, dy)), q.z2);
+  D r, ri;
+  ff::sqrt_rsqrt(r2, r, ri);
+  const D ri2 = ff::mul_nr(ri, ri);
+  const D ri3 = ff::mul_nr(ri2, ri);
+  D u[NL], c[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const D th = ff::mul_nr(q.lam[l], r);
+    D s;
+    if constexpr (ANY) ff::sincos_ds_any(th, tab, s, c[l]);
+    else ff::sincos_ds<float>(th, tab, s, c[l]);
+    u[l] = ff::add(ff::mul_nr(th, s), c[l]);
+  }
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const int lp = TIED ? 0 : p;
+    const D rb = ff::mul_nr(ri3, D{ld(2 + p, 0), ld(2 + p, 1)});
+    ff::acc_add(acc[p * NS], ff::mul_nr(u[lp], rb));
+    if constexpr (has_grad(VAR)) {
+      // psi b = (lambda^2 cos(lambda r) - 3 u / r^2) b / r^3
+      const D w = ff::sub(ff::mul_nr(q.lam2[lp], c[lp]),
+                          ff::mul_f_nr(ff::mul_nr(u[lp], ri2), 3.0f));
+      const D t1 = ff::mul_nr(w, rb);
+      ff::acc_add(acc[p * NS + 1], t1);
+      ff::acc_add(acc[p * NS + 2], ff::mul_nr(t1, dx));
+      ff::acc_add(acc[p * NS + 3], ff::mul_nr(t1, dy));
+    }
+  }
+}
+
 // Float-float sums of pixel t of each row of ROW pixels in [r0, r1).
 template <int VAR, bool TIED, bool ANY, int ROW>
 __device__ __forceinline__ void ff_rows(const float* tiles, int r0, int r1, int t, const ReQuery& q,
                                         const float4* tab, ff::ds (&acc)[3 * nsum_per_comp(VAR)]) {
-  using D = ff::ds;
-  constexpr int NS = nsum_per_comp(VAR);
-  constexpr int NL = TIED ? 1 : 3;
-  const D xq = D{q.x, 0.f}, yq = D{q.y, 0.f};
-  const D z2 = ff::two_prod(q.z, q.z);
-  D lam[NL], lam2[NL];
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    lam[l] = D{q.lh[l], q.ll[l]};
-    lam2[l] = ff::mul(lam[l], lam[l]);
-  }
+  const FfQuery<TIED> fq(q);
 #pragma unroll 1
   for (int row = r0; row < r1; ++row) {
     const float* T = tiles + (int64_t)(row / (TILE / ROW)) * (RE_NF * TILE);
     const int e = (row % (TILE / ROW)) * ROW + t;
-    const D X = D{re_load(T, 0, 0, e), re_load(T, 0, 1, e)};
-    const D Y = D{re_load(T, 1, 0, e), re_load(T, 1, 1, e)};
-    const D dx = ff::sub(xq, X);
-    const D dy = ff::sub(yq, Y);
-    // (products that feed a further float-float operation stay unnormalised: mul_nr)
-    const D r2 = ff::add(ff::add(ff::mul_nr(dx, dx), ff::mul_nr(dy, dy)), z2);
-    D r, ri;
-    ff::sqrt_rsqrt(r2, r, ri);
-    const D ri2 = ff::mul_nr(ri, ri);
-    const D ri3 = ff::mul_nr(ri2, ri);
-    D u[NL], c[NL];
-#pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      const D th = ff::mul_nr(lam[l], r);
-      D s;
-      if constexpr (ANY) ff::sincos_ds_any(th, tab, s, c[l]);
-      else ff::sincos_ds<float>(th, tab, s, c[l]);
-      u[l] = ff::add(ff::mul_nr(th, s), c[l]);
-    }
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-      const int lp = TIED ? 0 : p;
-      const D rb = ff::mul_nr(ri3, D{re_load(T, 2 + p, 0, e), re_load(T, 2 + p, 1, e)});
-      ff::acc_add(acc[p * NS], ff::mul_nr(u[lp], rb));
-      if constexpr (has_grad(VAR)) {
-        // psi b = (lambda^2 cos(lambda r) - 3 u / r^2) b / r^3
-        const D w = ff::sub(ff::mul_nr(lam2[lp], c[lp]),
-                            ff::mul_f_nr(ff::mul_nr(u[lp], ri2), 3.0f));
-        const D t1 = ff::mul_nr(w, rb);
-        ff::acc_add(acc[p * NS + 1], t1);
-        ff::acc_add(acc[p * NS + 2], ff::mul_nr(t1, dx));
-        ff::acc_add(acc[p * NS + 3], ff::mul_nr(t1, dy));
-      }
-    }
+    ff_pixel<VAR, TIED, ANY>(fq, tab, [&](int f, int part) { return re_load(T, f, part, e); }, acc);
   }
 }
 
@@ -120,11 +135,51 @@ __device__ __forceinline__ void sincos_delta(float d, float& s, float& c) {
   }
 }
 
+// Adds one pixel's difference terms to the FP32 block sums bs (ld as above; z2 = z^2).
+template <bool TIED, typename Load>
+__device__ __forceinline__ void dif_pixel(const ReQuery& q, float z2, Load ld, float (&bs)[12]) {
+  constexpr int NL = TIED ? 1 : 3;
+  const float dx = (q.x - ld(0, 0)) - ld(0, 1);
+  const float dy = (q.y - ld(1, 0)) - ld(1, 1);
+  const float r2 = fmaf(dx, dx, fmaf(dy, dy, z2));
+  const float ri = rsqrt_mufu(r2);
+  const float r = r2 * ri;
+  const float ri2 = ri * ri;
+  const float ri3 = ri2 * ri;
+  float du[NL], dw[NL];
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    const float sg = q.hs[l] * r, dl = q.hd[l] * r;
+    const float ss = sin_mufu(sg), cs = cos_mufu(sg);
+    float sd, cd;
+    sincos_delta(dl, sd, cd);
+    const float cs_sd = cs * sd, ss_sd = ss * sd;
+    du[l] = 2.0f * (fmaf(dl, ss * cd, sg * cs_sd) - ss_sd);
+    dw[l] = fmaf(q.pq[l], cs * cd, fmaf(-q.qq[l], ss_sd, -3.0f * du[l] * ri2));
+  }
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const int lp = TIED ? 0 : p;
+    const float rb = ri3 * ld(2 + p, 0);
+    const float t1 = dw[lp] * rb;
+    bs[4 * p + 0] = fmaf(du[lp], rb, bs[4 * p + 0]);
+    bs[4 * p + 1] += t1;
+    bs[4 * p + 2] = fmaf(t1, dx, bs[4 * p + 2]);
+    bs[4 * p + 3] = fmaf(t1, dy, bs[4 * p + 3]);
+  }
+}
+__device__ __forceinline__ void dif_fold(ff::ds (&acc)[12], const float (&bs)[12]) {
+#pragma unroll
+  for (int s = 0; s < 12; ++s) {
+    const ff::ds f = ff::two_sum(acc[s].hi, bs[s]);
+    acc[s] = ff::ds{f.hi, __fadd_rn(acc[s].lo, f.lo)};
+  }
+}
+
 // Difference sums: FP32 over blocks of DIF_BLK pixels of a thread, the block sums in float-float.
 template <bool TIED, int ROW>
 __device__ __forceinline__ void dif_rows(const float* tiles, int r0, int r1, int t, const ReQuery& q,
                                          ff::ds (&acc)[12]) {
-  constexpr int NL = TIED ? 1 : 3;
   const float z2 = q.z * q.z;
 #pragma unroll 1
   for (int b0 = r0; b0 < r1; b0 += DIF_BLK) {
@@ -136,40 +191,9 @@ __device__ __forceinline__ void dif_rows(const float* tiles, int r0, int r1, int
     for (int row = b0; row < b1; ++row) {
       const float* T = tiles + (int64_t)(row / (TILE / ROW)) * (RE_NF * TILE);
       const int e = (row % (TILE / ROW)) * ROW + t;
-      const float dx = (q.x - re_load(T, 0, 0, e)) - re_load(T, 0, 1, e);
-      const float dy = (q.y - re_load(T, 1, 0, e)) - re_load(T, 1, 1, e);
-      const float r2 = fmaf(dx, dx, fmaf(dy, dy, z2));
-      const float ri = rsqrt_mufu(r2);
-      const float r = r2 * ri;
-      const float ri2 = ri * ri;
-      const float ri3 = ri2 * ri;
-      float du[NL], dw[NL];
-#pragma unroll
-      for (int l = 0; l < NL; ++l) {
-        const float sg = q.hs[l] * r, dl = q.hd[l] * r;
-        const float ss = sin_mufu(sg), cs = cos_mufu(sg);
-        float sd, cd;
-        sincos_delta(dl, sd, cd);
-        const float cs_sd = cs * sd, ss_sd = ss * sd;
-        du[l] = 2.0f * (fmaf(dl, ss * cd, sg * cs_sd) - ss_sd);
-        dw[l] = fmaf(q.pq[l], cs * cd, fmaf(-q.qq[l], ss_sd, -3.0f * du[l] * ri2));
-      }
-#pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        const int lp = TIED ? 0 : p;
-        const float rb = ri3 * re_load(T, 2 + p, 0, e);
-        const float t1 = dw[lp] * rb;
-        bs[4 * p + 0] = fmaf(du[lp], rb, bs[4 * p + 0]);
-        bs[4 * p + 1] += t1;
-        bs[4 * p + 2] = fmaf(t1, dx, bs[4 * p + 2]);
-        bs[4 * p + 3] = fmaf(t1, dy, bs[4 * p + 3]);
-      }
+      dif_pixel<TIED>(q, z2, [&](int f, int part) { return re_load(T, f, part, e); }, bs);
     }
-#pragma unroll
-    for (int s = 0; s < 12; ++s) {
-      const ff::ds f = ff::two_sum(acc[s].hi, bs[s]);
-      acc[s] = ff::ds{f.hi, __fadd_rn(acc[s].lo, f.lo)};
-    }
+    dif_fold(acc, bs);
   }
 }
 

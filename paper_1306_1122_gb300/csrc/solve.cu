@@ -286,6 +286,7 @@ void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* ms
 
 // Difference sums of n queries of one problem (slots 0..n-1) and their bounds (debug entry).
 __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
+                                 const int32_t* __restrict__ item_off,
                                  const double* __restrict__ out, const Lam4* __restrict__ qlam,
                                  const Lam4* __restrict__ qlam0, const double* __restrict__ msc,
                                  const double* __restrict__ msc0, int dim, double* dS,
@@ -293,7 +294,7 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   const PlanHdr h = *plan;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    gather_sums<12>(out, h, nullptr, 0, i, dS + 12 * i);
+    gather_sums<12>(out, h, item_off, 0, i, dS + 12 * i);
     if (dS_bound) {
       const double la[3] = {qlam[i].x, qlam[i].y, qlam[i].z};
       const double l0[3] = {qlam0[i].x, qlam0[i].y, qlam0[i].z};
@@ -309,13 +310,13 @@ __global__ void dif_debug_kernel(int64_t n, const PlanHdr* __restrict__ plan,
   }
 }
 
-void launch_dif_debug(int64_t n, const PlanHdr* plan, const double* out, const Lam4* qlam,
-                      const Lam4* qlam0, const double* msc, const double* msc0,
+void launch_dif_debug(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
+                      const Lam4* qlam, const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s) {
   const int64_t nb = (n + 127) / 128;
   if (n > 0)
     dif_debug_kernel<<<(int)(nb < 1024 ? nb : 1024), 128, 0, s>>>(
-        n, plan, out, qlam, qlam0, msc, msc0, dim, dS, dS_bound);
+        n, plan, item_off, out, qlam, qlam0, msc, msc0, dim, dS, dS_bound);
 }
 
 // ------------------------------------------------------------------ certified B ----
