@@ -1047,7 +1047,8 @@ dbie_status dbie_eval_difference(dbie_ctx* c, int64_t n, const float* xyz,
   if (dS_bound) {
     DBIE_TRY(ensure(c->dmsc, sizeof(double) * 18 * n));
     msc = c->dmsc.as<double>();
-    launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n, c->sm_count, s);
+    launch_msc(c->prob.as<ProbDesc>(), n, c->qpos.as<float4>(), msc, msc + 15 * n, c->ntiles,
+               c->sm_count, s);
   }
   launch_dif_debug(n, &m->plan, m->item_off, c->out.as<double>(), c->qlam.as<Lam4>(),
                    c->qlam0.as<Lam4>(), msc, msc ? msc + 15 * n : nullptr, tied ? 1 : 3, dS,
@@ -1658,7 +1659,7 @@ static dbie_status solve_impl(int32_t nprob, dbie_ctx* const* ctxs, const int64_
   if (cert) {
     // the error bounds' lambda-independent absolute-value sums of every point
     launch_msc(b.probs.as<ProbDesc>(), N, b.ppos.as<float4>(), b.msc.as<float>(),
-               b.msc.as<float>() + 15 * N, c->sm_count, s);
+               b.msc.as<float>() + 15 * N, max_rows / RE_ROWS_PER_TILE, c->sm_count, s);
     CUDA_TRY(cudaGetLastError());
   }
   if (codes_stride) CUDA_TRY(cudaMemsetAsync(b.codes.p, 0, (size_t)codes_stride * N, s));

@@ -261,9 +261,9 @@ void launch_plan_round(const PlanArgs& a, cudaStream_t s);
 void launch_nm_step(const SolveArgs& a, int grid, cudaStream_t s);
 void launch_nm_refine(const SolveArgs& a, int grid, cudaStream_t s);
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, float* msc, float* msc0,
-                int sm_count, cudaStream_t s);
+                int ntiles, int sm_count, cudaStream_t s);
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
-                int sm_count, cudaStream_t s);
+                int ntiles, int sm_count, cudaStream_t s);
 void launch_dif_debug(int64_t n, const PlanHdr* plan, const int32_t* item_off, const double* out,
                       const Lam4* qlam, const Lam4* qlam0, const double* msc, const double* msc0,
                       int dim, double* dS, double* dS_bound, cudaStream_t s);

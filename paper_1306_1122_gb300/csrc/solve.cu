@@ -269,19 +269,75 @@ __global__ void __launch_bounds__(MSC_NT) msc_kernel(const ProbDesc* __restrict_
   }
 }
 
+// The same by a thread per point, for many points over few pixels, where the combination of a CTA's
+// sums outweighs the terms.  Measured (us, CTA / thread per point): 12,000 points over 16 x 16 pixels
+// 40 / 23, 400,000 1,330 / 250; 25,000 over 32 x 32 118 / 112; 50,000 over 64 x 48 (12 tiles) 339 / 343,
+// 100,000 672 / 502; 100,000 over 128 x 64 (32 tiles) 1,242 / 1,274, 200,000 2,471 / 2,243.
+template <typename T>
+__global__ void __launch_bounds__(MSC_NT) msc_points_kernel(const ProbDesc* __restrict__ probs,
+                                                            int64_t N,
+                                                            const float4* __restrict__ ppos,
+                                                            T* __restrict__ msc,
+                                                            T* __restrict__ msc0) {
+  for (int64_t g = blockIdx.x * (int64_t)MSC_NT + threadIdx.x; g < N;
+       g += (int64_t)gridDim.x * MSC_NT) {
+    const float4 pos = ppos[g];
+    const ProbDesc& pd = probs[__float_as_int(pos.w)];
+    const float z2 = __fmul_rn(pos.z, pos.z);
+    ff::ds tot[18];
+#pragma unroll
+    for (int i = 0; i < 18; ++i) tot[i] = ff::ds{0.f, 0.f};
+    for (int t = 0; t < pd.ntiles; ++t) {
+      const float* T32 = pd.tiles32 + (int64_t)t * pd.nf32 * TILE;
+      float acc[18];
+#pragma unroll
+      for (int i = 0; i < 18; ++i) acc[i] = 0.f;
+      for (int e = 0; e < TILE; ++e) {
+        const float dx = pos.x - __ldg(T32 + e), dy = pos.y - __ldg(T32 + TILE + e);
+        const float ri = rsqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, z2)));
+        float wj = 1.f;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {   // acc[3 j + p]: M_j of component p
+#pragma unroll
+          for (int p = 0; p < 3; ++p)
+            acc[3 * j + p] = __fmaf_rn(fabsf(__ldg(T32 + (2 + p) * TILE + e)), wj, acc[3 * j + p]);
+          wj *= ri;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 18; ++i) ff::acc_add(tot[i], ff::ds{acc[i], 0.f});
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j)
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const T v = (T)ff::to_double(tot[3 * j + p]);
+        if (j > 0) msc[15 * g + 5 * p + j - 1] = v;
+        else msc0[3 * g + p] = v;
+      }
+  }
+}
+
+// ntiles: of the largest problem.
 template <typename T>
 static void launch_msc_t(const ProbDesc* probs, int64_t N, const float4* ppos, T* msc, T* msc0,
-                         int sm_count, cudaStream_t s) {
+                         int ntiles, int sm_count, cudaStream_t s) {
+  if (N <= 0) return;
+  if (N >= 6000LL * ntiles) {
+    const int64_t nb = (N + MSC_NT - 1) / MSC_NT, most = 32LL * sm_count;
+    msc_points_kernel<T><<<(int)(nb < most ? nb : most), MSC_NT, 0, s>>>(probs, N, ppos, msc, msc0);
+    return;
+  }
   const int64_t most = 16LL * sm_count;
-  if (N > 0) msc_kernel<T><<<(int)(N < most ? N : most), MSC_NT, 0, s>>>(probs, N, ppos, msc, msc0);
+  msc_kernel<T><<<(int)(N < most ? N : most), MSC_NT, 0, s>>>(probs, N, ppos, msc, msc0);
 }
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, float* msc, float* msc0,
-                int sm_count, cudaStream_t s) {
-  launch_msc_t(probs, N, ppos, msc, msc0, sm_count, s);
+                int ntiles, int sm_count, cudaStream_t s) {
+  launch_msc_t(probs, N, ppos, msc, msc0, ntiles, sm_count, s);
 }
 void launch_msc(const ProbDesc* probs, int64_t N, const float4* ppos, double* msc, double* msc0,
-                int sm_count, cudaStream_t s) {
-  launch_msc_t(probs, N, ppos, msc, msc0, sm_count, s);
+                int ntiles, int sm_count, cudaStream_t s) {
+  launch_msc_t(probs, N, ppos, msc, msc0, ntiles, sm_count, s);
 }
 
 // Difference sums of n queries of one problem (slots 0..n-1) and their bounds (debug entry).
