@@ -17,7 +17,7 @@ LIB = os.path.join(PKG, "libdbie.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-diag-suppress", "1444",
           f"-I{INCLUDE}", f"-I{CSRC}"]
-# Translation units; the lambda-search file is compiled without FMA contraction so the simplex
+# Translation units; the lambda-search files are compiled without FMA contraction so the simplex
 # arithmetic rounds each operation as written.
 UNITS = {
     "capi.cu": [],

@@ -178,7 +178,9 @@ struct dbie_ctx {
   // Launch configuration per variant / tied until dbie_autotune picks one: uncapped, but the
   // objective variants at six CTAs of 128 threads per SM (80 registers), which keep the SFU busier.
   // (B, gradient, f and g at 20,000 points over 300 x 300 pixels 3.51 -> 3.16 ms, with dB/dlambda
-  // 3.67 -> 3.40; ten search iterations of 131,072 points over 128 x 128 94 -> 87 ms.)
+  // 3.67 -> 3.40; ten search iterations of 131,072 points over 128 x 128 94 -> 87 ms.)  With one tied
+  // lambda, three SFU results per pair, registers count for more and uncapped stays ahead (the same
+  // search 71.0 ms against 71.2, 20,000 points there 14.8 / 15.6, over 300 x 300 64.0 / 65.2).
   int cfg[NVAR][2] = {{0, 0}, {0, 0}, {3, 0}, {3, 0}, {0, 0}, {0, 0}, {0, 0}};
   int vjp_cfg = 0;
   cudaStream_t cap_stream = nullptr;  // streams and events used only to capture graphs

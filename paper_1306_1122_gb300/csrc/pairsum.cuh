@@ -15,7 +15,8 @@
 //  * Staging: one elected thread moves each tile with one cp.async.bulk (TMA bulk copy, no
 //    multicast) into an NSTAGE-deep ring of shared-memory buffers guarded by mbarriers (full:
 //    transaction bytes; empty: one arrival per warp).  Every wait is bounded in time.
-//  * Arithmetic (mixed form): FP32 pair terms (rsqrt, sin, cos on the SFU), plain FP32 sums
+//  * Arithmetic (mixed form): FP32 pair terms (rsqrt, sin, cos on the SFU, in the field sums and the
+//    adjoint one component's sin and cos on the FMA pipe: fma_sincos), plain FP32 sums
 //    over SUB elements, folded by an error-free two-sum (its error carried into the next
 //    block) and converted to FP64 at the end of the item.  FP64 form: the same sweep in double precision.
 #pragma once
@@ -39,8 +40,9 @@ namespace dbie {
 #define DBIE_PACKED 1     // FP32 pair sums on pixel pairs packed in f32x2 (0: one pixel per op)
 #endif
 constexpr int SUB = DBIE_FOLD_PIXELS;  // pixels summed in plain FP32 before a compensated fold
-constexpr int SUB1 = 32;  // elements per fold where one accumulator takes every element (adjoints,
-                          // the unpacked FP32 form): the per-accumulator length of the packed form
+constexpr int SUB1 = 32;  // elements per fold where one accumulator takes every element (the
+                          // seven-weight adjoint, the unpacked FP32 form): the per-accumulator
+                          // length of the packed form
 constexpr int GROUP_UNROLL = DBIE_GROUP_UNROLL;  // 4-pixel groups unrolled within a block
 constexpr int VJP_GROUPS = 8;                    // the same in the adjoint (4 points)
 static_assert(TILE % SUB == 0 && SUB % 4 == 0, "fold blocks must tile the 256-pixel tile");

@@ -28,7 +28,8 @@
 // cannot certify; dbie_eval offers the float-float sums as DBIE_PREC_FLOAT_FLOAT and
 // dbie_eval_difference the difference sums.
 //
-// Work distribution.  Both are bound by FP32 issue (824 and 153 instructions per pair), and their
+// Work distribution.  Both are bound by FP32 issue (838 and 183 instructions per pair, with the
+// combination of the threads' sums), and their
 // queries are few and scattered: a search round queues tens to thousands of them, over all
 // problems.  So the lanes of a CTA take pixels, not queries: an item is one query and a range of
 // rows of 128 pixels, one pixel per thread, and no lane idles whatever the number of queries

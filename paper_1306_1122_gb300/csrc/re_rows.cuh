@@ -21,8 +21,9 @@ struct ReQuery {
 // Whether lambda r may leave the range of sincos_ds for some pixel: |lambda| times the largest
 // distance to the quadrature grid's box (pixel centres, or Gauss points of elements two node
 // spacings wide, all inside [x0 - |hx|, x0 + 2 nx |hx|] with nx quadrature points per row); such a
-// query (rare: a far-out trial lambda, or not finite) takes the path with the FP64 fallback, so
-// the common path stays branch-free.
+// query (rare: a far-out or infinite trial lambda) takes the path with the FP64 fallback, so the
+// common path stays branch-free.  (A NaN lambda gives NaN on either path and reads no table entry
+// past the last.)
 __device__ __forceinline__ bool beyond_reduction(const ProbDesc& pd, float4 pos, float lmax) {
   const float x0 = (float)pd.x0, y0 = (float)pd.y0;
   const float ax = (float)fabs(pd.hx), ay = (float)fabs(pd.hy);

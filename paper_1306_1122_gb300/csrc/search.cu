@@ -111,8 +111,7 @@ __device__ __noinline__ long long rs_reeval(RsShared& S, const SolveArgs& a, int
     for (int i = 0; i < NL; ++i) {
       q.lh[i] = __shfl_sync(0xffffffffu, m.lh[0], i);
       q.ll[i] = __shfl_sync(0xffffffffu, m.ll[0], i);
-      const float al = fabsf(q.lh[i]);
-      lmax = al <= lmax ? lmax : al;   // (NaN is kept)
+      lmax = fmaxf(lmax, fabsf(q.lh[i]));   // (of NaN the others: its sums are NaN on either path)
       if constexpr (DIF) {
         q.hs[i] = __shfl_sync(0xffffffffu, m.hs[0], i);
         q.hd[i] = __shfl_sync(0xffffffffu, m.hd[0], i);

@@ -7,9 +7,11 @@
 //    (the fixed-lambda derivatives of Eq. 13), J = curl B (Eq. 14), f = |J x B| / (|J||B|)
 //    (Eq. 8), g = |div B| dV/dSigma / |B| (Eq. 9), Phi = f + w_g g.
 //  * simplex (Sect. 2.1; Nelder & Mead 1965, reflection 1, expansion 2, contraction 1/2,
-//    shrink 1/2, outside/inside contraction as in Lagarias et al. 1998): one thread per active
-//    point advances a state machine by one step per round; every round evaluates all pending
-//    trial points of all active points in one pair-sum pass.
+//    shrink 1/2, outside/inside contraction as in Lagarias et al. 1998): every active point is a
+//    state machine that advances by one step per round, the lanes of its warp sharing out the
+//    values and trial points of all its points (solve_step.cuh); every round evaluates all pending
+//    trial points of all active points in one pair-sum pass.  Few points on few pixels run all of
+//    it in one kernel (search.cu).
 #include "kernels.h"
 #include "solve_step.cuh"
 #include "warp_sums.cuh"
