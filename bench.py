@@ -647,6 +647,7 @@ def batch64_block(dev, sub_per_problem=128):
         sub_t[name] = (time.perf_counter() - t0, r)
     errs = [b_error_stats(f, w.mag, w.points[i], o["lam"].cpu().numpy()[i], dev)
             for f, w, i, o in zip(fields[:8], probs[:8], sub, outs[:8])]
+    obj_cfg = dbie._native.dbie_get_config(fields[0].handle)[4]   # the untied objective's
     for f in fields:
         f.close()
     n_sub = int(sum(len(i) for i in sub))
@@ -657,7 +658,7 @@ def batch64_block(dev, sub_per_problem=128):
             "roofline": {"bound": "alu", "kernel": "g1_kernel objective (batched)",
                          "achieved": mufu, "peak": peak, "unit": "T MUFU-op/s",
                          "frac": mufu / peak if mufu else None,
-                         "kernel_s": st["objective_ms"] / 1e3},
+                         "kernel_s": st["objective_ms"] / 1e3, "launch_config": obj_cfg},
             "iters_hist": hist.tolist(), "iters_mean": float(iters.mean()),
             "subsample": {"points": n_sub, "per_problem": sub_per_problem,
                           "mixed_s": sub_t["mixed"][0], "fp64_s": sub_t["fp64"][0],
