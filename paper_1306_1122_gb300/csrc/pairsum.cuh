@@ -682,7 +682,7 @@ __device__ __forceinline__ void vjp_body(const VjpArgs& a) {
                 const f32x2 th = vmul(pack2(l2[4 * p], l2[4 * p + 1]), r);
                 if (FMA_SC >> p & 1) {
                   f32x2 k;
-                  const f32x2 f = half_turns(th, k), f2 = vmul(f, f);
+                  const f32x2 f = half_turns(th, k), f2 = vsqr_sat(f);
                   phi = vmul(vfma(th, sin_half_turns(f, f2), cos_half_turns(f2)), vflip(ri3, k));
                 } else {
                   phi = vmul(vfma(th, vsin(th), vcos(th)), ri3);

@@ -68,7 +68,9 @@ __global__ void finalize_eval_kernel(int64_t n, const PlanHdr* __restrict__ plan
       const Lam4 l = qlam[i];
       const double lam[3] = {l.x, l.y, l.z};
       for (int p = 0; p < 3; ++p) {
-        const double d = z * lam[p] * S[p * NS + idx_sl(VAR)];
+        double d = z * lam[p] * S[p * NS + idx_sl(VAR)];
+        // an angle without a cosine: see half_turns
+        if (isinf(lam[p]) || (has_value(VAR) && isnan(S[p * NS]))) d = __longlong_as_double(0x7ff8000000000000LL);
         if (gB) {
           if (dBdl) dBdl[3 * i + p] = gB[3 * i + p] * d;
         } else if (dBdl) {
