@@ -324,7 +324,8 @@ dbie_status dbie_get_stats(dbie_ctx* ctx, dbie_stats* stats, int32_t reset);
 
 /* Pick launch parameters (CTA size, points per thread) for this device by timing candidates on
  * the context's boundary; results are cached per (device, variant, boundary size class) in
- * memory and in the file named by $DBIE_TUNE_CACHE when set.  Synchronises `stream`. */
+ * memory and in the file named by $DBIE_TUNE_CACHE when set.  Contexts on nine-node elements, whose
+ * kernels have one launch shape each, keep their parameters.  Synchronises `stream`. */
 dbie_status dbie_autotune(dbie_ctx* ctx, void* stream);
 
 /* Launch configuration indices in use (after dbie_autotune): cfg_out[2 * variant + tied] for the
